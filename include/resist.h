@@ -163,8 +163,8 @@ typedef struct {
 int resist_get_step_info(resist_ctx* ctx, resist_step_info* out);
 
 /* ---- Layer-level entry points: one layer on caller-owned device tensors, run by the kernels of the local step.
- * They allocate their own scratch with cudaMalloc, synchronise the stream before returning, and report
- * failures through resist_layer_last_error().  dtype: RESIST_F32 or RESIST_BF16 for activations and weights.
+ * They take their scratch from a bounded pool of cudaMalloc'ed blocks (resist_layer_release_scratch() frees the idle ones),
+ * synchronise the stream before returning, and report failures through resist_layer_last_error().  dtype: RESIST_F32 or RESIST_BF16 for activations and weights.
  *
  * resist_conv2d: a k x k convolution with zero padding (k-1)/2 and stride 1 or 2, the building block of the
  * residual blocks of Sec. 2.1.  Geometry is always that of the forward convolution: a [N,H,W,C], w [K,k,k,C],
@@ -202,6 +202,9 @@ int resist_conv2d_bn_relu(int32_t mode, int32_t backend, const void* act, const 
                           const void* bn_add, void* bn_out, float* dgamma, float* dbeta, float eps, float momentum,
                           int32_t* used_backend, resist_stream stream);
 const char* resist_layer_last_error(void);
+/* Frees the idle scratch blocks of the layer-level calls (at most 256 MiB in 16 blocks over all devices are kept between calls).
+ * Safe from any thread; blocks in use by other threads' calls are not touched. */
+int resist_layer_release_scratch(void);
 
 /* resist_bn_relu_forward for callers that cannot allocate device memory (the paper has no counterpart: this is a
  * property of the library, not of the method).  Who needs it: code running inside a fixed memory pool, loops

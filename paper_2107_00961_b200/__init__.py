@@ -108,7 +108,7 @@ def lib():
 EXPORTS = ["resist_init", "resist_destroy", "resist_partition", "resist_local_step", "resist_local_step_grouped",
            "resist_aggregate", "resist_eval", "resist_param_count", "resist_get_params", "resist_set_params",
            "resist_get_grads", "resist_get_logits", "resist_get_shadow", "resist_debug_set_wait_status", "resist_micro_mma_rate", "resist_get_step_info", "resist_splitmix64", "resist_last_error",
-           "resist_set_profiling", "resist_get_profile", "resist_conv2d", "resist_conv2d_bn_relu", "resist_bn_relu_forward", "resist_bn_relu_backward", "resist_layer_last_error",
+           "resist_set_profiling", "resist_get_profile", "resist_conv2d", "resist_conv2d_bn_relu", "resist_bn_relu_forward", "resist_bn_relu_backward", "resist_layer_last_error", "resist_layer_release_scratch",
            "resist_bn_relu_forward_noalloc", "resist_noalloc_last_error"]
 
 

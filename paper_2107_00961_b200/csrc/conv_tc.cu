@@ -58,6 +58,8 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     }
     return false;
 }
+// a plain store: the word lies in host memory (only ever written on the way out of a wait that gave up)
+__device__ __forceinline__ void report_wait(int* status, int code) { *(volatile int*)status = code; __threadfence_system(); }
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const void* tmap, uint32_t bar, int c0, int c1) {
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
                  ::"r"(dst), "l"(tmap), "r"(bar), "r"(c0), "r"(c1) : "memory");
@@ -238,7 +240,7 @@ __global__ void __launch_bounds__(TC_CONV_THREADS, 1) conv_tc_kernel(const TcPro
                 for (int sl = 0; sl < slabs && ok; ++sl) {
                     for (int g = 0; g < ngroups && ok; ++g) {
                         for (int j = 0; j < nt; ++j) {
-                            if (!mbar_wait(a_empty + 8 * sa, pha ^ 1u, &abort_s)) { atomicExch(&abort_s, 1); atomicExch(h.status, 1); ok = false; break; }
+                            if (!mbar_wait(a_empty + 8 * sa, pha ^ 1u, &abort_s)) { atomicExch(&abort_s, 1); report_wait(h.status, 1); ok = false; break; }
                             const int tm = tm0 + j;
                             const uint32_t dst = a_ring + (uint32_t)(sa * L.a_stage);
                             mbar_expect_tx(a_full + 8 * sa, (uint32_t)(nbox * a_box_bytes));
@@ -255,7 +257,7 @@ __global__ void __launch_bounds__(TC_CONV_THREADS, 1) conv_tc_kernel(const TcPro
                         if (!ok) break;
                         const int t_end = h.gbeg[g + 1];
                         for (int tap = h.gbeg[g]; tap < t_end; ++tap) {
-                            if (!mbar_wait(b_empty + 8 * sb_, phb ^ 1u, &abort_s)) { atomicExch(&abort_s, 1); atomicExch(h.status, 2); ok = false; break; }
+                            if (!mbar_wait(b_empty + 8 * sb_, phb ^ 1u, &abort_s)) { atomicExch(&abort_s, 1); report_wait(h.status, 2); ok = false; break; }
                             const uint32_t dst = b_ring + (uint32_t)(sb_ * L.b_stage);
                             const int wtap = h.wtap[tap];
                             mbar_expect_tx(b_full + 8 * sb_, (uint32_t)b_bytes);
@@ -298,7 +300,7 @@ __global__ void __launch_bounds__(TC_CONV_THREADS, 1) conv_tc_kernel(const TcPro
                 const uint32_t buf = (cnt % (uint32_t)L.nbuf) * 2u + (uint32_t)me, aph = (cnt / (uint32_t)L.nbuf) & 1u;
                 if (has) {
                     ++cnt;
-                    if (!mbar_wait(acc_empty + 8 * buf, aph ^ 1u, &abort_s)) { atomicExch(&abort_s, 1); atomicExch(h.status, 3); ok = false; break; }
+                    if (!mbar_wait(acc_empty + 8 * buf, aph ^ 1u, &abort_s)) { atomicExch(&abort_s, 1); report_wait(h.status, 3); ok = false; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 }
                 const uint32_t d_tmem = tmem_base + buf * (uint32_t)L.acc_stride;
@@ -314,13 +316,13 @@ __global__ void __launch_bounds__(TC_CONV_THREADS, 1) conv_tc_kernel(const TcPro
                         const uint32_t ai = a_cnt + (uint32_t)me; a_cnt += (uint32_t)nt;
                         const uint32_t sa = ai % (uint32_t)L.na, pha = (ai / (uint32_t)L.na) & 1u;
                         if (has) {
-                            if (!mbar_wait(a_full + 8 * sa, pha, &abort_s)) { atomicExch(&abort_s, 1); atomicExch(h.status, 4); ok = false; break; }
+                            if (!mbar_wait(a_full + 8 * sa, pha, &abort_s)) { atomicExch(&abort_s, 1); report_wait(h.status, 4); ok = false; break; }
                             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                         }
                         const uint32_t a_rows16 = ((a_ring + sa * (uint32_t)L.a_stage) >> 4) + (uint32_t)a_off * 8u;   // start address in 16-byte units
                         const int t_end = h.gbeg[g + 1];
                         for (int tap = h.gbeg[g]; tap < t_end; ++tap) {
-                            if (!mbar_wait(b_full + 8 * sb, phb, &abort_s)) { atomicExch(&abort_s, 1); atomicExch(h.status, 5); ok = false; break; }
+                            if (!mbar_wait(b_full + 8 * sb, phb, &abort_s)) { atomicExch(&abort_s, 1); report_wait(h.status, 5); ok = false; break; }
                             if (has) {
                                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                                 const uint32_t a16 = a_rows16 + (uint32_t)h.shift[tap] * 8u;
@@ -410,7 +412,7 @@ __global__ void __launch_bounds__(TC_CONV_THREADS, 1) conv_tc_kernel(const TcPro
             }
             ok = mbar_wait(acc_full + 8 * buf, aph, &abort_s);
             ok = bar_and_epi(bid, ok);                           // one decision for the four warps: they share the barriers below
-            if (!ok) { atomicExch(&abort_s, 1); atomicExch(h.status, 6); break; }
+            if (!ok) { atomicExch(&abort_s, 1); report_wait(h.status, 6); break; }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t t_row = tmem_base + buf * (uint32_t)L.acc_stride + ((uint32_t)(quad * 32) << 16);
             // The tile leaves in slabs of 64 columns: a slab is rounded and (with the residual added) written to a 16 KB staging
@@ -618,7 +620,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) conv_wgrad_tc_kernel(const TcWg
             int i = 0; bool ok = true; int s = 0; uint32_t ph = 0;
             const uint32_t tx = (uint32_t)(2 * nbox_dy * dy_box_bytes + a_slabs * nbox_a * a_box_bytes);
             for (; i < nc; ++i) {
-                if (!mbar_wait(bar_empty + 8 * s, ph ^ 1u, &abort_s)) { atomicExch(&abort_s, 1); atomicExch(p.status, 11); ok = false; break; }
+                if (!mbar_wait(bar_empty + 8 * s, ph ^ 1u, &abort_s)) { atomicExch(&abort_s, 1); report_wait(p.status, 11); ok = false; break; }
                 const int pos0 = (c_begin + i) * TILE_M;
                 const uint32_t dy_dst = ring + (uint32_t)(s * stage_bytes), a_dst = dy_dst + 2u * (uint32_t)dy_slab_bytes;
                 mbar_expect_tx(bar_full + 8 * s, tx);
@@ -664,7 +666,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) conv_wgrad_tc_kernel(const TcWg
             const uint64_t dy_const = desc_sw128(0, (uint32_t)dy_slab_bytes, 1024), a_const = desc_sw128(0, (uint32_t)a_slab_bytes, 1024);
             bool ok = true; int s = 0; uint32_t ph = 0;
             for (int i = 0; i < nc && ok; ++i) {
-                if (!mbar_wait(bar_full + 8 * s, ph, &abort_s)) { atomicExch(&abort_s, 1); atomicExch(p.status, 12); ok = false; break; }
+                if (!mbar_wait(bar_full + 8 * s, ph, &abort_s)) { atomicExch(&abort_s, 1); report_wait(p.status, 12); ok = false; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const int pos0 = (c_begin + i) * TILE_M;
                 const int dy_off = dy_flat ? 0 : pos0 - (pos0 / box_pos) * box_pos;
@@ -694,7 +696,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) conv_wgrad_tc_kernel(const TcWg
         float* const partial = p.partial; float* const outp = p.out;
         bool ok = nc > 0 ? mbar_wait(bar_acc, 0, &abort_s) : true;
         ok = __all_sync(0xffffffffu, ok);
-        if (!ok) { atomicExch(&abort_s, 1); atomicExch(p.status, 13); }
+        if (!ok) { atomicExch(&abort_s, 1); report_wait(p.status, 13); }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const int k = tm * 128 + m;
         if (ok && quad * 32 < cout - tm * 128) {              // warp-uniform: this lane quadrant holds real output channels
@@ -871,15 +873,17 @@ int conv_tc_stat_tiles(const ConvProb& p) {
     return (int)((pos + TILE_M - 1) / TILE_M);
 }
 
-static int* g_status = nullptr;      // one status word per process, zeroed at creation
+// One status word per process in pinned host memory that every device can write: a kernel stores into it only when a bounded wait
+// gives up, and the host reads it after a synchronisation without a copy (a 4-byte copy and its wait took 10 us of every layer call).
 int* conv_tc_status_word() {
-    if (!g_status) { cudaMalloc(&g_status, 256); cudaMemset(g_status, 0, 256); }
-    return g_status;
+    static int* word = [] { int* w = nullptr; if (cudaHostAlloc(&w, 256, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) { cudaGetLastError(); return (int*)nullptr; } *w = 0; return w; }();
+    return word;
 }
 int conv_tc_read_status() {
-    if (!g_status) return 0;
-    int v = 0; cudaMemcpy(&v, g_status, 4, cudaMemcpyDeviceToHost);
-    if (v) cudaMemset(g_status, 0, 4);              // reported once
+    volatile int* w = conv_tc_status_word();
+    if (!w) return 0;
+    const int v = *w;
+    if (v) *w = 0;                                  // reported once
     return v;
 }
 

@@ -1,6 +1,8 @@
 // Layer-level entry points: one convolution (forward, dgrad or wgrad) or one BN+ReLU (forward, backward)
 // on caller-owned device tensors, run by the same kernels the local step uses.
 #include <algorithm>
+#include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 #include "runtime.h"
@@ -43,6 +45,75 @@ using namespace resist;
 static thread_local std::string g_layer_error;
 extern "C" const char* resist_layer_last_error(void) { return g_layer_error.c_str(); }
 
+
+// Scratch of the layer-level calls.  cudaMalloc and cudaFree cost 100 to 300 us each (cudaFree also waits for the whole device), many
+// times the kernels of a small layer, so a call borrows a block and hands it back once its work is done (every call
+// synchronises its stream before it returns, so a block handed back is idle).  A block: device scratch plus pinned host memory for
+// the descriptors, which go up in one asynchronous copy.  A borrowed block belongs to one call alone, so any number of threads and
+// streams may be inside the calls.  Idle blocks are kept up to SCRATCH_IDLE_BYTES and SCRATCH_IDLE_BLOCKS over all devices, the rest is
+// freed at once; resist_layer_release_scratch() gives back the idle ones.
+namespace {
+constexpr size_t SCRATCH_IDLE_BYTES = (size_t)256 << 20, SCRATCH_HOST_BYTES = 16384;
+constexpr int SCRATCH_IDLE_BLOCKS = 16;
+struct ScratchBlock { char* dev = nullptr; char* host = nullptr; size_t bytes = 0; int device = -1; };
+std::mutex g_scratch_mutex;
+std::vector<ScratchBlock> g_scratch_idle;                     // guarded by the mutex
+
+void scratch_free(const ScratchBlock& b) { cudaFree(b.dev); cudaFreeHost(b.host); }
+
+struct Scratch {
+    ScratchBlock b;
+    cudaStream_t st; size_t staged = 0; bool busy = false;
+    explicit Scratch(cudaStream_t s) : st(s) {}
+    Scratch(const Scratch&) = delete;
+    cudaError_t take(size_t bytes) {
+        int dev = 0; cudaError_t e = cudaGetDevice(&dev); if (e != cudaSuccess) return e;
+        {
+            std::lock_guard<std::mutex> lock(g_scratch_mutex);
+            int best = -1;
+            for (int i = 0; i < (int)g_scratch_idle.size(); ++i)
+                if (g_scratch_idle[i].device == dev && g_scratch_idle[i].bytes >= bytes && (best < 0 || g_scratch_idle[i].bytes < g_scratch_idle[best].bytes)) best = i;
+            if (best >= 0) { b = g_scratch_idle[best]; g_scratch_idle.erase(g_scratch_idle.begin() + best); return cudaSuccess; }
+        }
+        size_t room = (size_t)1 << 20; while (room < bytes && room < ((size_t)64 << 20)) room *= 2;     // few sizes, so that blocks serve other layers too
+        b.bytes = std::max(room, bytes); b.device = dev;
+        e = cudaMalloc(&b.dev, b.bytes);
+        if (e == cudaSuccess) e = cudaHostAlloc(&b.host, SCRATCH_HOST_BYTES, cudaHostAllocPortable);
+        if (e != cudaSuccess) { cudaFree(b.dev); b = ScratchBlock(); }
+        return e;
+    }
+    // descriptors are laid out in the pinned memory at the offsets they have in the block, then sent as one copy
+    void stage(size_t at, const void* what, size_t bytes) { memcpy(b.host + at, what, bytes); staged = std::max(staged, at + bytes); }
+    cudaError_t send() { busy = true; return cudaMemcpyAsync(b.dev, b.host, staged, cudaMemcpyHostToDevice, st); }
+    cudaError_t wait() { const cudaError_t e = cudaStreamSynchronize(st); busy = false; return e; }
+    ~Scratch() {
+        if (!b.dev) return;
+        if (busy) cudaStreamSynchronize(st);                   // an error path left work in flight
+        std::vector<ScratchBlock> out;
+        {
+            std::lock_guard<std::mutex> lock(g_scratch_mutex);
+            g_scratch_idle.push_back(b);
+            size_t total = 0; for (const ScratchBlock& x : g_scratch_idle) total += x.bytes;
+            while (total > SCRATCH_IDLE_BYTES || (int)g_scratch_idle.size() > SCRATCH_IDLE_BLOCKS) {      // the largest goes first
+                int big = 0; for (int i = 1; i < (int)g_scratch_idle.size(); ++i) if (g_scratch_idle[i].bytes > g_scratch_idle[big].bytes) big = i;
+                total -= g_scratch_idle[big].bytes; out.push_back(g_scratch_idle[big]); g_scratch_idle.erase(g_scratch_idle.begin() + big);
+            }
+        }
+        for (const ScratchBlock& x : out) scratch_free(x);
+    }
+};
+}
+
+extern "C" int resist_layer_release_scratch(void) {
+    std::vector<ScratchBlock> out;
+    { std::lock_guard<std::mutex> lock(g_scratch_mutex); out.swap(g_scratch_idle); }
+    for (const ScratchBlock& x : out) scratch_free(x);
+    return RESIST_OK;
+}
+
+static int sm_count_of_device() {
+    int sm = 148, dev = 0; cudaGetDevice(&dev); cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev); return sm;
+}
 static int out_dim(int h, int k, int stride) { return (h + 2 * ((k - 1) / 2) - k) / stride + 1; }
 
 extern "C" int resist_conv2d(int32_t mode, int32_t dtype, int32_t backend, const void* act, const void* wgt, const void* add,
@@ -62,7 +133,7 @@ extern "C" int resist_conv2d(int32_t mode, int32_t dtype, int32_t backend, const
     else { p.M = K; p.Ncol = ksz * ksz * C; p.Kred = (int)rows_out; p.add = nullptr; }
     p.tiles_m = (p.M + 63) / 64; p.tiles_n = (p.Ncol + 63) / 64; p.splits = 1;
     const int ktiles = (p.Kred + 15) / 16; p.ktiles_per_split = ktiles;
-    int sm = 148; int dev = 0; cudaGetDevice(&dev); cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev);
+    const int sm = sm_count_of_device();
     // which kernel family: 0 CUDA cores, 1 tcgen05, 2 warp-level MMA
     auto pick = [&](const ConvProb& q, size_t* pb) -> int {
         if (dtype != RESIST_BF16 || backend == RESIST_CONV_CUDA_CORES) return 0;
@@ -77,21 +148,13 @@ extern "C" int resist_conv2d(int32_t mode, int32_t dtype, int32_t backend, const
         if (want_tc && conv_tc_supported(q, mode)) return 1;
         return 0;
     };
-    // backward of a stride-2 layer on the warp-MMA kernels: stride-1 problem on a zero-stuffed dy (the tcgen05 kernels take the
-    // stride-2 problem as it is)
-    char* up = nullptr;
+    // backward of a stride-2 layer on the warp-MMA kernels: a stride-1 problem that reads the compact dy through its pixel tables (odd
+    // positions are zero), as in the local step; the tcgen05 kernels take the stride-2 problem as it is
     if (stride == 2 && mode != CONV_FWD && K % 8 == 0) {
-        ConvProb q = p; q.stride = 1; q.P = H; q.Q = W;
+        ConvProb q = p; q.stride = 1; q.P = H; q.Q = W; q.dy_sub = 2; q.dy_P = p.P; q.dy_Q = p.Q;
         if (mode == CONV_DGRAD) q.M = (int)rows_in; else q.Kred = (int)rows_in;
         size_t pb = 0;
-        if (pick(q, &pb) == 2) {
-            if (cudaMalloc(&up, (size_t)N * H * W * K * 2 + 256) != cudaSuccess) { g_layer_error = "cudaMalloc failed"; return RESIST_ENOMEM; }
-            UpProb u{mode == CONV_DGRAD ? p.act : p.wgt, up + 256, N, H, W, K, p.P, p.Q};
-            cudaMemcpyAsync(up, &u, sizeof(u), cudaMemcpyHostToDevice, st);
-            launch_zero_stuff((const UpProb*)up, 1, (long long)N * H * W * (K / 8), st);
-            if (mode == CONV_DGRAD) q.act = up + 256; else q.wgt = up + 256;
-            p = q;
-        }
+        if (pick(q, &pb) == 2) p = q;
     }
     size_t wg_partial = 0;
     const int be = pick(p, &wg_partial);
@@ -109,9 +172,10 @@ extern "C" int resist_conv2d(int32_t mode, int32_t dtype, int32_t backend, const
         p.ktiles_per_split = (ktiles + want - 1) / want; p.splits = (ktiles + p.ktiles_per_split - 1) / p.ktiles_per_split;
         if (p.splits > 1) scratch = (size_t)p.splits * p.M * p.Ncol * 4;
     }
-    char* blob = nullptr;
-    cudaError_t e = cudaMalloc(&blob, 1024 + scratch);
-    if (e != cudaSuccess) { cudaFree(up); g_layer_error = cudaGetErrorString(e); return RESIST_ENOMEM; }
+    Scratch sc(st);
+    cudaError_t e = sc.take(1024 + scratch);
+    if (e != cudaSuccess) { g_layer_error = cudaGetErrorString(e); return RESIST_ENOMEM; }
+    char* const blob = sc.b.dev;
     if (!be && p.splits > 1) p.partial = (float*)(blob + 1024);
     if (be && mode == CONV_WGRAD) p.partial = (float*)(blob + 1024 + hd_room);
     bool filled = true;
@@ -123,9 +187,10 @@ extern "C" int resist_conv2d(int32_t mode, int32_t dtype, int32_t backend, const
         else cudaMemsetAsync(out, 0, (size_t)rows_in * C * 2, st);
     }
     if (be == 2) filled = mode == CONV_WGRAD ? conv_wgrad_mma_fill(p, 2 * sm, hd.data()) : conv_mma_fill(p, mode, hd.data());
-    if (!filled) { cudaFree(blob); cudaFree(up); g_layer_error = "descriptor set-up failed"; return RESIST_ECUDA; }
-    e = cudaMemcpyAsync(blob, &p, sizeof(p), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess && be) e = cudaMemcpyAsync(blob + 1024, hd.data(), hd.size(), cudaMemcpyHostToDevice, st);
+    if (!filled) { g_layer_error = "descriptor set-up failed"; return RESIST_ECUDA; }
+    sc.stage(0, &p, sizeof(p));
+    if (be) sc.stage(1024, hd.data(), hd.size());
+    e = sc.send();
     if (e == cudaSuccess) {
         if (be == 1 && mode == CONV_WGRAD) launch_conv_wgrad_tc_probs(blob + 1024, 1, conv_wgrad_tc_ctas(hd.data()), conv_wgrad_tc_smem(hd.data()), conv_wgrad_tc_out_elems(hd.data()), st);
         else if (be == 1) {
@@ -141,8 +206,7 @@ extern "C" int resist_conv2d(int32_t mode, int32_t dtype, int32_t backend, const
         }
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    cudaFree(blob); cudaFree(up);
+    if (e == cudaSuccess) e = sc.wait();
     if (e != cudaSuccess) { g_layer_error = cudaGetErrorString(e); return RESIST_ECUDA; }
     if (be == 1) { const int stv = conv_tc_read_status();
         if (stv) { g_layer_error = "a bounded device-side wait gave up (code " + std::to_string(stv) + ")"; return RESIST_ETIMEOUT; } }
@@ -161,18 +225,19 @@ extern "C" int resist_bn_relu_forward(int32_t dtype, const void* x, const float*
     cudaStream_t st = (cudaStream_t)stream;
     BnProb p{}; p.x = x; p.a = a; p.gamma = gamma; p.beta = beta; p.run_mean = run_mean; p.run_var = run_var; p.stat = stat;
     p.eps = eps; p.momentum = momentum; fill_bn(p, m, C, dtype == RESIST_BF16);
-    char* blob = nullptr;
-    cudaError_t e = cudaMalloc(&blob, 1024 + (size_t)p.chunks * 2 * C * 8);
+    Scratch sc(st);
+    cudaError_t e = sc.take(1024 + (size_t)p.chunks * 2 * C * 8);
     if (e != cudaSuccess) { g_layer_error = cudaGetErrorString(e); return RESIST_ENOMEM; }
+    char* const blob = sc.b.dev;
     p.partial = (double*)(blob + 1024);
-    e = cudaMemcpyAsync(blob, &p, sizeof(p), cudaMemcpyHostToDevice, st);
+    sc.stage(0, &p, sizeof(p));
+    e = sc.send();
     if (e == cudaSuccess) {
         launch_bn_stats((BnProb*)blob, 1, p.chunks, C, dtype == RESIST_BF16, st);
         launch_bn_apply((BnProb*)blob, 1, m * C, dtype == RESIST_BF16, st);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    cudaFree(blob);
+    if (e == cudaSuccess) e = sc.wait();
     if (e != cudaSuccess) { g_layer_error = cudaGetErrorString(e); return RESIST_ECUDA; }
     return RESIST_OK;
 }
@@ -184,18 +249,19 @@ extern "C" int resist_bn_relu_backward(int32_t dtype, const void* x, const void*
     cudaStream_t st = (cudaStream_t)stream;
     BnProb p{}; p.x = x; p.da = da; p.dx = dx; p.add = add; p.gamma = gamma; p.beta = beta; p.dgamma = dgamma; p.dbeta = dbeta; p.stat = stat;
     fill_bn(p, m, C, dtype == RESIST_BF16);
-    char* blob = nullptr;
-    cudaError_t e = cudaMalloc(&blob, 1024 + (size_t)p.chunks * 2 * C * 8);
+    Scratch sc(st);
+    cudaError_t e = sc.take(1024 + (size_t)p.chunks * 2 * C * 8);
     if (e != cudaSuccess) { g_layer_error = cudaGetErrorString(e); return RESIST_ENOMEM; }
+    char* const blob = sc.b.dev;
     p.partial = (double*)(blob + 1024);
-    e = cudaMemcpyAsync(blob, &p, sizeof(p), cudaMemcpyHostToDevice, st);
+    sc.stage(0, &p, sizeof(p));
+    e = sc.send();
     if (e == cudaSuccess) {
         launch_bn_bwd_reduce((BnProb*)blob, 1, p.chunks, C, dtype == RESIST_BF16, st);
         launch_bn_bwd_apply((BnProb*)blob, 1, m * C, dtype == RESIST_BF16, st);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    cudaFree(blob);
+    if (e == cudaSuccess) e = sc.wait();
     if (e != cudaSuccess) { g_layer_error = cudaGetErrorString(e); return RESIST_ECUDA; }
     return RESIST_OK;
 }
@@ -227,7 +293,7 @@ extern "C" int resist_conv2d_bn_relu(int32_t mode, int32_t backend, const void* 
     p.P = out_dim(H, ksz, stride); p.Q = out_dim(W, ksz, stride); p.scale = scale; p.add = add; p.out = out; p.act = act; p.wgt = wgt;
     const long long rows_out = (long long)N * p.P * p.Q, rows_in = (long long)N * H * W;
     if (mode == CONV_FWD) { p.M = (int)rows_out; p.Ncol = K; p.Kred = ksz * ksz * C; } else { p.M = (int)rows_in; p.Ncol = C; p.Kred = ksz * ksz * K; }
-    int sm = 148; int dev = 0; cudaGetDevice(&dev); cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev);
+    const int sm = sm_count_of_device();
     BnProb bn{};
     bn.gamma = gamma; bn.beta = beta; bn.stat = stat; bn.run_mean = run_mean; bn.run_var = run_var; bn.eps = eps; bn.momentum = momentum;
     bn.dgamma = dgamma; bn.dbeta = dbeta;
@@ -248,9 +314,10 @@ extern "C" int resist_conv2d_bn_relu(int32_t mode, int32_t backend, const void* 
     const int n_tc = be == 1 ? conv_tc_count(p, mode) : 1;
     std::vector<char> hd(be == 1 ? (size_t)n_tc * conv_tc_prob_bytes() : conv_mma_prob_bytes());
     const size_t hd_room = (hd.size() + 255) / 256 * 256;
-    char* blob = nullptr;
-    cudaError_t e = cudaMalloc(&blob, 1024 + hd_room + partial_bytes + 256);
+    Scratch sc(st);
+    cudaError_t e = sc.take(1024 + hd_room + partial_bytes + 256);
     if (e != cudaSuccess) { g_layer_error = cudaGetErrorString(e); return RESIST_ENOMEM; }
+    char* const blob = sc.b.dev;
     bn.partial = (double*)(blob + 1024 + hd_room);
     bool ok = true;
     if (be == 2) ok = conv_mma_fill(q, mode, hd.data(), &bn);
@@ -258,13 +325,14 @@ extern "C" int resist_conv2d_bn_relu(int32_t mode, int32_t backend, const void* 
         if (mode == CONV_FWD) { p.stat_tiles = (float*)bn.partial; bn.chunks = tiles; }
         ok = conv_tc_fill(p, mode, hd.data()) == n_tc;
     }
-    if (!ok) { cudaFree(blob); g_layer_error = "descriptor set-up failed"; return RESIST_ECUDA; }
-    e = cudaMemcpyAsync(blob, &bn, sizeof(bn), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(blob + 1024, hd.data(), hd.size(), cudaMemcpyHostToDevice, st);
+    if (!ok) { g_layer_error = "descriptor set-up failed"; return RESIST_ECUDA; }
+    sc.stage(0, &bn, sizeof(bn));
+    sc.stage(1024, hd.data(), hd.size());
+    e = sc.send();
     if (e == cudaSuccess) {
         if (be == 2) {
             if (!launch_conv_mma_probs(blob + 1024, 1, conv_mma_tiles(hd.data()), conv_mma_smem(hd.data()), conv_mma_pick_variant(q, mode) + 512, st)) {
-                cudaGetLastError(); cudaFree(blob); g_layer_error = "the fused launch was refused (cooperative grid too large?)"; return RESIST_ECUDA; }
+                cudaGetLastError(); g_layer_error = "the fused launch was refused (cooperative grid too large?)"; return RESIST_ECUDA; }
         } else {
             int t = 0; size_t packed = 0;
             for (int i = 0; i < n_tc; ++i) { const char* h = hd.data() + (size_t)i * conv_tc_prob_bytes(); t = std::max(t, conv_tc_tiles(h)); packed = conv_tc_merge(packed, conv_tc_smem(h)); }
@@ -277,8 +345,7 @@ extern "C" int resist_conv2d_bn_relu(int32_t mode, int32_t backend, const void* 
         }
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    cudaFree(blob);
+    if (e == cudaSuccess) e = sc.wait();
     if (e != cudaSuccess) { g_layer_error = cudaGetErrorString(e); return RESIST_ECUDA; }
     if (be == 1) { const int stv = conv_tc_read_status();
         if (stv) { g_layer_error = "a bounded device-side wait gave up (code " + std::to_string(stv) + ")"; return RESIST_ETIMEOUT; } }
