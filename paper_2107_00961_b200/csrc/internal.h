@@ -81,7 +81,7 @@ struct UpProb {           // zero stuffing of a stride-2 layer's dy: src [N,P,Q,
 };
 
 struct PoolProb {         // 3x3 stride-2 max-pool, pad 1: x [N,H,W,C] -> y [N,P,Q,C]
-    const void* x; void* y; int* arg; const void* dy; void* dx;
+    const void* x; void* y; uint8_t* arg; const void* dy; void* dx;     // arg: winning tap (3r + s) of each output
     int N, H, W, C, P, Q;
 };
 
@@ -98,8 +98,13 @@ struct HeadProb {         // global average pool + linear head + mean softmax cr
     float* loss_user;     // optional copy for the caller
     int* correct;         // optional top-1 count
     float* logits_user;   // optional copy for the caller
+    float* sample_loss;   // [B] loss of each sample, then [B] top-1 hits (0 or 1)
     int B, HW, C, classes;
+    unsigned done;        // samples' CTAs that have finished; wraps to 0 by itself (lives in the plan's blob, which starts zeroed)
 };
+// A head small enough for one CTA per sample to do pooling, logits, loss and the gradient of its input: every CTA reads all the head's
+// weights (32 KB at most, from L2).  Larger heads run as matrix products over the whole batch.
+inline bool head_small(int C, int classes) { return C <= 256 && classes <= 128 && C * classes <= 8192; }
 
 // A contiguous run of parameters treated alike by the bandwidth kernels.
 struct Segment {
@@ -119,7 +124,7 @@ struct ParamArrays {      // device pointers of the flat arrays
 constexpr int SEG_CHUNK = 4096;   // elements per CTA in the segment kernels
 constexpr int AGG_CHUNK = 8192;   // elements per CTA of the aggregate kernel (two rounds of four 16-byte groups per thread)
 
-// ---- launchers (kernels_ref.cu)
+// ---- launchers (kernels_ref.cu; pools, head and im2col: kernels_head.cu)
 void launch_conv_ref(const ConvProb* d, int nprob, int max_tiles, int mode, bool bf16, cudaStream_t s);
 void launch_splitk_reduce(const ConvProb* d, int nprob, int max_elems, cudaStream_t s);
 void launch_bn_stats(const BnProb* d, int nprob, int max_chunks, int max_c, bool bf16, cudaStream_t s);
@@ -128,13 +133,13 @@ void launch_bn_bwd_reduce(const BnProb* d, int nprob, int max_chunks, int max_c,
 void launch_bn_bwd_apply(const BnProb* d, int nprob, long long max_elems, bool bf16, cudaStream_t s);
 void launch_maxpool_fwd(const PoolProb* d, int nprob, long long max_elems, bool bf16, cudaStream_t s);
 void launch_maxpool_bwd(const PoolProb* d, int nprob, long long max_elems, bool bf16, cudaStream_t s);
-void launch_head_fwd(const HeadProb* d, int nprob, int maxB, int maxC, int max_classes, bool bf16, cudaStream_t s);
-void launch_head_bwd(const HeadProb* d, int nprob, int maxB, int maxC, int max_classes, long long max_elems,
-                     bool bf16, cudaStream_t s);
+int launch_head_fwd(const HeadProb* d, int nprob, int maxB, int maxC, int max_classes, bool bf16, cudaStream_t s);    // both return the number of kernels
+int launch_head_bwd(const HeadProb* d, int nprob, int maxB, int maxC, int max_classes, long long max_elems,
+                    bool bf16, cudaStream_t s);
 
 // statistics, finalisation and apply of BN+ReLU in one cooperative launch (bf16 vector path, training mode); false if the grid cannot be co-resident
 bool launch_bn_fused(const BnProb* d, int nprob, int max_chunks, int backward, cudaStream_t s);   // kernels_ref.cu
-void launch_im2col(const ColProb* d, int nprob, long long max_rows, cudaStream_t s);      // kernels_ref.cu
+void launch_im2col(const ColProb* d, int nprob, const ColProb& shape, cudaStream_t s);      // shape: the largest problem's
 void launch_repack_rows(const ConvProb* d, int nprob, int max_elems, cudaStream_t s);     // kernels_ref.cu
 void launch_zero_stuff(const UpProb* d, int nprob, long long max_vecs, cudaStream_t s);   // conv_tc.cu
 

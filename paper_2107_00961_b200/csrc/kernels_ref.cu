@@ -504,220 +504,6 @@ void launch_bn_bwd_apply(const BnProb* d, int nprob, long long max_elems, bool b
     else bn_bwd_apply_kernel<float><<<dim3(ew_grid(max_elems), nprob), 256, 0, s>>>(d);
 }
 
-// ------------------------------------------------------------------------------------------------
-// 3x3 stride-2 max-pool (padding 1, padded cells never win; first maximum in row-major window order)
-// ------------------------------------------------------------------------------------------------
-template <class T>
-__global__ void maxpool_fwd_kernel(const PoolProb* __restrict__ probs) {
-    const PoolProb& p = probs[blockIdx.y];
-    const long long n = (long long)p.N * p.P * p.Q * p.C;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        int c = (int)(i % p.C); long long t = i / p.C; int q = (int)(t % p.Q); t /= p.Q; int pp = (int)(t % p.P); int nn = (int)(t / p.P);
-        bool have = false; float best = 0.f; int bi = -1;
-        for (int r = 0; r < 3; ++r) { int h = 2 * pp + r - 1; if (h < 0 || h >= p.H) continue;
-            for (int s = 0; s < 3; ++s) { int w = 2 * q + s - 1; if (w < 0 || w >= p.W) continue;
-                float v = ldf<T>(p.x, (((long long)nn * p.H + h) * p.W + w) * p.C + c);
-                if (!have || v > best) { have = true; best = v; bi = h * p.W + w; } } }
-        stf<T>(p.y, i, best);
-        if (p.arg) p.arg[i] = bi;
-    }
-}
-template <class T>
-__global__ void maxpool_bwd_kernel(const PoolProb* __restrict__ probs) {
-    const PoolProb& p = probs[blockIdx.y];
-    const long long n = (long long)p.N * p.H * p.W * p.C;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        int c = (int)(i % p.C); long long t = i / p.C; int w = (int)(t % p.W); t /= p.W; int h = (int)(t % p.H); int nn = (int)(t / p.H);
-        float acc = 0.f;
-        for (int pp = h / 2; pp <= (h + 1) / 2; ++pp) { if (pp >= p.P) continue;          // windows with 2p-1 <= h <= 2p+1
-            for (int q = w / 2; q <= (w + 1) / 2; ++q) { if (q >= p.Q) continue;
-                long long o = (((long long)nn * p.P + pp) * p.Q + q) * p.C + c;
-                if (p.arg[o] == h * p.W + w) acc += ldf<T>(p.dy, o); } }
-        stf<T>(p.dx, i, acc);
-    }
-}
-void launch_maxpool_fwd(const PoolProb* d, int nprob, long long max_elems, bool bf16, cudaStream_t s) {
-    if (bf16) maxpool_fwd_kernel<__nv_bfloat16><<<dim3(ew_grid(max_elems), nprob), 256, 0, s>>>(d);
-    else maxpool_fwd_kernel<float><<<dim3(ew_grid(max_elems), nprob), 256, 0, s>>>(d);
-}
-void launch_maxpool_bwd(const PoolProb* d, int nprob, long long max_elems, bool bf16, cudaStream_t s) {
-    if (bf16) maxpool_bwd_kernel<__nv_bfloat16><<<dim3(ew_grid(max_elems), nprob), 256, 0, s>>>(d);
-    else maxpool_bwd_kernel<float><<<dim3(ew_grid(max_elems), nprob), 256, 0, s>>>(d);
-}
-
-// ------------------------------------------------------------------------------------------------
-// Global average pool, linear head, mean softmax cross-entropy and their gradients (fp32 math)
-// ------------------------------------------------------------------------------------------------
-template <class T>
-__global__ void avgpool_kernel(const HeadProb* __restrict__ probs) {
-    const HeadProb& p = probs[blockIdx.y];
-    const int n = p.B * p.C;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int c = i % p.C, b = i / p.C;
-        float s = 0.f;
-        int k = 0;
-        for (; k + 8 <= p.HW; k += 8) {                          // eight loads in flight, added in order
-            float v[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = ldf<T>(p.a, ((long long)b * p.HW + k + u) * p.C + c);
-#pragma unroll
-            for (int u = 0; u < 8; ++u) s += v[u];
-        }
-        for (; k < p.HW; ++k) s += ldf<T>(p.a, ((long long)b * p.HW + k) * p.C + c);
-        p.pooled[i] = s / (float)p.HW;
-    }
-}
-// one warp per logit
-__global__ void head_logits_kernel(const HeadProb* __restrict__ probs) {
-    const HeadProb& p = probs[blockIdx.y];
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) / 32, lane = threadIdx.x % 32;
-    const int nw = gridDim.x * blockDim.x / 32;
-    for (int o = warp; o < p.B * p.classes; o += nw) {
-        const int k = o % p.classes, b = o / p.classes;
-        float s = 0.f;
-        for (int c = lane; c < p.C; c += 32) s = fmaf(p.w[(long long)k * p.C + c], p.pooled[(long long)b * p.C + c], s);
-        for (int d = 16; d; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
-        if (lane == 0) { s += p.b[k]; p.logits[o] = s; if (p.logits_user) p.logits_user[o] = s; }
-    }
-}
-// one CTA per problem; one warp per sample, samples strided over the warps; fixed-order loss sum
-__global__ void __launch_bounds__(1024) loss_kernel(const HeadProb* __restrict__ probs) {
-    const HeadProb& p = probs[blockIdx.x];
-    __shared__ float sl[1024]; __shared__ int sc[1024];
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    for (int b = warp; b < p.B; b += (int)(blockDim.x >> 5)) {
-        const float* lg = p.logits + (long long)b * p.classes;
-        float mx = -INFINITY; int arg = 0x7fffffff;
-        for (int k = lane; k < p.classes; k += 32) { float v = lg[k]; if (v > mx) { mx = v; arg = k; } }
-        for (int d = 16; d; d >>= 1) {
-            float om = __shfl_xor_sync(0xffffffffu, mx, d); int oa = __shfl_xor_sync(0xffffffffu, arg, d);
-            if (om > mx || (om == mx && oa < arg)) { mx = om; arg = oa; }
-        }
-        float se = 0.f;
-        for (int k = lane; k < p.classes; k += 32) se += expf(lg[k] - mx);
-        for (int d = 16; d; d >>= 1) se += __shfl_xor_sync(0xffffffffu, se, d);
-        const float lse = mx + logf(se);
-        const int y = p.labels ? p.labels[b] : -1;
-        if (p.dlogits)
-            for (int k = lane; k < p.classes; k += 32)
-                p.dlogits[(long long)b * p.classes + k] = (expf(lg[k] - lse) - (k == y ? 1.f : 0.f)) / (float)p.B;
-        if (lane == 0) { sl[b] = y >= 0 ? lse - lg[y] : 0.f; sc[b] = (arg == y); }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float s = 0.f; int c = 0;
-        for (int b = 0; b < p.B; ++b) { s += sl[b]; c += sc[b]; }
-        s /= (float)p.B;
-        if (p.loss) *p.loss = s;
-        if (p.loss_user) *p.loss_user = s;
-        if (p.correct) *p.correct = c;
-    }
-}
-// one thread per element of dw (neighbouring threads = neighbouring input channels: the loads of `pooled` are coalesced and the
-// dlogits value is the same for a whole warp); samples added in order.  The last `classes` threads make the bias gradient.
-__global__ void head_bwd_w_kernel(const HeadProb* __restrict__ probs) {
-    const HeadProb& p = probs[blockIdx.y];
-    const int n = p.classes * p.C;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n + p.classes; i += gridDim.x * blockDim.x) {
-        float s = 0.f;
-        if (i < n) { const int c = i % p.C, k = i / p.C;
-#pragma unroll 4
-            for (int b = 0; b < p.B; ++b) s = fmaf(p.dlogits[(long long)b * p.classes + k], p.pooled[(long long)b * p.C + c], s);
-            p.dw[i] = s;
-        } else { const int k = i - n;
-            for (int b = 0; b < p.B; ++b) s += p.dlogits[(long long)b * p.classes + k];
-            p.db[k] = s; }
-    }
-}
-__global__ void head_bwd_x_kernel(const HeadProb* __restrict__ probs) {
-    const HeadProb& p = probs[blockIdx.y];
-    const int n = p.B * p.C;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int c = i % p.C, b = i / p.C;
-        float s = 0.f;
-        for (int k = 0; k < p.classes; ++k) s = fmaf(p.dlogits[(long long)b * p.classes + k], p.w[(long long)k * p.C + c], s);
-        p.dpooled[i] = s / (float)p.HW;
-    }
-}
-template <class T>
-__global__ void avgpool_bwd_kernel(const HeadProb* __restrict__ probs) {
-    const HeadProb& p = probs[blockIdx.y];
-    const long long n = (long long)p.B * p.HW * p.C;
-    if (sizeof(T) == 2 && p.C % 8 == 0 && (((uintptr_t)p.da | (uintptr_t)p.dpooled) & 15) == 0) {   // 8 channels per thread
-        const int G = p.C / 8; const long long nv = n / 8;
-        for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < nv; v += (long long)gridDim.x * blockDim.x) {
-            const int g = (int)(v % G); const long long b = v / ((long long)p.HW * G);
-            const float4 f0 = *reinterpret_cast<const float4*>(p.dpooled + b * p.C + g * 8), f1 = *reinterpret_cast<const float4*>(p.dpooled + b * p.C + g * 8 + 4);
-            const float f[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
-            reinterpret_cast<uint4*>(p.da)[v] = pack8(f);
-        }
-        return;
-    }
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(i % p.C); const long long b = i / ((long long)p.HW * p.C);
-        stf<T>(p.da, i, p.dpooled[b * p.C + c]);
-    }
-}
-
-void launch_head_fwd(const HeadProb* d, int nprob, int maxB, int maxC, int max_classes, bool bf16, cudaStream_t s) {
-    if (bf16) avgpool_kernel<__nv_bfloat16><<<dim3(ew_grid((long long)maxB * maxC), nprob), 256, 0, s>>>(d);
-    else avgpool_kernel<float><<<dim3(ew_grid((long long)maxB * maxC), nprob), 256, 0, s>>>(d);
-    head_logits_kernel<<<dim3(ew_grid((long long)maxB * max_classes * 32), nprob), 256, 0, s>>>(d);
-    loss_kernel<<<nprob, 1024, 0, s>>>(d);
-}
-void launch_head_bwd(const HeadProb* d, int nprob, int maxB, int maxC, int max_classes, long long max_elems,
-                     bool bf16, cudaStream_t s) {
-    head_bwd_w_kernel<<<dim3(ew_grid((long long)max_classes * (maxC + 1)), nprob), 256, 0, s>>>(d);
-    head_bwd_x_kernel<<<dim3(ew_grid((long long)maxB * maxC), nprob), 256, 0, s>>>(d);
-    if (bf16) avgpool_bwd_kernel<__nv_bfloat16><<<dim3(ew_grid(max_elems), nprob), 256, 0, s>>>(d);
-    else avgpool_bwd_kernel<float><<<dim3(ew_grid(max_elems), nprob), 256, 0, s>>>(d);
-}
-
-
-// ------------------------------------------------------------------------------------------------ im2col (few-channel stem)
-// One thread per (output position, 8-column group).  The first K*4 threads also pack the weights.
-__global__ void __launch_bounds__(256) im2col_kernel(const ColProb* __restrict__ probs) {
-    const ColProb& p = probs[blockIdx.y];
-    const __nv_bfloat16* __restrict__ src = (const __nv_bfloat16*)p.src;
-    const int cols = p.cols, G = cols >> 3;                       // row pitch in columns (a multiple of 8, at most 256), 8-column groups
-    const long long rows = (long long)p.N * p.P * p.Q, total = rows * G;
-    // column j of a row = tap (r, s), channel c: the three are looked up, not divided out, for every element
-    __shared__ int s_r[256], s_s[256], s_off[256];
-    for (int j = threadIdx.x; j < cols; j += blockDim.x) {
-        if (j < p.kk) { const int c = j % p.C, rs = j / p.C, ss = rs % p.ksz, r = rs / p.ksz; s_r[j] = r - p.pad; s_s[j] = ss - p.pad; s_off[j] = ((r - p.pad) * p.W + (ss - p.pad)) * p.C + c; }
-        else { s_r[j] = -(1 << 20); s_s[j] = 0; s_off[j] = 0; }   // beyond the taps: never inside the image
-    }
-    __syncthreads();
-    const unsigned short* __restrict__ src16 = reinterpret_cast<const unsigned short*>(src);
-    for (long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x; id < total; id += (long long)gridDim.x * blockDim.x) {
-        const int g = G == 4 ? (int)(id & 3) : (int)(id % G); const long long row = G == 4 ? id >> 2 : id / G;
-        const int q = (int)(row % p.Q); const long long t = row / p.Q; const int pr = (int)(t % p.P); const int n = (int)(t / p.P);
-        const int y0 = pr * p.stride, x0 = q * p.stride;
-        const long long base = (((long long)n * p.H + y0) * p.W + x0) * p.C;
-        unsigned short h[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const int j = g * 8 + e;
-            const int y = y0 + s_r[j], xx = x0 + s_s[j];
-            const bool in = y >= 0 && y < p.H && xx >= 0 && xx < p.W;
-            h[e] = in ? src16[base + s_off[j]] : (unsigned short)0;
-        }
-        *reinterpret_cast<uint4*>((__nv_bfloat16*)p.dst + row * cols + g * 8) =
-            make_uint4(h[0] | ((unsigned)h[1] << 16), h[2] | ((unsigned)h[3] << 16), h[4] | ((unsigned)h[5] << 16), h[6] | ((unsigned)h[7] << 16));
-        if (id < (long long)p.K * G) {                             // weights: w[k][kk] -> w32[k][cols]
-            const int kx = (int)(id / G);
-            __align__(16) __nv_bfloat16 wv[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) { const int j = g * 8 + e; wv[e] = j < p.kk ? ((const __nv_bfloat16*)p.w)[(long long)kx * p.kk + j] : __float2bfloat16(0.f); }
-            *reinterpret_cast<uint4*>((__nv_bfloat16*)p.w32 + (long long)kx * cols + g * 8) = *reinterpret_cast<const uint4*>(wv);
-        }
-    }
-}
-void launch_im2col(const ColProb* d, int nprob, long long max_rows, cudaStream_t s) {
-    long long gx = (max_rows * 4 + 255) / 256; if (gx > 148 * 16) gx = 148 * 16; if (gx < 1) gx = 1;
-    im2col_kernel<<<dim3((unsigned)gx, nprob), 256, 0, s>>>(d);
-}
-
 // dst[r][0..cols) = src[r][0..cols) for rows of different pitch (fp32): the weight gradient of an im2col'ed stem, computed with
 // the padded column count, goes to its place in the gradient vector
 __global__ void repack_rows_kernel(const ConvProb* __restrict__ probs) {

@@ -335,7 +335,7 @@ static size_t unroll_subnet(resist_ctx* ctx, Builder& bd, const std::vector<char
     // ---- stem
     const int Hs = out_dim(A.in_h, A.stem_k, A.stem_stride), Ws = out_dim(A.in_w, A.stem_k, A.stem_stride);
     const long long m_stem = (long long)B * Hs * Ws;
-    void* stem_y = bd.act(m_stem * A.stem_cout); void* stem_a = nullptr; void* stem_p = nullptr; int* stem_arg = nullptr; float* stem_stat = nullptr;
+    void* stem_y = bd.act(m_stem * A.stem_cout); void* stem_a = nullptr; void* stem_p = nullptr; uint8_t* stem_arg = nullptr; float* stem_stat = nullptr;
     const bool stem_col = bd.stem_as_im2col(L.stem);
     if (stem_col) { bd.stem_im2col(0, L.stem, B, A.in_h, A.in_w); bd.stem_conv(0, CONV_FWD, L.stem, nullptr, stem_y, B, A.in_h, A.in_w); }
     else bd.conv(0, CONV_FWD, nullptr, L.stem, nullptr, nullptr, stem_y, B, A.in_h, A.in_w, 1.f, true);
@@ -343,7 +343,7 @@ static size_t unroll_subnet(resist_ctx* ctx, Builder& bd, const std::vector<char
     if (A.stem_bn_relu) { stem_a = bd.act(m_stem * cC); stem_stat = bd.bn_fwd(1, stem_y, stem_a, L.stem_bn, m_stem); cur = stem_a; }
     if (A.stem_maxpool) {
         const int Hp = out_dim(cH, 3, 2), Wp = out_dim(cW, 3, 2);
-        stem_p = bd.act((long long)B * Hp * Wp * cC); stem_arg = (int*)bd.take((size_t)B * Hp * Wp * cC * 4);
+        stem_p = bd.act((long long)B * Hp * Wp * cC); stem_arg = bd.eval ? nullptr : (uint8_t*)bd.take((size_t)B * Hp * Wp * cC);
         Op op{}; op.key = 3; op.sub = bd.sub; op.kind = OP_POOL_FWD;
         op.pool = PoolProb{cur, stem_p, stem_arg, nullptr, nullptr, B, cH, cW, cC, Hp, Wp};
         bd.ops->push_back(op); bd.last_fwd_conv = -1; bd.last_tc_fwd = -1;
@@ -410,13 +410,14 @@ static size_t unroll_subnet(resist_ctx* ctx, Builder& bd, const std::vector<char
     hp.pooled = (float*)bd.take((size_t)B * cC * 4); hp.dpooled = (float*)bd.take((size_t)B * cC * 4);
     hp.logits = (float*)bd.take((size_t)B * A.classes * 4); hp.dlogits = bd.eval ? nullptr : (float*)bd.take((size_t)B * A.classes * 4);
     hp.loss = (float*)bd.take(256); hp.B = B; hp.HW = HW; hp.C = cC; hp.classes = A.classes;
+    hp.sample_loss = (float*)bd.take((size_t)B * 8);
     bd.logits = hp.logits;
+    int g_cur = -1;                                            // gradient w.r.t. the current tensor; a small head's forward kernel already writes it
+    if (!bd.eval) { g_cur = bd.gtake(); hp.da = bd.gbuf[g_cur]; }
     { Op op{}; op.key = FWD_END + 2; op.sub = bd.sub; op.kind = OP_HEAD_FWD; op.head = hp; bd.ops->push_back(op); }
     if (bd.eval) return bd.off;
 
     // ---- backward
-    int g_cur = bd.gtake();                                   // gradient w.r.t. the current tensor
-    hp.da = bd.gbuf[g_cur];
     { Op op{}; op.key = BWD0; op.sub = bd.sub; op.kind = OP_HEAD_BWD; op.head = hp; bd.ops->push_back(op); }
     { int g = bd.gtake(); bd.bn_bwd(BWD0 + 1, xF, bd.gbuf[g_cur], bd.gbuf[g], nullptr, L.final_bn, statF, mF); bd.grel(g_cur); g_cur = g; }
     for (int slot = (int)order.size() - 1; slot >= 0; --slot) {
@@ -630,7 +631,7 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
                 case OP_IM2COL: {
                     if (k == i) L.first = (int)col.size();
                     sites.push_back({2, (int)col.size(), 0, 0, slot});
-                    col.push_back(o.col);
+                    col.push_back(o.col); L.col = o.col;
                     const double rows = (double)o.col.N * o.col.P * o.col.Q;
                     L.max_elems = std::max<long long>(L.max_elems, (long long)rows);
                     L.bytes += 2.0 * o.col.cols * rows + 2.0 * o.col.N * o.col.H * o.col.W * o.col.C;
@@ -647,7 +648,7 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
                     pool.push_back(o.pool);
                     const PoolProb& p = o.pool;
                     L.max_elems = std::max<long long>(L.max_elems, (long long)p.N * (o.kind == OP_POOL_FWD ? p.P * p.Q : p.H * p.W) * p.C);
-                    L.bytes += (double)p.N * p.C * (es * ((double)p.H * p.W + (double)p.P * p.Q) + 4.0 * p.P * p.Q);
+                    L.bytes += (double)p.N * p.C * (es * ((double)p.H * p.W + (double)p.P * p.Q) + 1.0 * p.P * p.Q);
                     break; }
                 case OP_HEAD_FWD: case OP_HEAD_BWD: {
                     if (k == i) L.first = (int)head.size();
@@ -840,8 +841,8 @@ static int run_plan(resist_ctx* ctx, Plan& plan, const PatchArgs& pa, bool updat
             case OP_BN_BWD_APPLY: pk = PK_BN_BWD_APPLY; break;
             case OP_POOL_FWD: pk = PK_POOL_FWD; break;
             case OP_POOL_BWD: pk = PK_POOL_BWD; break;
-            case OP_HEAD_FWD: pk = PK_HEAD_FWD; nk = 3; break;
-            case OP_HEAD_BWD: pk = PK_HEAD_BWD; nk = 3; break;
+            case OP_HEAD_FWD: pk = PK_HEAD_FWD; nk = head_small(L.max_c, L.max_classes) ? 1 : 3; break;
+            case OP_HEAD_BWD: pk = PK_HEAD_BWD; nk = head_small(L.max_c, L.max_classes) ? 1 : 3; break;
             case OP_UPSAMPLE: pk = PK_UPSAMPLE; break;
             case OP_IM2COL: pk = PK_IM2COL; break;
             case OP_BN_FWD_FUSED: pk = PK_BN_FWD_FUSED; break;
@@ -869,10 +870,10 @@ static int run_plan(resist_ctx* ctx, Plan& plan, const PatchArgs& pa, bool updat
             case OP_BN_BWD_APPLY: launch_bn_bwd_apply(plan.d_bn + L.first, L.count, L.max_elems, bf, st); ++n_launch; break;
             case OP_POOL_FWD: launch_maxpool_fwd(plan.d_pool + L.first, L.count, L.max_elems, bf, st); ++n_launch; break;
             case OP_POOL_BWD: launch_maxpool_bwd(plan.d_pool + L.first, L.count, L.max_elems, bf, st); ++n_launch; break;
-            case OP_HEAD_FWD: launch_head_fwd(plan.d_head + L.first, L.count, L.max_b, L.max_c, L.max_classes, bf, st); n_launch += 3; break;
-            case OP_HEAD_BWD: launch_head_bwd(plan.d_head + L.first, L.count, L.max_b, L.max_c, L.max_classes, L.max_elems, bf, st); n_launch += 3; break;
+            case OP_HEAD_FWD: n_launch += launch_head_fwd(plan.d_head + L.first, L.count, L.max_b, L.max_c, L.max_classes, bf, st); break;
+            case OP_HEAD_BWD: n_launch += launch_head_bwd(plan.d_head + L.first, L.count, L.max_b, L.max_c, L.max_classes, L.max_elems, bf, st); break;
             case OP_UPSAMPLE: launch_zero_stuff(plan.d_up + L.first, L.count, L.max_elems, st); ++n_launch; break;
-            case OP_IM2COL: launch_im2col(plan.d_col + L.first, L.count, L.max_elems, st); ++n_launch; break;
+            case OP_IM2COL: launch_im2col(plan.d_col + L.first, L.count, L.col, st); ++n_launch; break;
             case OP_BN_TILE_STATS: launch_bn_finalize_tiles(plan.d_bn + L.first, L.count, L.max_c, st); ++n_launch; break;
             case OP_BN_FWD_FUSED:
                 if (launch_bn_fused(plan.d_bn + L.first, L.count, L.gx, 0, st)) ++n_launch;

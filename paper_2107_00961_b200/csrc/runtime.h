@@ -39,6 +39,7 @@ struct Launch {
     int gx; long long max_elems; int max_b, max_c, max_classes;
     double bytes, flops;                                      // algorithmic work of this launch
     bool join_before;                                         // the main stream first waits for the weight gradients in flight
+    ColProb col;                                              // im2col: the geometry its problems share
     char label[40];                                           // shape of the launch's first problem, for the per-launch trace
 };
 
