@@ -247,19 +247,21 @@ class Context:
                 setattr(self._blocks[i], name, int(a[10 + 8 * i + j]))
         arch = _Arch(*[int(v) for v in a[:10]], C.cast(self._blocks, C.POINTER(_Block)))
         opts = _Opts(dtype, momentum, weight_decay, bn_eps, bn_momentum, min_depth, momentum_policy, conv_backend, bn_stat_period)
-        # device memory comes from torch's caching allocator
-        self._held = {}
+        # device memory comes from torch's caching allocator.  The callbacks hold the table, not the context: a cycle through them would
+        # keep a dropped context's memory until the next garbage collection
+        held = self._held = {}
+        dev = self.device
 
         def _alloc(_user, nbytes):
             try:
-                t = torch.empty(int(nbytes), dtype=torch.uint8, device=self.device)
+                t = torch.empty(int(nbytes), dtype=torch.uint8, device=dev)
             except RuntimeError:
                 return None
-            self._held[t.data_ptr()] = t
+            held[t.data_ptr()] = t
             return t.data_ptr()
 
         def _free(_user, ptr):
-            self._held.pop(ptr, None)
+            held.pop(ptr, None)
 
         self._alloc_cb, self._free_cb = _ALLOC_FN(_alloc), _FREE_FN(_free)
         self._allocator = _Allocator(self._alloc_cb, self._free_cb, None)

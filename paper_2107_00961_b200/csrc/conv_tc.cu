@@ -17,11 +17,10 @@
 // Kernel structure of forward / dgrad (352 threads, one CTA per SM, persistent over the work of all problems of the launch).  A
 // unit of work is a PAIR of neighbouring 128-position tiles times one column tile of up to 256 output channels:
 // warp 0 = TMA producer (a ring of activation windows, two per step, and a ring of weight tiles, one per (slab, tap), shared by
-// the two tiles of the pair); warps 1 and 2 = MMA issuers, one per tile of the pair, each with its own accumulator in TMEM
-// (a single thread issues a tcgen05.mma only every ~150 cycles, see micro.cu, so one issuer cannot keep the tensor core busy);
-// warps 3..10 = two epilogue groups of four warps, one per tile of the pair (TMEM -> registers -> scale, residual add, bf16 ->
-// 16 KB staging slabs of 64 columns -> TMA store or row copy-out, with per-tile column sums for the BN that follows).
-// The weight-gradient kernel (192 threads) has one producer warp, one issuer warp and four epilogue warps.
+// the two tiles of the pair); warp 1 = MMA issuer, an accumulator in TMEM per tile; warps 2..9 = two epilogue groups of four warps,
+// one per tile of the pair (TMEM -> registers -> scale, residual add, bf16 -> staging slabs of 64 columns -> TMA store or row copy-out,
+// with per-tile column sums for the BN that follows); warp 10 = the residual, by TMA into the staging slabs.
+// The weight-gradient kernel (224 threads) has one producer warp, two issuer warps and four epilogue warps.
 // Every wait is bounded: on expiry the kernel records the place in the status word, drains its copies and MMAs, frees its
 // TMEM and returns.
 #include <cuda.h>
@@ -35,6 +34,15 @@ namespace resist {
 // ------------------------------------------------------------------------------------------------ device helpers
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+// One thread of a converged warp.  The compiler knows that elect.sync leaves a single thread, so the tcgen05 and TMA instructions
+// behind it take their operands from uniform registers; behind "lane == 0" it has to assume that several threads may be there and
+// wraps every one of them in a loop over the active threads (measured: 78 to 150 cycles per tcgen05.mma instead of the tensor
+// core's own 48 / 64 / 128 at N = 64 / 128 / 256).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
@@ -116,9 +124,54 @@ __device__ __forceinline__ uint4 lds128(uint32_t a) { uint4 v; asm volatile("ld.
 __device__ __forceinline__ void sts128(uint32_t a, uint4 v) { asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory"); }
 __device__ __forceinline__ uint32_t lds32(uint32_t a) { uint32_t v; asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(a)); return v; }
 
+// two fp32 operations per instruction
+__device__ __forceinline__ uint64_t f2_pack(uint32_t lo, uint32_t hi) { uint64_t r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi)); return r; }
+__device__ __forceinline__ void f2_unpack(uint64_t v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) { uint64_t r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
+__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) { uint64_t r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) { uint64_t r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+__device__ __forceinline__ uint64_t f2_of_bf16x2(uint32_t w) { return f2_pack(w << 16, w & 0xFFFF0000u); }
+__device__ __forceinline__ uint32_t bf16x2_of_f2(uint64_t v) { float lo, hi; f2_unpack(v, lo, hi); __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi); return *reinterpret_cast<uint32_t*>(&h); }
+
+// A thread's 32 columns of a tile: accumulator * scale (+ residual: RES from the staging slab it goes back to, GADD from registers),
+// rounded, into the staging slab; BN: relu(bn(.)) of the rounded value into a second slab.  st / st2: shared address of the row with the
+// row's swizzle phase folded in (a 16-byte chunk is st ^ chunk * 16); scale2: the scale twice, 0 for a position outside the map (whose sum
+// is of no pixel).  The kernel's epilogue is bound by instructions, not by the stores (skipping them changed nothing), hence the packed
+// arithmetic and one instance per kind.
+template <bool RES, bool GADD, bool BN>
+__device__ __forceinline__ void epi_cols(const uint32_t* v, uint32_t st, uint32_t st2, int chunk0, uint64_t scale2, const uint4* ga, const float4* bnc) {
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+        const uint32_t so = (uint32_t)(chunk0 + g) << 4;
+        uint32_t w[4];
+        if (RES || GADD) {
+            const uint4 a = RES ? lds128(st ^ so) : ga[g];
+            const uint32_t aw[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) w[k] = bf16x2_of_f2(f2_fma(f2_pack(v[g * 8 + 2 * k], v[g * 8 + 2 * k + 1]), scale2, f2_of_bf16x2(aw[k])));
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) w[k] = bf16x2_of_f2(f2_mul(f2_pack(v[g * 8 + 2 * k], v[g * 8 + 2 * k + 1]), scale2));
+        }
+        sts128(st ^ so, make_uint4(w[0], w[1], w[2], w[3]));
+        if (BN) {                                                // evaluation: with running statistics
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float4 q0 = bnc[g * 8 + 2 * k], q1 = bnc[g * 8 + 2 * k + 1];
+                const float z0 = (__uint_as_float(w[k] << 16) - q0.x) * q0.y * q0.z + q0.w, z1 = (__uint_as_float(w[k] & 0xFFFF0000u) - q1.x) * q1.y * q1.z + q1.w;
+                __nv_bfloat162 hh = __floats2bfloat162_rn(z0 > 0.f ? z0 : 0.f, z1 > 0.f ? z1 : 0.f);
+                w[k] = *reinterpret_cast<uint32_t*>(&hh);
+            }
+            sts128(st2 ^ so, make_uint4(w[0], w[1], w[2], w[3]));
+        }
+    }
+}
+
 constexpr int TC_THREADS = 224;              // wgrad kernel: producer warp, two MMA warps, four epilogue warps
-constexpr int TC_MAX_ISSUERS = 2;            // forward / dgrad kernel: MMA-issuing warps, one per tile of a pair
-constexpr int TC_CONV_THREADS = 32 * (1 + TC_MAX_ISSUERS + 8);   // forward / dgrad kernel: producer warp, MMA warps, two groups of four epilogue warps
+constexpr int TC_ISSUERS = 1;                // forward / dgrad kernel: MMA-issuing warps
+constexpr int TC_RES_WARP = 1 + TC_ISSUERS + 8;              // forward / dgrad kernel: fetches the residual
+constexpr int TC_CONV_THREADS = 32 * (TC_RES_WARP + 1);          // producer warp, MMA warps, two groups of four epilogue warps, residual warp
+constexpr int TC_MAX_EB = 4;                                     // 16 KB staging slabs per epilogue group
 constexpr int TC_MAX_STAGES = 12;
 constexpr int TILE_M = 128;
 constexpr int SLAB_BYTES = TILE_M * 128;      // 128 rows x 64 channels of bf16
@@ -137,6 +190,9 @@ struct TcHot {                // everything the kernel's loops read: each role k
     const __nv_bfloat16* add; __nv_bfloat16* out;
     float* stat_tiles;        // [tiles_m][2][ncol]: column sums and sums of squares of the stored tile, or nullptr
     int* status;
+    const float* bn_stat; const float* bn_gamma; const float* bn_beta; __nv_bfloat16* bn_out;   // evaluation: bn_out = relu(bn(y)) with mean | 1/std in bn_stat; nullptr otherwise
+    int store_y;              // 0: only bn_out is wanted
+    int res_tma;              // 1: the residual comes through map_add
     int a_flat;               // 1: a window is one box of 128 pixels of the (channel, pixel) map
     int dense;                // 1: position index == output pixel index
     int add_mode;             // 0 none; 2 residual read at the output pixel; 3 residual read from a compact tensor that applies at even (y, x) only
@@ -158,14 +214,16 @@ struct TcHot {                // everything the kernel's loops read: each role k
 struct alignas(64) TcProb {
     CUtensorMap map_a;        // activations (forward: a; dgrad: dy): (channel, pixel) or (channel, x, y, image), possibly element-strided
     CUtensorMap map_b;        // weights [K][taps][C] viewed as (C, tap, K)
-    CUtensorMap map_out;      // dense problems: the output as (channel, pixel), box 64 x 128
+    CUtensorMap map_out;      // dense problems: the output as (channel, pixel), box 64 x 32 (one warp's rows of a slab)
+    CUtensorMap map_bn;       // likewise bn_out
+    CUtensorMap map_add;      // dense problems: the residual, box 64 x 128
     TcHot h;
 };
 static_assert(sizeof(TcHot) % 4 == 0, "copied word by word");
 
-struct TcLaunch { int nprob, na, nb, a_stage, b_stage, tmem_cols, acc_stride, nbuf, groups, pg; };
-// nbuf: accumulators per tile of a pair (2: the next pair's MMAs run under this pair's epilogues); groups: epilogue groups (two: one
-// per tile of a pair; one: it takes both tiles in turn); pg: 16 KB staging buffers (one 64-column slab each) per group
+struct TcLaunch { int nprob, na, nb, a_stage, b_stage, tmem_cols, acc_stride, nbuf, groups, eb, res; };
+// nbuf: accumulators per tile of a pair (2: the next pair's MMAs run under this pair's epilogues); groups: epilogue groups (one per tile
+// of a pair); eb: 16 KB staging buffers (one 64-column slab each) per group; res: the staging buffers come through the residual warp
 constexpr int TC_MAX_PROBS = 128;             // descriptors per launch (sub-ResNets x output phases)
 
 __device__ __forceinline__ void copy_hot(TcHot* dst, const TcHot* src, int tid, int nthreads) {
@@ -176,28 +234,28 @@ __device__ __forceinline__ void copy_hot(TcHot* dst, const TcHot* src, int tid, 
 __global__ void __launch_bounds__(TC_CONV_THREADS, 1) conv_tc_kernel(const TcProb* __restrict__ probs, const TcLaunch L) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    __shared__ __align__(8) uint64_t bars[4 * TC_MAX_STAGES + 10];
+    __shared__ __align__(8) uint64_t bars[4 * TC_MAX_STAGES + 10 + 4 * TC_MAX_EB];
     __shared__ uint32_t tmem_base_s;
     __shared__ int abort_s;
-    __shared__ int pix_s2[2][TILE_M];
-    __shared__ float stat_s2[2][4][2][256];
+    __shared__ __align__(16) float stat_s2[2][4][2][256];
     __shared__ int unit_end_s[TC_MAX_PROBS];                      // running sum of the problems' unit counts (a unit: two row tiles x one column tile)
     __shared__ int tilesm_s[TC_MAX_PROBS], tilesn_s[TC_MAX_PROBS];
-    __shared__ TcHot hot_s[3 + TC_MAX_ISSUERS];                   // the current problem of the producer, the two epilogue groups, the MMA issuers
+    __shared__ TcHot hot_s[3 + TC_ISSUERS];                   // the current problem of the producer, the two epilogue groups, the MMA issuer
     const uint32_t a_full = smem_u32(&bars[0]), a_empty = smem_u32(&bars[TC_MAX_STAGES]);
     const uint32_t b_full = smem_u32(&bars[2 * TC_MAX_STAGES]), b_empty = smem_u32(&bars[3 * TC_MAX_STAGES]);
     const uint32_t acc_full = smem_u32(&bars[4 * TC_MAX_STAGES]), acc_empty = smem_u32(&bars[4 * TC_MAX_STAGES + 4]);
     const uint32_t drain = smem_u32(&bars[4 * TC_MAX_STAGES + 8]);
+    const uint32_t res_full = smem_u32(&bars[4 * TC_MAX_STAGES + 10]), res_empty = smem_u32(&bars[4 * TC_MAX_STAGES + 10 + 2 * TC_MAX_EB]);   // [group][slab buffer]
     const uint32_t a_ring = smem_u32(smem), b_ring = a_ring + (uint32_t)(L.na * L.a_stage), stg_base = b_ring + (uint32_t)(L.nb * L.b_stage);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp-uniform for the compiler too
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < TC_MAX_STAGES; ++s) {
-            mbar_init(a_full + 8 * s, 1); mbar_init(a_empty + 8 * s, 1); mbar_init(b_full + 8 * s, 1);
-            mbar_init(b_empty + 8 * s, TC_MAX_ISSUERS);          // a weight tile serves both tiles of a pair: both issuers release it
+            mbar_init(a_full + 8 * s, 1); mbar_init(a_empty + 8 * s, 1); mbar_init(b_full + 8 * s, 1); mbar_init(b_empty + 8 * s, 1);
         }
         for (int s = 0; s < 4; ++s) { mbar_init(acc_full + 8 * s, 1); mbar_init(acc_empty + 8 * s, 4); }
-        for (int s = 0; s < TC_MAX_ISSUERS; ++s) mbar_init(drain + 8 * s, 1);
+        mbar_init(drain, 1);
+        for (int s = 0; s < 2 * TC_MAX_EB; ++s) { mbar_init(res_full + 8 * s, 1); mbar_init(res_empty + 8 * s, 4); }
         abort_s = 0;
         int run = 0;
         for (int i = 0; i < L.nprob; ++i) {
@@ -216,54 +274,71 @@ __global__ void __launch_bounds__(TC_CONV_THREADS, 1) conv_tc_kernel(const TcPro
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = tmem_base_s;
     // A unit of work is a pair of neighbouring row tiles (2 x 128 positions) times one column tile: the two tiles share every weight
-    // tile, which is fetched once, and each has its own MMA-issuing warp and accumulator.  (One thread issues a tcgen05.mma only every
-    // ~150 cycles whatever its N (measured), more than the tensor core needs for it: two issuers keep it busy, and each tile's sum
-    // is still formed by one thread in a fixed order.)  The units of all problems, column tile innermost, are dealt round-robin: the
+    // tile, which is fetched once, and each has its own accumulator.  The units of all problems, column tile innermost, are dealt round-robin: the
     // CTAs that run side by side work on neighbouring tiles, share windows and weight tiles in L2 and read HBM as one moving front.
     // (Contiguous runs per CTA, with the column tile outermost, were measured too: no faster, and slower where the weights stream.)
-    const int u_begin = (int)blockIdx.x, u_stop = unit_end_s[L.nprob - 1], u_step = (int)gridDim.x;
+    // The last, partial wave: when at most half of the CTAs would get a pair of it, its pairs are split into single tiles (a pair of 256
+    // columns over 2304 reduction channels is 19 us of a launch of 60).
+    const int u_total = unit_end_s[L.nprob - 1], u_step = (int)gridDim.x, u_begin = (int)blockIdx.x;
+    const int u_full = u_total / u_step * u_step, u_rest = u_total - u_full;
+    const int u_split = 2 * u_rest <= u_step ? u_full : u_total, u_stop = u_split + 2 * (u_total - u_split);
+    struct Unit { int pi, tn, tm0, nt; };                        // problem, column tile, first row tile, row tiles (0: nothing to do)
+    auto decode = [&](int u) {
+        int half = -1;
+        if (u >= u_split) { half = (u - u_split) & 1; u = u_split + ((u - u_split) >> 1); }
+        Unit r; r.pi = 0; while (u >= unit_end_s[r.pi]) ++r.pi;
+        const int loc = u - (r.pi ? unit_end_s[r.pi - 1] : 0), tiles_n = tilesn_s[r.pi];
+        r.tm0 = 2 * (loc / tiles_n); r.tn = loc - (r.tm0 >> 1) * tiles_n;
+        r.nt = r.tm0 + 1 < tilesm_s[r.pi] ? 2 : 1;
+        if (half >= 0) { r.nt = half < r.nt ? 1 : 0; r.tm0 += half; }
+        return r;
+    };
 
     if (warp == 0) {
         // ---------------------------------------------------------------- TMA producer
-        if (lane == 0) {
+        if (elect_one()) {
             uint32_t a_cnt = 0, b_cnt = 0; bool ok = true;
             int cur = -1; TcHot& h = hot_s[0];
             int sa = 0, sb_ = 0; uint32_t pha = 0, phb = 0;       // ring positions and phases
             for (int u = u_begin; u < u_stop && ok; u += u_step) {
-                int pi = 0; while (u >= unit_end_s[pi]) ++pi;
+                const Unit un = decode(u);
+                if (!un.nt) continue;
+                const int pi = un.pi, tn = un.tn, tm0 = un.tm0, nt = un.nt;
                 if (pi != cur) { copy_hot(&h, &probs[pi].h, 0, 1); cur = pi; }
                 const TcProb* pp = probs + pi;
-                const int loc = u - (pi ? unit_end_s[pi - 1] : 0);
                 const int n_tile = h.n_tile, slabs = h.slabs, ngroups = h.ngroups, a_flat = h.a_flat, nbox = h.nbox,
                           a_box_bytes = h.a_box_bytes, R = h.R, Hp = h.Hp, pad = h.pad, es = h.es, b_bytes = h.b_bytes, mn = h.b_mn_major;
-                const int tiles_n = h.tiles_n, tn = loc % tiles_n, tm0 = 2 * (loc / tiles_n), nt = tm0 + 1 < h.tiles_m ? 2 : 1;
+                // first box of each tile's window: its image and its first tall row in that image (a box is rows of one image, or whole images)
+                int img0[2] = {0, 0}, row0[2] = {0, 0};
+                const int box_img = R > Hp ? R / max(Hp, 1) : 1, box_row = R > Hp ? Hp : R;
+                if (!a_flat)
+                    for (int j = 0; j < nt; ++j) { const int trow = floor_div((tm0 + j) * TILE_M - h.hb, h.box_pos) * R; img0[j] = floor_div(trow, Hp); row0[j] = trow - img0[j] * Hp; }
                 for (int sl = 0; sl < slabs && ok; ++sl) {
                     for (int g = 0; g < ngroups && ok; ++g) {
+                        const int gx = h.gxs[g], gy = h.gys[g], t_end = h.gbeg[g + 1];
                         for (int j = 0; j < nt; ++j) {
+                            const uint32_t dst = a_ring + (uint32_t)(sa * L.a_stage), full = a_full + 8 * sa;
                             if (!mbar_wait(a_empty + 8 * sa, pha ^ 1u, &abort_s)) { atomicExch(&abort_s, 1); report_wait(h.status, 1); ok = false; break; }
-                            const int tm = tm0 + j;
-                            const uint32_t dst = a_ring + (uint32_t)(sa * L.a_stage);
-                            mbar_expect_tx(a_full + 8 * sa, (uint32_t)(nbox * a_box_bytes));
-                            if (a_flat) tma_load_2d(dst, &pp->map_a, a_full + 8 * sa, sl * 64, tm * TILE_M);
+                            mbar_expect_tx(full, (uint32_t)(nbox * a_box_bytes));
+                            if (a_flat) tma_load_2d(dst, &pp->map_a, full, sl * 64, (tm0 + j) * TILE_M);
                             else {
-                                const int gx = h.gxs[g], gy = h.gys[g], bx0 = floor_div(tm * TILE_M - h.hb, h.box_pos);
+                                int img = img0[j], yy = row0[j];
                                 for (int i = 0; i < nbox; ++i) {
-                                    const int trow = (bx0 + i) * R, img = floor_div(trow, Hp), yy0 = trow - img * Hp;
-                                    tma_load_4d(dst + (uint32_t)(i * a_box_bytes), &pp->map_a, a_full + 8 * sa, sl * 64, gx, (yy0 - pad) * es + gy, img);
+                                    tma_load_4d(dst + (uint32_t)(i * a_box_bytes), &pp->map_a, full, sl * 64, gx, (yy - pad) * es + gy, img);
+                                    yy += box_row; if (yy >= Hp) { yy = 0; img += box_img; }
                                 }
                             }
                             ++a_cnt; if (++sa == L.na) { sa = 0; pha ^= 1u; }
                         }
                         if (!ok) break;
-                        const int t_end = h.gbeg[g + 1];
                         for (int tap = h.gbeg[g]; tap < t_end; ++tap) {
-                            if (!mbar_wait(b_empty + 8 * sb_, phb ^ 1u, &abort_s)) { atomicExch(&abort_s, 1); report_wait(h.status, 2); ok = false; break; }
-                            const uint32_t dst = b_ring + (uint32_t)(sb_ * L.b_stage);
+                            const uint32_t dst = b_ring + (uint32_t)(sb_ * L.b_stage), full = b_full + 8 * sb_;
                             const int wtap = h.wtap[tap];
-                            mbar_expect_tx(b_full + 8 * sb_, (uint32_t)b_bytes);
-                            if (!mn) tma_load_3d(dst, &pp->map_b, b_full + 8 * sb_, sl * 64, wtap, tn * n_tile);
+                            if (!mbar_wait(b_empty + 8 * sb_, phb ^ 1u, &abort_s)) { atomicExch(&abort_s, 1); report_wait(h.status, 2); ok = false; break; }
+                            mbar_expect_tx(full, (uint32_t)b_bytes);
+                            if (!mn) tma_load_3d(dst, &pp->map_b, full, sl * 64, wtap, tn * n_tile);
                             else for (int c = 0; c * 64 < n_tile; ++c)
-                                tma_load_3d(dst + (uint32_t)(c * 8192), &pp->map_b, b_full + 8 * sb_, tn * n_tile + c * 64, wtap, sl * 64);
+                                tma_load_3d(dst + (uint32_t)(c * 8192), &pp->map_b, full, tn * n_tile + c * 64, wtap, sl * 64);
                             ++b_cnt; if (++sb_ == L.nb) { sb_ = 0; phb ^= 1u; }
                         }
                     }
@@ -277,230 +352,243 @@ __global__ void __launch_bounds__(TC_CONV_THREADS, 1) conv_tc_kernel(const TcPro
                     for (int i = 0; i < 4096 && !mbar_try(b_full + 8 * (c % L.nb), (c / L.nb) & 1u); ++i) __nanosleep(64);
             }
         }
-    } else if (warp <= TC_MAX_ISSUERS) {
-        // ---------------------------------------------------------------- MMA issuers: warp 1 + j runs the reduction of tile j of every
-        // pair into its own accumulator.  Windows are per tile (the pair's two windows sit in consecutive ring stages); a weight stage
-        // is read by both issuers and released by both (an issuer whose pair has no second tile only passes the weight stages on).
-        const int me = warp - 1;
-        if (lane == 0) {
-            uint32_t a_cnt = 0, cnt = 0; bool ok = true;
-            int cur = -1; TcHot& h = hot_s[3 + me];
-            int sb = 0; uint32_t phb = 0;
-            // the constant part of a 128-byte-swizzle descriptor: stride between 8-row groups 1024 bytes, version, swizzle mode
-            const uint64_t desc_k = desc_sw128(0, 16, 1024), desc_mn = desc_sw128(0, 8192, 1024);
+    } else if (warp == 1) {
+        // ---------------------------------------------------------------- MMA issuer: the reductions of both tiles of a pair, each into its own
+        // accumulator.  (Everything the inner loops need sits in registers: between two asm statements the compiler would
+        // fetch a field of the shared descriptor again every time.)
+        if (elect_one()) {
+            uint32_t cnt[2] = {0u, 0u}; bool ok = true;
+            int cur = -1; TcHot& h = hot_s[3];
+            int sa = 0, sb = 0; uint32_t pha = 0, phb = 0;
+            const uint32_t nbuf1 = (uint32_t)L.nbuf - 1u;
+            // upper half of a 128-byte-swizzle descriptor: stride between 8-row groups 1024 bytes, version, swizzle mode; the lower half is the
+            // start address | leading-dimension offset << 16, both in 16-byte units
+            const uint32_t desc_hi = (uint32_t)(desc_sw128(0, 0, 1024) >> 32), a_lbo = 1u << 16;
             for (int u = u_begin; u < u_stop && ok; u += u_step) {
-                int pi = 0; while (u >= unit_end_s[pi]) ++pi;
-                if (pi != cur) { copy_hot(&h, &probs[pi].h, 0, 1); cur = pi; }
-                const int loc = u - (pi ? unit_end_s[pi - 1] : 0);
-                const int slabs = h.slabs, ngroups = h.ngroups, red = h.red, mn = h.b_mn_major;
-                const int tm0 = 2 * (loc / h.tiles_n), nt = tm0 + 1 < h.tiles_m ? 2 : 1, tm = tm0 + me;
-                const bool has = me < nt;
-                const int bx0 = h.a_flat ? 0 : floor_div(tm * TILE_M - h.hb, h.box_pos);
-                const int a_off = h.a_flat ? 0 : tm * TILE_M - h.hb - bx0 * h.box_pos;
-                const uint32_t buf = (cnt % (uint32_t)L.nbuf) * 2u + (uint32_t)me, aph = (cnt / (uint32_t)L.nbuf) & 1u;
-                if (has) {
-                    ++cnt;
+                const Unit un = decode(u);
+                if (!un.nt) continue;
+                const int nt = un.nt;
+                if (un.pi != cur) { copy_hot(&h, &probs[un.pi].h, 0, 1); cur = un.pi; }
+                const int slabs = h.slabs, ngroups = h.ngroups, red = h.red, mn = h.b_mn_major, a_flat = h.a_flat, hb = h.hb, box_pos = h.box_pos;
+                uint32_t a_off[2], d_tmem[2], full_bar[2];
+                for (int j = 0; j < nt; ++j) {
+                    const int p0 = (un.tm0 + j) * TILE_M - hb;
+                    a_off[j] = a_flat ? 0u : (uint32_t)(p0 - floor_div(p0, box_pos) * box_pos) * 8u;
+                    const uint32_t buf = (cnt[j] & nbuf1) * 2u + (uint32_t)j, aph = (cnt[j] >> nbuf1) & 1u;
+                    ++cnt[j];
+                    d_tmem[j] = tmem_base + buf * (uint32_t)L.acc_stride; full_bar[j] = acc_full + 8 * buf;
                     if (!mbar_wait(acc_empty + 8 * buf, aph ^ 1u, &abort_s)) { atomicExch(&abort_s, 1); report_wait(h.status, 3); ok = false; break; }
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 }
-                const uint32_t d_tmem = tmem_base + buf * (uint32_t)L.acc_stride;
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 // instruction descriptor: fp32 accumulate, bf16 x bf16, A K-major, B K-major or MN-major, N, M = 128
-                const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)mn << 16) |
-                                       ((uint32_t)(h.n_tile >> 3) << 17) | ((128u >> 4) << 24);
-                const uint64_t b_const = mn ? desc_mn : desc_k;
+                const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)mn << 16) | ((uint32_t)(h.n_tile >> 3) << 17) | ((128u >> 4) << 24);
+                const uint32_t b_lbo = mn ? (8192u >> 4) << 16 : 1u << 16;
                 const uint32_t b_step = mn ? 128u : 2u;           // one K = 16 step: 16 rows of 128 bytes (MN-major) or 32 bytes along the row (K-major), in 16-byte units
                 uint32_t acc = 0;
                 for (int sl = 0; sl < slabs && ok; ++sl) {
                     const int ksteps = (min(64, red - sl * 64) + 15) >> 4;
                     for (int g = 0; g < ngroups && ok; ++g) {
-                        const uint32_t ai = a_cnt + (uint32_t)me; a_cnt += (uint32_t)nt;
-                        const uint32_t sa = ai % (uint32_t)L.na, pha = (ai / (uint32_t)L.na) & 1u;
-                        if (has) {
-                            if (!mbar_wait(a_full + 8 * sa, pha, &abort_s)) { atomicExch(&abort_s, 1); report_wait(h.status, 4); ok = false; break; }
-                            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                        }
-                        const uint32_t a_rows16 = ((a_ring + sa * (uint32_t)L.a_stage) >> 4) + (uint32_t)a_off * 8u;   // start address in 16-byte units
+                        uint32_t a_lo[2], a_rel[2];
                         const int t_end = h.gbeg[g + 1];
-                        for (int tap = h.gbeg[g]; tap < t_end; ++tap) {
+                        for (int j = 0; j < nt; ++j) {
+                            if (!mbar_wait(a_full + 8 * sa, pha, &abort_s)) { atomicExch(&abort_s, 1); report_wait(h.status, 4); ok = false; break; }
+                            a_lo[j] = (((a_ring + (uint32_t)(sa * L.a_stage)) >> 4) + a_off[j]) | a_lbo; a_rel[j] = a_empty + 8 * sa;
+                            if (++sa == L.na) { sa = 0; pha ^= 1u; }
+                        }
+                        for (int tap = h.gbeg[g]; tap < t_end && ok; ++tap) {
+                            const uint32_t shift = (uint32_t)h.shift[tap] * 8u, b_lo = ((b_ring + (uint32_t)(sb * L.b_stage)) >> 4) | b_lbo;
                             if (!mbar_wait(b_full + 8 * sb, phb, &abort_s)) { atomicExch(&abort_s, 1); report_wait(h.status, 5); ok = false; break; }
-                            if (has) {
-                                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                                const uint32_t a16 = a_rows16 + (uint32_t)h.shift[tap] * 8u;
-                                const uint32_t b16 = (b_ring + (uint32_t)(sb * L.b_stage)) >> 4;
-                                for (int k16 = 0; k16 < ksteps; ++k16) {
-                                    umma_bf16(d_tmem, desc_k | (uint64_t)((a16 + 2u * (uint32_t)k16) & 0x3FFFu), b_const | (uint64_t)((b16 + b_step * (uint32_t)k16) & 0x3FFFu), idesc, acc);
-                                    acc = 1;
-                                }
-                                umma_commit(b_empty + 8 * sb);   // this issuer's share of the release: once its MMAs have read the weight tile
-                            } else mbar_arrive(b_empty + 8 * sb);
+#pragma unroll
+                            for (int j = 0; j < 2; ++j) {
+                                if (j >= nt) break;
+                                if (ksteps == 4) {
+#pragma unroll
+                                    for (int k16 = 0; k16 < 4; ++k16)
+                                        umma_bf16(d_tmem[j], f2_pack(a_lo[j] + shift + 2u * (uint32_t)k16, desc_hi), f2_pack(b_lo + b_step * (uint32_t)k16, desc_hi), idesc, k16 ? 1u : acc);
+                                } else
+                                    for (int k16 = 0; k16 < ksteps; ++k16)
+                                        umma_bf16(d_tmem[j], f2_pack(a_lo[j] + shift + 2u * (uint32_t)k16, desc_hi), f2_pack(b_lo + b_step * (uint32_t)k16, desc_hi), idesc, k16 ? 1u : acc);
+                            }
+                            acc = 1;
+                            umma_commit(b_empty + 8 * sb);       // released once these MMAs have read the weight tile
                             if (++sb == L.nb) { sb = 0; phb ^= 1u; }
                         }
-                        if (has && ok) umma_commit(a_empty + 8 * sa);
+                        if (ok) for (int j = 0; j < nt; ++j) umma_commit(a_rel[j]);
                     }
                 }
-                if (has && ok) umma_commit(acc_full + 8 * buf);  // accumulator complete
+                if (ok) for (int j = 0; j < nt; ++j) umma_commit(full_bar[j]);   // accumulators complete
             }
             if (!ok) {
                 // gave up: the MMAs already issued must have finished before the CTA frees its tensor memory
-                umma_commit(drain + 8 * me);
-                for (int i = 0; i < 65536 && !mbar_try(drain + 8 * me, 0u); ++i) __nanosleep(64);
+                umma_commit(drain);
+                for (int i = 0; i < 65536 && !mbar_try(drain, 0u); ++i) __nanosleep(64);
             }
+        }
+    } else if (warp == TC_RES_WARP) {
+        // ---------------------------------------------------------------- residual of dense problems: its 128 x 64 boxes go straight into
+        // the staging slabs the epilogue will add to and store from, up to L.eb slabs ahead per group
+        if (L.res && elect_one()) {
+            bool ok = true; uint32_t q[2] = {0u, 0u};
+            for (int u = u_begin; u < u_stop && ok; u += u_step) {
+                const Unit un = decode(u);
+                if (!un.nt) continue;
+                const TcHot* hp = &probs[un.pi].h;
+                const int load = __ldg(&hp->res_tma), out_slabs = __ldg(&hp->out_slabs), col0 = un.tn * __ldg(&hp->n_tile);
+                for (int sl = 0; sl < out_slabs && ok; ++sl)
+                    for (int j = 0; j < un.nt; ++j) {
+                        const uint32_t sb = (uint32_t)j * TC_MAX_EB + q[j] % (uint32_t)L.eb;
+                        if (!mbar_wait(res_empty + 8 * sb, ((q[j] / (uint32_t)L.eb) & 1u) ^ 1u, &abort_s)) { atomicExch(&abort_s, 1); report_wait(probs[un.pi].h.status, 7); ok = false; break; }
+                        if (!load) mbar_arrive(res_full + 8 * sb);           // a problem without residual in the same launch only passes through the ring
+                        else { mbar_expect_tx(res_full + 8 * sb, (uint32_t)SLAB_BYTES);
+                        tma_load_2d(stg_base + ((uint32_t)(j * L.eb) + q[j] % (uint32_t)L.eb) * SLAB_BYTES, &probs[un.pi].map_add, res_full + 8 * sb, col0 + sl * 64, (un.tm0 + j) * TILE_M); }
+                        ++q[j];
+                    }
+            }
+            if (!ok)
+                for (int j = 0; j < 2; ++j)
+                    for (uint32_t c = q[j] > (uint32_t)L.eb ? q[j] - L.eb : 0; c < q[j]; ++c)
+                        for (int i = 0; i < 4096 && !mbar_try(res_full + 8 * ((uint32_t)j * TC_MAX_EB + c % (uint32_t)L.eb), (c / (uint32_t)L.eb) & 1u); ++i) __nanosleep(64);
         }
     } else {
         // ---------------------------------------------------------------- epilogue: two groups of 4 warps (one TMEM lane quadrant each);
-        // group g takes tile g of every pair, so two epilogues run side by side (a single group takes both tiles in turn)
-        const int grp = (warp - 1 - TC_MAX_ISSUERS) >> 2, bid = 1 + grp;
+        // group g takes tile g of every pair.  Inside a tile the warps do not wait for one another: each stages and stores its own
+        // 32 rows, slab by slab of 64 columns, through its quarter of the group's slab buffers.
+        const int grp = (warp - 1 - TC_ISSUERS) >> 2, bid = 1 + grp;
         const int quad = warp & 3;
         const int m = quad * 32 + lane;                          // row of the tile = TMEM lane
-        const int et = threadIdx.x - 32 * (1 + TC_MAX_ISSUERS) - grp * 128;   // 0..127 among the group's threads
-        const bool leader = et == 0;
-        int* const pix_s = pix_s2[grp];
+        const int et = threadIdx.x - 32 * (1 + TC_ISSUERS) - grp * 128;   // 0..127 among the group's threads
         float (*const stat_s)[2][256] = stat_s2[grp];
+        float4* const bnc_s = reinterpret_cast<float4*>(&stat_s2[grp][0][0][0]);   // evaluation keeps no statistics: mean, 1/std, gamma, beta per column
         bool ok = true;
-        int cur = -1; const TcHot& h = hot_s[1 + grp];
-        uint32_t sc = 0, cnt[2] = {0u, 0u};                      // 64-column slabs this group has staged; tiles taken of each half of the pairs
-        for (int u = u_begin; grp < L.groups && u < u_stop && ok; u += u_step) {
-          int pi = 0; while (u >= unit_end_s[pi]) ++pi;
-          const TcProb* pp = probs + pi;
-          const int loc = u - (pi ? unit_end_s[pi - 1] : 0);
-          const int tn = loc % tilesn_s[pi], tm0 = 2 * (loc / tilesn_s[pi]), nt = tm0 + 1 < tilesm_s[pi] ? 2 : 1;
-          for (int hf = L.groups == 2 ? grp : 0; hf < nt && ok; hf += L.groups == 2 ? 2 : 1) {
-            const int tm = tm0 + hf;
-            const uint32_t buf = (cnt[hf] % (uint32_t)L.nbuf) * 2u + (uint32_t)hf, aph = (cnt[hf] / (uint32_t)L.nbuf) & 1u;
-            ++cnt[hf];
-            // every warp must have finished its share of the last tile's copy-out (it reads the pixel table)
-            bar_sync_epi(bid);
-            if (pi != cur) { copy_hot(&hot_s[1 + grp], &probs[pi].h, et, 128); cur = pi; bar_sync_epi(bid); }
-            const int n_tile = h.n_tile, ncol = h.ncol, add_mode = h.add_mode, dense = h.dense;
+        int cur = -1, cur_tn = -1; const TcHot& h = hot_s[1 + grp];
+        uint32_t sc = 0, cnt = 0;                                // slabs staged; tiles taken
+        const uint32_t eb = (uint32_t)L.eb, lag = eb >= 3u ? 2u : 1u;   // a slab is handed back to the residual warp when the store `lag` slabs later is due
+        for (int u = u_begin; u < u_stop; u += u_step) {
+            const Unit un = decode(u);
+            if (grp >= un.nt) continue;
+            const int pi = un.pi, tn = un.tn, tm = un.tm0 + grp;
+            const TcProb* pp = probs + pi;
+            const uint32_t buf = (cnt % (uint32_t)L.nbuf) * 2u + (uint32_t)grp, aph = (cnt / (uint32_t)L.nbuf) & 1u;
+            ++cnt;
+            if (pi != cur || (h.bn_out && tn != cur_tn)) {       // every warp of the group is through with the last problem's constants
+                bar_sync_epi(bid);
+                if (pi != cur) copy_hot(&hot_s[1 + grp], &probs[pi].h, et, 128);
+                bar_sync_epi(bid);
+                if (h.bn_out) {
+                    for (int c = et; c < h.n_tile; c += 128) {
+                        const int g = min(tn * h.n_tile + c, h.ncol - 1);
+                        bnc_s[c] = make_float4(__ldg(h.bn_stat + g), __ldg(h.bn_stat + h.ncol + g), __ldg(h.bn_gamma + g), __ldg(h.bn_beta + g));
+                    }
+                    bar_sync_epi(bid);
+                }
+                cur = pi; cur_tn = tn;
+            }
+            const int n_tile = h.n_tile, ncol = h.ncol, add_mode = h.add_mode, dense = h.dense, res_tma = h.res_tma, store_y = h.store_y;
             const float scale = h.scale;
-            const __nv_bfloat16* addp = h.add; __nv_bfloat16* outp = h.out; float* stat_tiles = h.stat_tiles;
+            const __nv_bfloat16* addp = h.add; __nv_bfloat16* outp = h.out; float* stat_tiles = h.stat_tiles; __nv_bfloat16* bn_out = h.bn_out;
             // position -> output pixel (and the residual's pixel)
             const int pos = tm * TILE_M + m;
             bool valid = pos < h.total_pos;
-            long long pix = pos, addpix = -1;
+            int pix = pos; long long addpix = -1;
             if (valid && (!dense || add_mode == 3)) {
                 const int Wp = h.Wp, Hp = h.Hp, pad = h.pad, os = h.os, OH = h.OH, OW = h.OW;
                 const int trow = pos / Wp, xx = pos - trow * Wp, img = trow / Hp, yy = trow - img * Hp;
                 const int y = (yy - pad) * os + h.oy, x = xx * os + h.ox;
                 valid = yy >= pad && xx < Wp - pad && y < OH && x < OW;
-                pix = ((long long)img * OH + y) * OW + x;
+                pix = (img * OH + y) * OW + x;
                 if (add_mode == 3 && !((y | x) & 1)) addpix = ((long long)img * ((OH + 1) >> 1) + (y >> 1)) * ((OW + 1) >> 1) + (x >> 1);
             }
             if (add_mode == 2) addpix = pix;
-            if (!dense) pix_s[m] = valid ? (int)pix : -1;
+            if (!valid) pix = -1;
             const int col0 = tn * n_tile;
-            const bool gadd = add_mode >= 2 && valid && addpix >= 0;
-            // the residual of a 32-column step is fetched one step ahead of its use (the first one ahead of the accumulator)
+            const bool gadd = !res_tma && add_mode >= 2 && valid && addpix >= 0;
+            // a residual that TMA cannot bring: the first slab's is read ahead of the accumulator, a later one's once the last has been used
             const __nv_bfloat16* addrow = addp + (gadd ? addpix : 0) * ncol + col0;
-            uint4 ga[4], gn[4];
+            uint4 ga[8];
+            auto load_add = [&](int c0) {                        // the 64 columns of a slab
 #pragma unroll
-            for (int g = 0; g < 4; ++g) gn[g] = (gadd && g * 8 < n_tile && col0 + g * 8 < ncol) ? __ldg(reinterpret_cast<const uint4*>(addrow + g * 8)) : make_uint4(0u, 0u, 0u, 0u);
-            if (add_mode == 2 && dense) {
-                // the residual rows of the group's next tile are asked into L2 now, a whole tile ahead of their use
-                int u2 = u, hf2 = hf + (L.groups == 2 ? 2 : 1);
-                if (hf2 >= nt) { u2 = u + u_step; hf2 = L.groups == 2 ? grp : 0; }
-                if (u2 < unit_end_s[pi]) {                       // same problem (else the next tile's own first loads have to do)
-                    const int loc2 = u2 - (pi ? unit_end_s[pi - 1] : 0);
-                    const int tn2 = loc2 % tilesn_s[pi], tm2 = 2 * (loc2 / tilesn_s[pi]) + hf2;
-                    const long long pos2 = (long long)tm2 * TILE_M + m;
-                    if (tm2 < tilesm_s[pi] && pos2 < h.total_pos) {
-                        const __nv_bfloat16* r2 = addp + pos2 * ncol + tn2 * n_tile;
-                        for (int c = 0; c < n_tile && tn2 * n_tile + c < ncol; c += 64)
-                            asm volatile("prefetch.global.L2 [%0];" ::"l"(r2 + c));
-                    }
-                }
-            }
+                for (int g = 0; g < 8; ++g) { const int c = c0 + g * 8; ga[g] = (gadd && c < n_tile && col0 + c < ncol) ? __ldg(reinterpret_cast<const uint4*>(addrow + c)) : make_uint4(0u, 0u, 0u, 0u); }
+            };
+            const bool any_gadd = !res_tma && add_mode >= 2;
+            if (any_gadd) load_add(0);
+            const uint32_t scw = __float_as_uint(valid ? scale : 0.f);
+            const uint64_t scale2 = f2_pack(scw, scw);
             ok = mbar_wait(acc_full + 8 * buf, aph, &abort_s);
-            ok = bar_and_epi(bid, ok);                           // one decision for the four warps: they share the barriers below
+            __syncwarp();
+            ok = bar_and_epi(bid, ok);                           // one decision for the four warps: they share the group's barriers
             if (!ok) { atomicExch(&abort_s, 1); report_wait(h.status, 6); break; }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t t_row = tmem_base + buf * (uint32_t)L.acc_stride + ((uint32_t)(quad * 32) << 16);
-            // The tile leaves in slabs of 64 columns: a slab is rounded and (with the residual added) written to a 16 KB staging
-            // buffer in the 128-byte-swizzle layout, then stored by TMA (dense problems) or copied out row by row, while the next
-            // slab is staged in the group's other buffer.
-            for (int c0 = 0; c0 < n_tile; c0 += 32) {
-                const int slab = c0 >> 6;
-                const bool slab_begin = !(c0 & 32), slab_end = (c0 & 32) || c0 + 32 >= n_tile, last = c0 + 32 >= n_tile;
-                const uint32_t stg = stg_base + ((uint32_t)(grp * L.pg) + sc % (uint32_t)L.pg) * SLAB_BYTES;
-                if (slab_begin) {
-                    if (leader) bulk_wait_read(L.pg - 1);        // the bulk store issued from this buffer has read it
-                    bar_sync_epi(bid);                           // ... and every warp is done with what it last held
+            for (int s0 = 0; s0 < n_tile; s0 += 64) {
+                const uint32_t sbuf = sc % eb;
+                const uint32_t stg = stg_base + ((uint32_t)grp * eb + sbuf) * SLAB_BYTES, stg2 = stg_base + ((uint32_t)L.groups * eb + (uint32_t)grp) * SLAB_BYTES;
+                if (elect_one()) {                               // the store last issued from this buffer has been read (with a BN: from the group's BN buffer too)
+                    bulk_wait_read(bn_out ? 0 : L.res ? (int)lag - 1 : (int)eb - 1);
+                    if (L.res && sc >= lag) mbar_arrive(res_empty + 8 * ((uint32_t)grp * TC_MAX_EB + (sc - lag) % eb));
                 }
-                uint32_t v[32];
-                tmem_ld32(t_row + (uint32_t)c0, v);
-#pragma unroll
-                for (int g = 0; g < 4; ++g) {
-                    ga[g] = gn[g];
-                    const int c = c0 + 32 + g * 8;
-                    gn[g] = (gadd && c < n_tile && col0 + c < ncol) ? __ldg(reinterpret_cast<const uint4*>(addrow + c)) : make_uint4(0u, 0u, 0u, 0u);
-                }
+                __syncwarp();
+                if (L.res && !mbar_wait(res_full + 8 * ((uint32_t)grp * TC_MAX_EB + sbuf), (sc / eb) & 1u, &abort_s)) { atomicExch(&abort_s, 1); report_wait(h.status, 8); }
+                __syncwarp();
+                ++sc;
+                // 64 columns, or 32 if the tile ends there: columns past the tile's own are never stored (n_tile is a multiple of 64 or covers
+                // all of the tensor's columns)
+                const uint32_t st = (stg + (uint32_t)m * 128u) ^ ((uint32_t)(m & 7) << 4), st2 = (stg2 + (uint32_t)m * 128u) ^ ((uint32_t)(m & 7) << 4);
+                const bool two = s0 + 32 < n_tile;
+                uint32_t v[2][32];
+                tmem_ld32(t_row + (uint32_t)s0, v[0]);
+                if (two) tmem_ld32(t_row + (uint32_t)(s0 + 32), v[1]);
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                if (last) {
+                if (s0 + 64 >= n_tile) {
                     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                     __syncwarp();
                     if (lane == 0) mbar_arrive(acc_empty + 8 * buf); // this warp has read its quadrant of the accumulator
                 }
-                const uint32_t s_row = stg + (uint32_t)m * 128u;
-#pragma unroll
-                for (int g = 0; g < 4; ++g) {
-                    const int c = c0 + g * 8;
-                    if (c < n_tile) {
-                        const uint32_t sa = s_row + ((uint32_t)(((c >> 3) & 7) ^ (m & 7)) << 4);
-                        float f[8];
-#pragma unroll
-                        for (int k = 0; k < 8; ++k) f[k] = valid ? __uint_as_float(v[g * 8 + k]) * scale : 0.f;
-                        if (gadd) {
-                            const uint32_t aw[4] = {ga[g].x, ga[g].y, ga[g].z, ga[g].w};
-#pragma unroll
-                            for (int k = 0; k < 4; ++k) {
-                                f[2 * k] += __uint_as_float(aw[k] << 16);
-                                f[2 * k + 1] += __uint_as_float(aw[k] & 0xFFFF0000u);
-                            }
-                        }
-                        uint32_t w[4];
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            __nv_bfloat162 hh = __floats2bfloat162_rn(f[2 * k], f[2 * k + 1]);
-                            w[k] = *reinterpret_cast<uint32_t*>(&hh);
-                        }
-                        sts128(sa, make_uint4(w[0], w[1], w[2], w[3]));
+                const float4* bq = bnc_s + s0;
+                if (!bn_out && res_tma) { epi_cols<true, false, false>(v[0], st, st2, 0, scale2, ga, bq); if (two) epi_cols<true, false, false>(v[1], st, st2, 4, scale2, ga, bq); }
+                else if (!bn_out && !any_gadd) { epi_cols<false, false, false>(v[0], st, st2, 0, scale2, ga, bq); if (two) epi_cols<false, false, false>(v[1], st, st2, 4, scale2, ga, bq); }
+                else if (!bn_out) { epi_cols<false, true, false>(v[0], st, st2, 0, scale2, ga, bq); if (two) epi_cols<false, true, false>(v[1], st, st2, 4, scale2, ga + 4, bq); }
+                else if (res_tma) { epi_cols<true, false, true>(v[0], st, st2, 0, scale2, ga, bq); if (two) epi_cols<true, false, true>(v[1], st, st2, 4, scale2, ga, bq + 32); }
+                else if (!any_gadd) { epi_cols<false, false, true>(v[0], st, st2, 0, scale2, ga, bq); if (two) epi_cols<false, false, true>(v[1], st, st2, 4, scale2, ga, bq + 32); }
+                else { epi_cols<false, true, true>(v[0], st, st2, 0, scale2, ga, bq); if (two) epi_cols<false, true, true>(v[1], st, st2, 4, scale2, ga + 4, bq + 32); }
+                if (any_gadd && s0 + 64 < n_tile) load_add(s0 + 64);
+                if (dense) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the bulk store reads what this thread wrote
+                __syncwarp();                                    // the warp's 32 rows of the slab are complete
+                if (dense) {
+                    if (elect_one()) {
+                        if (store_y) tma_store_2d(&pp->map_out, stg + (uint32_t)quad * 4096u, col0 + s0, tm * TILE_M + quad * 32);
+                        if (bn_out) tma_store_2d(&pp->map_bn, stg2 + (uint32_t)quad * 4096u, col0 + s0, tm * TILE_M + quad * 32);
+                        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                     }
-                }
-                if (!slab_end) continue;
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // the bulk store reads what this thread wrote
-                bar_sync_epi(bid);                               // the slab is complete
-                if (dense && leader) {
-                    tma_store_2d(&pp->map_out, stg, col0 + slab * 64, tm * TILE_M);
-                    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                } else {
+                    // copy-out of a tall slab: 16-byte chunks, eight consecutive lanes per 128-byte run of one output pixel
+                    const int ch = lane & 7, c = s0 + ch * 8;
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int row = i * 4 + (lane >> 3), px = __shfl_sync(0xffffffffu, pix, row);
+                        if (px >= 0 && c < n_tile && col0 + c < ncol) {
+                            const uint32_t so = (uint32_t)(quad * 32 + row) * 128u + ((uint32_t)(ch ^ (row & 7)) << 4);
+                            if (store_y) *reinterpret_cast<uint4*>(outp + (long long)px * ncol + col0 + c) = lds128(stg + so);
+                            if (bn_out) *reinterpret_cast<uint4*>(bn_out + (long long)px * ncol + col0 + c) = lds128(stg2 + so);
+                        }
+                    }
                 }
                 if (stat_tiles) {
                     // column sums of the stored (rounded) values: every warp over its own 32 rows, lane = two neighbouring columns;
                     // the four warps' sums are added in a fixed order once the tile's last slab is through
-                    float s0 = 0.f, s1 = 0.f, q0 = 0.f, q1 = 0.f;
+                    uint64_t su = 0, sq = 0;
 #pragma unroll 8
                     for (int r = 0; r < 32; ++r) {
-                        const int row = quad * 32 + r;
-                        const uint32_t uu = lds32(stg + (uint32_t)row * 128u + ((uint32_t)((lane >> 2) ^ (row & 7)) << 4) + ((uint32_t)(lane & 3) << 2));
-                        const float lo = __uint_as_float(uu << 16), hi = __uint_as_float(uu & 0xFFFF0000u);
-                        s0 += lo; q0 += lo * lo; s1 += hi; q1 += hi * hi;
+                        const uint64_t x = f2_of_bf16x2(lds32(stg + (uint32_t)(quad * 32 + r) * 128u + ((uint32_t)((lane >> 2) ^ (r & 7)) << 4) + ((uint32_t)(lane & 3) << 2)));
+                        su = f2_add(su, x); sq = f2_fma(x, x, sq);
                     }
-                    stat_s[quad][0][slab * 64 + 2 * lane] = s0; stat_s[quad][0][slab * 64 + 2 * lane + 1] = s1;
-                    stat_s[quad][1][slab * 64 + 2 * lane] = q0; stat_s[quad][1][slab * 64 + 2 * lane + 1] = q1;
+                    *reinterpret_cast<uint64_t*>(&stat_s[quad][0][s0 + 2 * lane]) = su;
+                    *reinterpret_cast<uint64_t*>(&stat_s[quad][1][s0 + 2 * lane]) = sq;
                 }
-                if (!dense) {
-                    // copy-out of a tall slab: 16-byte chunks, eight consecutive lanes per 128-byte run of one output pixel
-                    for (int idx = et; idx < TILE_M * 8; idx += 128) {
-                        const int ch = idx & 7, row = idx >> 3;
-                        const int c = slab * 64 + ch * 8, px = pix_s[row];
-                        if (px >= 0 && c < n_tile && col0 + c < ncol)
-                            *reinterpret_cast<uint4*>(outp + (long long)px * ncol + col0 + c) =
-                                lds128(stg + (uint32_t)row * 128u + ((uint32_t)(ch ^ (row & 7)) << 4));
-                    }
-                }
-                ++sc;
+                __syncwarp();
             }
             if (stat_tiles) {
-                bar_sync_epi(bid);
+                bar_sync_epi(bid);                               // (the next tile's barrier behind its accumulator keeps these sums until they are read)
                 for (int c = et; c < n_tile; c += 128) {
                     if (col0 + c < ncol) {
                         const float su = ((stat_s[0][0][c] + stat_s[1][0][c]) + stat_s[2][0][c]) + stat_s[3][0][c];
@@ -510,9 +598,8 @@ __global__ void __launch_bounds__(TC_CONV_THREADS, 1) conv_tc_kernel(const TcPro
                     }
                 }
             }
-          }
         }
-        if (leader) bulk_wait_read(0);                           // shared memory stays until the last bulk stores have read it
+        if (elect_one()) bulk_wait_read(0);                      // shared memory stays until the last bulk stores have read it
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -597,7 +684,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) conv_wgrad_tc_kernel(const TcWg
     const uint32_t bar_full = smem_u32(&bars[0]), bar_empty = smem_u32(&bars[TC_MAX_STAGES]), bar_acc = smem_u32(&bars[2 * TC_MAX_STAGES]);
     const uint32_t bar_drain = smem_u32(&bars[2 * TC_MAX_STAGES + 1]);
     const uint32_t ring = smem_u32(smem);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp-uniform for the compiler too
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < TC_MAX_STAGES; ++s) { mbar_init(bar_full + 8 * s, 1); mbar_init(bar_empty + 8 * s, 2); }   // both issuers release a stage
@@ -616,7 +703,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) conv_wgrad_tc_kernel(const TcWg
     const uint32_t tmem_d = tmem_base_s;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             int i = 0; bool ok = true; int s = 0; uint32_t ph = 0;
             const uint32_t tx = (uint32_t)(2 * nbox_dy * dy_box_bytes + a_slabs * nbox_a * a_box_bytes);
             for (; i < nc; ++i) {
@@ -656,7 +743,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) conv_wgrad_tc_kernel(const TcWg
         // group's taps are split between them; with an odd number of taps the last tap's 128 positions are split instead, each
         // half into an accumulator of its own (the epilogue adds the two, first half first).  So every accumulator is written
         // by one thread, in a fixed order.
-        if (lane == 0) {
+        if (elect_one()) {
             const int me = warp - 1, odd = ntap & 1, whole = (ntap - odd) >> 1;
             int it_tap[3], it_acc[3], it_k0[3], it_k1[3], nit = 0;
             for (int q = 0; q < whole; ++q) { it_tap[nit] = me * whole + q; it_acc[nit] = me * whole + q; it_k0[nit] = 0; it_k1[nit] = 8; ++nit; }
@@ -677,6 +764,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) conv_wgrad_tc_kernel(const TcWg
                     const uint32_t at16 = a16 + (uint32_t)shift8_s[it_tap[q]];
                     const uint32_t d_t = tmem_d + (uint32_t)(it_acc[q] * n_tile);
                     const int k0 = it_k0[q], k1 = it_k1[q];
+#pragma unroll 4
                     for (int k16 = k0; k16 < k1; ++k16)        // 16 positions = 16 rows of 128 bytes per step
                         umma_bf16(d_t, dy_const | (uint64_t)((dy16 + 128u * (uint32_t)k16) & 0x3FFFu), a_const | (uint64_t)((at16 + 128u * (uint32_t)k16) & 0x3FFFu), idesc, (i || k16 != k0) ? 1u : 0u);
                 }
@@ -800,9 +888,9 @@ static bool encode_map(CUtensorMap* m, const void* base, int rank, const uint64_
     return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(base), d, st, b, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
-// [pixels][chan] as (channel, pixel), box 64 x 128
-static bool encode_flat(CUtensorMap* m, const void* base, int chan, long long pixels) {
-    const uint64_t dims[2] = {(uint64_t)chan, (uint64_t)pixels}; const uint64_t st[1] = {(uint64_t)chan * 2}; const uint32_t box[2] = {64, 128};
+// [pixels][chan] as (channel, pixel), box 64 x rows
+static bool encode_flat(CUtensorMap* m, const void* base, int chan, long long pixels, int rows = 128) {
+    const uint64_t dims[2] = {(uint64_t)chan, (uint64_t)pixels}; const uint64_t st[1] = {(uint64_t)chan * 2}; const uint32_t box[2] = {64, (uint32_t)rows};
     return encode_map(m, base, 2, dims, st, box);
 }
 // [n_img][H][W][chan] as (channel, x, y, image): a box is box_h rows of Wp window positions of box_n images, every es-th pixel in x and y
@@ -976,8 +1064,12 @@ int conv_tc_fill(const ConvProb& p, int mode, void* host_tc) {
           const uint64_t st[2] = {(uint64_t)p.C * 2, (uint64_t)taps * p.C * 2};
           const uint32_t box[3] = {64, 1, mode == CONV_FWD ? (uint32_t)t.n_tile : 64u};
           if (!encode_map(&tp.map_b, p.wgt, 3, dims, st, box)) return 0; }
+        t.store_y = 1;
+        if (p.bn_out) { t.bn_out = (__nv_bfloat16*)p.bn_out; t.bn_stat = p.bn_stat; t.bn_gamma = p.bn_gamma; t.bn_beta = p.bn_beta; t.store_y = p.bn_only ? 0 : 1; }
         if (t.dense) {
-            if (!encode_flat(&tp.map_out, p.out, ncol, out_pixels)) return 0;
+            if (!encode_flat(&tp.map_out, p.out, ncol, out_pixels, 32)) return 0;
+            if (p.bn_out && !encode_flat(&tp.map_bn, p.bn_out, ncol, out_pixels, 32)) return 0;
+            if (t.add_mode == 2) { t.res_tma = 1; if (!encode_flat(&tp.map_add, p.add, ncol, out_pixels)) return 0; }
         }
         memcpy((char*)host_tc + (size_t)ph * sizeof(TcProb), &tp, sizeof(tp));
     }
@@ -986,16 +1078,16 @@ int conv_tc_fill(const ConvProb& p, int mode, void* host_tc) {
 size_t conv_tc_prob_bytes() { return sizeof(TcProb); }
 // units of work of a problem: pairs of row tiles x column tiles
 int conv_tc_tiles(const void* host_tc) { const TcHot* t = &((const TcProb*)host_tc)->h; return ((t->tiles_m + 1) / 2) * t->tiles_n; }
-// packs what a launch has to know about its largest problem into one number: window KB (12 bits), weight-tile KB (12), staging
-// tiles (4), KB of all weight tiles of a column tile (16), MMA N (20)
+// packs what a launch has to know about its largest problem into one number: window KB (12 bits), weight-tile KB (12), flags
+// (4; 1: residual through TMA, 2: BN of the output), KB of all weight tiles of a column tile (16), MMA N (20)
 size_t conv_tc_smem(const void* host_tc) {
     const TcHot* t = &((const TcProb*)host_tc)->h;
     const size_t a_stage = ((size_t)t->nbox * t->a_box_bytes + 1023) / 1024, b_stage = ((size_t)t->b_bytes + 1023) / 1024;
-    return (a_stage << 52) | (b_stage << 40) | ((size_t)(t->add_mode == 1 ? 2 : 1) << 36) | ((size_t)std::min(t->b_total / 1024, 0xFFFF) << 20) | (size_t)t->n_tile;
+    return (a_stage << 52) | (b_stage << 40) | ((size_t)((t->res_tma ? 1 : 0) | (t->bn_out ? 2 : 0)) << 36) | ((size_t)std::min(t->b_total / 1024, 0xFFFF) << 20) | (size_t)t->n_tile;
 }
 // field-wise maximum of two packed values
 size_t conv_tc_merge(size_t a, size_t b) {
-    return (std::max(a >> 52, b >> 52) << 52) | (std::max((a >> 40) & 0xFFF, (b >> 40) & 0xFFF) << 40) | (std::max((a >> 36) & 0xF, (b >> 36) & 0xF) << 36) |
+    return (std::max(a >> 52, b >> 52) << 52) | (std::max((a >> 40) & 0xFFF, (b >> 40) & 0xFFF) << 40) | ((((a >> 36) | (b >> 36)) & 0xF) << 36) |
            (std::max((a >> 20) & 0xFFFF, (b >> 20) & 0xFFFF) << 20) | std::max(a & 0xFFFFF, b & 0xFFFFF);
 }
 
@@ -1013,21 +1105,34 @@ void launch_conv_tc_probs(const void* d_tc, int nprob, int max_tiles, size_t pac
     L.nprob = nprob;
     L.a_stage = (int)(packed >> 52) * 1024; L.b_stage = (int)((packed >> 40) & 0xFFF) * 1024;
     const int n_tile = (int)(packed & 0xFFFFF);
-    // Shared memory.  Two epilogue groups, each with two 16 KB slab buffers (one where the rings need the room).  The windows' ring
-    // gets four stages (two pairs of tiles), the weights' ring what is left, up to eight tiles; any rest goes back to the windows.
-    // A layer runs at the bytes it keeps in flight.
+    // Shared memory.  Two epilogue groups of L.eb 16 KB slab buffers: a residual is fetched into them ahead of its use and wants three
+    // (one being added to, one being stored, one in flight), else two; a BN of the output takes one more per group.  A layer runs at the
+    // bytes it keeps in flight.  1x1 layers: four windows (two pairs of tiles), then weight tiles.  3x3 layers read a window nine times,
+    // so it is the weight tiles that stream: one slab buffer per group, two windows, four weight tiles, then more windows (measured
+    // at 128 channels on 16 x 16 maps, 1024 images: 148 us with two weight tiles and four windows, 125 us with four and three).
     const size_t a = (size_t)L.a_stage, b = (size_t)L.b_stage;
-    L.groups = 2; L.pg = 2;
-    if ((size_t)L.groups * L.pg * SLAB_BYTES + 4 * a + 3 * b > TC_SMEM_BUDGET) L.pg = 1;
-    const size_t rings = TC_SMEM_BUDGET - (size_t)L.groups * L.pg * SLAB_BYTES;
-    L.na = 4; while (L.na > 2 && (size_t)L.na * a + 2 * b > rings) --L.na;
-    L.nb = 2; while (L.nb < 8 && (size_t)L.na * a + (size_t)(L.nb + 1) * b <= rings) ++L.nb;
-    while (L.na < TC_MAX_STAGES && (size_t)(L.na + 1) * a + (size_t)L.nb * b <= rings) ++L.na;
+    const int flags = (int)((packed >> 36) & 0xF), extra = flags & 2 ? 1 : 0;
+    L.groups = 2; L.res = flags & 1;
+    auto staging = [&] { return (size_t)L.groups * (L.eb + extra) * SLAB_BYTES; };
+    if (a <= 16 * 1024) {                                        // 1x1 layers: windows of one box
+        L.eb = L.res ? 3 : 2;
+        while (L.eb > 1 && staging() + 4 * a + (L.res ? 1 : 3) * b > TC_SMEM_BUDGET) --L.eb;
+        const size_t rings = TC_SMEM_BUDGET - staging();
+        L.na = 4; while (L.na > 2 && (size_t)L.na * a + 2 * b > rings) --L.na;
+        L.nb = 1; while (L.nb < 8 && (size_t)L.na * a + (size_t)(L.nb + 1) * b <= rings) ++L.nb;
+        while (L.na < TC_MAX_STAGES && (size_t)(L.na + 1) * a + (size_t)L.nb * b <= rings) ++L.na;
+    } else {                                                     // several taps per window: weight tiles are what streams
+        L.eb = 1;
+        const size_t rings = TC_SMEM_BUDGET - staging();
+        L.na = 2; L.nb = 1; while (L.nb < 4 && 2 * a + (size_t)(L.nb + 1) * b <= rings) ++L.nb;
+        while (L.na < 4 && (size_t)(L.na + 1) * a + (size_t)L.nb * b <= rings) ++L.na;
+        while (L.nb < 8 && (size_t)L.na * a + (size_t)(L.nb + 1) * b <= rings) ++L.nb;
+    }
     L.acc_stride = (n_tile + 31) / 32 * 32;
     L.nbuf = L.acc_stride <= 128 ? 2 : 1;
     L.tmem_cols = 32; while (L.tmem_cols < 2 * L.nbuf * L.acc_stride) L.tmem_cols *= 2;
     // at least 120 KB of shared memory so that two CTAs that allocate tensor memory never share an SM
-    const size_t smem = std::max((size_t)L.na * a + (size_t)L.nb * b + (size_t)L.groups * L.pg * SLAB_BYTES, (size_t)120 * 1024) + 1024;
+    const size_t smem = std::max((size_t)L.na * a + (size_t)L.nb * b + staging(), (size_t)120 * 1024) + 1024;
     const long long total = (long long)max_tiles * nprob;
     const int grid = (int)std::max(1ll, std::min(total, (long long)sms));
     conv_tc_kernel<<<grid, TC_CONV_THREADS, smem, s>>>((const TcProb*)d_tc, L);

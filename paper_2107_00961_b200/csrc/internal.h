@@ -27,6 +27,9 @@ struct ConvProb {
     int dy_P, dy_Q;       //   zero-stuffed to H x W (only even positions exist); 0 or 1 = dy is stored at the problem's resolution
     int out_compact;      // dgrad of a stride-2 1x1 layer on tcgen05: out is [N,P,Q,C], the gradient at the even input positions (all others are zero)
     int add_sub;          // 2: `add` is such a compact tensor [N,(H+1)/2,(W+1)/2,Ncol] and is added at the even positions of the H x W result only
+    // evaluation: the BN+ReLU that consumes the output runs in the epilogue of the tensor-core kernels, bn_out = relu(bn(y)) of the rounded y
+    // with running statistics (bn_stat: mean [K] | 1/std [K]); bn_only: y itself is not needed
+    const float* bn_stat; const float* bn_gamma; const float* bn_beta; void* bn_out; int bn_only;
     float* stat_tiles;    // forward on tcgen05: per 128-position tile, the column sums and sums of squares of the stored output [tiles][2][K], or nullptr
 };
 
