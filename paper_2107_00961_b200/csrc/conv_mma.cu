@@ -48,7 +48,9 @@ struct alignas(16) MmaProb {
     int nsplit;                 // 1, or 2: a CTA computes one half of the output channels (its half of the filter resident)
     int variant, smem_bytes;    // which instantiation runs this problem (see mma_variant); dynamic shared memory
     float scale;
-    int fuse;                   // 0: convolution only; 1: + BN+ReLU forward of out; 2: + BN+ReLU backward with out as da
+    int fuse;                   // 0: convolution only; 1: + BN+ReLU forward of out; 2: + BN+ReLU backward with out as da (1, 2: cooperative launch);
+                                // 3: evaluation, bn.a = relu(bn(out)) with the statistics given, in the epilogue (store_y 0: out itself is not wanted)
+    int store_y;
     BnProb bn;                  // fuse 1: x = out, a; fuse 2: x, da = out, dx, add.  partial: [CTAs of the problem][2][C] doubles
 };
 
@@ -128,8 +130,9 @@ const MmaProb* __restrict__ probs) {
     const int ncol_all = ncol * nsplit, n_off = ((int)blockIdx.x % nsplit) * ncol;
     const int cta = blockIdx.x / nsplit, ncta = gridDim.x / nsplit;   // the launcher makes gridDim.x a multiple of nsplit
     constexpr bool FUSABLE = NB <= 4;                             // wider CTAs would pay for the sums with registers: the host never asks
-    const int fuse = FUSABLE ? p.fuse : 0;
-    if (cta >= units && !fuse) return;                            // fused: every CTA must reach the grid barrier
+    const int fuse = FUSABLE ? p.fuse : 0;                        // forward instances: 0, 1, 3; dgrad instances: 0, 2 (each carries the code of its own kinds only)
+    const bool coop = fuse == 1 || fuse == 2;
+    if (cta >= units && !coop) return;                            // fused: every CTA must reach the grid barrier
     extern __shared__ __align__(16) uint8_t sm[];
     __shared__ float s_red[8][2][NB * 8];                         // per-warp sums of the fused BN, over the CTA's whole walk
     __shared__ float s_bn[4][NB * 8];                             // fuse 2: mean, 1/std, gamma, beta of this CTA's channels
@@ -215,7 +218,7 @@ const MmaProb* __restrict__ probs) {
     const long long grp_in = (long long)p.G * (p.is == 2 ? p.iP * p.iQ : p.H * p.W) * ca;   // elements of a group of act
     const long long grp_out = (long long)p.G * (p.os == 1 ? p.H * p.W : p.P * p.Q) * ncol_all;
     const __nv_bfloat16* pf_add = addp;
-    const __nv_bfloat16* pf_x = fuse == 2 ? reinterpret_cast<const __nv_bfloat16*>(p.bn.x) : nullptr;
+    const __nv_bfloat16* pf_x = TRANS && fuse == 2 ? reinterpret_cast<const __nv_bfloat16*>(p.bn.x) : nullptr;
     auto issue = [&](int unit, int stage) {
         const int grp = unit / subs, j = unit - grp * subs;
         const __nv_bfloat16* ag = act + grp * grp_in + a_g * 8;
@@ -252,12 +255,12 @@ const MmaProb* __restrict__ probs) {
     const uint32_t b_lane = TRANS ? (uint32_t)(((lane >> 3) & 1) * 8 + (lane & 7)) * wpitch + (lane >> 4) * 16
                                   : (uint32_t)((lane >> 4) * 8 + (lane & 7)) * wpitch + ((lane >> 3) & 1) * 16;
     const float scale = p.scale;
-    if (fuse) for (int i = tid; i < 8 * 2 * ncol; i += MMA_THREADS) (&s_red[0][0][0])[i] = 0.f;
+    if (coop) for (int i = tid; i < 8 * 2 * ncol; i += MMA_THREADS) (&s_red[0][0][0])[i] = 0.f;
 
     __syncthreads();                                              // tables complete
     pdl_wait();                                                   // from here on: tensors the previous kernel may have written
     const __nv_bfloat16* __restrict__ bnx = reinterpret_cast<const __nv_bfloat16*>(p.bn.x);
-    if (fuse == 2 && tid < ncol) {
+    if (fuse >= 2 && tid < ncol) {
         const int c = n_off + tid;
         s_bn[0][tid] = p.bn.stat[c]; s_bn[1][tid] = p.bn.stat[p.bn.C + c]; s_bn[2][tid] = p.bn.gamma[c]; s_bn[3][tid] = p.bn.beta[c];
     }
@@ -308,6 +311,7 @@ const MmaProb* __restrict__ probs) {
         const __nv_bfloat16* __restrict__ add_g = addp + obase;
         const __nv_bfloat16* __restrict__ bnx_g = bnx + obase;
         __nv_bfloat16* __restrict__ out_g = outp + obase;
+        __nv_bfloat16* __restrict__ bna_g = reinterpret_cast<__nv_bfloat16*>(p.bn.a) + obase;
         int opx[MBW][2];
 #pragma unroll
         for (int mb = 0; mb < MBW; ++mb) {
@@ -336,7 +340,7 @@ const MmaProb* __restrict__ probs) {
                         for (int c2 = 0; c2 < NB / 2; ++c2) { const uint2 v = *reinterpret_cast<const uint2*>(add_g + o + c2 * 4); wv[c2 * 2] = v.x; wv[c2 * 2 + 1] = v.y; }
                     }
                 }
-                if (fuse == 2) {
+                if (TRANS && fuse == 2) {
                     if constexpr (NB % 4 == 0) {
 #pragma unroll
                         for (int c4 = 0; c4 < NB / 4; ++c4) { const uint4 v = *reinterpret_cast<const uint4*>(bnx_g + o + c4 * 8); xv[c4 * 4] = v.x; xv[c4 * 4 + 1] = v.y; xv[c4 * 4 + 2] = v.z; xv[c4 * 4 + 3] = v.w; }
@@ -352,13 +356,13 @@ const MmaProb* __restrict__ probs) {
                     __nv_bfloat162 h = __floats2bfloat162_rn(v0, v1);
                     wv[j] = *reinterpret_cast<uint32_t*>(&h);
                 }
-                if (fuse == 1) {                                  // sums of the STORED values: x, x^2
+                if (!TRANS && fuse == 1) {                        // sums of the STORED values: x, x^2
 #pragma unroll
                     for (int j = 0; j < NB; ++j) {
                         const float r0 = valid ? __uint_as_float(wv[j] << 16) : 0.f, r1 = valid ? __uint_as_float(wv[j] & 0xFFFF0000u) : 0.f;
                         ps[2 * j] += r0; pq[2 * j] += r0 * r0; ps[2 * j + 1] += r1; pq[2 * j + 1] += r1 * r1;
                     }
-                } else if (fuse == 2) {                           // sums of dz = da * [relu input > 0] and dz * xhat
+                } else if (TRANS && fuse == 2) {                  // sums of dz = da * [relu input > 0] and dz * xhat
 #pragma unroll
                     for (int j = 0; j < NB; ++j) {
                         const int c = t4 * (2 * NB) + 2 * j;
@@ -370,7 +374,7 @@ const MmaProb* __restrict__ probs) {
                         ps[2 * j] += dz0; pq[2 * j] += dz0 * xh0; ps[2 * j + 1] += dz1; pq[2 * j + 1] += dz1 * xh1;
                     }
                 }
-                if (valid) {
+                if (valid && (TRANS || fuse != 3 || p.store_y)) {
                     if constexpr (NB % 4 == 0) {
 #pragma unroll
                         for (int c4 = 0; c4 < NB / 4; ++c4) *reinterpret_cast<uint4*>(out_g + o + c4 * 8) = make_uint4(wv[c4 * 4], wv[c4 * 4 + 1], wv[c4 * 4 + 2], wv[c4 * 4 + 3]);
@@ -379,8 +383,26 @@ const MmaProb* __restrict__ probs) {
                         for (int c2 = 0; c2 < NB / 2; ++c2) *reinterpret_cast<uint2*>(out_g + o + c2 * 4) = make_uint2(wv[c2 * 2], wv[c2 * 2 + 1]);
                     }
                 }
+                if (!TRANS && fuse == 3 && valid) {
+#pragma unroll
+                    for (int j = 0; j < NB; ++j) {
+                        const int c = t4 * (2 * NB) + 2 * j;
+                        const float2 mean = *reinterpret_cast<const float2*>(&s_bn[0][c]), istd = *reinterpret_cast<const float2*>(&s_bn[1][c]);
+                        const float2 ga = *reinterpret_cast<const float2*>(&s_bn[2][c]), be = *reinterpret_cast<const float2*>(&s_bn[3][c]);
+                        const float z0 = (__uint_as_float(wv[j] << 16) - mean.x) * istd.x * ga.x + be.x, z1 = (__uint_as_float(wv[j] & 0xFFFF0000u) - mean.y) * istd.y * ga.y + be.y;
+                        __nv_bfloat162 h = __floats2bfloat162_rn(z0 > 0.f ? z0 : 0.f, z1 > 0.f ? z1 : 0.f);
+                        wv[j] = *reinterpret_cast<uint32_t*>(&h);
+                    }
+                    if constexpr (NB % 4 == 0) {
+#pragma unroll
+                        for (int c4 = 0; c4 < NB / 4; ++c4) *reinterpret_cast<uint4*>(bna_g + o + c4 * 8) = make_uint4(wv[c4 * 4], wv[c4 * 4 + 1], wv[c4 * 4 + 2], wv[c4 * 4 + 3]);
+                    } else {
+#pragma unroll
+                        for (int c2 = 0; c2 < NB / 2; ++c2) *reinterpret_cast<uint2*>(bna_g + o + c2 * 4) = make_uint2(wv[c2 * 2], wv[c2 * 2 + 1]);
+                    }
+                }
             }
-        if (fuse) {                                               // the 8 lanes that own the same channels, fixed butterfly; lane g8 = 0 keeps the warp's running sum
+        if (coop) {                                               // the 8 lanes that own the same channels, fixed butterfly; lane g8 = 0 keeps the warp's running sum
 #pragma unroll
             for (int i = 0; i < 2 * NB; ++i) {
 #pragma unroll
@@ -395,7 +417,7 @@ const MmaProb* __restrict__ probs) {
         stage = stage + 1 == stages ? 0 : stage + 1;
     }
     cp_async_wait<0>();
-    if (!fuse) return;
+    if (!coop) return;
 
     // ---- fused BN: this CTA's sums (warps added in order, in double) -> partial[cta][2][C]; grid barrier; statistics; elementwise pass
     const BnProb& bn = p.bn;
@@ -433,7 +455,7 @@ const MmaProb* __restrict__ probs) {
         if (q == 0) {
             a0 = 0.0; a1 = 0.0;
             for (int k = 0; k < Q; ++k) { a0 += s_dred[k * C + c]; a1 += s_dred[256 + k * C + c]; }
-            if (fuse == 1) {
+            if (!TRANS) {
                 const double m = (double)bn.m, mean = a0 / m;
                 double var = a1 / m - mean * mean; if (var < 0.0) var = 0.0;
                 const float fm = (float)mean, fi = (float)(1.0 / sqrt(var + (double)bn.eps));
@@ -465,11 +487,11 @@ const MmaProb* __restrict__ probs) {
         const uint4* xv = reinterpret_cast<const uint4*>(bn.x);
         const uint4* dv = reinterpret_cast<const uint4*>(bn.da);
         const uint4* av = reinterpret_cast<const uint4*>(bn.add);
-        uint4* ov = reinterpret_cast<uint4*>(fuse == 1 ? bn.a : bn.dx);
+        uint4* ov = reinterpret_cast<uint4*>(!TRANS ? bn.a : bn.dx);
         for (long long v = (long long)blockIdx.x * MMA_THREADS + tid; v < nv; v += stride) {
             const float* st = s_stat + ((int)v & (G - 1)) * 8;
             float x[8], o[8]; bf8_unpack(__ldcg(xv + v), x);
-            if (fuse == 1) {
+            if (!TRANS) {
 #pragma unroll
                 for (int j = 0; j < 8; ++j) { const float z = (x[j] - st[j]) * st[C + j] * st[4 * C + j] + st[5 * C + j]; o[j] = z > 0.f ? z : 0.f; }
             } else {
@@ -569,6 +591,11 @@ bool conv_mma_fill(const ConvProb& p, int mode, void* host, const BnProb* bn) {
     t.os = mode == CONV_FWD ? p.stride : 1; t.P = p.P; t.Q = p.Q;
     t.is = (mode == CONV_DGRAD && p.dy_sub == 2) ? 2 : 1; t.iP = p.dy_P; t.iQ = p.dy_Q;
     t.stages = g.stages; t.nsplit = g.nsplit; t.variant = g.variant; t.smem_bytes = (int)g.smem; t.scale = p.scale;
+    t.store_y = 1;
+    if (p.bn_out) {
+        t.fuse = 3; t.bn.stat = const_cast<float*>(p.bn_stat); t.bn.gamma = p.bn_gamma; t.bn.beta = p.bn_beta; t.bn.a = p.bn_out; t.bn.C = g.ncol;
+        t.store_y = p.bn_only ? 0 : 1;
+    }
     if (bn) {
         if (!conv_mma_can_fuse_bn(p, mode, bn->C)) return false;
         t.fuse = mode == CONV_FWD ? 1 : 2; t.bn = *bn; t.variant |= MMA_VARIANT_FUSED;

@@ -131,6 +131,7 @@ constexpr int AGG_CHUNK = 8192;   // elements per CTA of the aggregate kernel (t
 void launch_conv_ref(const ConvProb* d, int nprob, int max_tiles, int mode, bool bf16, cudaStream_t s);
 void launch_splitk_reduce(const ConvProb* d, int nprob, int max_elems, cudaStream_t s);
 void launch_bn_stats(const BnProb* d, int nprob, int max_chunks, int max_c, bool bf16, cudaStream_t s);
+void launch_bn_eval_stats(const BnProb* d, int nprob, int max_c, cudaStream_t s);      // mean | 1/std from the running statistics
 void launch_bn_apply(const BnProb* d, int nprob, long long max_elems, bool bf16, cudaStream_t s);
 void launch_bn_bwd_reduce(const BnProb* d, int nprob, int max_chunks, int max_c, bool bf16, cudaStream_t s);
 void launch_bn_bwd_apply(const BnProb* d, int nprob, long long max_elems, bool bf16, cudaStream_t s);
@@ -151,6 +152,7 @@ void launch_sgd(const Segment* d, int nseg, long long nchunks, ParamArrays pa, f
                 bool shadow, cudaStream_t s);
 void launch_scatter(const Segment* d, int nseg, long long nchunks, ParamArrays pa, bool zero_momentum, bool shadow,
                     cudaStream_t s);
+void launch_shadow(const float* src, __nv_bfloat16* dst, long long n, cudaStream_t s);   // dst = round(src); both 16-byte aligned
 void launch_scatter_buffers(const Segment* d, int nseg, long long nchunks, ParamArrays pa, cudaStream_t s);
 struct AggArrays { const float* sub_p; const float* sub_b; long long stride_p, stride_b; float* global_p; float* global_b; };   // _p parameters, _b BN running statistics
 void launch_aggregate(const Segment* d, int nseg, long long nchunks, const AggArrays& arr, int S, cudaStream_t s);

@@ -79,6 +79,18 @@ __global__ void __launch_bounds__(256) scatter_kernel(const Segment* __restrict_
     }
 }
 
+__global__ void __launch_bounds__(256) shadow_kernel(const float* __restrict__ src, __nv_bfloat16* __restrict__ dst, long long n) {
+    const long long nq = n >> 2, step = (long long)gridDim.x * 256;
+    for (long long q = blockIdx.x * 256ll + threadIdx.x; q < nq; q += 4 * step) {        // four 16-byte loads in flight
+        float4 x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = q + u * step < nq ? __ldg(reinterpret_cast<const float4*>(src) + q + u * step) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) if (q + u * step < nq) reinterpret_cast<uint2*>(dst)[q + u * step] = make_uint2(pack_bf16x2(x[u].x, x[u].y), pack_bf16x2(x[u].z, x[u].w));
+    }
+    for (long long i = 4 * nq + blockIdx.x * 256ll + threadIdx.x; i < n; i += step) dst[i] = __float2bfloat16_rn(src[i]);
+}
+
 __global__ void __launch_bounds__(256) scatter_buffers_kernel(const Segment* __restrict__ segs, int nseg, ParamArrays pa) {
     const Segment& sg = find_segment(segs, nseg, blockIdx.x);
     const Range r = chunk_range(sg, blockIdx.x);
@@ -188,6 +200,10 @@ void launch_scatter(const Segment* d, int nseg, long long nchunks, ParamArrays p
                   else scatter_kernel<true, false><<<g, 256, 0, s>>>(d, nseg, pa); }
     else { if (zero_momentum) scatter_kernel<false, true><<<g, 256, 0, s>>>(d, nseg, pa);
            else scatter_kernel<false, false><<<g, 256, 0, s>>>(d, nseg, pa); }
+}
+void launch_shadow(const float* src, __nv_bfloat16* dst, long long n, cudaStream_t s) {
+    const long long g = (n / 4 + 1023) / 1024;
+    shadow_kernel<<<(unsigned)(g < 1 ? 1 : g > 148 * 8 ? 148 * 8 : g), 256, 0, s>>>(src, dst, n);
 }
 void launch_scatter_buffers(const Segment* d, int nseg, long long nchunks, ParamArrays pa, cudaStream_t s) {
     if (nchunks <= 0) return;

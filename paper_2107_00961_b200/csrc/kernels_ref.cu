@@ -488,6 +488,9 @@ void launch_bn_stats(const BnProb* d, int nprob, int max_chunks, int max_c, bool
     if (bf16) bn_finalize_kernel<__nv_bfloat16, 0><<<dim3((max_c + 7) / 8, nprob), 256, 0, s>>>(d);
     else bn_finalize_kernel<float, 0><<<dim3((max_c + 7) / 8, nprob), 256, 0, s>>>(d);
 }
+void launch_bn_eval_stats(const BnProb* d, int nprob, int max_c, cudaStream_t s) {
+    bn_finalize_kernel<float, 0><<<dim3((max_c + 7) / 8, nprob), 256, 0, s>>>(d);
+}
 // the vector path takes at least 32768 elements per CTA (see bn_stream_vec), and about 16 CTAs per SM over the launch
 static int stream_grid(long long n, int nprob) { long long g = (n + 32767) / 32768; const long long cap = std::max(1, 148 * 16 / std::max(1, nprob)); if (g > cap) g = cap; if (g < 1) g = 1; return (int)g; }
 void launch_bn_apply(const BnProb* d, int nprob, long long max_elems, bool bf16, cudaStream_t s) {

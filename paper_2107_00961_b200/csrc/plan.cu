@@ -110,6 +110,7 @@ struct Builder {
     double* bn_partial = nullptr; float* wgrad_partial = nullptr; size_t bn_partial_need = 0, wgrad_partial_need = 0;
     char* up_buf = nullptr; size_t up_need = 0; const void* up_src = nullptr;      // zero-stuffed dy of the current stride-2 layer
     char* col_buf = nullptr; char* col_w = nullptr;                                 // im2col of the input images and the stem's weights packed alike
+    static constexpr long long EVAL_STATS_KEY = -1;
     static constexpr int NGBUF = 12;           // rotating gradient buffers: the more, the further the main stream runs ahead of the weight gradients
     char* gbuf[NGBUF] = {}; bool gused[NGBUF] = {}; size_t gbig = 0;
     float* logits = nullptr;
@@ -133,9 +134,10 @@ struct Builder {
     int gtake() { int best = -1; for (int i = 0; i < NGBUF; ++i) if (!gused[i] && (best < 0 || gstamp[i] < gstamp[best])) best = i; if (best >= 0) gused[best] = true; return best; }
     void grel(int i) { if (i >= 0) { gused[i] = false; gstamp[i] = ++gclock; } }
 
-    float* W() const { return ctx->pa.w + (long long)copy * ctx->pa.n; }
+    // evaluation reads the global parameters and statistics where they are; only the convolutions' bf16 copy is refreshed
+    float* W() const { return eval ? ctx->pa.global : ctx->pa.w + (long long)copy * ctx->pa.n; }
     float* G() const { return ctx->pa.g + (long long)copy * ctx->pa.n; }
-    float* Bf() const { return ctx->pa.buf + (long long)copy * ctx->pa.nbuf; }
+    float* Bf() const { return eval ? ctx->pa.global_buf : ctx->pa.buf + (long long)copy * ctx->pa.nbuf; }
     const void* CW(long long o) const {           // the convolutions' copy of the weights
         if (ctx->opts.dtype == RESIST_BF16) return ctx->pa.wb + (long long)copy * ctx->pa.n + o;
         return W() + o;
@@ -260,8 +262,8 @@ struct Builder {
 
     // chunks per BN problem that give the fused (cooperative) kernels about two CTAs per SM over all sub-ResNets
     int fused_chunks() const { return std::max(8, 2 * ctx->sm_count / std::max(1, ctx->S)); }
-    // forward BN+ReLU: statistics (or running statistics in evaluation) then apply
-    float* bn_fwd(long long key, const void* x, void* a, const BNRef& r, long long m) {
+    // forward BN+ReLU: statistics (or running statistics in evaluation) then apply.  x_used: x is read by more than this BN
+    float* bn_fwd(long long key, const void* x, void* a, const BNRef& r, long long m, bool x_used) {
         float* stat = (float*)take((size_t)4 * r.c * 4);
         Op op{}; op.key = key; op.sub = sub; op.kind = OP_BN_STATS;
         BnProb& p = op.bn;
@@ -273,6 +275,20 @@ struct Builder {
         p.partial = bn_partial;
         const int producer = last_fwd_conv; last_fwd_conv = -1;
         const int tc_producer = last_tc_fwd; last_tc_fwd = -1;
+        if (eval) {
+            // all layers' mean | 1/std come from one launch at the start; behind a tensor-core convolution the elementwise pass runs in
+            // that convolution's epilogue
+            op.key = EVAL_STATS_KEY; op.kind = OP_BN_EVAL_STATS; ops->push_back(op);
+            const int prod = producer >= 0 ? producer : tc_producer;
+            if (prod >= 0 && (*ops)[prod].conv.out == x && (*ops)[prod].conv.K == r.c &&
+                (tc_producer >= 0 || (p.vec && conv_mma_can_fuse_bn((*ops)[prod].conv, CONV_FWD, r.c)))) {
+                ConvProb& c = (*ops)[prod].conv;
+                c.bn_stat = stat; c.bn_gamma = p.gamma; c.bn_beta = p.beta; c.bn_out = a; c.bn_only = x_used ? 0 : 1;
+                return stat;
+            }
+            op.key = key + 1; op.kind = OP_BN_APPLY; ops->push_back(op);
+            return stat;
+        }
         if (fusable(producer, x, p)) { fuse_into(producer, p, 1); return stat; }                            // inside the producing convolution's launch
         if (!eval && p.vec && tc_producer >= 0 && (*ops)[tc_producer].conv.out == x && (*ops)[tc_producer].conv.K == r.c) {
             // the tcgen05 convolution that produces x leaves per-tile column sums: a small launch turns them into statistics, then one elementwise pass
@@ -340,7 +356,7 @@ static size_t unroll_subnet(resist_ctx* ctx, Builder& bd, const std::vector<char
     if (stem_col) { bd.stem_im2col(0, L.stem, B, A.in_h, A.in_w); bd.stem_conv(0, CONV_FWD, L.stem, nullptr, stem_y, B, A.in_h, A.in_w); }
     else bd.conv(0, CONV_FWD, nullptr, L.stem, nullptr, nullptr, stem_y, B, A.in_h, A.in_w, 1.f, true);
     void* cur = stem_y; int cH = Hs, cW = Ws, cC = A.stem_cout;
-    if (A.stem_bn_relu) { stem_a = bd.act(m_stem * cC); stem_stat = bd.bn_fwd(1, stem_y, stem_a, L.stem_bn, m_stem); cur = stem_a; }
+    if (A.stem_bn_relu) { stem_a = bd.act(m_stem * cC); stem_stat = bd.bn_fwd(1, stem_y, stem_a, L.stem_bn, m_stem, false); cur = stem_a; }
     if (A.stem_maxpool) {
         const int Hp = out_dim(cH, 3, 2), Wp = out_dim(cW, 3, 2);
         stem_p = bd.act((long long)B * Hp * Wp * cC); stem_arg = bd.eval ? nullptr : (uint8_t*)bd.take((size_t)B * Hp * Wp * cC);
@@ -381,21 +397,21 @@ static size_t unroll_subnet(resist_ctx* ctx, Builder& bd, const std::vector<char
         const long long m_in = (long long)B * s.H * s.W, m_out = (long long)B * s.Ho * s.Wo;
         const float scale = (bd.eval && K.partitionable) ? inv_S : 1.f;
         s.x = cur; s.a1 = bd.act(m_in * K.cin);
-        s.stat[0] = bd.bn_fwd(key + 0, s.x, s.a1, r.bn[0], m_in);
+        s.stat[0] = bd.bn_fwd(key + 0, s.x, s.a1, r.bn[0], m_in, !K.has_projection);
         const void* sc = s.x;
         if (K.has_projection) { void* scb = bd.act(m_out * K.cout); bd.conv(key + 2, CONV_FWD, s.a1, r.proj, nullptr, nullptr, scb, B, s.H, s.W, 1.f); sc = scb; }
         void* out = bd.act(m_out * K.cout);
         if (K.kind == RESIST_BASIC) {
             s.y1 = bd.act(m_out * K.cout); s.a2 = bd.act(m_out * K.cout);
             bd.conv(key + 3, CONV_FWD, s.a1, r.conv[0], nullptr, nullptr, s.y1, B, s.H, s.W, 1.f);
-            s.stat[1] = bd.bn_fwd(key + 4, s.y1, s.a2, r.bn[1], m_out);
+            s.stat[1] = bd.bn_fwd(key + 4, s.y1, s.a2, r.bn[1], m_out, false);
             bd.conv(key + 6, CONV_FWD, s.a2, r.conv[1], nullptr, sc, out, B, s.Ho, s.Wo, scale);
         } else {
             s.y1 = bd.act(m_in * K.cmid); s.a2 = bd.act(m_in * K.cmid); s.y2 = bd.act(m_out * K.cmid); s.a3 = bd.act(m_out * K.cmid);
             bd.conv(key + 3, CONV_FWD, s.a1, r.conv[0], nullptr, nullptr, s.y1, B, s.H, s.W, 1.f);
-            s.stat[1] = bd.bn_fwd(key + 4, s.y1, s.a2, r.bn[1], m_in);
+            s.stat[1] = bd.bn_fwd(key + 4, s.y1, s.a2, r.bn[1], m_in, false);
             bd.conv(key + 6, CONV_FWD, s.a2, r.conv[1], nullptr, nullptr, s.y2, B, s.H, s.W, 1.f);
-            s.stat[2] = bd.bn_fwd(key + 7, s.y2, s.a3, r.bn[2], m_out);
+            s.stat[2] = bd.bn_fwd(key + 7, s.y2, s.a3, r.bn[2], m_out, false);
             bd.conv(key + 9, CONV_FWD, s.a3, r.conv[2], nullptr, sc, out, B, s.Ho, s.Wo, scale);
         }
         cur = out; cH = s.Ho; cW = s.Wo; cC = K.cout;
@@ -404,7 +420,7 @@ static size_t unroll_subnet(resist_ctx* ctx, Builder& bd, const std::vector<char
     // ---- final BN + ReLU, pool, head, loss
     const long long mF = (long long)B * cH * cW; const int HW = cH * cW;
     void* xF = cur; void* aF = bd.act(mF * cC);
-    float* statF = bd.bn_fwd(FWD_END, xF, aF, L.final_bn, mF);
+    float* statF = bd.bn_fwd(FWD_END, xF, aF, L.final_bn, mF, false);
     HeadProb hp{};
     hp.a = aF; hp.w = bd.W() + L.head_w; hp.b = bd.W() + L.head_b; hp.dw = bd.G() + L.head_w; hp.db = bd.G() + L.head_b;
     hp.pooled = (float*)bd.take((size_t)B * cC * 4); hp.dpooled = (float*)bd.take((size_t)B * cC * 4);
@@ -614,14 +630,15 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
                         if (o.kind == OP_CONV_WGRAD) L.bytes += es * (in_e + out_e) + 4.0 * w_e;
                         else L.bytes += es * (in_e + out_e + w_e + (p.add ? (o.kind == OP_CONV_FWD ? out_e : in_e) : 0.0)); }
                     break; }
-                case OP_BN_STATS: case OP_BN_APPLY: case OP_BN_BWD_REDUCE: case OP_BN_BWD_APPLY: case OP_BN_FWD_FUSED: case OP_BN_BWD_FUSED: case OP_BN_TILE_STATS: {
+                case OP_BN_STATS: case OP_BN_APPLY: case OP_BN_BWD_REDUCE: case OP_BN_BWD_APPLY: case OP_BN_FWD_FUSED: case OP_BN_BWD_FUSED: case OP_BN_TILE_STATS: case OP_BN_EVAL_STATS: {
                     if (k == i) L.first = (int)bn.size();
                     bn.push_back(o.bn);
                     L.gx = std::max(L.gx, o.bn.chunks); L.max_c = std::max(L.max_c, o.bn.C);
                     L.max_elems = std::max<long long>(L.max_elems, o.bn.m * o.bn.C);
                     { const double e = (double)o.bn.m * o.bn.C;
                       if (o.kind == OP_BN_TILE_STATS) L.bytes += 8.0 * o.bn.chunks * o.bn.C;
-                      else if (o.kind == OP_BN_STATS) L.bytes += o.bn.eval ? 0.0 : es * e;
+                      else if (o.kind == OP_BN_EVAL_STATS) L.bytes += 16.0 * o.bn.C;
+                      else if (o.kind == OP_BN_STATS) L.bytes += es * e;
                       else if (o.kind == OP_BN_APPLY) L.bytes += 2 * es * e;
                       else if (o.kind == OP_BN_BWD_REDUCE) L.bytes += 2 * es * e;
                       else if (o.kind == OP_BN_FWD_FUSED) L.bytes += 2 * es * e;          // x once from HBM (the second read is an L2 hit), a once
@@ -673,7 +690,7 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
                         if (o.fuse == 1) wr.push_back(o.bn.a); else if (o.fuse == 2) wr.push_back(o.bn.dx);
                         break;
                     case OP_CONV_WGRAD: case OP_SPLITK: case OP_REPACK: break;
-                    case OP_BN_STATS: case OP_BN_BWD_REDUCE: case OP_BN_TILE_STATS: break;
+                    case OP_BN_STATS: case OP_BN_BWD_REDUCE: case OP_BN_TILE_STATS: case OP_BN_EVAL_STATS: break;
                     case OP_BN_APPLY: case OP_BN_FWD_FUSED: wr.push_back(o.bn.a); break;
                     case OP_BN_BWD_APPLY: case OP_BN_BWD_FUSED: wr.push_back(o.bn.dx); break;
                     default: always = true; break;
@@ -836,6 +853,7 @@ static int run_plan(resist_ctx* ctx, Plan& plan, const PatchArgs& pa, bool updat
             case OP_CONV_WGRAD: pk = L.backend >= 200 ? PK_CONV_WGRAD_MMA : L.backend ? PK_CONV_WGRAD_TC : PK_CONV_WGRAD_CC; break;
             case OP_SPLITK: case OP_REPACK: pk = PK_SPLITK; break;
             case OP_BN_STATS: pk = PK_BN_STATS; nk = 2; break;
+            case OP_BN_EVAL_STATS: pk = PK_BN_STATS; break;
             case OP_BN_APPLY: pk = PK_BN_APPLY; break;
             case OP_BN_BWD_REDUCE: pk = PK_BN_BWD_REDUCE; nk = 2; break;
             case OP_BN_BWD_APPLY: pk = PK_BN_BWD_APPLY; break;
@@ -865,6 +883,7 @@ static int run_plan(resist_ctx* ctx, Plan& plan, const PatchArgs& pa, bool updat
             case OP_SPLITK: launch_splitk_reduce(plan.d_conv + L.first, L.count, (int)L.max_elems, st); ++n_launch; break;
             case OP_REPACK: launch_repack_rows(plan.d_conv + L.first, L.count, (int)L.max_elems, st); ++n_launch; break;
             case OP_BN_STATS: launch_bn_stats(plan.d_bn + L.first, L.count, L.gx, L.max_c, bf, st); n_launch += 2; break;
+            case OP_BN_EVAL_STATS: launch_bn_eval_stats(plan.d_bn + L.first, L.count, L.max_c, st); ++n_launch; break;
             case OP_BN_APPLY: launch_bn_apply(plan.d_bn + L.first, L.count, L.max_elems, bf, st); ++n_launch; break;
             case OP_BN_BWD_REDUCE: launch_bn_bwd_reduce(plan.d_bn + L.first, L.count, L.gx, L.max_c, bf, st); n_launch += 2; break;
             case OP_BN_BWD_APPLY: launch_bn_bwd_apply(plan.d_bn + L.first, L.count, L.max_elems, bf, st); ++n_launch; break;
@@ -952,15 +971,8 @@ int resist_eval(resist_ctx* ctx, const void* images, const int32_t* labels, int3
     if (rc) return rc;
     const int copy = ctx->S_cap;                               // the evaluation copy sits after the working copies
     const int S = std::max(ctx->S, 1);
-    // refresh the evaluation copy from the global parameters
-    Segment sp{0, ctx->L.n_params, 0, 0u, copy}, sb{0, ctx->L.n_buffers, 0, 0u, copy};
-    rc = ensure_seg_table(ctx, 2); if (rc) return rc;
-    Segment both[2] = {sp, sb};
-    cudaError_t e = cudaMemcpyAsync(ctx->d_seg, both, sizeof(both), cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) { ctx->err = cudaGetErrorString(e); return RESIST_ECUDA; }
-    launch_scatter(ctx->d_seg, 1, (sp.len + SEG_CHUNK - 1) / SEG_CHUNK, ctx->pa, false, ctx->opts.dtype == RESIST_BF16, st);
-    launch_scatter_buffers(ctx->d_seg + 1, 1, (sb.len + SEG_CHUNK - 1) / SEG_CHUNK, ctx->pa, st);
-    cudaStreamSynchronize(st);
+    // refresh the convolutions' bf16 copy from the global parameters (everything else is read from the global arrays in place)
+    if (ctx->opts.dtype == RESIST_BF16) launch_shadow(ctx->pa.global, ctx->pa.wb + (long long)copy * ctx->pa.n, ctx->L.n_params, st);
     Plan& plan = ctx->plans[ctx->S_cap + 1];
     if (!plan.valid || plan.B != B || plan.generation != (unsigned long long)S) {
         std::vector<char> all(ctx->arch.num_blocks, 1);
