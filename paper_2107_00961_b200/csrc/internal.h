@@ -141,6 +141,13 @@ int launch_head_fwd(const HeadProb* d, int nprob, int maxB, int maxC, int max_cl
 int launch_head_bwd(const HeadProb* d, int nprob, int maxB, int maxC, int max_classes, long long max_elems,
                     bool bf16, cudaStream_t s);
 
+// ---- launchers (kernels_small.cu): layers of a few thousand positions on CUDA cores
+bool conv_small_ok(const ConvProb& p, int mode);
+int conv_small_ctas(const ConvProb& p, int mode);
+void launch_conv_small(const ConvProb* d, int nprob, int max_ctas, int mode, int ksz, bool bf16, cudaStream_t s);
+bool bn_small_ok(const BnProb& p);
+void launch_bn_small(const BnProb* d, int nprob, int max_c, int backward, bool bf16, cudaStream_t s);
+
 // statistics, finalisation and apply of BN+ReLU in one cooperative launch (bf16 vector path, training mode); false if the grid cannot be co-resident
 bool launch_bn_fused(const BnProb* d, int nprob, int max_chunks, int backward, cudaStream_t s);   // kernels_ref.cu
 void launch_im2col(const ColProb* d, int nprob, const ColProb& shape, cudaStream_t s);      // shape: the largest problem's

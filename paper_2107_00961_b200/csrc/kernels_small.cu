@@ -1,0 +1,246 @@
+// Layers of a few thousand positions on CUDA cores (fp32 mode on small nets, and bf16 shapes no tensor-core family takes).  Such a layer is
+// microseconds of arithmetic, so the 64 x 64 GEMM tiles of kernels_ref.cu leave all but one or two SMs idle and walk the reduction
+// serially (a 32-channel 3x3 layer on 2 x 2 maps: 18 slices of dependent loads, 46-60 us), and BN pays three launches.  Here the
+// reduction of an output is spread over the warps of a CTA (one filter tap each) and added in tap order, and BN is one launch.
+// All sums have a fixed order.
+#include <algorithm>
+#include "internal.h"
+
+namespace resist {
+
+template <class T> __device__ __forceinline__ float sm_ld(const T* p);
+template <> __device__ __forceinline__ float sm_ld<float>(const float* p) { return __ldg(p); }
+template <> __device__ __forceinline__ float sm_ld<__nv_bfloat16>(const __nv_bfloat16* p) { return __bfloat162float(__ldg(p)); }
+template <class T> __device__ __forceinline__ float4 sm_ld4(const T* p);
+template <> __device__ __forceinline__ float4 sm_ld4<float>(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
+template <> __device__ __forceinline__ float4 sm_ld4<__nv_bfloat16>(const __nv_bfloat16* p) {
+    const uint2 v = __ldg(reinterpret_cast<const uint2*>(p));
+    return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xFFFF0000u), __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xFFFF0000u));
+}
+template <class T> __device__ __forceinline__ void sm_st(T* p, float v);
+template <> __device__ __forceinline__ void sm_st<float>(float* p, float v) { *p = v; }
+template <> __device__ __forceinline__ void sm_st<__nv_bfloat16>(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
+
+constexpr int SMALL_PB = 8;                                      // positions per CTA of the forward / dgrad kernel
+
+// Forward and dgrad: a CTA takes 8 positions x 32 output columns (lanes); warp = filter tap (3x3) or quarter of the reduction (1x1).  The
+// activations are the same address for a whole warp, the weights are read once per 8 positions.
+template <class T, int MODE, int KS>
+__global__ void __launch_bounds__(KS == 3 ? 288 : 128) conv_small_kernel(const ConvProb* __restrict__ probs) {
+    constexpr int TAPS = KS * KS, NW = KS == 3 ? 9 : 4;
+    const ConvProb& p = probs[blockIdx.y];
+    const int M = p.M, Ncol = p.Ncol, ctiles = (Ncol + 31) >> 5;
+    const int tile = blockIdx.x / ctiles, ct = blockIdx.x - tile * ctiles, m0 = tile * SMALL_PB;
+    if (m0 >= M) return;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, col = ct * 32 + lane;
+    const int tap = KS == 3 ? warp : 0, red = MODE == CONV_FWD ? p.C : p.K;
+    int lo = 0, hi = red;
+    if (KS == 1) { const int q = ((red + 3) / 4 + 3) / 4 * 4; lo = min(warp * q, red); hi = min(lo + q, red); }
+    // lane i < 8: element offset of position i's operand row for this tap, -1 outside the image
+    int off_l = -1;
+    {
+        const int m = m0 + (lane & 7), r = tap / KS, s = tap % KS;
+        if (m < M) {
+            if (MODE == CONV_FWD) {
+                const int q = m % p.Q, t = m / p.Q, pp = t % p.P, n = t / p.P, h = pp * p.stride + r - p.pad, x = q * p.stride + s - p.pad;
+                if (h >= 0 && h < p.H && x >= 0 && x < p.W) off_l = ((n * p.H + h) * p.W + x) * red;
+            } else {
+                const int x = m % p.W, t = m / p.W, h = t % p.H, n = t / p.H, ph = h + p.pad - r, qx = x + p.pad - s;
+                if (ph >= 0 && qx >= 0 && ph % p.stride == 0 && qx % p.stride == 0) {
+                    const int pp = ph / p.stride, q = qx / p.stride;
+                    if (pp < p.P && q < p.Q) off_l = ((n * p.P + pp) * p.Q + q) * red;
+                }
+            }
+        }
+    }
+    int off[SMALL_PB];
+#pragma unroll
+    for (int i = 0; i < SMALL_PB; ++i) off[i] = __shfl_sync(0xffffffffu, off_l, i);
+    float acc[SMALL_PB] = {};
+    const T* __restrict__ act = (const T*)p.act; const T* __restrict__ wgt = (const T*)p.wgt;
+    const int colc = min(col, Ncol - 1);
+    const bool vec = red % 4 == 0 && ((uintptr_t)act & 15) == 0 && (MODE != CONV_FWD || (p.C % 4 == 0 && ((uintptr_t)wgt & 15) == 0));
+    int c = lo;
+    if (vec) {
+#pragma unroll 2
+        for (; c + 4 <= hi; c += 4) {
+            float w[4];
+            if (MODE == CONV_FWD) { const float4 v = sm_ld4<T>(wgt + ((long long)colc * TAPS + tap) * p.C + c); w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w; }
+            else {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) w[k] = sm_ld<T>(wgt + ((long long)(c + k) * TAPS + tap) * p.C + colc);
+            }
+            float4 a[SMALL_PB];
+#pragma unroll
+            for (int i = 0; i < SMALL_PB; ++i) a[i] = off[i] >= 0 ? sm_ld4<T>(act + off[i] + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int i = 0; i < SMALL_PB; ++i) acc[i] = fmaf(a[i].w, w[3], fmaf(a[i].z, w[2], fmaf(a[i].y, w[1], fmaf(a[i].x, w[0], acc[i]))));
+        }
+    }
+    for (; c < hi; ++c) {
+        const float w = MODE == CONV_FWD ? sm_ld<T>(wgt + ((long long)colc * TAPS + tap) * p.C + c) : sm_ld<T>(wgt + ((long long)c * TAPS + tap) * p.C + colc);
+#pragma unroll
+        for (int i = 0; i < SMALL_PB; ++i) acc[i] = fmaf(off[i] >= 0 ? sm_ld<T>(act + off[i] + c) : 0.f, w, acc[i]);
+    }
+    __shared__ float part[NW][SMALL_PB][32];
+#pragma unroll
+    for (int i = 0; i < SMALL_PB; ++i) part[warp][i][lane] = acc[i];
+    __syncthreads();
+    for (int i = warp; i < SMALL_PB; i += NW) {
+        const int m = m0 + i;
+        if (m >= M || col >= Ncol) continue;
+        float v = 0.f;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) v += part[w][i][lane];
+        v *= p.scale;
+        const long long o = (long long)m * Ncol + col;
+        if (p.add) v += sm_ld<T>((const T*)p.add + o);
+        sm_st<T>((T*)p.out + o, v);
+    }
+}
+
+// Weight gradient: a CTA takes 32 (tap, input channel) columns (lanes) x 8 output channels; its 32 warps take every 32nd position (few
+// enough that the loads of all of a warp's positions are in flight together) and their sums are added in warp order.
+template <class T>
+__global__ void __launch_bounds__(1024) wgrad_small_kernel(const ConvProb* __restrict__ probs) {
+    const ConvProb& p = probs[blockIdx.y];
+    const int K = p.K, C = p.C, Ncol = p.Ncol, M = p.Kred, ctiles = (Ncol + 31) >> 5, ktiles = (K + 7) >> 3;
+    if ((int)blockIdx.x >= ctiles * ktiles) return;
+    const int kt = blockIdx.x / ctiles, ct = blockIdx.x - kt * ctiles;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, col = ct * 32 + lane, k0 = kt * 8;
+    __shared__ int4 pos[1024];                                    // per position of a run of 1024: image row base, h, w of tap (0, 0), dy row
+    __shared__ float part[32][8][32];
+    const int cc = min(col, Ncol - 1), tap = cc / C, c = cc - tap * C, r = tap / p.ksz, s = tap - r * p.ksz;
+    const T* __restrict__ act = (const T*)p.act; const T* __restrict__ dy = (const T*)p.wgt;
+    const bool vec = k0 + 8 <= K && K % 4 == 0 && ((uintptr_t)dy & 15) == 0;
+    float acc[8] = {};
+    for (int mb = 0; mb < M; mb += 1024) {
+        __syncthreads();
+        { const int m = mb + threadIdx.x, q = m % p.Q, t = m / p.Q, pp = t % p.P, n = t / p.P; pos[threadIdx.x] = make_int4(n * p.H, pp * p.stride - p.pad, q * p.stride - p.pad, m * K + k0); }
+        __syncthreads();
+        const int run = min(1024, M - mb);
+#pragma unroll 4
+        for (int j = warp; j < run; j += 32) {
+            const int4 q = pos[j];
+            const int h = q.y + r, x = q.z + s;
+            const float a = (h >= 0 && h < p.H && x >= 0 && x < p.W) ? sm_ld<T>(act + (long long)((q.x + h) * p.W + x) * C + c) : 0.f;
+            if (vec) {
+                const float4 d0 = sm_ld4<T>(dy + q.w), d1 = sm_ld4<T>(dy + q.w + 4);
+                acc[0] = fmaf(d0.x, a, acc[0]); acc[1] = fmaf(d0.y, a, acc[1]); acc[2] = fmaf(d0.z, a, acc[2]); acc[3] = fmaf(d0.w, a, acc[3]);
+                acc[4] = fmaf(d1.x, a, acc[4]); acc[5] = fmaf(d1.y, a, acc[5]); acc[6] = fmaf(d1.z, a, acc[6]); acc[7] = fmaf(d1.w, a, acc[7]);
+            } else {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) if (k0 + k < K) acc[k] = fmaf(sm_ld<T>(dy + q.w + k), a, acc[k]);
+            }
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) part[warp][k][lane] = acc[k];
+    __syncthreads();
+    if (warp < 8 && k0 + warp < K && col < Ncol) {
+        float v = 0.f;
+#pragma unroll
+        for (int w = 0; w < 32; ++w) v += part[w][warp][lane];
+        ((float*)p.out)[(long long)(k0 + warp) * Ncol + col] = v;
+    }
+}
+
+// The line: up to 64 M multiply-adds (about where one GEMM tile per SM exists and the tiles' reuse starts to pay), filters of at most nine
+// taps, and for the weight gradient at most 2048 positions (its CTAs walk all of them).
+bool conv_small_ok(const ConvProb& p, int mode) {
+    if ((p.ksz != 1 && p.ksz != 3) || (double)p.M * p.Ncol * p.Kred > 64e6) return false;
+    if ((long long)p.N * p.H * p.W * p.C >= (1ll << 31) || (long long)p.N * p.P * p.Q * p.K >= (1ll << 31)) return false;
+    return mode != CONV_WGRAD || p.Kred <= 2048;
+}
+int conv_small_ctas(const ConvProb& p, int mode) {
+    if (mode == CONV_WGRAD) return ((p.Ncol + 31) / 32) * ((p.K + 7) / 8);
+    return ((p.M + SMALL_PB - 1) / SMALL_PB) * ((p.Ncol + 31) / 32);
+}
+template <class T>
+static void launch_small_t(const ConvProb* d, dim3 g, int mode, int ksz, cudaStream_t s) {
+    if (mode == CONV_WGRAD) wgrad_small_kernel<T><<<g, 1024, 0, s>>>(d);
+    else if (mode == CONV_FWD) { if (ksz == 3) conv_small_kernel<T, CONV_FWD, 3><<<g, 288, 0, s>>>(d); else conv_small_kernel<T, CONV_FWD, 1><<<g, 128, 0, s>>>(d); }
+    else { if (ksz == 3) conv_small_kernel<T, CONV_DGRAD, 3><<<g, 288, 0, s>>>(d); else conv_small_kernel<T, CONV_DGRAD, 1><<<g, 128, 0, s>>>(d); }
+}
+// all problems of a launch have the same filter size (max_ctas: the most conv_small_ctas() over them)
+void launch_conv_small(const ConvProb* d, int nprob, int max_ctas, int mode, int ksz, bool bf16, cudaStream_t s) {
+    if (bf16) launch_small_t<__nv_bfloat16>(d, dim3(max_ctas, nprob), mode, ksz, s); else launch_small_t<float>(d, dim3(max_ctas, nprob), mode, ksz, s);
+}
+
+// ------------------------------------------------------------------------------------------------ BN+ReLU in one launch
+// A CTA owns 8 channels over all rows: sums (of x - x[0] as in the other BN kernels; fp32 per thread, double across threads), statistics,
+// then the elementwise pass, whose second read comes from L1 or L2.
+template <class T, int MODE>
+__global__ void __launch_bounds__(512) bn_small_kernel(const BnProb* __restrict__ probs) {
+    const BnProb& p = probs[blockIdx.y];
+    const int C = p.C, c = blockIdx.x * 8 + (threadIdx.x & 7), m = (int)p.m, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if ((int)blockIdx.x * 8 >= C) return;
+    const bool on = c < C; const int cs = on ? c : C - 1;
+    const T* __restrict__ x = (const T*)p.x; const T* __restrict__ da = (const T*)p.da;
+    __shared__ double red[2][16][8];
+    __shared__ float st[4][8];
+    float mean = 0.f, istd = 0.f; const float ga = p.gamma[cs], be = p.beta[cs];
+    const float shift = MODE == 0 ? sm_ld<T>(x + cs) : 0.f;
+    if (MODE == 1) { mean = p.stat[cs]; istd = p.stat[C + cs]; }
+    float s0 = 0.f, s1 = 0.f;
+#pragma unroll 8
+    for (int r = threadIdx.x >> 3; r < m; r += 64) {
+        const float v = sm_ld<T>(x + (long long)r * C + cs);
+        if (MODE == 0) { const float d = v - shift; s0 += d; s1 += d * d; }
+        else { const float xh = (v - mean) * istd, dz = xh * ga + be > 0.f ? sm_ld<T>(da + (long long)r * C + cs) : 0.f; s0 += dz; s1 += dz * xh; }
+    }
+    double d0 = s0, d1 = s1;
+    d0 += __shfl_xor_sync(0xffffffffu, d0, 8); d1 += __shfl_xor_sync(0xffffffffu, d1, 8);
+    d0 += __shfl_xor_sync(0xffffffffu, d0, 16); d1 += __shfl_xor_sync(0xffffffffu, d1, 16);
+    if (lane < 8) { red[0][warp][lane] = d0; red[1][warp][lane] = d1; }
+    __syncthreads();
+    if (threadIdx.x < 8) {
+        double a0 = 0.0, a1 = 0.0;
+#pragma unroll
+        for (int w = 0; w < 16; ++w) { a0 += red[0][w][threadIdx.x]; a1 += red[1][w][threadIdx.x]; }
+        if (MODE == 0) {
+            const double dm_ = (double)m, dm = a0 / dm_;
+            double var = a1 / dm_ - dm * dm; if (var < 0.0) var = 0.0;
+            const double mu = dm + (double)shift;
+            st[0][threadIdx.x] = (float)mu; st[1][threadIdx.x] = (float)(1.0 / sqrt(var + (double)p.eps));
+            if (on) {
+                p.stat[c] = st[0][threadIdx.x]; p.stat[C + c] = st[1][threadIdx.x];
+                if (p.run_mean) {
+                    const double unb = m > 1 ? var * dm_ / (dm_ - 1.0) : var, mo = (double)p.momentum;
+                    p.run_mean[c] = (float)((1.0 - mo) * (double)p.run_mean[c] + mo * mu);
+                    p.run_var[c] = (float)((1.0 - mo) * (double)p.run_var[c] + mo * unb);
+                }
+            }
+        } else {
+            st[2][threadIdx.x] = (float)a0; st[3][threadIdx.x] = (float)a1;
+            if (on) { p.stat[2 * C + c] = (float)a0; p.stat[3 * C + c] = (float)a1; p.dbeta[c] = (float)a0; p.dgamma[c] = (float)a1; }
+        }
+    }
+    __syncthreads();
+    if (!on) return;
+    const int j = threadIdx.x & 7;
+    const float inv_m = 1.f / (float)m;
+    if (MODE == 0) { mean = st[0][j]; istd = st[1][j]; }
+    const float sb = MODE == 1 ? st[2][j] * inv_m : 0.f, sg = MODE == 1 ? st[3][j] * inv_m : 0.f;
+#pragma unroll 4
+    for (int r = threadIdx.x >> 3; r < m; r += 64) {
+        const long long i = (long long)r * C + c;
+        const float xh = (sm_ld<T>(x + i) - mean) * istd;
+        if (MODE == 0) { const float z = xh * ga + be; sm_st<T>((T*)p.a + i, z > 0.f ? z : 0.f); }
+        else {
+            const float dz = xh * ga + be > 0.f ? sm_ld<T>(da + i) : 0.f;
+            float v = ga * istd * (dz - sb - xh * sg);
+            if (p.add) v += sm_ld<T>((const T*)p.add + i);
+            sm_st<T>((T*)p.dx + i, v);
+        }
+    }
+}
+// Up to 8192 rows a CTA's walk over all of them costs less than the two launches saved (128 rows per thread, twice).
+bool bn_small_ok(const BnProb& p) { return !p.vec && !p.eval && p.m <= 8192; }
+void launch_bn_small(const BnProb* d, int nprob, int max_c, int backward, bool bf16, cudaStream_t s) {
+    const dim3 g((max_c + 7) / 8, nprob);
+    if (bf16) { if (backward) bn_small_kernel<__nv_bfloat16, 1><<<g, 512, 0, s>>>(d); else bn_small_kernel<__nv_bfloat16, 0><<<g, 512, 0, s>>>(d); }
+    else { if (backward) bn_small_kernel<float, 1><<<g, 512, 0, s>>>(d); else bn_small_kernel<float, 0><<<g, 512, 0, s>>>(d); }
+}
+
+}  // namespace resist

@@ -166,7 +166,8 @@ extern "C" int resist_conv2d(int32_t mode, int32_t dtype, int32_t backend, const
     if (be == 2) hd.resize(mode == CONV_WGRAD ? conv_wgrad_mma_prob_bytes() : conv_mma_prob_bytes());
     const size_t hd_room = (hd.size() + 255) / 256 * 256;
     if (be && mode == CONV_WGRAD) scratch = hd_room + wg_partial; else if (be) scratch = hd_room;
-    if (!be && mode == CONV_WGRAD) {
+    const bool small = !be && conv_small_ok(p, mode);
+    if (!be && mode == CONV_WGRAD && !small) {
         const int tiles = p.tiles_m * p.tiles_n;
         int want = (2 * sm + tiles - 1) / tiles; want = std::max(1, std::min(std::min(want, 64), ktiles));
         p.ktiles_per_split = (ktiles + want - 1) / want; p.splits = (ktiles + p.ktiles_per_split - 1) / p.ktiles_per_split;
@@ -200,6 +201,7 @@ extern "C" int resist_conv2d(int32_t mode, int32_t dtype, int32_t backend, const
         }
         else if (be == 2 && mode == CONV_WGRAD) launch_conv_wgrad_mma_probs(blob + 1024, 1, conv_wgrad_mma_ctas(hd.data()), conv_wgrad_mma_smem(hd.data()), conv_wgrad_mma_out_elems(hd.data()), conv_wgrad_mma_pick_variant(p, 2 * sm), st);
         else if (be == 2) launch_conv_mma_probs(blob + 1024, 1, conv_mma_tiles(hd.data()), conv_mma_smem(hd.data()), conv_mma_pick_variant(p, mode), st);
+        else if (small) launch_conv_small((ConvProb*)blob, 1, conv_small_ctas(p, mode), mode, ksz, dtype == RESIST_BF16, st);
         else {
             launch_conv_ref((ConvProb*)blob, 1, p.tiles_m * p.tiles_n * p.splits, mode, dtype == RESIST_BF16, st);
             if (mode == CONV_WGRAD && p.splits > 1) launch_splitk_reduce((ConvProb*)blob, 1, p.M * p.Ncol, st);

@@ -190,7 +190,7 @@ struct Builder {
                 ops->push_back(u); p.add = up_buf;
             }
         }
-        if (mode == CONV_WGRAD && !op.backend) {
+        if (mode == CONV_WGRAD && !op.backend && !conv_small_ok(p, mode)) {
             const int tiles = p.tiles_m * p.tiles_n;
             int want = (2 * ctx->sm_count + tiles - 1) / tiles; if (want > 64) want = 64; if (want > ktiles) want = ktiles; if (want < 1) want = 1;
             p.ktiles_per_split = (ktiles + want - 1) / want; p.splits = (ktiles + p.ktiles_per_split - 1) / p.ktiles_per_split;
@@ -301,6 +301,7 @@ struct Builder {
             return stat;
         }
         if (p.vec && !eval && r.c <= 512 && (long long)p.chunks * ctx->S <= bn_fused_capacity(0)) { op.kind = OP_BN_FWD_FUSED; ops->push_back(op); return stat; }   // one cooperative launch
+        if (bn_small_ok(p)) { op.kind = OP_BN_FWD_SMALL; ops->push_back(op); return stat; }
         ops->push_back(op);
         op.key = key + 1; op.kind = OP_BN_APPLY; ops->push_back(op);
         return stat;
@@ -318,6 +319,7 @@ struct Builder {
         bn_partial_need = std::max(bn_partial_need, (size_t)p.chunks * 2 * r.c * 8);
         p.partial = bn_partial;
         const int producer = last_dgrad; last_dgrad = -1;
+        if (bn_small_ok(p)) { op.kind = OP_BN_BWD_SMALL; ops->push_back(op); return; }
         if (fusable(producer, da, p)) { fuse_into(producer, p, 2); return; }
         // one cooperative launch where all sub-ResNets' chunks can be resident together (the kernel holds 128 registers: one CTA
         // per SM), else the reduction and the elementwise pass as launches of their own
@@ -625,12 +627,15 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
                     if (o.kind == OP_SPLITK) { L.max_elems = std::max<long long>(L.max_elems, (long long)p.M * p.Ncol);
                         L.bytes += 4.0 * p.M * p.Ncol * (p.splits + 1); }
                     else { L.gx = std::max(L.gx, p.tiles_m * p.tiles_n * p.splits);
+                        { const int mode = o.kind == OP_CONV_FWD ? CONV_FWD : o.kind == OP_CONV_DGRAD ? CONV_DGRAD : CONV_WGRAD;
+                          if (k == i) { L.ksz = p.ksz; L.small_ctas = 1; }
+                          L.small_ctas = L.small_ctas && p.splits == 1 && p.ksz == L.ksz && conv_small_ok(p, mode) ? std::max(L.small_ctas, conv_small_ctas(p, mode)) : 0; }
                         const double in_e = (double)p.N * p.H * p.W * p.C, out_e = (double)p.N * p.P * p.Q * p.K, w_e = (double)p.K * p.ksz * p.ksz * p.C;
                         L.flops += 2.0 * out_e * p.ksz * p.ksz * p.C;
                         if (o.kind == OP_CONV_WGRAD) L.bytes += es * (in_e + out_e) + 4.0 * w_e;
                         else L.bytes += es * (in_e + out_e + w_e + (p.add ? (o.kind == OP_CONV_FWD ? out_e : in_e) : 0.0)); }
                     break; }
-                case OP_BN_STATS: case OP_BN_APPLY: case OP_BN_BWD_REDUCE: case OP_BN_BWD_APPLY: case OP_BN_FWD_FUSED: case OP_BN_BWD_FUSED: case OP_BN_TILE_STATS: case OP_BN_EVAL_STATS: {
+                case OP_BN_STATS: case OP_BN_APPLY: case OP_BN_BWD_REDUCE: case OP_BN_BWD_APPLY: case OP_BN_FWD_FUSED: case OP_BN_BWD_FUSED: case OP_BN_TILE_STATS: case OP_BN_EVAL_STATS: case OP_BN_FWD_SMALL: case OP_BN_BWD_SMALL: {
                     if (k == i) L.first = (int)bn.size();
                     bn.push_back(o.bn);
                     L.gx = std::max(L.gx, o.bn.chunks); L.max_c = std::max(L.max_c, o.bn.C);
@@ -641,7 +646,7 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
                       else if (o.kind == OP_BN_STATS) L.bytes += es * e;
                       else if (o.kind == OP_BN_APPLY) L.bytes += 2 * es * e;
                       else if (o.kind == OP_BN_BWD_REDUCE) L.bytes += 2 * es * e;
-                      else if (o.kind == OP_BN_FWD_FUSED) L.bytes += 2 * es * e;          // x once from HBM (the second read is an L2 hit), a once
+                      else if (o.kind == OP_BN_FWD_FUSED || o.kind == OP_BN_FWD_SMALL) L.bytes += 2 * es * e;          // x once from HBM (the second read is an L2 hit), a once
                       else if (o.kind == OP_BN_BWD_FUSED) L.bytes += es * e * (o.bn.add ? 4 : 3);
                       else L.bytes += es * e * (o.bn.add ? 4 : 3); }
                     break; }
@@ -691,8 +696,8 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
                         break;
                     case OP_CONV_WGRAD: case OP_SPLITK: case OP_REPACK: break;
                     case OP_BN_STATS: case OP_BN_BWD_REDUCE: case OP_BN_TILE_STATS: case OP_BN_EVAL_STATS: break;
-                    case OP_BN_APPLY: case OP_BN_FWD_FUSED: wr.push_back(o.bn.a); break;
-                    case OP_BN_BWD_APPLY: case OP_BN_BWD_FUSED: wr.push_back(o.bn.dx); break;
+                    case OP_BN_APPLY: case OP_BN_FWD_FUSED: case OP_BN_FWD_SMALL: wr.push_back(o.bn.a); break;
+                    case OP_BN_BWD_APPLY: case OP_BN_BWD_FUSED: case OP_BN_BWD_SMALL: wr.push_back(o.bn.dx); break;
                     default: always = true; break;
                 }
             }
@@ -863,9 +868,9 @@ static int run_plan(resist_ctx* ctx, Plan& plan, const PatchArgs& pa, bool updat
             case OP_HEAD_BWD: pk = PK_HEAD_BWD; nk = head_small(L.max_c, L.max_classes) ? 1 : 3; break;
             case OP_UPSAMPLE: pk = PK_UPSAMPLE; break;
             case OP_IM2COL: pk = PK_IM2COL; break;
-            case OP_BN_FWD_FUSED: pk = PK_BN_FWD_FUSED; break;
+            case OP_BN_FWD_FUSED: case OP_BN_FWD_SMALL: pk = PK_BN_FWD_FUSED; break;
             case OP_BN_TILE_STATS: pk = PK_BN_TILE_STATS; break;
-            case OP_BN_BWD_FUSED: pk = PK_BN_BWD_FUSED; break;
+            case OP_BN_BWD_FUSED: case OP_BN_BWD_SMALL: pk = PK_BN_BWD_FUSED; break;
         }
         pf.begin(pk, nk, L.bytes, L.flops, st, L.label);
         switch (L.kind) {
@@ -878,11 +883,14 @@ static int run_plan(resist_ctx* ctx, Plan& plan, const PatchArgs& pa, bool updat
                 }
                 else if (L.backend && mode == CONV_WGRAD) { launch_conv_wgrad_tc_probs((const char*)plan.d_wtc + (size_t)L.first * plan.wtc_stride, L.count, L.gx, (size_t)L.max_elems, L.max_b, st); ++n_launch; }
                 else if (L.backend) launch_conv_tc_probs((const char*)plan.d_tc + (size_t)L.first * plan.tc_stride, L.ndesc, L.gx, (size_t)L.max_elems, st);
+                else if (L.small_ctas) launch_conv_small(plan.d_conv + L.first, L.count, L.small_ctas, mode, L.ksz, bf, st);
                 else launch_conv_ref(plan.d_conv + L.first, L.count, L.gx, mode, bf, st);
                 ++n_launch; break; }
             case OP_SPLITK: launch_splitk_reduce(plan.d_conv + L.first, L.count, (int)L.max_elems, st); ++n_launch; break;
             case OP_REPACK: launch_repack_rows(plan.d_conv + L.first, L.count, (int)L.max_elems, st); ++n_launch; break;
             case OP_BN_STATS: launch_bn_stats(plan.d_bn + L.first, L.count, L.gx, L.max_c, bf, st); n_launch += 2; break;
+            case OP_BN_FWD_SMALL: launch_bn_small(plan.d_bn + L.first, L.count, L.max_c, 0, bf, st); ++n_launch; break;
+            case OP_BN_BWD_SMALL: launch_bn_small(plan.d_bn + L.first, L.count, L.max_c, 1, bf, st); ++n_launch; break;
             case OP_BN_EVAL_STATS: launch_bn_eval_stats(plan.d_bn + L.first, L.count, L.max_c, st); ++n_launch; break;
             case OP_BN_APPLY: launch_bn_apply(plan.d_bn + L.first, L.count, L.max_elems, bf, st); ++n_launch; break;
             case OP_BN_BWD_REDUCE: launch_bn_bwd_reduce(plan.d_bn + L.first, L.count, L.gx, L.max_c, bf, st); n_launch += 2; break;
