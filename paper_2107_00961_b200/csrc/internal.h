@@ -155,7 +155,7 @@ void launch_repack_rows(const ConvProb* d, int nprob, int max_elems, cudaStream_
 void launch_zero_stuff(const UpProb* d, int nprob, long long max_vecs, cudaStream_t s);   // conv_tc.cu
 
 // ---- launchers (kernels_bw.cu)
-void launch_sgd(const Segment* d, int nseg, long long nchunks, ParamArrays pa, float lr, float mu, float wd,
+void launch_sgd(const Segment* d, int nseg, long long nchunks, ParamArrays pa, const float* lr, float mu, float wd,
                 bool shadow, cudaStream_t s);
 void launch_scatter(const Segment* d, int nseg, long long nchunks, ParamArrays pa, bool zero_momentum, bool shadow,
                     cudaStream_t s);

@@ -29,7 +29,8 @@ __device__ __forceinline__ unsigned pack_bf16x2(float a, float b) {
 // v = mu*v + (g + wd*w);  w = w - lr*v;  bf16 copy of w refreshed for the convolutions
 template <bool SHADOW>
 __global__ void __launch_bounds__(256) sgd_kernel(const Segment* __restrict__ segs, int nseg, ParamArrays pa,
-                                                  float lr, float mu, float wd) {
+                                                  const float* __restrict__ lr_dev, float mu, float wd) {
+    const float lr = __ldg(lr_dev);                               // in device memory, so that a recorded step serves every learning rate
     const Segment& sg = find_segment(segs, nseg, blockIdx.x);
     const Range r = chunk_range(sg, blockIdx.x);
     const long long o = (long long)sg.sub * pa.n + r.base;
@@ -186,7 +187,7 @@ __global__ void __launch_bounds__(256, 3) aggregate_kernel(const Segment* __rest
     }
 }
 
-void launch_sgd(const Segment* d, int nseg, long long nchunks, ParamArrays pa, float lr, float mu, float wd,
+void launch_sgd(const Segment* d, int nseg, long long nchunks, ParamArrays pa, const float* lr, float mu, float wd,
                 bool shadow, cudaStream_t s) {
     if (nchunks <= 0) return;
     if (shadow) sgd_kernel<true><<<(unsigned)nchunks, 256, 0, s>>>(d, nseg, pa, lr, mu, wd);

@@ -77,6 +77,7 @@ static size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 static int out_dim(int h, int k, int stride) { return (h + 2 * ((k - 1) / 2) - k) / stride + 1; }
 
 void free_plan(resist_ctx* ctx, Plan& p) {
+    if (p.graph) cudaGraphExecDestroy(p.graph);
     ctx_free(ctx, p.d_blob);
     p = Plan();
 }
@@ -84,9 +85,11 @@ void free_plan(resist_ctx* ctx, Plan& p) {
 struct PatchArgs {
     const void* images[RESIST_MAX_SUBNETS]; const int* labels[RESIST_MAX_SUBNETS];
     float* loss_out; float* logits_out; int* correct;
+    float* lr_slot; float lr;
 };
 __global__ void patch_kernel(const PatchSite* sites, int n, PatchArgs a) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0 && a.lr_slot) *a.lr_slot = a.lr;
     if (i >= n) return;
     const PatchSite s = sites[i];
     void* v = nullptr;
@@ -729,8 +732,10 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
     const size_t o_mm = off;   off += align_up(mm.size(), 256);
     const size_t o_col = off;  off += align_up(col.size() * sizeof(ColProb), 256);
     const size_t o_wmm = off;  off += align_up(wmm.size(), 256);
+    if (plan.graph) cudaGraphExecDestroy(plan.graph);
+    plan.graph = nullptr; plan.runs = 0; plan.graph_failed = false;
     ctx_free(ctx, plan.d_blob);
-    plan.d_blob = ctx_alloc(ctx, off + 256); plan.blob_bytes = off;
+    plan.d_blob = ctx_alloc(ctx, off + 256); plan.blob_bytes = off; plan.d_lr = (float*)((char*)plan.d_blob + off);
     if (!plan.d_blob) { ctx->err = "allocator returned NULL for the launch plan"; return RESIST_ENOMEM; }
     char* base = (char*)plan.d_blob;
     plan.d_conv = (ConvProb*)(base + o_conv); plan.d_bn = (BnProb*)(base + o_bn); plan.d_pool = (PoolProb*)(base + o_pool);
@@ -813,30 +818,31 @@ static int build_plan(resist_ctx* ctx, Plan& plan, int sub, int B, cudaStream_t 
     return RESIST_OK;
 }
 
-static int run_plan(resist_ctx* ctx, Plan& plan, const PatchArgs& pa, bool update, float lr, cudaStream_t st) {
-    const bool bf = ctx->opts.dtype == RESIST_BF16;
-    long long n_launch = 0;
-    Profiler& pf = ctx->prof;
-    const cudaStream_t caller_st = st;
-    const bool overlap = !pf.on && update;
-    if (overlap && !ctx->main_stream) {
+// The streams a step runs on beside the caller's (created on first use).
+static int ensure_streams(resist_ctx* ctx) {
+    if (!ctx->main_stream) {
         int lo = 0, hi = 0; cudaDeviceGetStreamPriorityRange(&lo, &hi);      // hi: numerically lowest = greatest priority
         if (cudaStreamCreateWithPriority(&ctx->main_stream, cudaStreamNonBlocking, hi) != cudaSuccess ||
             cudaEventCreateWithFlags(&ctx->ev_enter, cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&ctx->ev_leave, cudaEventDisableTiming) != cudaSuccess) { ctx->err = "cannot create the main stream"; return RESIST_ECUDA; }
     }
-    if (overlap) { cudaEventRecord(ctx->ev_enter, caller_st); cudaStreamWaitEvent(ctx->main_stream, ctx->ev_enter, 0); st = ctx->main_stream; }
-    if (plan.nsites) { pf.begin(PK_PATCH, 1, 0, 0, st); patch_kernel<<<(plan.nsites + 63) / 64, 64, 0, st>>>(plan.d_sites, plan.nsites, pa); pf.end(st); ++n_launch; }
+    if (!ctx->side_stream) {
+        if (cudaStreamCreateWithFlags(&ctx->side_stream, cudaStreamNonBlocking) != cudaSuccess ||
+            cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
+            cudaEventCreateWithFlags(&ctx->ev_side_done, cudaEventDisableTiming) != cudaSuccess) { ctx->err = "cannot create the second stream"; return RESIST_ECUDA; }
+    }
+    return RESIST_OK;
+}
+
+// Enqueues the plan's launches on `st` (and, with overlap, the weight gradients on the second stream, joined at the end).
+static int enqueue_launches(resist_ctx* ctx, Plan& plan, bool update, bool overlap, cudaStream_t st, long long& n_launch) {
+    const bool bf = ctx->opts.dtype == RESIST_BF16;
+    Profiler& pf = ctx->prof;
     // A layer's weight gradient and data gradient both read dy and are independent of each other: the weight gradients
     // (and their partial-sum reductions) go to a second stream, one after another, while the main stream carries on
     // down the network.  Gradient buffers are recycled, so a launch that writes a buffer which a weight gradient in
     // flight still reads first waits for the second stream (join_before, worked out when the plan was built).
     // Per-kernel profiling keeps everything on one stream.
-    if (overlap && !ctx->side_stream) {
-        if (cudaStreamCreateWithFlags(&ctx->side_stream, cudaStreamNonBlocking) != cudaSuccess ||
-            cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-            cudaEventCreateWithFlags(&ctx->ev_side_done, cudaEventDisableTiming) != cudaSuccess) { ctx->err = "cannot create the second stream"; return RESIST_ECUDA; }
-    }
     bool side_pending = false;
     const cudaStream_t main_st = st;
     OpKind prev_kind = OP_HEAD_FWD;
@@ -918,11 +924,51 @@ static int run_plan(resist_ctx* ctx, Plan& plan, const PatchArgs& pa, bool updat
     if (side_pending) cudaStreamWaitEvent(main_st, ctx->ev_side_done, 0);
     if (update && plan.sgd_chunks) {
         pf.begin(PK_SGD, 1, (bf ? 22.0 : 20.0) * plan.sgd_params, 0, st);
-        launch_sgd(plan.d_sgd, plan.n_sgd_seg, plan.sgd_chunks, ctx->pa, lr, ctx->opts.momentum, ctx->opts.weight_decay, bf, st);
+        launch_sgd(plan.d_sgd, plan.n_sgd_seg, plan.sgd_chunks, ctx->pa, plan.d_lr, ctx->opts.momentum, ctx->opts.weight_decay, bf, st);
         pf.end(st);
         ++n_launch;
     }
-    if (overlap) { cudaEventRecord(ctx->ev_leave, st); cudaStreamWaitEvent(caller_st, ctx->ev_leave, 0); }
+    return RESIST_OK;
+}
+
+// Records the plan's launches (everything but the patching of the call's pointers) as a graph.  A step is up to 400 launches, two
+// events around every weight gradient among them: enqueueing them costs the host 0.3 to 1 ms, and each dependent pair of launches
+// a few microseconds of idle GPU.  Failing to record is no error: the plan keeps being enqueued launch by launch.
+static void record_plan(resist_ctx* ctx, Plan& plan, bool update) {
+    plan.graph_failed = true;
+    cudaGraph_t g = nullptr;
+    if (cudaStreamBeginCapture(ctx->main_stream, cudaStreamCaptureModeRelaxed) != cudaSuccess) { cudaGetLastError(); return; }
+    long long n = 0;
+    const int rc = enqueue_launches(ctx, plan, update, update, ctx->main_stream, n);
+    const cudaError_t e = cudaStreamEndCapture(ctx->main_stream, &g);
+    if (rc == RESIST_OK && e == cudaSuccess && g && cudaGraphInstantiate(&plan.graph, g, cudaGraphInstantiateFlagUseNodePriority) == cudaSuccess) { plan.graph_failed = false; plan.graph_launches = n; }
+    else plan.graph = nullptr;
+    if (g) cudaGraphDestroy(g);
+    cudaGetLastError();
+}
+
+static int run_plan(resist_ctx* ctx, Plan& plan, PatchArgs pa, bool update, float lr, cudaStream_t st) {
+    long long n_launch = 0;
+    Profiler& pf = ctx->prof;
+    const cudaStream_t caller_st = st;
+    const bool overlap = !pf.on && update;
+    { const int rc = ensure_streams(ctx); if (rc) return rc; }
+    // a caller that is recording a graph of its own gets the launches, not a graph inside it
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(caller_st, &cap) != cudaSuccess) { cudaGetLastError(); cap = cudaStreamCaptureStatusActive; }
+    if (!pf.on && cap == cudaStreamCaptureStatusNone) {
+        if (plan.runs < 2) ++plan.runs;
+        else if (!plan.graph && !plan.graph_failed) record_plan(ctx, plan, update);
+    }
+    const bool use_graph = plan.graph && !pf.on && cap == cudaStreamCaptureStatusNone;
+    if (overlap && !use_graph) { cudaEventRecord(ctx->ev_enter, caller_st); cudaStreamWaitEvent(ctx->main_stream, ctx->ev_enter, 0); st = ctx->main_stream; }
+    pa.lr_slot = update ? plan.d_lr : nullptr; pa.lr = lr;
+    if (plan.nsites || update) { pf.begin(PK_PATCH, 1, 0, 0, st); patch_kernel<<<(plan.nsites + 64) / 64, 64, 0, st>>>(plan.d_sites, plan.nsites, pa); pf.end(st); ++n_launch; }
+    if (use_graph) {
+        if (cudaGraphLaunch(plan.graph, caller_st) != cudaSuccess) { ctx->err = "the recorded step failed to launch"; cudaGetLastError(); return RESIST_ECUDA; }
+        n_launch += plan.graph_launches;
+    } else { const int rc = enqueue_launches(ctx, plan, update, overlap, st, n_launch); if (rc) return rc; }
+    if (overlap && !use_graph) { cudaEventRecord(ctx->ev_leave, st); cudaStreamWaitEvent(caller_st, ctx->ev_leave, 0); }
     pf.collect(st);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) { ctx->err = std::string("launch failed: ") + cudaGetErrorString(e); return RESIST_ECUDA; }

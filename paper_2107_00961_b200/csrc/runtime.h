@@ -83,6 +83,9 @@ struct Plan {
     void* d_wtc = nullptr; size_t wtc_stride = 0;            // tensor-core wgrad descriptors
     void* d_mm = nullptr; size_t mm_stride = 0; void* d_wmm = nullptr; size_t wmm_stride = 0;   // warp-level MMA descriptors
     Segment* d_sgd = nullptr; int n_sgd_seg = 0; long long sgd_chunks = 0; double sgd_params = 0;
+    float* d_lr = nullptr;                                    // learning rate of the step at hand (written with the patched pointers)
+    // The plan's launches as a graph, recorded when the plan runs for the third time (a round of one or two steps does not pay for it)
+    cudaGraphExec_t graph = nullptr; int runs = 0; bool graph_failed = false; long long graph_launches = 0;
     resist_step_info info{};
 };
 
