@@ -91,11 +91,7 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint32
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");   // src_bytes 0: zeros
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-// Programmatic dependent launch: a kernel launched with the attribute may start while the kernel before it in the
-// stream is still running; it must not touch anything that kernel writes before pdl_wait() returns (which is when that
-// kernel has finished and its writes are visible).  pdl_trigger() lets the NEXT kernel of the stream start early.
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Programmatic dependent launch (internal.h).  These kernels read their weights ahead of the wait: the kernel before must not write them.
 template <class K, class A>
 static void launch_pdl(K kernel, dim3 grid, size_t smem, cudaStream_t s, bool pdl, A arg) {
     cudaLaunchConfig_t cfg = {}; cfg.gridDim = grid; cfg.blockDim = dim3(256); cfg.dynamicSmemBytes = smem; cfg.stream = s;
@@ -124,7 +120,6 @@ const MmaProb* __restrict__ probs) {
     __shared__ MmaProb p;
     if (threadIdx.x < sizeof(MmaProb) / 4) reinterpret_cast<uint32_t*>(&p)[threadIdx.x] = reinterpret_cast<const uint32_t*>(probs + blockIdx.y)[threadIdx.x];
     __syncthreads();
-    pdl_trigger();
     constexpr int TAPS = KSZ * KSZ, PAD = KSZ / 2, ncol = NB * 8;   // ncol: output channels of THIS CTA
     const int units = p.units, nsplit = p.nsplit;
     const int ncol_all = ncol * nsplit, n_off = ((int)blockIdx.x % nsplit) * ncol;
@@ -258,7 +253,7 @@ const MmaProb* __restrict__ probs) {
     if (coop) for (int i = tid; i < 8 * 2 * ncol; i += MMA_THREADS) (&s_red[0][0][0])[i] = 0.f;
 
     __syncthreads();                                              // tables complete
-    pdl_wait();                                                   // from here on: tensors the previous kernel may have written
+    chain_wait();                                                 // from here on: tensors the previous kernel may have written
     const __nv_bfloat16* __restrict__ bnx = reinterpret_cast<const __nv_bfloat16*>(p.bn.x);
     if (fuse >= 2 && tid < ncol) {
         const int c = n_off + tid;
@@ -706,7 +701,6 @@ __global__ void __launch_bounds__(MMA_THREADS) conv_wgrad_mma_kernel(const MmaWg
     __shared__ MmaWgradProb p;
     if (threadIdx.x < sizeof(MmaWgradProb) / 4) reinterpret_cast<uint32_t*>(&p)[threadIdx.x] = reinterpret_cast<const uint32_t*>(probs + blockIdx.y)[threadIdx.x];
     __syncthreads();
-    pdl_trigger();
     if ((int)blockIdx.x >= p.tap_groups * p.splits) return;
     const int split = blockIdx.x % p.splits, tg = blockIdx.x / p.splits;
     const int tap0 = tg * p.taps_per_group; int ntap = p.taps - tap0; if (ntap > p.taps_per_group) ntap = p.taps_per_group;
@@ -800,7 +794,7 @@ __global__ void __launch_bounds__(MMA_THREADS) conv_wgrad_mma_kernel(const MmaWg
     const int ksteps = sub / 16;
 
     __syncthreads();                                              // table complete
-    pdl_wait();                                                   // from here on: tensors the previous kernel may have written
+    chain_wait();                                                 // from here on: tensors the previous kernel may have written
     const int units = p.units;
     int nxt = split;
     for (int st = 0; st < stages - 1; ++st) { if (nxt < units) issue(nxt, st); cp_async_commit(); nxt += p.splits; }
@@ -862,8 +856,7 @@ __global__ void __launch_bounds__(MMA_THREADS) conv_wgrad_mma_kernel(const MmaWg
 // out[k][t][c] = sum over splits of partial[split][t][k][c], in a fixed order: a block owns 32 consecutive elements,
 // warp w adds the splits w, w+8, ... (ascending), then the 8 sums are added in warp order.
 __global__ void __launch_bounds__(256) wgrad_mma_reduce_kernel(const MmaWgradProb* __restrict__ probs) {
-    pdl_trigger();
-    pdl_wait();                                                   // launched programmatically behind the kernel that writes the partial sums
+    chain_wait();                                                 // launched programmatically behind the kernel that writes the partial sums
     const MmaWgradProb& p = probs[blockIdx.y];
     const int n = p.taps * p.K * p.C, splits = p.splits, taps = p.taps, K = p.K, C = p.C;
     const float* __restrict__ partial = p.partial;

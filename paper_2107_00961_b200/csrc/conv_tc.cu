@@ -272,6 +272,7 @@ __global__ void __launch_bounds__(TC_CONV_THREADS, 1) conv_tc_kernel(const TcPro
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    chain_wait();                                                // from here on: tensors the previous kernel may have written or read
     const uint32_t tmem_base = tmem_base_s;
     // A unit of work is a pair of neighbouring row tiles (2 x 128 positions) times one column tile: the two tiles share every weight
     // tile, which is fetched once, and each has its own accumulator.  The units of all problems, column tile innermost, are dealt round-robin: the
@@ -936,6 +937,10 @@ static int phase_taps(int u, int v, int rs[4][2]) {
     return n;
 }
 
+static int device_sms() {
+    static const int n = [] { int dev = 0, v = 0; cudaGetDevice(&dev); cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev); return v > 0 ? v : 148; }();
+    return n;
+}
 static bool tc_shape_ok(const ConvProb& p) {
     if ((p.ksz != 1 && p.ksz != 3) || p.stride < 1 || p.stride > 2) return false;
     if (p.C % 8 || p.K % 8) return false;
@@ -973,6 +978,36 @@ int conv_tc_read_status() {
     const int v = *w;
     if (v) *w = 0;                                  // reported once
     return v;
+}
+
+// Columns per tile: up to 256, a multiple of 64 when there are several tiles.  A launch ends with its slowest CTA, so a launch of few units
+// takes the width with the least (waves of pairs) x (clocks per pair) over `group` such problems, the last partial wave possibly in
+// single tiles (see the kernel).  Clocks per tile: the tensor core needs 128 / 68 / 52 per MMA of 256 / 128 / 64 columns; the rings are fed
+// from L2 at about 28 bytes per clock and SM (all SMs at once); an epilogue takes about 20 per column, and only runs under the next tile's
+// MMAs when two accumulators per tile fit TMEM (up to 128 columns).  Narrower tiles read every window once more, so they have to promise
+// 12 %, and from two full waves of the widest tiles on there is nothing to fill.  (50 images of 14 x 14 x 256, 3x3: 88 tiles of 256
+// columns are 88 busy SMs of 148; 74 -> 63 us for the layer call.  Evaluation of 50 ImageNet-shaped images 2.19 -> 1.95 ms.)
+static void pick_n_tile(TcHot& t, int ntaps, int group, int phases) {
+    const int sms = device_sms();
+    double best = 0; int best_n = 0; long long wide_pairs = 0;
+    const int first = (t.ncol + 255) / 256;
+    for (int tn = first; tn <= std::max(first, (t.ncol + 63) / 64); ++tn) {
+        int n = (t.ncol + tn - 1) / tn;
+        n = tn > 1 ? (n + 63) / 64 * 64 : (n + 15) / 16 * 16;
+        if ((t.ncol + n - 1) / n != tn) continue;
+        const double mma = n > 128 ? n / 2.0 : n > 64 ? 68 : 52, steps = (double)ntaps * t.slabs * std::min(4, (t.red + 15) / 16);
+        const double epi = 20.0 * n + 500, a_bytes = (double)t.slabs * t.ngroups * t.nbox * t.a_box_bytes, b_bytes = (double)t.slabs * ntaps * n * 128;
+        auto unit = [&](int tiles) {
+            const double run = std::max(tiles * steps * mma, (tiles * a_bytes + b_bytes) / 28) + 300;
+            return n > 128 ? run + epi : std::max(run, epi);
+        };
+        const long long pairs = (long long)((t.tiles_m + 1) / 2) * tn * group * phases, rest = pairs % sms;
+        const double time = (double)(pairs / sms) * unit(2) + (rest == 0 ? 0 : 2 * rest <= sms ? unit(1) : unit(2)) + (n > 128 ? 0 : epi);
+        if (best_n && wide_pairs >= 2 * sms) break;
+        if (!best_n) wide_pairs = pairs;
+        if (!best_n || time < 0.88 * best) { best = time; best_n = n; }
+    }
+    t.n_tile = best_n; t.tiles_n = (t.ncol + best_n - 1) / best_n;
 }
 
 // Fills conv_tc_count() host-side TcProbs for this problem.  Returns the number written (0: not supported or encoding failed).
@@ -1045,17 +1080,12 @@ int conv_tc_fill(const ConvProb& p, int mode, void* host_tc) {
         }
         // residual
         t.add_mode = !p.add ? 0 : p.add_sub == 2 ? 3 : 2;
-        // output tiles: up to 256 columns, a multiple of 64 when there are several
-        const int n_cap = 256;
         const int ntaps = t.gbeg[t.ngroups];
         auto b_tile = [&](int nt) { return mode == CONV_FWD ? nt * 128 : ((nt + 63) / 64) * 8192; };
         auto b_total = [&](int nt) { return (size_t)t.slabs * ntaps * ((b_tile(nt) + 1023) / 1024 * 1024); };
-        t.tiles_n = (ncol + n_cap - 1) / n_cap;
-        t.n_tile = (ncol + t.tiles_n - 1) / t.tiles_n;
-        t.n_tile = t.tiles_n > 1 ? (t.n_tile + 63) / 64 * 64 : (t.n_tile + 15) / 16 * 16;
-        t.tiles_n = (ncol + t.n_tile - 1) / t.n_tile;
-        t.out_slabs = (t.n_tile + 63) / 64;
         t.tiles_m = (t.total_pos + TILE_M - 1) / TILE_M;
+        pick_n_tile(t, ntaps, p.group > 0 ? p.group : 1, count);
+        t.out_slabs = (t.n_tile + 63) / 64;
         t.b_bytes = b_tile(t.n_tile);
         t.b_total = (int)b_total(t.n_tile);
         // weights [K][taps][C] viewed as (C, tap, K).  Forward: a tile is n_tile output channels (rows) x 64 input channels.
@@ -1094,7 +1124,9 @@ size_t conv_tc_merge(size_t a, size_t b) {
 constexpr size_t TC_SMEM_BUDGET = 204 * 1024;
 
 // total_tiles: an upper bound of the tiles of all problems of the launch (max_tiles * nprob); packed: conv_tc_merge over its problems
-void launch_conv_tc_probs(const void* d_tc, int nprob, int max_tiles, size_t packed, cudaStream_t s) {
+// pdl: programmatic launch.  For evaluation, a chain of convolutions; in training the linked launches made the steps slower (ImageNet-shaped
+// 22.6 -> 24.4 ms with the forward half linked): between the convolutions run streaming kernels that want the whole SM.
+void launch_conv_tc_probs(const void* d_tc, int nprob, int max_tiles, size_t packed, cudaStream_t s, bool pdl) {
     static bool configured = false; static int sms = 0;
     if (!configured) {
         cudaFuncSetAttribute(conv_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(TC_SMEM_BUDGET + 1024));
@@ -1135,7 +1167,10 @@ void launch_conv_tc_probs(const void* d_tc, int nprob, int max_tiles, size_t pac
     const size_t smem = std::max((size_t)L.na * a + (size_t)L.nb * b + staging(), (size_t)120 * 1024) + 1024;
     const long long total = (long long)max_tiles * nprob;
     const int grid = (int)std::max(1ll, std::min(total, (long long)sms));
-    conv_tc_kernel<<<grid, TC_CONV_THREADS, smem, s>>>((const TcProb*)d_tc, L);
+    cudaLaunchConfig_t cfg = {}; cfg.gridDim = dim3(grid); cfg.blockDim = dim3(TC_CONV_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = s;
+    cudaLaunchAttribute at[1]; at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization; at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at; cfg.numAttrs = pdl ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, conv_tc_kernel, (const TcProb*)d_tc, (const TcLaunch)L);
 }
 
 // ---- wgrad host side

@@ -22,6 +22,7 @@ struct ConvProb {
     int M, Ncol, Kred;    // GEMM extents of this mode
     int tiles_m, tiles_n, splits, ktiles_per_split;
     float scale;          // result = scale*acc + add
+    int group;            // problems of the launch this one is part of (0: alone); tcgen05 column tiles are chosen by it
     int wg_ld, wg_cols;   // wgrad of a 1x1 problem on an im2col'ed input: row stride and valid columns of dw (0: K x C dense)
     int dy_sub;           // backward of a stride-2 layer as a stride-1 problem: 2 = dy is stored compact [N,dy_P,dy_Q,K] and read as if
     int dy_P, dy_Q;       //   zero-stuffed to H x W (only even positions exist); 0 or 1 = dy is stored at the problem's resolution
@@ -123,6 +124,14 @@ struct ParamArrays {      // device pointers of the flat arrays
     float* w;  float* v;  float* g;  __nv_bfloat16* wb;  float* buf;   // [S][n] each (buf: [S][n_buffers])
     long long n, nbuf;
 };
+
+#ifdef __CUDACC__
+// Programmatic dependent launch.  A kernel launched with that attribute takes its places and makes its set-up while the last CTAs of the
+// kernel before still run; when the wait returns, that kernel has finished and its writes are visible.  Every thread waits before it
+// touches anything an earlier kernel of the stream writes or reads, and only then lets the NEXT kernel in: with one kernel running and
+// one waiting, no line that a kernel reads can have been cached before its last write.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+#endif
 
 constexpr int SEG_CHUNK = 4096;   // elements per CTA in the segment kernels
 constexpr int AGG_CHUNK = 8192;   // elements per CTA of the aggregate kernel (two rounds of four 16-byte groups per thread)

@@ -15,7 +15,7 @@ size_t conv_tc_merge(size_t a, size_t b);
 size_t conv_tc_prob_bytes();
 int conv_tc_tiles(const void* host_tc);
 size_t conv_tc_smem(const void* host_tc);
-void launch_conv_tc_probs(const void* d_tc, int nprob, int max_tiles, size_t max_smem, cudaStream_t s);
+void launch_conv_tc_probs(const void* d_tc, int nprob, int max_tiles, size_t max_smem, cudaStream_t s, bool pdl = false);
 int conv_tc_read_status();
 bool conv_wgrad_tc_supported(const ConvProb& p, int target_ctas, size_t* partial_bytes);
 bool conv_wgrad_tc_fill(const ConvProb& p, int target_ctas, void* host_tc);

@@ -24,7 +24,7 @@ size_t conv_tc_prob_bytes();
 int conv_tc_tiles(const void* host_tc);
 size_t conv_tc_smem(const void* host_tc);
 size_t conv_tc_merge(size_t a, size_t b);
-void launch_conv_tc_probs(const void* d_tc, int nprob, int max_tiles, size_t max_smem, cudaStream_t s);
+void launch_conv_tc_probs(const void* d_tc, int nprob, int max_tiles, size_t max_smem, cudaStream_t s, bool pdl = false);
 bool conv_wgrad_tc_supported(const ConvProb& p, int target_ctas, size_t* partial_bytes);
 bool conv_wgrad_tc_fill(const ConvProb& p, int target_ctas, void* host_tc);
 size_t conv_wgrad_tc_prob_bytes();
@@ -556,6 +556,7 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
                    ops[i].kind != OP_UPSAMPLE && ops[i].kind != OP_IM2COL && ops[i].kind != OP_SPLITK && ops[i].kind != OP_REPACK)
             snprintf(L.label, sizeof(L.label), "bn m%lld C%d x%d", ops[i].bn.m, ops[i].bn.C, L.count);
         for (size_t k = i; k < j; ++k) {
+            ops[k].conv.group = (int)(j - i);
             const Op& o = ops[k]; const int slot = single ? 0 : o.sub;
             switch (o.kind) {
                 case OP_REPACK: {
@@ -888,7 +889,7 @@ static int enqueue_launches(resist_ctx* ctx, Plan& plan, bool update, bool overl
                         ctx->err = "warp-MMA convolution launch failed"; cudaGetLastError(); return RESIST_ECUDA; }
                 }
                 else if (L.backend && mode == CONV_WGRAD) { launch_conv_wgrad_tc_probs((const char*)plan.d_wtc + (size_t)L.first * plan.wtc_stride, L.count, L.gx, (size_t)L.max_elems, L.max_b, st); ++n_launch; }
-                else if (L.backend) launch_conv_tc_probs((const char*)plan.d_tc + (size_t)L.first * plan.tc_stride, L.ndesc, L.gx, (size_t)L.max_elems, st);
+                else if (L.backend) launch_conv_tc_probs((const char*)plan.d_tc + (size_t)L.first * plan.tc_stride, L.ndesc, L.gx, (size_t)L.max_elems, st, pdl_ok && !update);
                 else if (L.small_ctas) launch_conv_small(plan.d_conv + L.first, L.count, L.small_ctas, mode, L.ksz, bf, st);
                 else launch_conv_ref(plan.d_conv + L.first, L.count, L.gx, mode, bf, st);
                 ++n_launch; break; }
