@@ -188,7 +188,8 @@ struct TapRef { int wtap; int shift; };       // weight tap index (r*ksz + s); r
 // problems, one per output phase, do the same for a stride-2 dgrad.
 struct TcHot {                // everything the kernel's loops read: each role keeps a copy in shared memory
     const __nv_bfloat16* add; __nv_bfloat16* out;
-    float* stat_tiles;        // [tiles_m][2][ncol]: column sums and sums of squares of the stored tile, or nullptr
+    float* stat_tiles;        // [tiles_m][2][ncol]: column sums of the stored tile (of y and y^2, or with bwd_x of dz and dz * xhat), or nullptr
+    const __nv_bfloat16* bwd_x;   // dgrad whose output feeds a BN+ReLU backward: input of that BN (constants in bn_stat, bn_gamma, bn_beta)
     int* status;
     const float* bn_stat; const float* bn_gamma; const float* bn_beta; __nv_bfloat16* bn_out;   // evaluation: bn_out = relu(bn(y)) with mean | 1/std in bn_stat; nullptr otherwise
     int store_y;              // 0: only bn_out is wanted
@@ -231,6 +232,8 @@ __device__ __forceinline__ void copy_hot(TcHot* dst, const TcHot* src, int tid, 
     for (int i = tid; i < (int)(sizeof(TcHot) / 4); i += nthreads) d4[i] = __ldg(s4 + i);
 }
 
+// BWD: the instance of dgrad launches (sums of the BN backward, no BN of the output); the other one is forward's and evaluation's.
+template <bool BWD>
 __global__ void __launch_bounds__(TC_CONV_THREADS, 1) conv_tc_kernel(const TcProb* __restrict__ probs, const TcLaunch L) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -238,6 +241,7 @@ __global__ void __launch_bounds__(TC_CONV_THREADS, 1) conv_tc_kernel(const TcPro
     __shared__ uint32_t tmem_base_s;
     __shared__ int abort_s;
     __shared__ __align__(16) float stat_s2[2][4][2][256];
+    __shared__ __align__(16) float bwd_s2[BWD ? 2 : 1][4][BWD ? 256 : 4];   // per group: -mean, 1/std, gamma, beta of the column tile (from L2 they cost a slab 1000 clocks)
     __shared__ int unit_end_s[TC_MAX_PROBS];                      // running sum of the problems' unit counts (a unit: two row tiles x one column tile)
     __shared__ int tilesm_s[TC_MAX_PROBS], tilesn_s[TC_MAX_PROBS];
     __shared__ TcHot hot_s[3 + TC_ISSUERS];                   // the current problem of the producer, the two epilogue groups, the MMA issuer
@@ -472,7 +476,7 @@ __global__ void __launch_bounds__(TC_CONV_THREADS, 1) conv_tc_kernel(const TcPro
             const TcProb* pp = probs + pi;
             const uint32_t buf = (cnt % (uint32_t)L.nbuf) * 2u + (uint32_t)grp, aph = (cnt / (uint32_t)L.nbuf) & 1u;
             ++cnt;
-            if (pi != cur || (h.bn_out && tn != cur_tn)) {       // every warp of the group is through with the last problem's constants
+            if (pi != cur || ((h.bn_out || h.bwd_x) && tn != cur_tn)) {   // every warp of the group is through with the last problem's constants
                 bar_sync_epi(bid);
                 if (pi != cur) copy_hot(&hot_s[1 + grp], &probs[pi].h, et, 128);
                 bar_sync_epi(bid);
@@ -483,25 +487,35 @@ __global__ void __launch_bounds__(TC_CONV_THREADS, 1) conv_tc_kernel(const TcPro
                     }
                     bar_sync_epi(bid);
                 }
+                if (BWD && h.bwd_x) {
+                    float (*const w)[256] = reinterpret_cast<float (*)[256]>(&bwd_s2[BWD ? grp : 0][0][0]);
+                    for (int c = et; c < h.n_tile; c += 128) {
+                        const int g = min(tn * h.n_tile + c, h.ncol - 1);
+                        w[0][c] = -__ldg(h.bn_stat + g); w[1][c] = __ldg(h.bn_stat + h.ncol + g); w[2][c] = __ldg(h.bn_gamma + g); w[3][c] = __ldg(h.bn_beta + g);
+                    }
+                    bar_sync_epi(bid);
+                }
                 cur = pi; cur_tn = tn;
             }
             const int n_tile = h.n_tile, ncol = h.ncol, add_mode = h.add_mode, dense = h.dense, res_tma = h.res_tma, store_y = h.store_y;
             const float scale = h.scale;
-            const __nv_bfloat16* addp = h.add; __nv_bfloat16* outp = h.out; float* stat_tiles = h.stat_tiles; __nv_bfloat16* bn_out = h.bn_out;
+            const __nv_bfloat16* addp = h.add; __nv_bfloat16* outp = h.out; float* stat_tiles = h.stat_tiles; __nv_bfloat16* bn_out = BWD ? nullptr : h.bn_out;
             // position -> output pixel (and the residual's pixel)
-            const int pos = tm * TILE_M + m;
-            bool valid = pos < h.total_pos;
-            int pix = pos; long long addpix = -1;
-            if (valid && (!dense || add_mode == 3)) {
+            long long addpix = -1;
+            auto pixel_of = [&](int pos) -> int {                // -1: a padding position; sets addpix of a compact residual
+                addpix = -1;
+                if (pos >= h.total_pos) return -1;
+                if (dense && add_mode != 3) return pos;
                 const int Wp = h.Wp, Hp = h.Hp, pad = h.pad, os = h.os, OH = h.OH, OW = h.OW;
                 const int trow = pos / Wp, xx = pos - trow * Wp, img = trow / Hp, yy = trow - img * Hp;
                 const int y = (yy - pad) * os + h.oy, x = xx * os + h.ox;
-                valid = yy >= pad && xx < Wp - pad && y < OH && x < OW;
-                pix = (img * OH + y) * OW + x;
+                if (!(yy >= pad && xx < Wp - pad && y < OH && x < OW)) return -1;
                 if (add_mode == 3 && !((y | x) & 1)) addpix = ((long long)img * ((OH + 1) >> 1) + (y >> 1)) * ((OW + 1) >> 1) + (x >> 1);
-            }
+                return (img * OH + y) * OW + x;
+            };
+            const int pix = pixel_of(tm * TILE_M + m);
+            const bool valid = pix >= 0;
             if (add_mode == 2) addpix = pix;
-            if (!valid) pix = -1;
             const int col0 = tn * n_tile;
             const bool gadd = !res_tma && add_mode >= 2 && valid && addpix >= 0;
             // a residual that TMA cannot bring: the first slab's is read ahead of the accumulator, a later one's once the last has been used
@@ -513,6 +527,29 @@ __global__ void __launch_bounds__(TC_CONV_THREADS, 1) conv_tc_kernel(const TcPro
             };
             const bool any_gadd = !res_tma && add_mode >= 2;
             if (any_gadd) load_add(0);
+            // BN backward: lane (row group lane >> 3, chunk lane & 7) reads x the way the copy-out writes, a slab ahead of its use
+            const __nv_bfloat16* bwd_x = BWD ? h.bwd_x : nullptr;
+            uint4 xr[8];
+            auto load_x = [&](int s0) {
+                const int c = s0 + (lane & 7) * 8;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int px = __shfl_sync(0xffffffffu, pix, i * 4 + (lane >> 3));
+                    xr[i] = (px >= 0 && c < n_tile && col0 + c < ncol) ? __ldg(reinterpret_cast<const uint4*>(bwd_x + (long long)px * ncol + col0 + c)) : make_uint4(0u, 0u, 0u, 0u);
+                }
+            };
+            if (bwd_x) {
+                load_x(0);
+                // the rows of the group's next tile are asked into L2 now, a whole tile ahead of their use (the 64 -> 256
+                // channel dgrad of 8 x 128 images of 32 x 32: 342 us with the sums, 131 + 193 us with a reduction pass of its own; the epilogue is the
+                // limit, and the little L1 beside 225 KB of shared memory; 3x3 layers at 128 channels 118 instead of 105 + 43 us)
+                const Unit nx = u + u_step < u_stop ? decode(u + u_step) : Unit{-1, 0, 0, 0};
+                if (nx.pi == pi && grp < nx.nt) {
+                    const int px2 = pixel_of((nx.tm0 + grp) * TILE_M + m);
+                    if (px2 >= 0)
+                        for (int c = nx.tn * n_tile; c < min((nx.tn + 1) * n_tile, ncol); c += 64) asm volatile("prefetch.global.L2 [%0];" ::"l"(bwd_x + (long long)px2 * ncol + c));
+                }
+            }
             const uint32_t scw = __float_as_uint(valid ? scale : 0.f);
             const uint64_t scale2 = f2_pack(scw, scw);
             ok = mbar_wait(acc_full + 8 * buf, aph, &abort_s);
@@ -574,7 +611,42 @@ __global__ void __launch_bounds__(TC_CONV_THREADS, 1) conv_tc_kernel(const TcPro
                         }
                     }
                 }
-                if (stat_tiles) {
+                if (bwd_x) {
+                    // the sums the BN backward needs, of the stored (rounded) da: dz = da where relu's input was positive, and dz * xhat.  A lane
+                    // has 8 columns of 8 rows; the four lanes of a column group are added in a fixed order, the warps as below.
+                    const int ch = lane & 7;
+                    uint64_t nm[4], is[4], ga2[4], be2[4], su[4] = {0, 0, 0, 0}, sq[4] = {0, 0, 0, 0};
+                    const uint32_t w0 = smem_u32(&bwd_s2[BWD ? grp : 0][0][0]) + (uint32_t)(s0 + ch * 8) * 4u;
+#pragma unroll
+                    for (int k = 0; k < 4; k += 2) {
+                        const uint4 a = lds128(w0 + 8u * k), b = lds128(w0 + 1024u + 8u * k), g = lds128(w0 + 2048u + 8u * k), e = lds128(w0 + 3072u + 8u * k);
+                        nm[k] = f2_pack(a.x, a.y); nm[k + 1] = f2_pack(a.z, a.w); is[k] = f2_pack(b.x, b.y); is[k + 1] = f2_pack(b.z, b.w);
+                        ga2[k] = f2_pack(g.x, g.y); ga2[k + 1] = f2_pack(g.z, g.w); be2[k] = f2_pack(e.x, e.y); be2[k + 1] = f2_pack(e.z, e.w);
+                    }
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int row = i * 4 + (lane >> 3);
+                        const uint4 d = lds128(stg + (uint32_t)(quad * 32 + row) * 128u + ((uint32_t)(ch ^ (row & 7)) << 4));
+                        const uint32_t dw[4] = {d.x, d.y, d.z, d.w}, xw[4] = {xr[i].x, xr[i].y, xr[i].z, xr[i].w};
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const uint64_t xh = f2_mul(f2_add(f2_of_bf16x2(xw[k]), nm[k]), is[k]);
+                            float z0, z1; f2_unpack(f2_fma(xh, ga2[k], be2[k]), z0, z1);
+                            const uint64_t dz = f2_of_bf16x2(dw[k] & ((z0 > 0.f ? 0x0000FFFFu : 0u) | (z1 > 0.f ? 0xFFFF0000u : 0u)));
+                            su[k] = f2_add(su[k], dz); sq[k] = f2_fma(dz, xh, sq[k]);
+                        }
+                    }
+                    if (s0 + 64 < n_tile) load_x(s0 + 64);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+#pragma unroll
+                        for (int d = 8; d < 32; d <<= 1) { su[k] = f2_add(su[k], __shfl_xor_sync(0xffffffffu, su[k], d)); sq[k] = f2_add(sq[k], __shfl_xor_sync(0xffffffffu, sq[k], d)); }
+                        if (lane < 8) {
+                            *reinterpret_cast<uint64_t*>(&stat_s[quad][0][s0 + ch * 8 + 2 * k]) = su[k];
+                            *reinterpret_cast<uint64_t*>(&stat_s[quad][1][s0 + ch * 8 + 2 * k]) = sq[k];
+                        }
+                    }
+                } else if (stat_tiles) {
                     // column sums of the stored (rounded) values: every warp over its own 32 rows, lane = two neighbouring columns;
                     // the four warps' sums are added in a fixed order once the tile's last slab is through
                     uint64_t su = 0, sq = 0;
@@ -839,30 +911,54 @@ __global__ void __launch_bounds__(256) wgrad_tc_reduce_kernel(const TcWgradProb*
 }
 
 // ------------------------------------------------------------------------------------------------ BN statistics from the tiles' sums
-// The forward kernel leaves, per 128-position tile, the column sums and sums of squares of the values it stored.  One warp
-// per channel adds them in a fixed order in double and turns them into mean, 1/sqrt(var + eps) and the running statistics.
-__global__ void __launch_bounds__(256) bn_finalize_tiles_kernel(const BnProb* __restrict__ probs) {
+// The convolution kernel leaves, per 128-position tile, the column sums of what it stored.  Here they are added in a fixed order in
+// double: a CTA takes 16 channels, 32 rows of threads every 32nd tile (all of a thread's loads in flight for up to 256 tiles; latency is
+// all there is to this kernel), then the 32 sums.  MODE 0, forward: mean, 1/sqrt(var + eps) and the running statistics.
+// MODE 1, backward: the two reduction sums and the gradients of beta and gamma.
+template <int MODE>
+__global__ void __launch_bounds__(512) bn_finalize_tiles_kernel(const BnProb* __restrict__ probs) {
     const BnProb& p = probs[blockIdx.y];
-    const int lane = threadIdx.x & 31;
-    const int c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (c >= p.C) return;
-    const float* tiles = reinterpret_cast<const float*>(p.partial);
+    const int C = p.C, ch = threadIdx.x & 15, row = threadIdx.x >> 4, c = blockIdx.x * 16 + ch, n = p.chunks;
+    if ((int)blockIdx.x * 16 >= C) return;
+    __shared__ double red[2][32][17];
+    const float* __restrict__ t = reinterpret_cast<const float*>(p.partial) + (c < C ? c : 0);
     double a0 = 0.0, a1 = 0.0;
-    for (int k = lane; k < p.chunks; k += 32) { a0 += (double)tiles[((long long)k * 2 + 0) * p.C + c]; a1 += (double)tiles[((long long)k * 2 + 1) * p.C + c]; }
+    for (int k = row; k < n; k += 8 * 32) {                      // eight tiles of loads in flight per thread
+        float v0[8], v1[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int kk = k + 32 * u;
+            v0[u] = kk < n ? __ldcg(t + (long long)kk * 2 * C) : 0.f; v1[u] = kk < n ? __ldcg(t + ((long long)kk * 2 + 1) * C) : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) { a0 += (double)v0[u]; a1 += (double)v1[u]; }
+    }
+    red[0][row][ch] = a0; red[1][row][ch] = a1;
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // warp = channel of the 16, lane = row of sums; fixed butterfly
+    a0 = red[0][lane][warp]; a1 = red[1][lane][warp];
     for (int d = 16; d; d >>= 1) { a0 += __shfl_xor_sync(0xffffffffu, a0, d); a1 += __shfl_xor_sync(0xffffffffu, a1, d); }
-    if (lane != 0) return;
+    const int cc = blockIdx.x * 16 + warp;
+    if (lane != 0 || cc >= C) return;
+    if (MODE == 1) {
+        p.stat[2 * C + cc] = (float)a0; p.stat[3 * C + cc] = (float)a1;
+        p.dbeta[cc] = (float)a0; p.dgamma[cc] = (float)a1;
+        return;
+    }
     const double m = (double)p.m, mean = a0 / m;
     double var = a1 / m - mean * mean; if (var < 0.0) var = 0.0;
-    p.stat[c] = (float)mean;
-    p.stat[p.C + c] = (float)(1.0 / sqrt(var + (double)p.eps));
+    p.stat[cc] = (float)mean;
+    p.stat[C + cc] = (float)(1.0 / sqrt(var + (double)p.eps));
     if (p.run_mean) {
         const double unb = p.m > 1 ? var * m / (m - 1.0) : var, mo = (double)p.momentum;
-        p.run_mean[c] = (float)((1.0 - mo) * (double)p.run_mean[c] + mo * mean);
-        p.run_var[c] = (float)((1.0 - mo) * (double)p.run_var[c] + mo * unb);
+        p.run_mean[cc] = (float)((1.0 - mo) * (double)p.run_mean[cc] + mo * mean);
+        p.run_var[cc] = (float)((1.0 - mo) * (double)p.run_var[cc] + mo * unb);
     }
 }
-void launch_bn_finalize_tiles(const BnProb* d, int nprob, int max_c, cudaStream_t s) {
-    bn_finalize_tiles_kernel<<<dim3((max_c + 7) / 8, nprob), 256, 0, s>>>(d);
+void launch_bn_finalize_tiles(const BnProb* d, int nprob, int max_c, int backward, cudaStream_t s) {
+    const dim3 g((max_c + 15) / 16, nprob);
+    if (backward) bn_finalize_tiles_kernel<1><<<g, 512, 0, s>>>(d); else bn_finalize_tiles_kernel<0><<<g, 512, 0, s>>>(d);
 }
 
 // ------------------------------------------------------------------------------------------------ host side
@@ -966,6 +1062,13 @@ int conv_tc_stat_tiles(const ConvProb& p) {
     return (int)((pos + TILE_M - 1) / TILE_M);
 }
 
+// likewise of a dgrad problem, over its descriptors
+int conv_tc_dgrad_tiles(const ConvProb& p) {
+    if (p.ksz == 1) return (int)(((long long)p.N * p.P * p.Q + TILE_M - 1) / TILE_M);
+    Tall g; tall_of(p.stride == 2 ? p.P : p.H, p.stride == 2 ? p.Q : p.W, 1, 1, g);
+    return (int)(((long long)p.N * g.Hp * g.Wp + TILE_M - 1) / TILE_M) * (p.stride == 2 ? 4 : 1);
+}
+
 // One status word per process in pinned host memory that every device can write: a kernel stores into it only when a bounded wait
 // gives up, and the host reads it after a synchronisation without a copy (a 4-byte copy and its wait took 10 us of every layer call).
 int* conv_tc_status_word() {
@@ -1019,7 +1122,8 @@ int conv_tc_fill(const ConvProb& p, int mode, void* host_tc) {
     for (int ph = 0; ph < count; ++ph) {
         TcProb tp; memset(&tp, 0, sizeof(tp)); TcHot& t = tp.h;
         t.add = (const __nv_bfloat16*)p.add; t.out = (__nv_bfloat16*)p.out; t.status = conv_tc_status_word();
-        t.stat_tiles = mode == CONV_FWD ? p.stat_tiles : nullptr;
+        t.stat_tiles = p.stat_tiles;
+        if (mode == CONV_DGRAD && p.bn_x) { t.bwd_x = (const __nv_bfloat16*)p.bn_x; t.bn_stat = p.bn_stat; t.bn_gamma = p.bn_gamma; t.bn_beta = p.bn_beta; }
         t.n_img = p.N; t.ncol = ncol; t.red = chan_a; t.slabs = (chan_a + 63) / 64; t.scale = p.scale;
         t.b_mn_major = mode == CONV_DGRAD ? 1 : 0;
         t.es = 1; t.pad = 0; t.os = 1; t.oy = 0; t.ox = 0; t.ngroups = 1; t.gbeg[0] = 0;
@@ -1084,6 +1188,7 @@ int conv_tc_fill(const ConvProb& p, int mode, void* host_tc) {
         auto b_tile = [&](int nt) { return mode == CONV_FWD ? nt * 128 : ((nt + 63) / 64) * 8192; };
         auto b_total = [&](int nt) { return (size_t)t.slabs * ntaps * ((b_tile(nt) + 1023) / 1024 * 1024); };
         t.tiles_m = (t.total_pos + TILE_M - 1) / TILE_M;
+        if (t.stat_tiles) t.stat_tiles += (long long)ph * t.tiles_m * 2 * ncol;        // one run of tiles per output phase
         pick_n_tile(t, ntaps, p.group > 0 ? p.group : 1, count);
         t.out_slabs = (t.n_tile + 63) / 64;
         t.b_bytes = b_tile(t.n_tile);
@@ -1109,11 +1214,11 @@ size_t conv_tc_prob_bytes() { return sizeof(TcProb); }
 // units of work of a problem: pairs of row tiles x column tiles
 int conv_tc_tiles(const void* host_tc) { const TcHot* t = &((const TcProb*)host_tc)->h; return ((t->tiles_m + 1) / 2) * t->tiles_n; }
 // packs what a launch has to know about its largest problem into one number: window KB (12 bits), weight-tile KB (12), flags
-// (4; 1: residual through TMA, 2: BN of the output), KB of all weight tiles of a column tile (16), MMA N (20)
+// (4; 1: residual through TMA, 2: BN of the output, 4: dgrad), KB of all weight tiles of a column tile (16), MMA N (20)
 size_t conv_tc_smem(const void* host_tc) {
     const TcHot* t = &((const TcProb*)host_tc)->h;
     const size_t a_stage = ((size_t)t->nbox * t->a_box_bytes + 1023) / 1024, b_stage = ((size_t)t->b_bytes + 1023) / 1024;
-    return (a_stage << 52) | (b_stage << 40) | ((size_t)((t->res_tma ? 1 : 0) | (t->bn_out ? 2 : 0)) << 36) | ((size_t)std::min(t->b_total / 1024, 0xFFFF) << 20) | (size_t)t->n_tile;
+    return (a_stage << 52) | (b_stage << 40) | ((size_t)((t->res_tma ? 1 : 0) | (t->bn_out ? 2 : 0) | (t->b_mn_major ? 4 : 0)) << 36) | ((size_t)std::min(t->b_total / 1024, 0xFFFF) << 20) | (size_t)t->n_tile;
 }
 // field-wise maximum of two packed values
 size_t conv_tc_merge(size_t a, size_t b) {
@@ -1129,7 +1234,8 @@ constexpr size_t TC_SMEM_BUDGET = 204 * 1024;
 void launch_conv_tc_probs(const void* d_tc, int nprob, int max_tiles, size_t packed, cudaStream_t s, bool pdl) {
     static bool configured = false; static int sms = 0;
     if (!configured) {
-        cudaFuncSetAttribute(conv_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(TC_SMEM_BUDGET + 1024));
+        cudaFuncSetAttribute(conv_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(TC_SMEM_BUDGET + 1024));
+        cudaFuncSetAttribute(conv_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(TC_SMEM_BUDGET - 8 * 1024 + 1024));
         int dev = 0; cudaGetDevice(&dev); cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         configured = true;
     }
@@ -1143,19 +1249,20 @@ void launch_conv_tc_probs(const void* d_tc, int nprob, int max_tiles, size_t pac
     // so it is the weight tiles that stream: one slab buffer per group, two windows, four weight tiles, then more windows (measured
     // at 128 channels on 16 x 16 maps, 1024 images: 148 us with two weight tiles and four windows, 125 us with four and three).
     const size_t a = (size_t)L.a_stage, b = (size_t)L.b_stage;
+    const size_t budget = (packed >> 36) & 4 ? TC_SMEM_BUDGET - 8 * 1024 : TC_SMEM_BUDGET;      // dgrad keeps 8 KB of BN constants beside the rings
     const int flags = (int)((packed >> 36) & 0xF), extra = flags & 2 ? 1 : 0;
     L.groups = 2; L.res = flags & 1;
     auto staging = [&] { return (size_t)L.groups * (L.eb + extra) * SLAB_BYTES; };
     if (a <= 16 * 1024) {                                        // 1x1 layers: windows of one box
         L.eb = L.res ? 3 : 2;
-        while (L.eb > 1 && staging() + 4 * a + (L.res ? 1 : 3) * b > TC_SMEM_BUDGET) --L.eb;
-        const size_t rings = TC_SMEM_BUDGET - staging();
+        while (L.eb > 1 && staging() + 4 * a + (L.res ? 1 : 3) * b > budget) --L.eb;
+        const size_t rings = budget - staging();
         L.na = 4; while (L.na > 2 && (size_t)L.na * a + 2 * b > rings) --L.na;
         L.nb = 1; while (L.nb < 8 && (size_t)L.na * a + (size_t)(L.nb + 1) * b <= rings) ++L.nb;
         while (L.na < TC_MAX_STAGES && (size_t)(L.na + 1) * a + (size_t)L.nb * b <= rings) ++L.na;
     } else {                                                     // several taps per window: weight tiles are what streams
         L.eb = 1;
-        const size_t rings = TC_SMEM_BUDGET - staging();
+        const size_t rings = budget - staging();
         L.na = 2; L.nb = 1; while (L.nb < 4 && 2 * a + (size_t)(L.nb + 1) * b <= rings) ++L.nb;
         while (L.na < 4 && (size_t)(L.na + 1) * a + (size_t)L.nb * b <= rings) ++L.na;
         while (L.nb < 8 && (size_t)L.na * a + (size_t)(L.nb + 1) * b <= rings) ++L.nb;
@@ -1170,7 +1277,7 @@ void launch_conv_tc_probs(const void* d_tc, int nprob, int max_tiles, size_t pac
     cudaLaunchConfig_t cfg = {}; cfg.gridDim = dim3(grid); cfg.blockDim = dim3(TC_CONV_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = s;
     cudaLaunchAttribute at[1]; at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization; at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at; cfg.numAttrs = pdl ? 1 : 0;
-    cudaLaunchKernelEx(&cfg, conv_tc_kernel, (const TcProb*)d_tc, (const TcLaunch)L);
+    cudaLaunchKernelEx(&cfg, flags & 4 ? conv_tc_kernel<true> : conv_tc_kernel<false>, (const TcProb*)d_tc, (const TcLaunch)L);
 }
 
 // ---- wgrad host side

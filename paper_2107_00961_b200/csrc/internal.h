@@ -31,7 +31,9 @@ struct ConvProb {
     // evaluation: the BN+ReLU that consumes the output runs in the epilogue of the tensor-core kernels, bn_out = relu(bn(y)) of the rounded y
     // with running statistics (bn_stat: mean [K] | 1/std [K]); bn_only: y itself is not needed
     const float* bn_stat; const float* bn_gamma; const float* bn_beta; void* bn_out; int bn_only;
-    float* stat_tiles;    // forward on tcgen05: per 128-position tile, the column sums and sums of squares of the stored output [tiles][2][K], or nullptr
+    float* stat_tiles;    // tcgen05: per 128-position tile [tiles][2][columns], forward: the column sums and sums of squares of the stored output;
+                          // dgrad (with bn_x): the sums of dz and dz * xhat of the BN+ReLU whose output gradient is the output; or nullptr
+    const void* bn_x;     // dgrad on tcgen05: input of that BN (shape of out); bn_stat, bn_gamma, bn_beta as above
 };
 
 // One batch-normalisation + ReLU problem over x [m, C] (forward or backward).

@@ -19,7 +19,8 @@ int conv_tc_fill(const ConvProb& p, int mode, void* host_tc);
 int conv_tc_count(const ConvProb& p, int mode);
 int conv_tc_stat_tiles(const ConvProb& p);
 int bn_fused_capacity(int backward);                                                    // kernels_ref.cu
-void launch_bn_finalize_tiles(const BnProb* d, int nprob, int max_c, cudaStream_t s);
+void launch_bn_finalize_tiles(const BnProb* d, int nprob, int max_c, int backward, cudaStream_t s);
+int conv_tc_dgrad_tiles(const ConvProb& p);
 size_t conv_tc_prob_bytes();
 int conv_tc_tiles(const void* host_tc);
 size_t conv_tc_smem(const void* host_tc);
@@ -121,6 +122,7 @@ struct Builder {
     // The BN+ReLU that consumes a warp-MMA convolution's output joins that convolution's launch (forward: the BN of the
     // output; backward: the BN backward whose da the data gradient produces).  Index of the candidate in *ops, or -1.
     int last_fwd_conv = -1, last_dgrad = -1;
+    int last_tc_dgrad = -1;   // likewise the last data gradient, for the BN backward behind it
     int last_tc_fwd = -1;     // the last forward convolution if it runs on tcgen05: its epilogue can leave the sums the BN of its output needs
     bool fusable(int idx, const void* tensor, const BnProb& p) const {
         if (idx < 0 || eval || ctx->opts.dtype != RESIST_BF16 || (ctx->opts.conv_backend != RESIST_CONV_AUTO && ctx->opts.conv_backend != RESIST_CONV_WARP_MMA)) return false;
@@ -204,7 +206,7 @@ struct Builder {
         }
         ops->push_back(op);
         if (mode == CONV_FWD) { last_fwd_conv = op.backend >= 1000 ? (int)ops->size() - 1 : -1; last_tc_fwd = op.backend == 1 ? (int)ops->size() - 1 : -1; }
-        if (mode == CONV_DGRAD) last_dgrad = op.backend >= 1000 ? (int)ops->size() - 1 : -1;
+        if (mode == CONV_DGRAD) { last_dgrad = op.backend >= 1000 ? (int)ops->size() - 1 : -1; last_tc_dgrad = op.backend == 1 && !out_compact ? (int)ops->size() - 1 : -1; }
         if (mode == CONV_WGRAD && p.splits > 1) { Op r = op; r.key = key + 1; r.kind = OP_SPLITK; r.patch_images = 0; ops->push_back(r); }
         return out_compact;
     }
@@ -322,6 +324,20 @@ struct Builder {
         bn_partial_need = std::max(bn_partial_need, (size_t)p.chunks * 2 * r.c * 8);
         p.partial = bn_partial;
         const int producer = last_dgrad; last_dgrad = -1;
+        const int tc_producer = last_tc_dgrad; last_tc_dgrad = -1;
+        if (tc_producer >= 0 && (*ops)[tc_producer].conv.out == da && (*ops)[tc_producer].conv.C == r.c && (*ops)[tc_producer].conv.stride == 1) {
+            // the tcgen05 data gradient that produces da reads x beside it and leaves the per-tile sums; one small launch adds them up, then
+            // one elementwise pass.  (The reduction as a pass of its own read x and da once more: 2.8 of 26 ms of the wide net's launches, and
+            // the cooperative form of small layers was 27 us of barrier and re-added partial sums whatever its size.  Not at stride 2: the
+            // scattered rows of x cost the four phases 171 us where the pass took 130.)
+            ConvProb& c = (*ops)[tc_producer].conv;
+            const int tiles = conv_tc_dgrad_tiles(c);
+            bn_partial_need = std::max(bn_partial_need, (size_t)tiles * 2 * r.c * 4);
+            c.bn_x = x; c.bn_stat = stat; c.bn_gamma = p.gamma; c.bn_beta = p.beta; c.stat_tiles = (float*)bn_partial; p.partial = bn_partial; p.chunks = tiles;
+            op.kind = OP_BN_BWD_TILE_SUMS; ops->push_back(op);
+            op.key = key + 1; op.kind = OP_BN_BWD_APPLY; ops->push_back(op);
+            return;
+        }
         if (bn_small_ok(p)) { op.kind = OP_BN_BWD_SMALL; ops->push_back(op); return; }
         if (fusable(producer, da, p)) { fuse_into(producer, p, 2); return; }
         // one cooperative launch where all sub-ResNets' chunks can be resident together (the kernel holds 128 registers: one CTA
@@ -496,7 +512,7 @@ static size_t unroll_subnet(resist_ctx* ctx, Builder& bd, const std::vector<char
         Op op{}; op.key = BWD_END; op.sub = bd.sub; op.kind = OP_POOL_BWD;
         op.pool = PoolProb{stem_a ? stem_a : stem_y, nullptr, stem_arg, bd.gbuf[g_cur], bd.gbuf[g], B, Hs, Ws, A.stem_cout, cH, cW};
         op.pool.P = out_dim(Hs, 3, 2); op.pool.Q = out_dim(Ws, 3, 2);
-        bd.ops->push_back(op); bd.grel(g_cur); g_cur = g; bd.last_dgrad = -1;
+        bd.ops->push_back(op); bd.grel(g_cur); g_cur = g; bd.last_dgrad = -1; bd.last_tc_dgrad = -1;
     }
     if (A.stem_bn_relu) { const int g = bd.gtake(); bd.bn_bwd(BWD_END + 1, stem_y, bd.gbuf[g_cur], bd.gbuf[g], nullptr, L.stem_bn, stem_stat, m_stem); bd.grel(g_cur); g_cur = g; }
     if (stem_col) bd.stem_conv(BWD_END + 3, CONV_WGRAD, L.stem, bd.gbuf[g_cur], nullptr, B, A.in_h, A.in_w);
@@ -621,7 +637,7 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
                         const double in_e = (double)p.N * p.H * p.W * p.C, out_e = (double)p.N * p.P * p.Q * p.K, w_e = (double)p.K * p.ksz * p.ksz * p.C;
                         L.flops += 2.0 * out_e * p.ksz * p.ksz * p.C;
                         if (o.kind == OP_CONV_WGRAD) L.bytes += es * (in_e + out_e) + 4.0 * w_e;
-                        else L.bytes += es * (in_e + out_e + w_e + (p.add ? (o.kind == OP_CONV_FWD ? out_e : in_e) : 0.0));
+                        else L.bytes += es * (in_e + out_e + w_e + (p.add ? (o.kind == OP_CONV_FWD ? out_e : in_e) : 0.0) + (p.bn_x ? in_e : 0.0));
                         break;
                     }
                     if (k == i) L.first = (int)conv.size();
@@ -639,13 +655,13 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
                         if (o.kind == OP_CONV_WGRAD) L.bytes += es * (in_e + out_e) + 4.0 * w_e;
                         else L.bytes += es * (in_e + out_e + w_e + (p.add ? (o.kind == OP_CONV_FWD ? out_e : in_e) : 0.0)); }
                     break; }
-                case OP_BN_STATS: case OP_BN_APPLY: case OP_BN_BWD_REDUCE: case OP_BN_BWD_APPLY: case OP_BN_FWD_FUSED: case OP_BN_BWD_FUSED: case OP_BN_TILE_STATS: case OP_BN_EVAL_STATS: case OP_BN_FWD_SMALL: case OP_BN_BWD_SMALL: {
+                case OP_BN_STATS: case OP_BN_APPLY: case OP_BN_BWD_REDUCE: case OP_BN_BWD_APPLY: case OP_BN_FWD_FUSED: case OP_BN_BWD_FUSED: case OP_BN_TILE_STATS: case OP_BN_EVAL_STATS: case OP_BN_FWD_SMALL: case OP_BN_BWD_SMALL: case OP_BN_BWD_TILE_SUMS: {
                     if (k == i) L.first = (int)bn.size();
                     bn.push_back(o.bn);
                     L.gx = std::max(L.gx, o.bn.chunks); L.max_c = std::max(L.max_c, o.bn.C);
                     L.max_elems = std::max<long long>(L.max_elems, o.bn.m * o.bn.C);
                     { const double e = (double)o.bn.m * o.bn.C;
-                      if (o.kind == OP_BN_TILE_STATS) L.bytes += 8.0 * o.bn.chunks * o.bn.C;
+                      if (o.kind == OP_BN_TILE_STATS || o.kind == OP_BN_BWD_TILE_SUMS) L.bytes += 8.0 * o.bn.chunks * o.bn.C;
                       else if (o.kind == OP_BN_EVAL_STATS) L.bytes += 16.0 * o.bn.C;
                       else if (o.kind == OP_BN_STATS) L.bytes += es * e;
                       else if (o.kind == OP_BN_APPLY) L.bytes += 2 * es * e;
@@ -699,7 +715,7 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
                         if (o.fuse == 1) wr.push_back(o.bn.a); else if (o.fuse == 2) wr.push_back(o.bn.dx);
                         break;
                     case OP_CONV_WGRAD: case OP_SPLITK: case OP_REPACK: break;
-                    case OP_BN_STATS: case OP_BN_BWD_REDUCE: case OP_BN_TILE_STATS: case OP_BN_EVAL_STATS: break;
+                    case OP_BN_STATS: case OP_BN_BWD_REDUCE: case OP_BN_TILE_STATS: case OP_BN_EVAL_STATS: case OP_BN_BWD_TILE_SUMS: break;
                     case OP_BN_APPLY: case OP_BN_FWD_FUSED: case OP_BN_FWD_SMALL: wr.push_back(o.bn.a); break;
                     case OP_BN_BWD_APPLY: case OP_BN_BWD_FUSED: case OP_BN_BWD_SMALL: wr.push_back(o.bn.dx); break;
                     default: always = true; break;
@@ -876,7 +892,7 @@ static int enqueue_launches(resist_ctx* ctx, Plan& plan, bool update, bool overl
             case OP_UPSAMPLE: pk = PK_UPSAMPLE; break;
             case OP_IM2COL: pk = PK_IM2COL; break;
             case OP_BN_FWD_FUSED: case OP_BN_FWD_SMALL: pk = PK_BN_FWD_FUSED; break;
-            case OP_BN_TILE_STATS: pk = PK_BN_TILE_STATS; break;
+            case OP_BN_TILE_STATS: case OP_BN_BWD_TILE_SUMS: pk = PK_BN_TILE_STATS; break;
             case OP_BN_BWD_FUSED: case OP_BN_BWD_SMALL: pk = PK_BN_BWD_FUSED; break;
         }
         pf.begin(pk, nk, L.bytes, L.flops, st, L.label);
@@ -908,7 +924,8 @@ static int enqueue_launches(resist_ctx* ctx, Plan& plan, bool update, bool overl
             case OP_HEAD_BWD: n_launch += launch_head_bwd(plan.d_head + L.first, L.count, L.max_b, L.max_c, L.max_classes, L.max_elems, bf, st); break;
             case OP_UPSAMPLE: launch_zero_stuff(plan.d_up + L.first, L.count, L.max_elems, st); ++n_launch; break;
             case OP_IM2COL: launch_im2col(plan.d_col + L.first, L.count, L.col, st); ++n_launch; break;
-            case OP_BN_TILE_STATS: launch_bn_finalize_tiles(plan.d_bn + L.first, L.count, L.max_c, st); ++n_launch; break;
+            case OP_BN_TILE_STATS: launch_bn_finalize_tiles(plan.d_bn + L.first, L.count, L.max_c, 0, st); ++n_launch; break;
+            case OP_BN_BWD_TILE_SUMS: launch_bn_finalize_tiles(plan.d_bn + L.first, L.count, L.max_c, 1, st); ++n_launch; break;
             case OP_BN_FWD_FUSED:
                 if (launch_bn_fused(plan.d_bn + L.first, L.count, L.gx, 0, st)) ++n_launch;
                 else { launch_bn_stats(plan.d_bn + L.first, L.count, L.gx, L.max_c, bf, st); launch_bn_apply(plan.d_bn + L.first, L.count, L.max_elems, bf, st); n_launch += 3; }
