@@ -58,12 +58,12 @@ int conv_wgrad_mma_pick_variant(const ConvProb& p, int target_ctas);
 // Which kernel family takes a bf16 convolution: 0 = CUDA cores, 1 = tcgen05, >= 200 = warp-level MMA (wgrad: 200 +
 // output channels; forward and dgrad: 1000 + the kernel variant, so that the value also separates launches by what
 // the kernel is specialised on).
-static int pick_backend(const ConvProb& p, int mode, int target_ctas, size_t* partial_bytes, int pref = RESIST_CONV_AUTO) {
+static int pick_backend(const ConvProb& p, int mode, int group, int target_ctas, size_t* partial_bytes, int pref = RESIST_CONV_AUTO) {
     bool want_mma = pref == RESIST_CONV_AUTO || pref == RESIST_CONV_WARP_MMA || pref == RESIST_CONV_WARP_MMA_UNFUSED; const bool want_tc = pref == RESIST_CONV_AUTO || pref == RESIST_CONV_TCGEN05;
-    // 3x3 layers of 64 channels and more with many positions run faster on tcgen05 followed by the streaming BN kernels than on
-    // the warp-level MMA kernels with the BN inside (measured at 8 x 128 images of 32 x 32: 450 -> 218 us forward, 668 -> 211 +
-    // 195 us backward); small ones stay (a ResNet-110 stage of 8 x 8 maps measured the same either way)
-    if (pref == RESIST_CONV_AUTO && p.C >= 64 && p.K >= 64 && p.ksz == 3 && (long long)p.N * p.H * p.W >= 65536) want_mma = false;
+    // 3x3 layers of 64 channels and more run faster on tcgen05, followed by the streaming BN kernels, than on the warp-level MMA kernels
+    // with the BN inside, once the launch has enough positions: ResNet-110's 8 x 8 stage at 4 x 128 images 3.44 -> 3.24 ms per step, its
+    // evaluation of 1000 images 3.68 -> 3.32 ms; one worker's 84 images alone (5376 positions) 1.28 -> 1.46 ms, so they stay.
+    if (pref == RESIST_CONV_AUTO && p.C >= 64 && p.K >= 64 && p.ksz == 3 && (long long)group * p.N * p.H * p.W >= 24576) want_mma = false;
     if (mode == CONV_WGRAD) {
         if (want_mma && conv_wgrad_mma_supported(p, target_ctas, partial_bytes)) return 200 + conv_wgrad_mma_pick_variant(p, target_ctas);
         if (want_tc && conv_wgrad_tc_supported(p, target_ctas, partial_bytes)) return 1;
@@ -107,7 +107,7 @@ __global__ void patch_kernel(const PatchSite* sites, int n, PatchArgs a) {
 // sub-ResNet's workspace slice; with base == nullptr the pass only measures.
 // ------------------------------------------------------------------------------------------------
 struct Builder {
-    resist_ctx* ctx; int B; int sub; int copy; bool eval; int slot_for_patch;
+    resist_ctx* ctx; int B; int sub; int copy; bool eval; int group;      // group: sub-ResNets that share the launches now being built
     char* base; size_t off = 0; size_t es;
     std::vector<Op>* ops;
     // scratch shared by the operations of this sub-ResNet (they run one after another)
@@ -173,16 +173,16 @@ struct Builder {
             ConvProb q = p; q.stride = 1; q.P = p.H; q.Q = p.W; q.dy_sub = 2; q.dy_P = p.P; q.dy_Q = p.Q;
             if (mode == CONV_DGRAD) q.M = (int)rows_in; else q.Kred = (int)rows_in;
             size_t pb = 0;
-            if (pick_backend(q, mode, wgrad_target_ctas(ctx), &pb, pref) >= 200) {
+            if (pick_backend(q, mode, group, wgrad_target_ctas(ctx), &pb, pref) >= 200) {
                 p = q;
                 if (mode == CONV_WGRAD) wgrad_partial_need = std::max(wgrad_partial_need, pb);
             }
         }
         if (mode == CONV_WGRAD) {
             size_t pb = 0;
-            op.backend = (tc_ok && !patch) ? pick_backend(p, mode, wgrad_target_ctas(ctx), &pb, pref) : 0;
+            op.backend = (tc_ok && !patch) ? pick_backend(p, mode, group, wgrad_target_ctas(ctx), &pb, pref) : 0;
             if (op.backend) { wgrad_partial_need = std::max(wgrad_partial_need, pb); p.partial = wgrad_partial; }
-        } else op.backend = tc_ok ? pick_backend(p, mode, 0, nullptr, pref) : 0;
+        } else op.backend = tc_ok ? pick_backend(p, mode, group, 0, nullptr, pref) : 0;
         if (op.backend) ++n_tc; else ++n_cc;
         const bool out_compact = mode == CONV_DGRAD && op.backend == 1 && p.ksz == 1 && p.stride == 2;
         if (out_compact) p.out_compact = 1;
@@ -253,7 +253,7 @@ struct Builder {
         p.tiles_m = (p.M + 63) / 64; p.tiles_n = (p.Ncol + 63) / 64; p.splits = 1; p.ktiles_per_split = (p.Kred + 15) / 16;
         flops += 2LL * rows * p.K * kk;
         size_t pb = 0;
-        op.backend = pick_backend(p, mode, wgrad_target_ctas(ctx), &pb, wide ? RESIST_CONV_TCGEN05 : RESIST_CONV_WARP_MMA);
+        op.backend = pick_backend(p, mode, group, wgrad_target_ctas(ctx), &pb, wide ? RESIST_CONV_TCGEN05 : RESIST_CONV_WARP_MMA);
         if (mode == CONV_WGRAD) { wgrad_partial_need = std::max(wgrad_partial_need, pb); p.partial = wgrad_partial; }
         ++n_tc;
         ops->push_back(op);
@@ -394,25 +394,28 @@ static size_t unroll_subnet(resist_ctx* ctx, Builder& bd, const std::vector<char
     // the earlier stages, the largest number of blocks any sub-ResNet of this round holds there.  Sub-ResNets then share a
     // launch only with blocks of the same stage (same shapes, same kernel variant), instead of splitting a slot's launch
     // whenever their block counts per stage differ.
-    std::vector<int> aslot(order.size(), 0); int n_aslots = 0;
+    std::vector<int> aslot(order.size(), 0), share(order.size(), 1); int n_aslots = 0;       // share: sub-ResNets in the slot's launches
     {
         int n_stage = 0; for (int b = 0; b < nb; ++b) n_stage = std::max(n_stage, ctx->blocks[b].stage + 1);
         std::vector<int> stage_max(std::max(n_stage, 1), 0), cnt(std::max(n_stage, 1), 0);
         for (int b = 0; b < nb; ++b) if (present[b]) ++cnt[std::max(0, ctx->blocks[b].stage)];
         stage_max = cnt;
+        std::vector<std::vector<int>> held;                          // blocks per stage of every sub-ResNet that runs in this plan
         for (int s2 = 0; s2 < ctx->S && (int)ctx->mask.size() == nb; ++s2) {
             std::fill(cnt.begin(), cnt.end(), 0);
             for (int b = 0; b < nb; ++b) if (ctx->mask[b] >> s2 & 1u) ++cnt[std::max(0, ctx->blocks[b].stage)];
+            if (bd.group > 1) held.push_back(cnt);
             for (size_t t = 0; t < cnt.size(); ++t) stage_max[t] = std::max(stage_max[t], cnt[t]);
         }
         std::vector<int> base(stage_max.size() + 1, 0);
         for (size_t t = 0; t < stage_max.size(); ++t) base[t + 1] = base[t] + stage_max[t];
         n_aslots = base.back();
         std::fill(cnt.begin(), cnt.end(), 0);
-        for (size_t i = 0; i < order.size(); ++i) { const int t = std::max(0, ctx->blocks[order[i]].stage); aslot[i] = base[t] + cnt[t]++; }
+        for (size_t i = 0; i < order.size(); ++i) { const int t = std::max(0, ctx->blocks[order[i]].stage); share[i] = 0; for (const auto& h : held) share[i] += h[t] > cnt[t]; share[i] = std::max(share[i], 1); aslot[i] = base[t] + cnt[t]++; }
     }
     for (size_t slot = 0; slot < order.size(); ++slot) {
         const int b = order[slot]; const resist_block& K = ctx->blocks[b]; const BlockRef& r = L.blk[b]; BlockMem& s = bm[b];
+        bd.group = share[slot];
         const long long key = KEY_BLOCK0 + 20LL * (long long)aslot[slot];
         s.H = cH; s.W = cW; s.Ho = out_dim(cH, 3, K.stride); s.Wo = out_dim(cW, 3, K.stride);
         const long long m_in = (long long)B * s.H * s.W, m_out = (long long)B * s.Ho * s.Wo;
@@ -459,6 +462,7 @@ static size_t unroll_subnet(resist_ctx* ctx, Builder& bd, const std::vector<char
     { int g = bd.gtake(); bd.bn_bwd(BWD0 + 1, xF, bd.gbuf[g_cur], bd.gbuf[g], nullptr, L.final_bn, statF, mF); bd.grel(g_cur); g_cur = g; }
     for (int slot = (int)order.size() - 1; slot >= 0; --slot) {
         const int b = order[slot]; const resist_block& K = ctx->blocks[b]; const BlockRef& r = L.blk[b]; BlockMem& s = bm[b];
+        bd.group = share[slot];
         const long long key = BWD_BLOCK0 + 40LL * ((long long)n_aslots - 1 - aslot[slot]);
         const long long m_in = (long long)B * s.H * s.W, m_out = (long long)B * s.Ho * s.Wo;
         const char* dout = bd.gbuf[g_cur];
@@ -525,13 +529,13 @@ static size_t unroll_subnet(resist_ctx* ctx, Builder& bd, const std::vector<char
 // ------------------------------------------------------------------------------------------------
 struct Needs { size_t bn_partial = 0, wgrad_partial = 0, gbig = 0, up = 0, total = 0; };
 
-static Needs measure_subnet(resist_ctx* ctx, int sub, int copy, const std::vector<char>& present, int B, bool eval, float inv_S) {
+static Needs measure_subnet(resist_ctx* ctx, int sub, int copy, const std::vector<char>& present, int B, bool eval, float inv_S, int group) {
     std::vector<Op> scratch;
-    Builder b1{ctx, B, sub, copy, eval, 0, nullptr}; b1.es = ctx->opts.dtype == RESIST_BF16 ? 2 : 4; b1.ops = &scratch;
+    Builder b1{ctx, B, sub, copy, eval, group, nullptr}; b1.es = ctx->opts.dtype == RESIST_BF16 ? 2 : 4; b1.ops = &scratch;
     unroll_subnet(ctx, b1, present, inv_S);
     Needs n; n.bn_partial = b1.bn_partial_need; n.wgrad_partial = b1.wgrad_partial_need; n.gbig = b1.gbig; n.up = b1.up_need;
     scratch.clear();
-    Builder b2{ctx, B, sub, copy, eval, 0, nullptr}; b2.es = b1.es; b2.ops = &scratch;
+    Builder b2{ctx, B, sub, copy, eval, group, nullptr}; b2.es = b1.es; b2.ops = &scratch;
     b2.bn_partial_need = n.bn_partial; b2.wgrad_partial_need = n.wgrad_partial; b2.gbig = n.gbig; b2.up_need = n.up;
     n.total = align_up(unroll_subnet(ctx, b2, present, inv_S), 256);
     return n;
@@ -794,10 +798,10 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
     return RESIST_OK;
 }
 
-static int ensure_workspace(resist_ctx* ctx, int B, std::vector<Needs>& needs) {
+static int ensure_workspace(resist_ctx* ctx, int B, int group, std::vector<Needs>& needs) {
     needs.resize(ctx->S);
     size_t slice = 0;
-    for (int s = 0; s < ctx->S; ++s) { needs[s] = measure_subnet(ctx, s, s, present_of(ctx, s), B, false, 1.f); slice = std::max(slice, needs[s].total); }
+    for (int s = 0; s < ctx->S; ++s) { needs[s] = measure_subnet(ctx, s, s, present_of(ctx, s), B, false, 1.f, group); slice = std::max(slice, needs[s].total); }
     if (slice <= ctx->ws_slice && (size_t)ctx->S * ctx->ws_slice <= ctx->ws_bytes) return RESIST_OK;
     if (slice <= ctx->ws_slice) slice = ctx->ws_slice;
     slice = align_up(slice + slice / 16, 1 << 20);               // a little slack: partitions differ slightly in size
@@ -814,12 +818,13 @@ static int ensure_workspace(resist_ctx* ctx, int B, std::vector<Needs>& needs) {
 // sub >= 0: one sub-ResNet; sub == -1: all S grouped
 static int build_plan(resist_ctx* ctx, Plan& plan, int sub, int B, cudaStream_t st) {
     std::vector<Needs> needs;
-    int rc = ensure_workspace(ctx, B, needs);
+    const int group = sub >= 0 ? 1 : ctx->S;
+    int rc = ensure_workspace(ctx, B, group, needs);
     if (rc) return rc;
     std::vector<Op> ops; plan.info = resist_step_info{};
     const int s0 = sub >= 0 ? sub : 0, s1 = sub >= 0 ? sub + 1 : ctx->S;
     for (int s = s0; s < s1; ++s) {
-        Builder bd{ctx, B, s, s, false, 0, (char*)ctx->d_ws + (size_t)s * ctx->ws_slice};
+        Builder bd{ctx, B, s, s, false, group, (char*)ctx->d_ws + (size_t)s * ctx->ws_slice};
         bd.es = ctx->opts.dtype == RESIST_BF16 ? 2 : 4; bd.ops = &ops;
         bd.bn_partial_need = needs[s].bn_partial; bd.wgrad_partial_need = needs[s].wgrad_partial; bd.gbig = needs[s].gbig; bd.up_need = needs[s].up;
         const size_t used = unroll_subnet(ctx, bd, present_of(ctx, s), 1.f);
@@ -1048,14 +1053,14 @@ int resist_eval(resist_ctx* ctx, const void* images, const int32_t* labels, int3
     Plan& plan = ctx->plans[ctx->S_cap + 1];
     if (!plan.valid || plan.B != B || plan.generation != (unsigned long long)S) {
         std::vector<char> all(ctx->arch.num_blocks, 1);
-        Needs n = measure_subnet(ctx, 0, copy, all, B, true, 1.f / (float)S);
+        Needs n = measure_subnet(ctx, 0, copy, all, B, true, 1.f / (float)S, 1);
         if (n.total > ctx->eval_ws_bytes) {
             cudaDeviceSynchronize(); ctx_free(ctx, ctx->d_eval_ws);
             ctx->d_eval_ws = ctx_alloc(ctx, n.total); ctx->eval_ws_bytes = ctx->d_eval_ws ? n.total : 0;
             if (!ctx->d_eval_ws) { ctx->err = "allocator returned NULL for the evaluation workspace"; return RESIST_ENOMEM; }
         }
         std::vector<Op> ops;
-        Builder bd{ctx, B, 0, copy, true, 0, (char*)ctx->d_eval_ws}; bd.es = ctx->opts.dtype == RESIST_BF16 ? 2 : 4; bd.ops = &ops;
+        Builder bd{ctx, B, 0, copy, true, 1, (char*)ctx->d_eval_ws}; bd.es = ctx->opts.dtype == RESIST_BF16 ? 2 : 4; bd.ops = &ops;
         bd.bn_partial_need = n.bn_partial; bd.wgrad_partial_need = n.wgrad_partial; bd.gbig = n.gbig; bd.up_need = n.up;
         unroll_subnet(ctx, bd, all, 1.f / (float)S);
         plan.sub = -2;
