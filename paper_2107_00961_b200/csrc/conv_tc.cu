@@ -167,7 +167,7 @@ __device__ __forceinline__ void epi_cols(const uint32_t* v, uint32_t st, uint32_
     }
 }
 
-constexpr int TC_THREADS = 224;              // wgrad kernel: producer warp, two MMA warps, four epilogue warps
+constexpr int TC_THREADS = 224;              // wgrad kernel: producer warp of dy, MMA warp, producer warp of a, four epilogue warps
 constexpr int TC_ISSUERS = 1;                // forward / dgrad kernel: MMA-issuing warps
 constexpr int TC_RES_WARP = 1 + TC_ISSUERS + 8;              // forward / dgrad kernel: fetches the residual
 constexpr int TC_CONV_THREADS = 32 * (TC_RES_WARP + 1);          // producer warp, MMA warps, two groups of four epilogue warps, residual warp
@@ -708,9 +708,15 @@ void launch_zero_stuff(const UpProb* d, int nprob, long long max_vecs, cudaStrea
 // dw[k][r][s][c] = sum over output positions of dy[pos][k] * a[pos + shift(r,s)][c].  The reduction runs over the
 // positions of the forward problem (pixels in order, or the tall zero-padded map, where dy reads as zero at the padding
 // positions and adds nothing), 128 per pipeline stage: D[cout (128 lanes), cin] per tap, A = dy^T and B = shifted a,
-// both MN-major straight from their 128-byte rows.  A CTA accumulates a range of position chunks for one group of taps
+// both MN-major straight from their 128-byte rows.  A CTA of the three-tap form accumulates a range of position chunks for one group of taps
 // (taps that read the same window: up to three taps of a stride-1 layer, the taps of one input parity phase of a stride-2
 // layer) and writes an fp32 partial, or, alone on its tile, the result; a second kernel adds the partials in a fixed order.
+// The nine-tap form (stride 1): the two 64-row halves of A are the same 64 channels of dy, the second one map row further (the descriptor's
+// leading offset is Wp rows instead of a slab), and the three 64-column parts of B the same channels of a, one position apart each.  One MMA
+// of 128 x 192 then holds the taps (row 1; 0, 1, 2) in its lower and (row 0; 0, 1, 2) in its upper lanes, a second one row 2 (and row 1 again, unused).
+// What bounds it: the boxes' way from L2 into shared memory, 20 to 25 bytes per clock and SM; the MMAs alone would take 1536 clocks of a chunk's
+// ~2500.  One thread producing both operands with two divisions per box took ~5500 clocks per chunk.  8 x 128 images, us: 64 channels 32 x 32 294 -> 94,
+// 128 16 x 16 143 -> 102, 256 8 x 8 205 -> 101, 512 4 x 4 171 -> 134.
 struct alignas(64) TcWgradProb {
     CUtensorMap map_dy;       // (channel k, pixel) or (channel k, x, y, image)
     CUtensorMap map_a;        // likewise for a, possibly element-strided
@@ -719,13 +725,15 @@ struct alignas(64) TcWgradProb {
     int* status;
     int dy_flat, a_flat, taps;
     int es, pad, Hp, Wp, n_img;
-    int R, box_pos, nbox_dy, nbox_a, hb, dy_box_bytes, a_box_bytes;
+    int R, box_pos, nbox_dy, nbox_a, hb, hb_step, dy_box_bytes, a_box_bytes;
     int chunks;                                   // position chunks of 128 in total
     int cout, cin, m_tiles, n_tile, n_tiles, a_slabs;
     int tap_groups; int gbeg[10]; int gxs[9], gys[9];
     TapRef tap[9];                                // wtap = index of the tap in dw; shift = row shift inside the a window
     int splits, chunks_per_split;
     int dy_slab_bytes, a_slab_bytes;              // one 64-channel slab of a stage
+    int nine, m_tile, dy_slabs, mma_n;            // nine: all taps of a 64 x 64 tile in one CTA (m_tile 64, one slab each)
+    int dy_lead, a_lead;                          // byte step from 64 rows (columns) of an MMA's operand to the next 64
     int stage_bytes, stages, tmem_cols;
 };
 
@@ -736,7 +744,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) conv_wgrad_tc_kernel(const TcWg
     // everything the loops read, in registers (the descriptor lives in global memory)
     const int splits = p.splits, tap_groups = p.tap_groups, n_tiles = p.n_tiles, chunks = p.chunks, chunks_per_split = p.chunks_per_split;
     const int stages = p.stages, stage_bytes = p.stage_bytes, dy_slab_bytes = p.dy_slab_bytes, a_slab_bytes = p.a_slab_bytes, a_slabs = p.a_slabs;
-    const int n_tile = p.n_tile, dy_flat = p.dy_flat, a_flat = p.a_flat, box_pos = p.box_pos, hb = p.hb, R = p.R, Hp = p.Hp, pad = p.pad, es = p.es;
+    const int n_tile = p.n_tile, dy_flat = p.dy_flat, a_flat = p.a_flat, box_pos = p.box_pos, R = p.R, Hp = p.Hp, pad = p.pad, es = p.es;
+    const int nine = p.nine, m_tile = p.m_tile, dy_slabs = p.dy_slabs;
     const int nbox_dy = p.nbox_dy, nbox_a = p.nbox_a, dy_box_bytes = p.dy_box_bytes, a_box_bytes = p.a_box_bytes, tmem_cols = p.tmem_cols;
     int id = blockIdx.x;
     const int split = id % splits; id /= splits;
@@ -744,13 +753,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1) conv_wgrad_tc_kernel(const TcWg
     const int tn = id % n_tiles; const int tm = id / n_tiles;
     const int c_begin = split * chunks_per_split;
     const int c_end = min(c_begin + chunks_per_split, chunks);
-    const int tap0 = p.gbeg[tg], ntap = p.gbeg[tg + 1] - tap0;
+    const int tap0 = p.gbeg[tg], ntap = nine ? 2 : p.gbeg[tg + 1] - tap0;      // nine: one accumulator per issuing warp
     const int gx = p.gxs[tg], gy = p.gys[tg];
+    const int hb = p.hb - tg * p.hb_step;                        // the group's window of a starts hb positions before the chunk
     const int nc = c_end - c_begin;
 
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    __shared__ __align__(8) uint64_t bars[2 * TC_MAX_STAGES + 3];
+    __shared__ __align__(8) uint64_t bars[2 * TC_MAX_STAGES + 2];
     __shared__ uint32_t tmem_base_s;
     __shared__ int abort_s;
     __shared__ int shift8_s[4], wtap_s[4];                       // the group's taps: row shift in 16-byte units, index in dw
@@ -760,10 +770,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) conv_wgrad_tc_kernel(const TcWg
     const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp-uniform for the compiler too
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < TC_MAX_STAGES; ++s) { mbar_init(bar_full + 8 * s, 1); mbar_init(bar_empty + 8 * s, 2); }   // both issuers release a stage
-        mbar_init(bar_acc, 2); mbar_init(bar_drain, 1); mbar_init(bar_drain + 8, 1);
+        for (int s = 0; s < TC_MAX_STAGES; ++s) { mbar_init(bar_full + 8 * s, 2); mbar_init(bar_empty + 8 * s, 1); }   // each operand's producer announces its bytes
+        mbar_init(bar_acc, 1); mbar_init(bar_drain, 1);
         abort_s = 0;
-        for (int i = 0; i < ntap; ++i) { shift8_s[i] = p.tap[tap0 + i].shift * 8; wtap_s[i] = p.tap[tap0 + i].wtap; }
+        for (int i = 0; i < ntap; ++i) { shift8_s[i] = p.tap[tap0 + (nine ? 3 * i : i)].shift * 8; wtap_s[i] = p.tap[tap0 + i].wtap; }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -775,35 +785,36 @@ __global__ void __launch_bounds__(TC_THREADS, 1) conv_wgrad_tc_kernel(const TcWg
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_d = tmem_base_s;
 
-    if (warp == 0) {
+    if (warp == 0 || warp == 2) {
+        // One producer per operand: warp 0 loads dy, warp 2 a.  A stage is up to two dozen boxes, and where each one lies is kept as (image, row)
+        // counters: with both operands in one thread and a division or two per box, this thread was what the launch waited for.
         if (elect_one()) {
+            const bool is_dy = warp == 0;
+            const CUtensorMap* map = is_dy ? &p.map_dy : &p.map_a;
+            const int flat = is_dy ? dy_flat : a_flat, slabs = is_dy ? dy_slabs : a_slabs, nbox = is_dy ? nbox_dy : nbox_a;
+            const int c0 = is_dy ? tm * m_tile : tn * n_tile, box_bytes = is_dy ? dy_box_bytes : a_box_bytes, slab_bytes = is_dy ? dy_slab_bytes : a_slab_bytes;
+            const int mul = is_dy ? 1 : es, x0 = is_dy ? 0 : gx, y0 = is_dy ? 0 : gy;
+            const uint32_t first = ring + (is_dy ? 0u : (uint32_t)(dy_slabs * dy_slab_bytes)), tx = (uint32_t)(slabs * nbox * box_bytes);
+            const int box_img = R > Hp ? R / max(Hp, 1) : 1, box_row = R > Hp ? Hp : R;      // a box is rows of one image, or whole images
+            int pos = c_begin * TILE_M - (is_dy ? 0 : hb), img0 = 0, row0 = 0;
+            if (!flat) { const int b = floor_div(pos, box_pos), trow = b * R; img0 = floor_div(trow, Hp); row0 = trow - img0 * Hp; pos -= b * box_pos; }   // pos: from the first box's start
             int i = 0; bool ok = true; int s = 0; uint32_t ph = 0;
-            const uint32_t tx = (uint32_t)(2 * nbox_dy * dy_box_bytes + a_slabs * nbox_a * a_box_bytes);
             for (; i < nc; ++i) {
                 if (!mbar_wait(bar_empty + 8 * s, ph ^ 1u, &abort_s)) { atomicExch(&abort_s, 1); report_wait(p.status, 11); ok = false; break; }
-                const int pos0 = (c_begin + i) * TILE_M;
-                const uint32_t dy_dst = ring + (uint32_t)(s * stage_bytes), a_dst = dy_dst + 2u * (uint32_t)dy_slab_bytes;
-                mbar_expect_tx(bar_full + 8 * s, tx);
-                if (dy_flat) {
-                    for (int j = 0; j < 2; ++j) tma_load_2d(dy_dst + (uint32_t)(j * dy_slab_bytes), &p.map_dy, bar_full + 8 * s, tm * 128 + j * 64, pos0);
+                const uint32_t dst = first + (uint32_t)(s * stage_bytes), full = bar_full + 8 * s;
+                mbar_expect_tx(full, tx);
+                if (flat) {
+                    for (int j = 0; j < slabs; ++j) tma_load_2d(dst + (uint32_t)(j * slab_bytes), map, full, c0 + j * 64, pos);
+                    pos += TILE_M;
                 } else {
-                    const int bd0 = pos0 / box_pos;
-                    for (int b = 0; b < nbox_dy; ++b) {
-                        const int trow = (bd0 + b) * R, img = trow / Hp, yy0 = trow - img * Hp;
-                        for (int j = 0; j < 2; ++j)
-                            tma_load_4d(dy_dst + (uint32_t)(j * dy_slab_bytes + b * dy_box_bytes), &p.map_dy, bar_full + 8 * s, tm * 128 + j * 64, 0, yy0 - pad, img);
+                    int img = img0, row = row0; uint32_t to = dst;
+                    for (int b = 0; b < nbox; ++b) {
+                        const int y = (row - pad) * mul + y0;
+                        tma_load_4d(to, map, full, c0, x0, y, img);
+                        for (int j = 1; j < slabs; ++j) tma_load_4d(to + (uint32_t)(j * slab_bytes), map, full, c0 + j * 64, x0, y, img);
+                        to += (uint32_t)box_bytes; row += box_row; if (row >= Hp) { row = 0; img += box_img; }
                     }
-                }
-                if (a_flat) {
-                    for (int j = 0; j < a_slabs; ++j) tma_load_2d(a_dst + (uint32_t)(j * a_slab_bytes), &p.map_a, bar_full + 8 * s, tn * n_tile + j * 64, pos0);
-                } else {
-                    const int ba0 = floor_div(pos0 - hb, box_pos);
-                    for (int b = 0; b < nbox_a; ++b) {
-                        const int trow = (ba0 + b) * R, img = floor_div(trow, Hp), yy0 = trow - img * Hp;
-                        for (int j = 0; j < a_slabs; ++j)
-                            tma_load_4d(a_dst + (uint32_t)(j * a_slab_bytes + b * a_box_bytes), &p.map_a, bar_full + 8 * s, tn * n_tile + j * 64,
-                                        gx, (yy0 - pad) * es + gy, img);
-                    }
+                    for (pos += TILE_M; pos >= box_pos; pos -= box_pos) { row0 += box_row; if (row0 >= Hp) { row0 = 0; img0 += box_img; } }
                 }
                 if (++s == stages) { s = 0; ph ^= 1u; }
             }
@@ -811,44 +822,45 @@ __global__ void __launch_bounds__(TC_THREADS, 1) conv_wgrad_tc_kernel(const TcWg
                 for (int c = max(0, i - stages); c < i; ++c)
                     for (int w = 0; w < 4096 && !mbar_try(bar_full + 8 * (c % stages), (uint32_t)(c / stages) & 1u); ++w) __nanosleep(64);
         }
-    } else if (warp <= 2) {
-        // Two issuing warps (one thread issues a tcgen05.mma only every ~150 cycles, more than the tensor core needs for it).  The
-        // group's taps are split between them; with an odd number of taps the last tap's 128 positions are split instead, each
-        // half into an accumulator of its own (the epilogue adds the two, first half first).  So every accumulator is written
-        // by one thread, in a fixed order.
+    } else if (warp == 1) {
+        // The issuer: every tap of the group into its own accumulator, so each is summed over the positions in order.
         if (elect_one()) {
-            const int me = warp - 1, odd = ntap & 1, whole = (ntap - odd) >> 1;
-            int it_tap[3], it_acc[3], it_k0[3], it_k1[3], nit = 0;
-            for (int q = 0; q < whole; ++q) { it_tap[nit] = me * whole + q; it_acc[nit] = me * whole + q; it_k0[nit] = 0; it_k1[nit] = 8; ++nit; }
-            if (odd) { it_tap[nit] = ntap - 1; it_acc[nit] = ntap - 1 + me; it_k0[nit] = me * 4; it_k1[nit] = me * 4 + 4; ++nit; }
-            // fp32 accumulate, bf16 x bf16, A and B MN-major, N = n_tile, M = 128
-            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((uint32_t)(n_tile >> 3) << 17) | ((128u >> 4) << 24);
-            const uint64_t dy_const = desc_sw128(0, (uint32_t)dy_slab_bytes, 1024), a_const = desc_sw128(0, (uint32_t)a_slab_bytes, 1024);
-            bool ok = true; int s = 0; uint32_t ph = 0;
-            for (int i = 0; i < nc && ok; ++i) {
+            // fp32 accumulate, bf16 x bf16, A and B MN-major, N = mma_n, M = 128
+            const int mma_n = p.mma_n;
+            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((uint32_t)(mma_n >> 3) << 17) | ((128u >> 4) << 24);
+            const uint32_t desc_hi = (uint32_t)(desc_sw128(0, 0, 1024) >> 32), dy_lbo = (uint32_t)(p.dy_lead >> 4) << 16, a_lbo = (uint32_t)(p.a_lead >> 4) << 16;
+            const uint32_t a_at = (uint32_t)(dy_slabs * dy_slab_bytes) >> 4, inc = (uint32_t)(TILE_M % box_pos);
+            uint32_t sh[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) sh[q] = q < ntap ? (uint32_t)shift8_s[q] : 0u;
+            // the chunk's first position inside the first box of either window
+            const int pos = c_begin * TILE_M;
+            uint32_t dy_off = dy_flat ? 0u : (uint32_t)(pos % box_pos), a_off = a_flat ? 0u : (uint32_t)(pos - hb - floor_div(pos - hb, box_pos) * box_pos);
+            bool ok = true; int s = 0; uint32_t ph = 0, acc = 0;
+            for (int i = 0; i < nc; ++i) {
                 if (!mbar_wait(bar_full + 8 * s, ph, &abort_s)) { atomicExch(&abort_s, 1); report_wait(p.status, 12); ok = false; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const int pos0 = (c_begin + i) * TILE_M;
-                const int dy_off = dy_flat ? 0 : pos0 - (pos0 / box_pos) * box_pos;
-                const int a_off = a_flat ? 0 : pos0 - hb - floor_div(pos0 - hb, box_pos) * box_pos;
-                const uint32_t dy16 = ((ring + (uint32_t)(s * stage_bytes)) >> 4) + (uint32_t)dy_off * 8u;       // start addresses in 16-byte units
-                const uint32_t a16 = ((ring + (uint32_t)(s * stage_bytes) + 2u * (uint32_t)dy_slab_bytes) >> 4) + (uint32_t)a_off * 8u;
-                for (int q = 0; q < nit; ++q) {
-                    const uint32_t at16 = a16 + (uint32_t)shift8_s[it_tap[q]];
-                    const uint32_t d_t = tmem_d + (uint32_t)(it_acc[q] * n_tile);
-                    const int k0 = it_k0[q], k1 = it_k1[q];
-#pragma unroll 4
-                    for (int k16 = k0; k16 < k1; ++k16)        // 16 positions = 16 rows of 128 bytes per step
-                        umma_bf16(d_t, dy_const | (uint64_t)((dy16 + 128u * (uint32_t)k16) & 0x3FFFu), a_const | (uint64_t)((at16 + 128u * (uint32_t)k16) & 0x3FFFu), idesc, (i || k16 != k0) ? 1u : 0u);
+                const uint32_t stage16 = (ring + (uint32_t)(s * stage_bytes)) >> 4;           // addresses in 16-byte units
+                const uint32_t dy_lo = (stage16 + dy_off * 8u) | dy_lbo, a_lo = (stage16 + a_at + a_off * 8u) | a_lbo;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (q >= ntap) break;
+                    const uint32_t d_t = tmem_d + (uint32_t)(q * mma_n), at = a_lo + sh[q];
+#pragma unroll
+                    for (int k16 = 0; k16 < 8; ++k16)          // 16 positions = 16 rows of 128 bytes per step
+                        umma_bf16(d_t, f2_pack(dy_lo + 128u * (uint32_t)k16, desc_hi), f2_pack(at + 128u * (uint32_t)k16, desc_hi), idesc, k16 ? 1u : acc);
                 }
+                acc = 1;
                 umma_commit(bar_empty + 8 * s);
+                if (!dy_flat) { dy_off += inc; if (dy_off >= (uint32_t)box_pos) dy_off -= (uint32_t)box_pos; }
+                if (!a_flat) { a_off += inc; if (a_off >= (uint32_t)box_pos) a_off -= (uint32_t)box_pos; }
                 if (++s == stages) { s = 0; ph ^= 1u; }
             }
             if (ok) umma_commit(bar_acc);
             else {
                 // gave up: the MMAs already issued must have finished before the CTA frees its tensor memory
-                umma_commit(bar_drain + 8 * me);
-                for (int w = 0; w < 65536 && !mbar_try(bar_drain + 8 * me, 0u); ++w) __nanosleep(64);
+                umma_commit(bar_drain);
+                for (int w = 0; w < 65536 && !mbar_try(bar_drain, 0u); ++w) __nanosleep(64);
             }
         }
     } else {
@@ -859,8 +871,31 @@ __global__ void __launch_bounds__(TC_THREADS, 1) conv_wgrad_tc_kernel(const TcWg
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) { atomicExch(&abort_s, 1); report_wait(p.status, 13); }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const int k = tm * 128 + m;
-        if (ok && quad * 32 < cout - tm * 128) {              // warp-uniform: this lane quadrant holds real output channels
+        // nine: lanes 0 - 63 hold the taps of rows 1 (first accumulator) and 2 (second) of the tile's channels, lanes 64 - 127 those of row 0
+        // (first) and row 1 once more (second, not read)
+        const bool upper = nine && quad >= 2;
+        const int k = tm * m_tile + (upper ? m - 64 : m);
+        if (ok && nine) {
+            if ((quad & 1) * 32 < cout - tm * 64) {
+                for (int q = 0; q < (upper ? 3 : 6); ++q) {
+                    const int wt = upper ? q : 3 + q;
+                    float* dst = splits > 1 ? partial + (((long long)split * taps + wt) * cout + k) * cin + tn * 64
+                                            : outp + ((long long)k * taps + wt) * cin + tn * 64;
+                    for (int c0 = 0; c0 < 64; c0 += 32) {
+                        uint32_t v[32];
+                        if (nc > 0) {
+                            tmem_ld32(tmem_d + ((uint32_t)(quad * 32) << 16) + (uint32_t)(q * 64 + c0), v);
+                            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                        } else { for (int j = 0; j < 32; ++j) v[j] = 0u; }
+                        if (k < cout) {
+#pragma unroll
+                            for (int j = 0; j < 32; j += 4)
+                                if (tn * 64 + c0 + j < cin) *reinterpret_cast<uint4*>(dst + c0 + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                        }
+                    }
+                }
+            }
+        } else if (ok && quad * 32 < cout - tm * 128) {              // warp-uniform: this lane quadrant holds real output channels
             for (int tt = 0; tt < ntap; ++tt) {
                 const int wt = wtap_s[tt];
                 float* dst = splits > 1 ? partial + (((long long)split * taps + wt) * cout + k) * cin + tn * n_tile
@@ -870,13 +905,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) conv_wgrad_tc_kernel(const TcWg
                     if (nc > 0) {
                         tmem_ld32(tmem_d + ((uint32_t)(quad * 32) << 16) + (uint32_t)(tt * n_tile + c0), v);
                         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                        if ((ntap & 1) && tt == ntap - 1) {      // the tap whose positions were split: first half + second half
-                            uint32_t v2[32];
-                            tmem_ld32(tmem_d + ((uint32_t)(quad * 32) << 16) + (uint32_t)(ntap * n_tile + c0), v2);
-                            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-                            for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + __uint_as_float(v2[j]));
-                        }
                     } else { for (int j = 0; j < 32; ++j) v[j] = 0u; }
                     if (k < cout) {
 #pragma unroll
@@ -1281,26 +1309,31 @@ void launch_conv_tc_probs(const void* d_tc, int nprob, int max_tiles, size_t pac
 }
 
 // ---- wgrad host side
-struct WgGeom { TcWgradProb t; size_t smem, partial_bytes; int box_h, box_n; };
+struct WgGeom { TcWgradProb t; size_t smem, partial_bytes; long long cost; int box_h, box_n; };
 
-static bool wg_geometry_box(const ConvProb& p, int target_ctas, WgGeom& w, int max_box);
+static bool wg_geometry_box(const ConvProb& p, int target_ctas, WgGeom& w, int max_box, bool nine);
 // Both operands of a 3x3 weight gradient are windows of boxes, so a stage is large and the boxes' rounding decides how many stages
 // fit: the largest boxes that still leave two stages are taken (fewer TMA issues), else the size with the most stages.
+// A stride-1 3x3 layer has two forms: 128 x 128 tiles with one filter row's three taps per CTA, or 64 x 64 tiles with all nine taps, which load
+// both operands once and, at 64 channels, leave no half of the MMA's lanes idle.  The cheaper one by the split's cost is taken.  us at
+// 8 x 128 images, three taps | nine: 64 channels 32 x 32 294 | 94, 128 16 x 16 102 | 119, 256 8 x 8 146 | 101 (96 against 128 CTAs), 512 4 x 4 134 | 150.
 static bool wg_geometry(const ConvProb& p, int target_ctas, WgGeom& w) {
-    if (p.ksz == 1) return wg_geometry_box(p, target_ctas, w, 96);
+    if (p.ksz == 1) return wg_geometry_box(p, target_ctas, w, 96, false);
     const int caps[5] = {96, 64, 48, 32, 24};
-    WgGeom best; int best_stages = 0;
-    for (int i = 0; i < 5; ++i) {
-        WgGeom g;
-        if (!wg_geometry_box(p, target_ctas, g, caps[i])) continue;
-        if (g.t.stages > best_stages) { best = g; best_stages = g.t.stages; }
-        if (best_stages >= 2) break;
+    bool found = false;
+    for (int nine = 0; nine < (p.stride == 1 ? 2 : 1); ++nine) {
+        WgGeom best; int best_stages = 0;
+        for (int i = 0; i < 5 && best_stages < 2; ++i) {
+            WgGeom g;
+            if (!wg_geometry_box(p, target_ctas, g, caps[i], nine != 0)) continue;
+            if (g.t.stages > best_stages) { best = g; best_stages = g.t.stages; }
+        }
+        if (!best_stages || (found && best.cost >= w.cost)) continue;
+        w = best; found = true;
     }
-    if (!best_stages) return false;
-    w = best;
-    return true;
+    return found;
 }
-static bool wg_geometry_box(const ConvProb& p, int target_ctas, WgGeom& w, int max_box) {
+static bool wg_geometry_box(const ConvProb& p, int target_ctas, WgGeom& w, int max_box, bool nine) {
     if (!tc_shape_ok(p)) return false;
     if (((uintptr_t)p.act | (uintptr_t)p.wgt) & 15) return false;
     TcWgradProb& t = w.t; memset(&t, 0, sizeof(t));
@@ -1323,9 +1356,16 @@ static bool wg_geometry_box(const ConvProb& p, int target_ctas, WgGeom& w, int m
         Tall g; if (!tall_of(p.H, p.W, 1, 1, g, max_box)) return false;
         w.box_h = g.box_h; w.box_n = g.box_n;
         t.dy_flat = 0; t.a_flat = 0; t.pad = 1; t.Hp = g.Hp; t.Wp = g.Wp; t.R = g.R; t.box_pos = g.box_pos; t.hb = g.Wp + 1;
-        t.nbox_dy = boxes_for(TILE_M, g.box_pos); t.nbox_a = boxes_for(TILE_M + 2 * t.hb, g.box_pos); t.dy_box_bytes = g.box_bytes; t.a_box_bytes = g.box_bytes;
+        t.dy_box_bytes = g.box_bytes; t.a_box_bytes = g.box_bytes;
+        if (nine) {
+            t.nine = 1; t.hb = 1;                        // dy from the chunk on, a from one position before it, both for one more row of the map
+            t.nbox_dy = boxes_for(TILE_M + g.Wp, g.box_pos); t.nbox_a = boxes_for(TILE_M + g.Wp + 2, g.box_pos);
+            t.tap[0] = TapRef{0, 0}; t.tap[3] = TapRef{3, g.Wp};       // where the two accumulators' windows start
+        } else {
+            t.nbox_dy = boxes_for(TILE_M, g.box_pos); t.nbox_a = boxes_for(TILE_M + 2, g.box_pos); t.hb_step = g.Wp;      // a group is the three taps of a filter row
+            for (int i = 0; i < 9; ++i) t.tap[i] = TapRef{i, i % 3};
+        }
         total_pos = (long long)p.N * g.Hp * g.Wp;
-        for (int i = 0; i < 9; ++i) t.tap[i] = TapRef{i, (i / 3) * g.Wp + (i % 3)};
         t.tap_groups = 0;                                // groups of up to three taps: set below, once the column tile is known
     } else {
         Tall g; if (!tall_of(p.P, p.Q, 1, 2, g, max_box)) return false;
@@ -1344,39 +1384,43 @@ static bool wg_geometry_box(const ConvProb& p, int target_ctas, WgGeom& w, int m
         }
     }
     t.chunks = (int)((total_pos + TILE_M - 1) / TILE_M);
-    t.m_tiles = (p.K + 127) / 128;
+    t.m_tile = t.nine ? 64 : 128; t.dy_slabs = t.m_tile / 64;
+    t.m_tiles = (p.K + t.m_tile - 1) / t.m_tile;
     // columns of one CTA: the input channels in tiles of at most 256 (1x1) or 128 (3x3: up to four taps in 512 columns of tensor memory)
-    const int n_cap = taps == 1 ? 256 : 128;
+    const int n_cap = taps == 1 ? 256 : t.nine ? 64 : 128;
     t.n_tiles = (p.C + n_cap - 1) / n_cap;
     t.n_tile = (p.C + t.n_tiles - 1) / t.n_tiles;
     t.n_tile = t.n_tiles > 1 ? (t.n_tile + 63) / 64 * 64 : (t.n_tile + 15) / 16 * 16;
     t.n_tiles = (p.C + t.n_tile - 1) / t.n_tile;
+    if (t.nine) t.n_tile = 64;
     t.a_slabs = (t.n_tile + 63) / 64;
-    if (taps == 9 && p.stride == 1) { for (int g = 0; g < 3; ++g) { t.gbeg[g + 1] = 3 * (g + 1); t.gxs[g] = 0; t.gys[g] = 0; } t.tap_groups = 3; }
-    int max_group = 0; for (int g = 0; g < t.tap_groups; ++g) max_group = std::max(max_group, t.gbeg[g + 1] - t.gbeg[g]);
-    int max_acc = 0; for (int g = 0; g < t.tap_groups; ++g) { const int n = t.gbeg[g + 1] - t.gbeg[g]; max_acc = std::max(max_acc, n + (n & 1)); }   // an odd group's last tap takes two accumulators
-    (void)max_group;
-    t.tmem_cols = 32; while (t.tmem_cols < max_acc * t.n_tile) t.tmem_cols *= 2;
+    if (t.nine) { t.tap_groups = 1; t.gbeg[1] = 9; }
+    else if (taps == 9 && p.stride == 1) { for (int g = 0; g < 3; ++g) { t.gbeg[g + 1] = 3 * (g + 1); t.gxs[g] = 0; t.gys[g] = 0; } t.tap_groups = 3; }
+    int max_acc = 0; for (int g = 0; g < t.tap_groups; ++g) max_acc = std::max(max_acc, t.gbeg[g + 1] - t.gbeg[g]);
+    t.mma_n = t.nine ? 192 : t.n_tile;
+    if (t.nine) max_acc = 2;
+    t.tmem_cols = 32; while (t.tmem_cols < max_acc * t.mma_n) t.tmem_cols *= 2;
     if (t.tmem_cols > 512) return false;
     t.dy_slab_bytes = (t.nbox_dy * t.dy_box_bytes + 1023) / 1024 * 1024;
     t.a_slab_bytes = (t.nbox_a * t.a_box_bytes + 1023) / 1024 * 1024;
-    t.stage_bytes = 2 * t.dy_slab_bytes + t.a_slabs * t.a_slab_bytes;
+    t.dy_lead = t.nine ? t.Wp * 128 : t.dy_slab_bytes; t.a_lead = t.nine ? 128 : t.a_slab_bytes;
+    t.stage_bytes = t.dy_slabs * t.dy_slab_bytes + t.a_slabs * t.a_slab_bytes;
     t.stages = TC_MAX_STAGES; while (t.stages > 1 && (size_t)t.stages * t.stage_bytes > TC_SMEM_BUDGET) --t.stages;
     if ((size_t)t.stages * t.stage_bytes > TC_SMEM_BUDGET) return false;
     w.smem = std::max((size_t)t.stages * t.stage_bytes, (size_t)120 * 1024) + 1024;
     // Split of the positions.  target_ctas is twice this problem's share of the SMs.  Every CTA pays a fixed cost (set-up, the
     // accumulators' way out) worth about six chunks, and a launch takes whole waves, so the split is the one that minimises
-    // waves x (chunks per CTA + 6): mostly one full wave.  The partial buffer is sized for the most splits any share could pick.
+    // waves x (chunks per CTA + 6): mostly one full wave.  (A chunk of the nine-tap form takes 3/4 of the others' time.)  The partial buffer is sized for the most splits any share could pick.
     const int fixed = t.m_tiles * t.n_tiles * t.tap_groups;
     const int want_max = std::max(1, std::min(std::min(t.chunks, 256), target_ctas / fixed));
     const int share = std::max(1, target_ctas / 2);
     long long best_cost = -1; int best_cps = t.chunks;
     for (int sp = 1; sp <= want_max; ++sp) {
         const int cps = (t.chunks + sp - 1) / sp, eff = (t.chunks + cps - 1) / cps;
-        const long long waves = ((long long)fixed * eff + share - 1) / share, cost = waves * (cps + 6);
+        const long long waves = ((long long)fixed * eff + share - 1) / share, cost = waves * ((t.nine ? 3 : 4) * (long long)cps + 24);
         if (best_cost < 0 || cost < best_cost) { best_cost = cost; best_cps = cps; }
     }
-    t.chunks_per_split = best_cps; t.splits = (t.chunks + best_cps - 1) / best_cps;
+    w.cost = best_cost; t.chunks_per_split = best_cps; t.splits = (t.chunks + best_cps - 1) / best_cps;
     w.partial_bytes = want_max > 1 ? (size_t)want_max * taps * p.K * p.C * 4 : 0;
     return true;
 }
