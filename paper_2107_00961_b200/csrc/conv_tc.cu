@@ -940,22 +940,23 @@ __global__ void __launch_bounds__(256) wgrad_tc_reduce_kernel(const TcWgradProb*
 
 // ------------------------------------------------------------------------------------------------ BN statistics from the tiles' sums
 // The convolution kernel leaves, per 128-position tile, the column sums of what it stored.  Here they are added in a fixed order in
-// double: a CTA takes 16 channels, 32 rows of threads every 32nd tile (all of a thread's loads in flight for up to 256 tiles; latency is
-// all there is to this kernel), then the 32 sums.  MODE 0, forward: mean, 1/sqrt(var + eps) and the running statistics.
+// double: a CTA takes CH channels, 512 / CH rows of threads every (512 / CH)-th tile (eight tiles' loads in flight per thread; latency is
+// all there is to this kernel), then the rows' sums.  MODE 0, forward: mean, 1/sqrt(var + eps) and the running statistics.
 // MODE 1, backward: the two reduction sums and the gradients of beta and gamma.
-template <int MODE>
+template <int MODE, int CH>
 __global__ void __launch_bounds__(512) bn_finalize_tiles_kernel(const BnProb* __restrict__ probs) {
     const BnProb& p = probs[blockIdx.y];
-    const int C = p.C, ch = threadIdx.x & 15, row = threadIdx.x >> 4, c = blockIdx.x * 16 + ch, n = p.chunks;
-    if ((int)blockIdx.x * 16 >= C) return;
-    __shared__ double red[2][32][17];
+    constexpr int ROWS = 512 / CH;
+    const int C = p.C, ch = threadIdx.x % CH, row = threadIdx.x / CH, c = blockIdx.x * CH + ch, n = p.chunks;
+    if ((int)blockIdx.x * CH >= C) return;
+    __shared__ double red[2][ROWS][CH + 1];
     const float* __restrict__ t = reinterpret_cast<const float*>(p.partial) + (c < C ? c : 0);
     double a0 = 0.0, a1 = 0.0;
-    for (int k = row; k < n; k += 8 * 32) {                      // eight tiles of loads in flight per thread
+    for (int k = row; k < n; k += 8 * ROWS) {                    // eight tiles of loads in flight per thread
         float v0[8], v1[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-            const int kk = k + 32 * u;
+            const int kk = k + ROWS * u;
             v0[u] = kk < n ? __ldcg(t + (long long)kk * 2 * C) : 0.f; v1[u] = kk < n ? __ldcg(t + ((long long)kk * 2 + 1) * C) : 0.f;
         }
 #pragma unroll
@@ -964,10 +965,12 @@ __global__ void __launch_bounds__(512) bn_finalize_tiles_kernel(const BnProb* __
     red[0][row][ch] = a0; red[1][row][ch] = a1;
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // warp = channel of the 16, lane = row of sums; fixed butterfly
+    if (warp >= CH) return;
+    // warp = channel, lane = every 32nd row of sums; fixed butterfly
     a0 = red[0][lane][warp]; a1 = red[1][lane][warp];
+    for (int r = lane + 32; r < ROWS; r += 32) { a0 += red[0][r][warp]; a1 += red[1][r][warp]; }
     for (int d = 16; d; d >>= 1) { a0 += __shfl_xor_sync(0xffffffffu, a0, d); a1 += __shfl_xor_sync(0xffffffffu, a1, d); }
-    const int cc = blockIdx.x * 16 + warp;
+    const int cc = blockIdx.x * CH + warp;
     if (lane != 0 || cc >= C) return;
     if (MODE == 1) {
         p.stat[2 * C + cc] = (float)a0; p.stat[3 * C + cc] = (float)a1;
@@ -984,9 +987,14 @@ __global__ void __launch_bounds__(512) bn_finalize_tiles_kernel(const BnProb* __
         p.run_var[cc] = (float)((1.0 - mo) * (double)p.run_var[cc] + mo * unb);
     }
 }
+// 16 channels per CTA while that gives every SM one, 4 below: the fewer channels, the fewer CTAs, and the tiles are then many
+// (the ImageNet-stem step, whose 64-channel layers have 1568 tiles and filled 16 SMs: 21.40 -> 21.21 ms).
 void launch_bn_finalize_tiles(const BnProb* d, int nprob, int max_c, int backward, cudaStream_t s) {
-    const dim3 g((max_c + 15) / 16, nprob);
-    if (backward) bn_finalize_tiles_kernel<1><<<g, 512, 0, s>>>(d); else bn_finalize_tiles_kernel<0><<<g, 512, 0, s>>>(d);
+    const bool few = (max_c + 15) / 16 * nprob < 148;
+    const int ch = few ? 4 : 16;
+    const dim3 g((max_c + ch - 1) / ch, nprob);
+    if (backward) { if (few) bn_finalize_tiles_kernel<1, 4><<<g, 512, 0, s>>>(d); else bn_finalize_tiles_kernel<1, 16><<<g, 512, 0, s>>>(d); }
+    else { if (few) bn_finalize_tiles_kernel<0, 4><<<g, 512, 0, s>>>(d); else bn_finalize_tiles_kernel<0, 16><<<g, 512, 0, s>>>(d); }
 }
 
 // ------------------------------------------------------------------------------------------------ host side
