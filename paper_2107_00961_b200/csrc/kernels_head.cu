@@ -422,7 +422,8 @@ __global__ void __launch_bounds__(256) im2col_kernel(const ColProb* __restrict__
     const int per_img = (P + rp - 1) / rp;
     const int n = blockIdx.x / per_img, p0 = (blockIdx.x - n * per_img) * rp;
     if (n >= p.N) return;
-    if (blockIdx.x < 8) pack_stem_weights(p, blockIdx.x * 256 + tid, 8 * 256);
+    const int packers = min(8, (int)gridDim.x);                  // a few small images are fewer than eight CTAs
+    if ((int)blockIdx.x < packers) pack_stem_weights(p, blockIdx.x * 256 + tid, packers * 256);
     const unsigned short* __restrict__ src = (const unsigned short*)p.src;
     const int WC = W * C, y0 = p0 * stride - p.pad;
     if ((WC & 7) == 0 && ((uintptr_t)src & 15) == 0) {            // rows are whole 16-byte runs
