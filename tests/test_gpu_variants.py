@@ -1,0 +1,207 @@
+"""The kernel variants and the dispatch rules between them, at the sizes where one ends and the next begins: edges of tiles, remainders,
+the smallest and largest sizes of a range.  References: the oracle's layer and network routines, or, where two runs must agree to the
+bit, the same work done the other way.
+"""
+from concurrent.futures import ThreadPoolExecutor
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import synth
+from parity import LR, max_rel_err, norm_max_abs, per_tensor, run_protocol_both, to_dev
+
+pytestmark = pytest.mark.gpu
+
+# One bf16 rounding that falls on the other side moves an element by one ulp, at most 2^-7 of it; the criterion is relative to the largest.
+BF16_TOL = 2.0 ** -7
+# fp32 sums of n products: every addition rounds by at most 2^-24 of the partial sum, a random walk of sqrt(n) steps; against the 1 % floor
+# of max_rel_err that is 100 sqrt(n) 2^-24: 1e-3 up to n = 28000.  The longer sums below are split over CTAs into much shorter ones.
+F32_TOL = 1e-3
+
+
+@pytest.fixture(scope="module")
+def m():
+    import paper_2107_00961_b200 as mod
+    mod.lib()
+    return mod
+
+
+def rnd(seed, *shape, bf16=True):
+    x = synth.standard_normal(seed, int(np.prod(shape))).astype(np.float32).reshape(shape)
+    return synth.round_to_bf16(x) if bf16 else x
+
+
+def dev(x, bf16=True):
+    t = torch.from_numpy(np.ascontiguousarray(x)).cuda()
+    return t.to(torch.bfloat16) if bf16 else t
+
+
+# (backend, N, H, W, C, K, ksz, stride)
+CONVS = [
+    # tap-per-warp kernels: one position, ragged channels, 2048 positions and one more (the weight gradient's line), 64 M multiply-adds and just above
+    (1, 1, 1, 1, 5, 3, 3, 1), (1, 3, 5, 7, 5, 9, 3, 1), (1, 2, 9, 9, 33, 17, 1, 2), (1, 1, 32, 64, 8, 16, 3, 1), (1, 1, 3, 683, 8, 8, 3, 1),
+    (1, 4, 20, 25, 40, 88, 3, 1), (1, 4, 20, 26, 40, 88, 3, 1),
+    # weight gradient with nine taps per CTA: one chunk, two images in a box, ragged channels, rows wider than the largest box, many splits
+    (2, 1, 3, 3, 64, 64, 3, 1), (2, 9, 5, 7, 64, 64, 3, 1), (2, 2, 33, 31, 48, 40, 3, 1), (2, 1, 4, 100, 64, 64, 3, 1), (2, 20, 32, 32, 64, 64, 3, 1),
+    # both forms of it: three taps of 128 x 128 tiles where the split fills the SMs, nine where it does not; stride 2 keeps its phases
+    (2, 4, 17, 15, 136, 72, 3, 1), (2, 2, 8, 8, 256, 256, 3, 1), (2, 3, 11, 13, 72, 200, 3, 2),
+    # forward and data gradient: one tile, a last wave of single tiles (298 tiles), column tiles narrower than the channels
+    (2, 1, 2, 2, 64, 64, 1, 1), (2, 4, 97, 98, 64, 72, 1, 1), (2, 5, 14, 14, 256, 256, 3, 1),
+]
+
+
+@pytest.mark.parametrize("case", CONVS)
+def test_convolutions_at_the_edges_of_the_variants(m, case):
+    backend, N, H, W, C, K, k, s = case
+    geom = (N, H, W, C, K, k, s)
+    a, w = rnd(1, N, H, W, C), synth.round_to_bf16(rnd(2, K, k, k, C) * np.float32(0.25))
+    y_ref = oracle.conv_fwd(a, w, s, quant=1)
+    dy = rnd(4, *y_ref.shape)
+    y, _ = m.resist_conv2d(0, dev(a), dev(w), geom, backend=backend)
+    da, _ = m.resist_conv2d(1, dev(dy), dev(w), geom, backend=backend)
+    dw, _ = m.resist_conv2d(2, dev(a), dev(dy), geom, backend=backend)
+    assert norm_max_abs(y.float().cpu().numpy(), y_ref) < BF16_TOL
+    assert norm_max_abs(da.float().cpu().numpy(), oracle.conv_dgrad(dy, w, (H, W), s, quant=1)) < BF16_TOL
+    assert max_rel_err(dw.cpu().numpy(), oracle.conv_wgrad(dy, a, k, s)) < F32_TOL
+
+
+# a single tile of sums, two partial tiles, more tiles than one pass of loads holds, stride-1 3x3 over several column tiles
+@pytest.mark.parametrize("shape", [(1, 2, 3, 64, 64, 1), (1, 13, 11, 256, 64, 1), (2, 160, 207, 64, 64, 1), (3, 9, 7, 512, 128, 3)])
+def test_backward_sums_from_the_data_gradients_tiles(m, shape):
+    N, H, W, C, K, k = shape
+    w, dy = synth.round_to_bf16(rnd(2, K, k, k, C) * np.float32(0.25)), rnd(4, N, H, W, K)
+    x = synth.round_to_bf16(rnd(5, N, H, W, C) * np.float32(1.7) + rnd(6, C)[None, None, None, :])
+    g, b = (1 + 0.2 * rnd(13, C)).astype(np.float32), (0.3 * rnd(14, C)).astype(np.float32)
+    _, mean, invstd = oracle.bn_relu_fwd(x.reshape(-1, C), g, b, quant=1)
+    stat = torch.zeros(4 * C, device="cuda")
+    stat[:C], stat[C:2 * C] = dev(mean.astype(np.float32), False), dev(invstd.astype(np.float32), False)
+    da, dx, dg, db, used = m.resist_conv2d_bn_relu(1, dev(dy), dev(w), (N, H, W, C, K, k, 1), dev(g, False), dev(b, False), stat=stat, x=dev(x), backend=2)
+    assert used == 1
+    # from the library's own da on, so that only this pass's arithmetic is compared: sums of n terms in fp32 per tile, then double
+    dx_ref, dg_ref, db_ref = oracle.bn_relu_bwd(da.float().cpu().numpy().reshape(-1, C), x.reshape(-1, C), g, b, mean, invstd, quant=1)
+    # A ReLU mask is taken from gamma * xhat + beta, which fp32 decides differently within about 1e-6 of zero: one element in a million, worth
+    # one term of the sum, 5 sigma against the sum's sqrt(n) sigma: below 2e-3 of the largest sum from n = 1000 on, none is expected below.
+    assert norm_max_abs(dg.cpu().numpy(), dg_ref) < 2e-3 and norm_max_abs(db.cpu().numpy(), db_ref) < 2e-3
+    assert norm_max_abs(dx.float().cpu().numpy().reshape(-1, C), dx_ref) < 2 * BF16_TOL      # rounded twice: the term and its sum
+    assert norm_max_abs(da.float().cpu().numpy(), oracle.conv_dgrad(dy, w, (H, W), 1, quant=1)) < BF16_TOL
+
+
+@pytest.mark.parametrize("rows,C", [(1, 64), (65535, 64), (200001, 16), (8192, 24), (8193, 24)])
+def test_bn_passes_at_wave_and_small_layer_edges(m, rows, C):
+    x, da = synth.round_to_bf16(rnd(11, rows, C) * np.float32(1.7) + rnd(12, C)[None, :]), rnd(17, rows, C)
+    g, b = (1 + 0.2 * rnd(13, C)).astype(np.float32), (0.3 * rnd(14, C)).astype(np.float32)
+    a_ref, mean, invstd = oracle.bn_relu_fwd(x, g, b, quant=1)
+    dx_ref, dg_ref, db_ref = oracle.bn_relu_bwd(da, x, g, b, mean, invstd, quant=1)
+    a, stat = m.resist_bn_relu_forward(dev(x), dev(g, False), dev(b, False))
+    dx, dg, db = m.resist_bn_relu_backward(dev(x), dev(da), dev(g, False), dev(b, False), stat)
+    assert norm_max_abs(a.float().cpu().numpy(), a_ref) < BF16_TOL
+    assert norm_max_abs(dx.float().cpu().numpy(), dx_ref) < 2 * BF16_TOL
+    assert norm_max_abs(dg.cpu().numpy(), dg_ref) < 2e-3 and norm_max_abs(db.cpu().numpy(), db_ref) < 2e-3      # as above
+
+
+@pytest.mark.parametrize("release", [False, True])
+def test_layer_calls_from_many_threads_and_streams_share_the_scratch_pool(m, release):
+    shapes = [(2, 8, 8, 64, 64, 3, 1), (4, 16, 16, 32, 32, 3, 1), (1, 28, 28, 128, 128, 3, 1), (3, 5, 7, 5, 9, 3, 1), (2, 16, 16, 256, 64, 1, 1), (2, 16, 16, 64, 64, 3, 2)]
+    data = [(dev(rnd(10 + i, *g[:4])), dev(rnd(30 + i, g[4], g[5], g[5], g[3]))) for i, g in enumerate(shapes)]
+    torch.cuda.synchronize()
+    alone = [m.resist_conv2d(0, a, w, g)[0].cpu() for (a, w), g in zip(data, shapes)]
+
+    def work(i):
+        st = torch.cuda.Stream()
+        out = []
+        with torch.cuda.stream(st):
+            for j in range(12):
+                q = (i + j) % len(shapes)
+                out.append((q, m.resist_conv2d(0, *data[q], shapes[q], stream=st)[0]))
+                if release and j % 5 == i % 5:
+                    assert m.lib().resist_layer_release_scratch() == 0
+        st.synchronize()
+        return [(q, y.cpu()) for q, y in out]
+
+    with ThreadPoolExecutor(max_workers=8) as ex:
+        for got in ex.map(work, range(8)):
+            for q, y in got:
+                assert torch.equal(y, alone[q])
+    assert m.lib().resist_layer_release_scratch() == 0
+
+
+def net(h, w, classes, stem, width, pool, kind=synth.BASIC, depth=(2, 2)):
+    mids = tuple(width * (i + 1) for i in range(len(depth)))
+    widths = mids if kind == synth.BASIC else tuple(4 * x for x in mids)
+    k, s = (7, 2) if pool else (3, 1)
+    return synth.Arch(h, w, 3, classes, k, s, stem, 1 if pool else 0, pool, synth._stack(kind, stem, depth, widths, mids, "stage_first_shared"))
+
+
+# head: one kernel up to 8192 weights, 256 channels and 128 classes, tiled products beyond; max-pool: odd maps (windows that leave the map on one
+# side), channels with and without the vector width.  The 7x7 stem's scale has a zero gradient in exact arithmetic (scale invariance): left out.
+NETS = [net(8, 8, 128, 8, 32, 0), net(8, 8, 129, 8, 32, 0), net(6, 5, 32, 8, 128, 0), net(6, 5, 31, 8, 129, 0), net(5, 6, 2, 8, 8, 0), net(6, 6, 1000, 8, 16, 0),
+        net(37, 29, 10, 8, 8, 1), net(33, 42, 11, 12, 12, 1)]
+
+
+@pytest.mark.parametrize("arch", NETS, ids=lambda a: f"{a.in_h}x{a.in_w}_stem{a.stem_cout}_classes{a.classes}")
+def test_heads_and_pooling_in_a_step(m, arch):
+    out = run_protocol_both(arch, 2, 5, 1, 23, "f32", 0, True, m)
+    # behind the max-pool almost constant channels multiply upstream rounding by up to 1 / sqrt(eps) = 316
+    tol = 5e-3 if arch.stem_maxpool else 1e-4
+    for s, r in enumerate(out["steps"][0]["subs"]):
+        assert max_rel_err(r["logits_gpu"], r["logits_cpu"]) < tol
+        v, name = per_tensor(arch, r["grads_gpu"], r["grads_cpu"], max_rel_err, skip_names=("stem.bn.gamma",))
+        assert v < tol, (name, v)
+
+
+@pytest.mark.parametrize("dtype,grouped", [("f32", True), ("bf16", True), ("bf16", False)])
+def test_recorded_steps_equal_launched_steps(m, dtype, grouped):
+    """Two rounds of four steps, new tensors and a new learning rate each: a plan is launched twice and replayed from its recording from then
+    on; a context that profiles launches every step.  Same bits."""
+    arch = net(16, 16, 10, 16, 16, 0, depth=(2, 3))
+    a, S, B = arch.to_int32(), 3, 12
+    p0, buf0 = synth.perturbed_params(arch, 4)
+    tdt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    got = []
+    for profile in (False, True):
+        ctx = m.Context(a, dtype=m.BF16 if dtype == "bf16" else m.F32)
+        ctx.set_params(p0, buf0)
+        ctx.set_profiling(profile)
+        for r in range(2):
+            ctx.partition(50 + r, S)
+            for step in range(4):
+                xs = [to_dev(rnd(100 * r + 10 * step + s, B, 16, 16, 3), tdt) for s in range(S)]
+                ys = [to_dev((synth.splitmix64_words(7 * step + s, B) % np.uint64(10)).astype(np.int32), None) for s in range(S)]
+                loss, lr = torch.zeros(S, device="cuda"), LR / (1 + 4 * r + step)
+                if grouped:
+                    ctx.local_step_grouped(xs, ys, lr, loss)
+                else:
+                    for s in range(S):
+                        ctx.local_step(s, xs[s], ys[s], lr, loss[s:s + 1])
+                torch.cuda.synchronize()
+                got.append((profile, loss.cpu().numpy()))
+            ctx.aggregate()
+        got.append((profile, *ctx.get_params(-1)))
+    n = len(got) // 2
+    for one, two in zip(got[:n], got[n:]):
+        for u, v in zip(one[1:], two[1:]):
+            np.testing.assert_array_equal(u, v)
+
+
+# BN in the epilogues of evaluation's convolutions, three calls so that the recorded form runs too: warp-level layers, tcgen05 layers with more than
+# one slab and column tile, the pooled stem; 1 image, a ragged batch and one that fills several waves of tiles
+@pytest.mark.parametrize("kind,width,pool", [(synth.BASIC, 16, 0), (synth.BOTTLENECK, 64, 0), (synth.BOTTLENECK, 64, 1)])
+@pytest.mark.parametrize("B", [1, 13, 150])
+def test_evaluation_with_bn_in_the_epilogues(m, kind, width, pool, B):
+    hw = 40 if pool else 16
+    arch = net(hw, hw - 3, 10, width, width, pool, kind)
+    a = arch.to_int32()
+    p, buf = synth.perturbed_params(arch, 3)
+    ctx = m.Context(a, dtype=m.BF16)
+    ctx.set_params(p, buf)
+    ctx.partition(1, 2)
+    for call in range(3):
+        x = rnd(8 + call, B, arch.in_h, arch.in_w, 3)
+        y = (synth.splitmix64_words(9 + call, B) % np.uint64(10)).astype(np.int32)
+        logits, loss, _ = ctx.eval(to_dev(x, torch.bfloat16), to_dev(y, None))
+        ref = oracle.evaluate(a, p, buf, 2, x, y, quant=1)
+        # seven layers of one-ulp differences (2^-8 each of what they touch), averaged by the sums that follow: 2e-2 as for whole steps
+        assert norm_max_abs(logits.cpu().numpy(), ref["logits"]) < 2e-2
+        assert abs(loss.item() - ref["loss"]) < 2e-2 * max(1.0, abs(ref["loss"]))
