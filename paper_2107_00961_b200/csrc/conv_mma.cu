@@ -1,11 +1,11 @@
 // Convolutions of NARROW layers (C and K multiples of 16, at most 64) on warp-level MMA (mma.sync m16n8k16, bf16
 // inputs, fp32 accumulation).
 //
-// Why not tcgen05 here: one thread issues a tcgen05.mma (M = 128, K = 16) only every 114-165 cycles whatever its N, two
-// issuing warps every 57-82 (resist_micro_mma_rate in micro.cu measures it), while the tensor core needs N / 2 cycles: a layer
-// with 16 or 32 output channels would spend 4-10 times its tensor time on issue, and its TMA rows would be 32-64 bytes.  The
-// warp-level MMA has no such granularity (n = 8), cp.async has no per-row cost, and these HBM-bound layers need far less
-// than its rate.  Wider layers, and 64-channel 3x3 layers with many positions, run on tcgen05 (conv_tc.cu).
+// Why not tcgen05 here: a tcgen05.mma of 16 or 32 columns takes as long as one of 48, TMA rows of 32 to 64 bytes cost as much as rows of
+// 128, and what every role does per tile (~5800 clocks) is then more than the tile's MMAs.  Built and measured with 32- and 64-byte
+// swizzled rows and the whole filter resident: 16 channels, 1000 x 32 x 32, 108 us against 37 here; 32 channels 40 against 29.  The
+// warp-level MMA has no such granularity (n = 8), cp.async has no per-row cost, and these HBM-bound layers need far less than its
+// rate.  Wider layers, and 64-channel 3x3 layers with many positions, run on tcgen05 (conv_tc.cu).
 //
 // Tiling: a GROUP of G whole images is one tall zero-padded map.  With pad = k/2, image n occupies rows
 // n*Hp .. n*Hp+H-1 (Hp = H + pad) of a map that is Wp = W + pad wide; row H of every image and column W of every

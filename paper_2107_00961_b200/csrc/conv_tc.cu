@@ -714,8 +714,9 @@ void launch_zero_stuff(const UpProb* d, int nprob, long long max_vecs, cudaStrea
 // The nine-tap form (stride 1): the two 64-row halves of A are the same 64 channels of dy, the second one map row further (the descriptor's
 // leading offset is Wp rows instead of a slab), and the three 64-column parts of B the same channels of a, one position apart each.  One MMA
 // of 128 x 192 then holds the taps (row 1; 0, 1, 2) in its lower and (row 0; 0, 1, 2) in its upper lanes, a second one row 2 (and row 1 again, unused).
-// What bounds it: the boxes' way from L2 into shared memory, 20 to 25 bytes per clock and SM; the MMAs alone would take 1536 clocks of a chunk's
-// ~2500.  One thread producing both operands with two divisions per box took ~5500 clocks per chunk.  8 x 128 images, us: 64 channels 32 x 32 294 -> 94,
+// What bounds it: the tensor pipe, 74 % active at 64 channels and 1024 x 32 x 32 positions (a quarter of that is row 1 computed twice), then the
+// boxes' way into shared memory.  Before, one thread produced both operands with two divisions per box and a chunk of 1536 clocks of MMAs took
+// ~5500.  8 x 128 images, us: 64 channels 32 x 32 294 -> 94,
 // 128 16 x 16 143 -> 102, 256 8 x 8 205 -> 101, 512 4 x 4 171 -> 134.
 struct alignas(64) TcWgradProb {
     CUtensorMap map_dy;       // (channel k, pixel) or (channel k, x, y, image)
