@@ -321,13 +321,19 @@ __global__ void __launch_bounds__(256) bn_reduce_kernel(const BnProb* __restrict
             float mean = 0.f, istd = 0.f, g = 0.f, b = 0.f, shift = 0.f;
             if (MODE == 1) { mean = p.stat[c]; istd = p.stat[C + c]; g = p.gamma[c]; b = p.beta[c]; }
             else shift = ldf<T>(p.x, c);      // sums of (x - x[0,c]): no cancellation when |mean| >> std
-            for (long long r = r0 + rg; r < r1; r += R) {
-                float x = ldf<T>(p.x, r * C + c);
-                if (MODE == 0) { x -= shift; s0 += x; s1 += x * x; }
-                else {
-                    float xh = (x - mean) * istd;
-                    float dz = (xh * g + b > 0.f) ? ldf<T>(p.da, r * C + c) : 0.f;
-                    s0 += dz; s1 += dz * xh;
+            // eight rows of loads in flight per thread, added in ascending order
+            for (long long r = r0 + rg; r < r1; r += 8 * R) {
+                float xs[8], ds[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const long long i = (r + u * R) * C + c; const bool in = r + u * R < r1;
+                    xs[u] = in ? ldf<T>(p.x, i) : 0.f; ds[u] = MODE == 1 && in ? ldf<T>(p.da, i) : 0.f;
+                }
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    if (r + u * R >= r1) break;
+                    if (MODE == 0) { const float x = xs[u] - shift; s0 += x; s1 += x * x; }
+                    else { const float xh = (xs[u] - mean) * istd, dz = xh * g + b > 0.f ? ds[u] : 0.f; s0 += dz; s1 += dz * xh; }
                 }
             }
         }
@@ -375,35 +381,51 @@ __global__ void bn_finalize_kernel(const BnProb* __restrict__ probs) {
     }
 }
 
+// The elementwise pass of the other types and channel counts, laid out like the sums: a thread keeps one channel with its constants in registers
+// and walks down its rows, eight of them in flight; a CTA takes an even share of the rows.  (A thread per element, with a 64-bit division
+// for the channel and its four constants loaded anew: GENERIC_US2.)
+template <class T, int MODE>
+__device__ void bn_stream_scalar(const BnProb& p) {
+    const int C = p.C, nl = C < 256 ? C : 256, R = 256 / nl, rg = threadIdx.x / nl, lane = threadIdx.x % nl;
+    long long rows = (p.m + gridDim.x - 1) / gridDim.x; rows = (rows + R - 1) / R * R;
+    const long long r0 = blockIdx.x * rows, r1 = r0 + rows < p.m ? r0 + rows : p.m;
+    const float inv_m = 1.f / (float)p.m;
+    if (rg >= R) return;
+    for (int c = lane; c < C; c += nl) {
+        const float mean = p.stat[c], istd = p.stat[C + c], g = p.gamma[c], b = p.beta[c];
+        const float sb = MODE == 1 ? p.stat[2 * C + c] * inv_m : 0.f, sg = MODE == 1 ? p.stat[3 * C + c] * inv_m : 0.f;
+        for (long long r = r0 + rg; r < r1; r += 8 * R) {
+            float xs[8], ds[8], as[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const long long i = (r + u * R) * C + c; const bool in = r + u * R < r1;
+                xs[u] = in ? ldf<T>(p.x, i) : 0.f; ds[u] = MODE == 1 && in ? ldf<T>(p.da, i) : 0.f; as[u] = MODE == 1 && in && p.add ? ldf<T>(p.add, i) : 0.f;
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                if (r + u * R >= r1) break;
+                const long long i = (r + u * R) * C + c;
+                if (MODE == 0) { const float z = (xs[u] - mean) * istd * g + b; stf<T>(p.a, i, z > 0.f ? z : 0.f); }
+                else {
+                    const float xh = (xs[u] - mean) * istd, dz = xh * g + b > 0.f ? ds[u] : 0.f;
+                    float v = g * istd * (dz - sb - xh * sg);
+                    if (p.add) v += as[u];
+                    stf<T>(p.dx, i, v);
+                }
+            }
+        }
+    }
+}
 template <class T>
 __global__ void __launch_bounds__(256) bn_apply_kernel(const BnProb* __restrict__ probs) {
     const BnProb& p = probs[blockIdx.y];
-    if (p.vec) { bn_stream_vec<0>(p, p.stat); return; }
-    const long long n = p.m * p.C;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(i % p.C);
-        float z = (ldf<T>(p.x, i) - p.stat[c]) * p.stat[p.C + c] * p.gamma[c] + p.beta[c];
-        stf<T>(p.a, i, z > 0.f ? z : 0.f);
-    }
+    if (p.vec) bn_stream_vec<0>(p, p.stat); else bn_stream_scalar<T, 0>(p);
 }
-
 template <class T>
 __global__ void __launch_bounds__(256, 2) bn_bwd_apply_kernel(const BnProb* __restrict__ probs) {
     const BnProb& p = probs[blockIdx.y];
-    if (p.vec) { bn_stream_vec<1>(p, p.stat); return; }
-    const long long n = p.m * p.C;
-    const float inv_m = 1.f / (float)p.m;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(i % p.C);
-        const float istd = p.stat[p.C + c], g = p.gamma[c];
-        const float xh = (ldf<T>(p.x, i) - p.stat[c]) * istd;
-        const float dz = (xh * g + p.beta[c] > 0.f) ? ldf<T>(p.da, i) : 0.f;
-        float v = g * istd * (dz - p.stat[2 * p.C + c] * inv_m - xh * p.stat[3 * p.C + c] * inv_m);
-        if (p.add) v += ldf<T>(p.add, i);
-        stf<T>(p.dx, i, v);
-    }
+    if (p.vec) bn_stream_vec<1>(p, p.stat); else bn_stream_scalar<T, 1>(p);
 }
-
 
 // ------------------------------------------------------------------------------------------------ fused BN+ReLU (cooperative)
 // One launch per BN layer and direction: partial sums per chunk, a grid-wide barrier, then EVERY CTA adds the
@@ -502,7 +524,8 @@ static int stream_grid(K kernel, int& slots, long long n, int nprob) {
         slots = std::max(1, sms * per);
     }
     const long long total = std::max(1ll, (n + 32767) / 32768 * nprob);
-    if (total <= slots) return (int)std::max(1ll, (n + 32767) / 32768);
+    // below one wave the other path gets a CTA per 4096 elements (the vector path's surplus CTAs find no rows and leave)
+    if (total <= slots) return (int)std::max(1ll, std::min<long long>(slots / nprob, (n + 4095) / 4096));
     const long long waves = std::min((total + slots / 2) / slots, std::max(1ll, 2368ll / slots));
     return (int)std::max(1ll, waves * slots / nprob);
 }
