@@ -88,8 +88,8 @@ def test_backward_sums_from_the_data_gradients_tiles(m, shape):
     assert norm_max_abs(da.float().cpu().numpy(), oracle.conv_dgrad(dy, w, (H, W), 1, quant=1)) < BF16_TOL
 
 
-@pytest.mark.parametrize("rows,C", [(1, 64), (65535, 64), (200001, 16), (8192, 24), (8193, 24)])
-def test_bn_passes_at_wave_and_small_layer_edges(m, rows, C):
+@pytest.mark.parametrize("rows,C", [(1, 64), (65535, 64), (200001, 16), (8192, 24), (8193, 24), (9001, 30), (5000, 300), (600, 261), (600, 1100)])
+def test_bn_passes_at_the_edges_of_waves_and_channel_groups(m, rows, C):
     x, da = synth.round_to_bf16(rnd(11, rows, C) * np.float32(1.7) + rnd(12, C)[None, :]), rnd(17, rows, C)
     g, b = (1 + 0.2 * rnd(13, C)).astype(np.float32), (0.3 * rnd(14, C)).astype(np.float32)
     a_ref, mean, invstd = oracle.bn_relu_fwd(x, g, b, quant=1)
