@@ -59,15 +59,6 @@ struct ScratchBlock { char* dev = nullptr; char* host = nullptr; size_t bytes = 
 std::mutex g_scratch_mutex;
 std::vector<ScratchBlock> g_scratch_idle;                     // guarded by the mutex
 
-// Descriptors travel as a kernel's parameters: a copy from pinned memory goes through a copy engine, and the kernel behind it waits
-// for that engine (forward + backward of 65535 x 64: 122 -> 106 us).  Not those with tensor maps: TMA reads them through a path of its own, which
-// a copy is known to keep coherent.
-constexpr int PUT_WORDS = 64;
-struct PutArgs { uint4 v[PUT_WORDS]; };
-__global__ void __launch_bounds__(PUT_WORDS) put_kernel(const __grid_constant__ PutArgs a, uint4* dst, int n) {
-    if ((int)threadIdx.x < n) dst[threadIdx.x] = a.v[threadIdx.x];
-}
-
 void scratch_free(const ScratchBlock& b) { cudaFree(b.dev); cudaFreeHost(b.host); }
 
 struct Scratch {
@@ -94,13 +85,6 @@ struct Scratch {
     // descriptors are laid out in the pinned memory at the offsets they have in the block, then sent as one copy
     void stage(size_t at, const void* what, size_t bytes) { memcpy(b.host + at, what, bytes); staged = std::max(staged, at + bytes); }
     cudaError_t send() { busy = true; return cudaMemcpyAsync(b.dev, b.host, staged, cudaMemcpyHostToDevice, st); }
-    // a descriptor without tensor maps
-    template <class P> cudaError_t send(const P& p) {
-        static_assert(sizeof(P) <= sizeof(PutArgs), "descriptor too large for the parameters");
-        PutArgs a; memcpy(&a, &p, sizeof(P)); busy = true;
-        put_kernel<<<1, PUT_WORDS, 0, st>>>(a, reinterpret_cast<uint4*>(b.dev), (int)((sizeof(P) + 15) / 16));
-        return cudaGetLastError();
-    }
     cudaError_t wait() { const cudaError_t e = cudaStreamSynchronize(st); busy = false; return e; }
     ~Scratch() {
         if (!b.dev) return;
@@ -205,7 +189,9 @@ extern "C" int resist_conv2d(int32_t mode, int32_t dtype, int32_t backend, const
     }
     if (be == 2) filled = mode == CONV_WGRAD ? conv_wgrad_mma_fill(p, 2 * sm, hd.data()) : conv_mma_fill(p, mode, hd.data());
     if (!filled) { g_layer_error = "descriptor set-up failed"; return RESIST_ECUDA; }
-    if (be) { sc.stage(0, &p, sizeof(p)); sc.stage(1024, hd.data(), hd.size()); e = sc.send(); } else e = sc.send(p);
+    sc.stage(0, &p, sizeof(p));
+    if (be) sc.stage(1024, hd.data(), hd.size());
+    e = sc.send();
     if (e == cudaSuccess) {
         if (be == 1 && mode == CONV_WGRAD) launch_conv_wgrad_tc_probs(blob + 1024, 1, conv_wgrad_tc_ctas(hd.data()), conv_wgrad_tc_smem(hd.data()), conv_wgrad_tc_out_elems(hd.data()), st);
         else if (be == 1) {
@@ -246,7 +232,8 @@ extern "C" int resist_bn_relu_forward(int32_t dtype, const void* x, const float*
     if (e != cudaSuccess) { g_layer_error = cudaGetErrorString(e); return RESIST_ENOMEM; }
     char* const blob = sc.b.dev;
     p.partial = (double*)(blob + 1024);
-    e = sc.send(p);
+    sc.stage(0, &p, sizeof(p));
+    e = sc.send();
     if (e == cudaSuccess) {
         launch_bn_stats((BnProb*)blob, 1, p.chunks, C, dtype == RESIST_BF16, st);
         launch_bn_apply((BnProb*)blob, 1, m * C, dtype == RESIST_BF16, st);
@@ -269,7 +256,8 @@ extern "C" int resist_bn_relu_backward(int32_t dtype, const void* x, const void*
     if (e != cudaSuccess) { g_layer_error = cudaGetErrorString(e); return RESIST_ENOMEM; }
     char* const blob = sc.b.dev;
     p.partial = (double*)(blob + 1024);
-    e = sc.send(p);
+    sc.stage(0, &p, sizeof(p));
+    e = sc.send();
     if (e == cudaSuccess) {
         launch_bn_bwd_reduce((BnProb*)blob, 1, p.chunks, C, dtype == RESIST_BF16, st);
         launch_bn_bwd_apply((BnProb*)blob, 1, m * C, dtype == RESIST_BF16, st);
