@@ -141,11 +141,11 @@ constexpr int AGG_CHUNK = 8192;   // elements per CTA of the aggregate kernel (t
 // ---- launchers (kernels_ref.cu; pools, head and im2col: kernels_head.cu)
 void launch_conv_ref(const ConvProb* d, int nprob, int max_tiles, int mode, bool bf16, cudaStream_t s);
 void launch_splitk_reduce(const ConvProb* d, int nprob, int max_elems, cudaStream_t s);
-void launch_bn_stats(const BnProb* d, int nprob, int max_chunks, int max_c, bool bf16, cudaStream_t s);
+void launch_bn_stats(const BnProb* d, int nprob, int max_chunks, int max_c, bool bf16, bool vec, cudaStream_t s);
 void launch_bn_eval_stats(const BnProb* d, int nprob, int max_c, cudaStream_t s);      // mean | 1/std from the running statistics
-void launch_bn_apply(const BnProb* d, int nprob, long long max_elems, bool bf16, cudaStream_t s);
-void launch_bn_bwd_reduce(const BnProb* d, int nprob, int max_chunks, int max_c, bool bf16, cudaStream_t s);
-void launch_bn_bwd_apply(const BnProb* d, int nprob, long long max_elems, bool bf16, cudaStream_t s);
+void launch_bn_apply(const BnProb* d, int nprob, long long max_elems, bool bf16, bool vec, cudaStream_t s);
+void launch_bn_bwd_reduce(const BnProb* d, int nprob, int max_chunks, int max_c, bool bf16, bool vec, cudaStream_t s);
+void launch_bn_bwd_apply(const BnProb* d, int nprob, long long max_elems, bool bf16, bool vec, cudaStream_t s);
 void launch_maxpool_fwd(const PoolProb* d, int nprob, long long max_elems, bool bf16, cudaStream_t s);
 void launch_maxpool_bwd(const PoolProb* d, int nprob, long long max_elems, bool bf16, cudaStream_t s);
 int launch_head_fwd(const HeadProb* d, int nprob, int maxB, int maxC, int max_classes, bool bf16, cudaStream_t s);    // both return the number of kernels

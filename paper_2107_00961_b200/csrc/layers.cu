@@ -235,8 +235,8 @@ extern "C" int resist_bn_relu_forward(int32_t dtype, const void* x, const float*
     sc.stage(0, &p, sizeof(p));
     e = sc.send();
     if (e == cudaSuccess) {
-        launch_bn_stats((BnProb*)blob, 1, p.chunks, C, dtype == RESIST_BF16, st);
-        launch_bn_apply((BnProb*)blob, 1, m * C, dtype == RESIST_BF16, st);
+        launch_bn_stats((BnProb*)blob, 1, p.chunks, C, dtype == RESIST_BF16, p.vec != 0, st);
+        launch_bn_apply((BnProb*)blob, 1, m * C, dtype == RESIST_BF16, p.vec != 0, st);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = sc.wait();
@@ -259,8 +259,8 @@ extern "C" int resist_bn_relu_backward(int32_t dtype, const void* x, const void*
     sc.stage(0, &p, sizeof(p));
     e = sc.send();
     if (e == cudaSuccess) {
-        launch_bn_bwd_reduce((BnProb*)blob, 1, p.chunks, C, dtype == RESIST_BF16, st);
-        launch_bn_bwd_apply((BnProb*)blob, 1, m * C, dtype == RESIST_BF16, st);
+        launch_bn_bwd_reduce((BnProb*)blob, 1, p.chunks, C, dtype == RESIST_BF16, p.vec != 0, st);
+        launch_bn_bwd_apply((BnProb*)blob, 1, m * C, dtype == RESIST_BF16, p.vec != 0, st);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = sc.wait();
@@ -341,8 +341,8 @@ extern "C" int resist_conv2d_bn_relu(int32_t mode, int32_t backend, const void* 
             for (int i = 0; i < n_tc; ++i) { const char* h = hd.data() + (size_t)i * conv_tc_prob_bytes(); t = std::max(t, conv_tc_tiles(h)); packed = conv_tc_merge(packed, conv_tc_smem(h)); }
             launch_conv_tc_probs(blob + 1024, n_tc, t, packed, st);
             launch_bn_finalize_tiles((BnProb*)blob, 1, bn.C, mode == CONV_FWD ? 0 : 1, st);
-            if (mode == CONV_FWD) launch_bn_apply((BnProb*)blob, 1, bn.m * bn.C, true, st);
-            else launch_bn_bwd_apply((BnProb*)blob, 1, bn.m * bn.C, true, st);
+            if (mode == CONV_FWD) launch_bn_apply((BnProb*)blob, 1, bn.m * bn.C, true, true, st);
+            else launch_bn_bwd_apply((BnProb*)blob, 1, bn.m * bn.C, true, true, st);
         }
         e = cudaGetLastError();
     }

@@ -64,8 +64,8 @@ extern "C" int resist_bn_relu_forward_noalloc(int32_t dtype, const void* x, cons
     // the reduction of this same call, and the descriptor is rewritten here.
     store_descriptor<<<1, 1, 0, st>>>(p);
     const BnProb* d = reinterpret_cast<const BnProb*>(base);
-    launch_bn_stats(d, 1, p.chunks, C, dtype == RESIST_BF16, st);
-    launch_bn_apply(d, 1, m * C, dtype == RESIST_BF16, st);
+    launch_bn_stats(d, 1, p.chunks, C, dtype == RESIST_BF16, p.vec != 0, st);
+    launch_bn_apply(d, 1, m * C, dtype == RESIST_BF16, p.vec != 0, st);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) { g_noalloc_error = std::string("launch failed: ") + cudaGetErrorString(e); return RESIST_ECUDA; }
     return RESIST_OK;

@@ -662,7 +662,7 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
                 case OP_BN_STATS: case OP_BN_APPLY: case OP_BN_BWD_REDUCE: case OP_BN_BWD_APPLY: case OP_BN_FWD_FUSED: case OP_BN_BWD_FUSED: case OP_BN_TILE_STATS: case OP_BN_EVAL_STATS: case OP_BN_FWD_SMALL: case OP_BN_BWD_SMALL: case OP_BN_BWD_TILE_SUMS: {
                     if (k == i) L.first = (int)bn.size();
                     bn.push_back(o.bn);
-                    L.gx = std::max(L.gx, o.bn.chunks); L.max_c = std::max(L.max_c, o.bn.C);
+                    L.gx = std::max(L.gx, o.bn.chunks); L.max_c = std::max(L.max_c, o.bn.C); L.non_vec |= !o.bn.vec;
                     L.max_elems = std::max<long long>(L.max_elems, o.bn.m * o.bn.C);
                     { const double e = (double)o.bn.m * o.bn.C;
                       if (o.kind == OP_BN_TILE_STATS || o.kind == OP_BN_BWD_TILE_SUMS) L.bytes += 8.0 * o.bn.chunks * o.bn.C;
@@ -916,13 +916,13 @@ static int enqueue_launches(resist_ctx* ctx, Plan& plan, bool update, bool overl
                 ++n_launch; break; }
             case OP_SPLITK: launch_splitk_reduce(plan.d_conv + L.first, L.count, (int)L.max_elems, st); ++n_launch; break;
             case OP_REPACK: launch_repack_rows(plan.d_conv + L.first, L.count, (int)L.max_elems, st); ++n_launch; break;
-            case OP_BN_STATS: launch_bn_stats(plan.d_bn + L.first, L.count, L.gx, L.max_c, bf, st); n_launch += 2; break;
+            case OP_BN_STATS: launch_bn_stats(plan.d_bn + L.first, L.count, L.gx, L.max_c, bf, !L.non_vec, st); n_launch += 2; break;
             case OP_BN_FWD_SMALL: launch_bn_small(plan.d_bn + L.first, L.count, L.max_c, 0, bf, st); ++n_launch; break;
             case OP_BN_BWD_SMALL: launch_bn_small(plan.d_bn + L.first, L.count, L.max_c, 1, bf, st); ++n_launch; break;
             case OP_BN_EVAL_STATS: launch_bn_eval_stats(plan.d_bn + L.first, L.count, L.max_c, st); ++n_launch; break;
-            case OP_BN_APPLY: launch_bn_apply(plan.d_bn + L.first, L.count, L.max_elems, bf, st); ++n_launch; break;
-            case OP_BN_BWD_REDUCE: launch_bn_bwd_reduce(plan.d_bn + L.first, L.count, L.gx, L.max_c, bf, st); n_launch += 2; break;
-            case OP_BN_BWD_APPLY: launch_bn_bwd_apply(plan.d_bn + L.first, L.count, L.max_elems, bf, st); ++n_launch; break;
+            case OP_BN_APPLY: launch_bn_apply(plan.d_bn + L.first, L.count, L.max_elems, bf, !L.non_vec, st); ++n_launch; break;
+            case OP_BN_BWD_REDUCE: launch_bn_bwd_reduce(plan.d_bn + L.first, L.count, L.gx, L.max_c, bf, !L.non_vec, st); n_launch += 2; break;
+            case OP_BN_BWD_APPLY: launch_bn_bwd_apply(plan.d_bn + L.first, L.count, L.max_elems, bf, !L.non_vec, st); ++n_launch; break;
             case OP_POOL_FWD: launch_maxpool_fwd(plan.d_pool + L.first, L.count, L.max_elems, bf, st); ++n_launch; break;
             case OP_POOL_BWD: launch_maxpool_bwd(plan.d_pool + L.first, L.count, L.max_elems, bf, st); ++n_launch; break;
             case OP_HEAD_FWD: n_launch += launch_head_fwd(plan.d_head + L.first, L.count, L.max_b, L.max_c, L.max_classes, bf, st); break;
@@ -933,11 +933,11 @@ static int enqueue_launches(resist_ctx* ctx, Plan& plan, bool update, bool overl
             case OP_BN_BWD_TILE_SUMS: launch_bn_finalize_tiles(plan.d_bn + L.first, L.count, L.max_c, 1, st); ++n_launch; break;
             case OP_BN_FWD_FUSED:
                 if (launch_bn_fused(plan.d_bn + L.first, L.count, L.gx, 0, st)) ++n_launch;
-                else { launch_bn_stats(plan.d_bn + L.first, L.count, L.gx, L.max_c, bf, st); launch_bn_apply(plan.d_bn + L.first, L.count, L.max_elems, bf, st); n_launch += 3; }
+                else { launch_bn_stats(plan.d_bn + L.first, L.count, L.gx, L.max_c, bf, !L.non_vec, st); launch_bn_apply(plan.d_bn + L.first, L.count, L.max_elems, bf, !L.non_vec, st); n_launch += 3; }
                 break;
             case OP_BN_BWD_FUSED:
                 if (launch_bn_fused(plan.d_bn + L.first, L.count, L.gx, 1, st)) ++n_launch;
-                else { launch_bn_bwd_reduce(plan.d_bn + L.first, L.count, L.gx, L.max_c, bf, st); launch_bn_bwd_apply(plan.d_bn + L.first, L.count, L.max_elems, bf, st); n_launch += 3; }
+                else { launch_bn_bwd_reduce(plan.d_bn + L.first, L.count, L.gx, L.max_c, bf, !L.non_vec, st); launch_bn_bwd_apply(plan.d_bn + L.first, L.count, L.max_elems, bf, !L.non_vec, st); n_launch += 3; }
                 break;
         }
         pf.end(st);

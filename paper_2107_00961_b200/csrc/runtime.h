@@ -37,6 +37,7 @@ struct Launch {
     OpKind kind; int backend; int first, count;               // range in the typed device array
     int ndesc;                                                // tcgen05 forward / dgrad: descriptors of the launch (a stride-2 dgrad has one per output phase)
     int gx; long long max_elems; int max_b, max_c, max_classes;
+    bool non_vec;                                             // BN: not every problem takes the vector path
     double bytes, flops;                                      // algorithmic work of this launch
     bool join_before;                                         // the main stream first waits for the weight gradients in flight
     int small_ctas, ksz;                                      // CUDA-core convolutions: CTAs per problem of the small-layer kernels (0: not all problems are small)
