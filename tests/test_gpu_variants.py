@@ -185,6 +185,34 @@ def test_recorded_steps_equal_launched_steps(m, dtype, grouped):
             np.testing.assert_array_equal(u, v)
 
 
+@pytest.mark.parametrize("replayed", [0, 1, 4])
+def test_steps_on_different_streams_run_in_the_order_of_the_calls(m, replayed):
+    """Two steps of one sub-ResNet, the first on a stream that is busy for a while: the second waits for it, whether steps are
+    launched, the second is the first to be replayed, or both are replayed.  Same bits as on one stream."""
+    arch = net(16, 16, 10, 16, 16, 0)
+    p0, buf0 = synth.perturbed_params(arch, 4)
+    xs = [to_dev(rnd(60 + i, 12, 16, 16, 3), torch.bfloat16) for i in range(2)]
+    ys = [to_dev((synth.splitmix64_words(70 + i, 12) % np.uint64(10)).astype(np.int32), None) for i in range(2)]
+    got = []
+    for streams in (1, 2):
+        ctx = m.Context(arch.to_int32(), dtype=m.BF16)
+        ctx.set_params(p0, buf0)
+        ctx.partition(5, 2)
+        for _ in range(replayed):
+            ctx.local_step(0, xs[0], ys[0], LR)
+        torch.cuda.synchronize()
+        one = torch.cuda.Stream()
+        two = torch.cuda.Stream() if streams == 2 else one
+        with torch.cuda.stream(one):
+            torch.cuda._sleep(40_000_000)                        # about 20 ms
+        ctx.local_step(0, xs[0], ys[0], LR, stream=one)
+        ctx.local_step(0, xs[1], ys[1], 3 * LR, stream=two)
+        torch.cuda.synchronize()
+        got.append(ctx.get_params(0))
+    for u, v in zip(*got):
+        np.testing.assert_array_equal(u, v)
+
+
 # BN in the epilogues of evaluation's convolutions, three calls so that the recorded form runs too: warp-level layers, tcgen05 layers with more than
 # one slab and column tile, the pooled stem; 1 image, a ragged batch and one that fills several waves of tiles
 @pytest.mark.parametrize("kind,width,pool", [(synth.BASIC, 16, 0), (synth.BOTTLENECK, 64, 0), (synth.BOTTLENECK, 64, 1)])
