@@ -851,6 +851,7 @@ static int ensure_streams(resist_ctx* ctx) {
     if (!ctx->side_stream) {
         if (cudaStreamCreateWithFlags(&ctx->side_stream, cudaStreamNonBlocking) != cudaSuccess ||
             cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
+            cudaEventCreateWithFlags(&ctx->ev_eval, cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&ctx->ev_side_done, cudaEventDisableTiming) != cudaSuccess) { ctx->err = "cannot create the second stream"; return RESIST_ECUDA; }
     }
     return RESIST_OK;
@@ -1047,7 +1048,12 @@ int resist_eval(resist_ctx* ctx, const void* images, const int32_t* labels, int3
     if (!ctx) return RESIST_EINVAL;
     if (!images || B < 1 || B > 1024) { ctx->err = "need images and 1 <= B <= 1024"; return RESIST_EINVAL; }
     cudaStream_t st = (cudaStream_t)stream;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError(); ctx->err = "an evaluation cannot be part of a caller's graph"; return RESIST_ECUDA; }
     int rc = ensure_param_arrays(ctx, std::max(ctx->S_cap, 1));
+    if (rc) return rc;
+    rc = ensure_streams(ctx);
     if (rc) return rc;
     const int copy = ctx->S_cap;                               // the evaluation copy sits after the working copies
     const int S = std::max(ctx->S, 1);
@@ -1075,6 +1081,8 @@ int resist_eval(resist_ctx* ctx, const void* images, const int32_t* labels, int3
     const resist_step_info keep = ctx->info;
     rc = run_plan(ctx, plan, pa, false, 0.f, st);
     ctx->info = keep;
+    // it reads the global arrays in place: the next aggregate, whatever its stream, overwrites them only afterwards
+    if (cudaEventRecord(ctx->ev_eval, st) != cudaSuccess && rc == RESIST_OK) { cudaGetLastError(); ctx->err = "cannot record the end of the evaluation"; rc = RESIST_ECUDA; }
     return rc;
 }
 

@@ -215,7 +215,7 @@ int resist_destroy(resist_ctx* ctx) {
     for (Plan& p : ctx->plans) free_plan(ctx, p);
     ctx_free(ctx, ctx->d_param_blob); ctx_free(ctx, ctx->pa.global); ctx_free(ctx, ctx->d_ws); ctx_free(ctx, ctx->d_eval_ws);
     ctx_free(ctx, ctx->d_seg);
-    if (ctx->side_stream) { cudaStreamDestroy(ctx->side_stream); cudaEventDestroy(ctx->ev_fork); cudaEventDestroy(ctx->ev_side_done); }
+    if (ctx->side_stream) { cudaStreamDestroy(ctx->side_stream); cudaEventDestroy(ctx->ev_fork); cudaEventDestroy(ctx->ev_side_done); cudaEventDestroy(ctx->ev_eval); }
     if (ctx->main_stream) { cudaStreamDestroy(ctx->main_stream); cudaEventDestroy(ctx->ev_enter); cudaEventDestroy(ctx->ev_leave); }
     delete ctx;
     return RESIST_OK;
@@ -389,6 +389,7 @@ int resist_aggregate(resist_ctx* ctx, resist_stream stream) {
     CK(cudaMemcpyAsync(ctx->d_seg, segs.data(), segs.size() * sizeof(Segment), cudaMemcpyHostToDevice, st));
     double rd = 0, wr = 0;
     for (const Segment& g : segs) { rd += (double)g.len * __builtin_popcount(g.mask); wr += (double)g.len; }
+    if (ctx->ev_eval) CK(cudaStreamWaitEvent(st, ctx->ev_eval, 0));   // an evaluation in flight on another stream still reads what is overwritten here
     ctx->prof.begin(PK_AGGREGATE, 1, 4.0 * (rd + wr), 0, st);
     const AggArrays arr{ctx->pa.w, ctx->pa.buf, ctx->pa.n, ctx->pa.nbuf, ctx->pa.global, ctx->pa.global_buf};
     launch_aggregate(ctx->d_seg, (int)segs.size(), bchunks, arr, S, st);

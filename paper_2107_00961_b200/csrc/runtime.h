@@ -121,5 +121,6 @@ struct resist_ctx {
     // while they overlap, the main chain of the step runs on a stream of the library's own with the highest priority
     // (forked from and joined to the caller's stream), so that its CTAs are placed before those of the weight gradients
     cudaStream_t main_stream = nullptr; cudaEvent_t ev_enter = nullptr, ev_leave = nullptr;
+    cudaEvent_t ev_eval = nullptr;                             // end of the last evaluation's reads of the global parameters
     std::string err;
 };

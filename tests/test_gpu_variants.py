@@ -213,6 +213,50 @@ def test_steps_on_different_streams_run_in_the_order_of_the_calls(m, replayed):
         np.testing.assert_array_equal(u, v)
 
 
+@pytest.mark.parametrize("calls", [0, 3])
+def test_an_evaluation_sees_the_parameters_of_its_call(m, calls):
+    """Its stream is busy when it is called, and the next aggregate comes on another stream: launched and replayed evaluations alike
+    return what they would have returned alone."""
+    arch = net(16, 16, 10, 16, 16, 0)
+    p0, buf0 = synth.perturbed_params(arch, 4)
+    ctx = m.Context(arch.to_int32(), dtype=m.BF16)
+    ctx.set_params(p0, buf0)
+    ctx.partition(5, 2)
+    x, y = to_dev(rnd(60, 12, 16, 16, 3), torch.bfloat16), to_dev((synth.splitmix64_words(70, 12) % np.uint64(10)).astype(np.int32), None)
+    ref = ctx.eval(x, y)[0].cpu()
+    for _ in range(calls):
+        ctx.eval(x, y)
+    ctx.local_step(0, x, y, 30 * LR)
+    torch.cuda.synchronize()
+    one, two = torch.cuda.Stream(), torch.cuda.Stream()
+    with torch.cuda.stream(one):
+        torch.cuda._sleep(40_000_000)                            # about 20 ms
+        logits = ctx.eval(x, y, stream=one)[0]
+    ctx.aggregate(stream=two)
+    torch.cuda.synchronize()
+    assert torch.equal(logits.cpu(), ref)
+    assert not torch.equal(ctx.eval(x, y)[0].cpu(), ref)
+
+
+def test_an_evaluation_is_refused_while_the_callers_stream_is_recorded(m):
+    """Its plan and workspace do not live as long as the caller's graph would.  The recording itself goes on."""
+    arch = net(8, 8, 10, 16, 16, 0)
+    ctx = m.Context(arch.to_int32(), dtype=m.BF16)
+    x = to_dev(rnd(60, 4, 8, 8, 3), torch.bfloat16)
+    ref = ctx.eval(x)[0].cpu()
+    t = torch.ones(8, device="cuda")
+    st, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=st):
+        t.mul_(2)
+        with pytest.raises(m.ResistError, match="graph"):
+            ctx.eval(x, stream=st)
+        t.add_(1)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert t.cpu().tolist() == [3.0] * 8
+    assert torch.equal(ctx.eval(x)[0].cpu(), ref)
+
+
 # BN in the epilogues of evaluation's convolutions, three calls so that the recorded form runs too: warp-level layers, tcgen05 layers with more than
 # one slab and column tile, the pooled stem; 1 image, a ragged batch and one that fills several waves of tiles
 @pytest.mark.parametrize("kind,width,pool", [(synth.BASIC, 16, 0), (synth.BOTTLENECK, 64, 0), (synth.BOTTLENECK, 64, 1)])
