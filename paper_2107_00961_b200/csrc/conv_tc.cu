@@ -206,7 +206,6 @@ struct TcHot {                // everything the kernel's loops read: each role k
     int red, slabs;                          // reduction channels, 64-channel slabs
     int b_mn_major;                          // 0: forward (weights K-major); 1: dgrad (weights MN-major)
     int b_bytes;                             // bytes of one weight tile (one slab, one tap)
-    int b_total;                             // bytes of all weight tiles of one column tile, each rounded up to 1 KB
     int out_slabs;                           // 64-column slabs of the output tile
     int total_pos;
     float scale;
@@ -1081,14 +1080,45 @@ static bool tc_shape_ok(const ConvProb& p) {
     return true;
 }
 
+// The window of a forward / dgrad tile: its tall map, the positions before the tile's first (hb) and the boxes that cover it.  "flat": one
+// box of 128 pixels of a dense problem.
+struct TcWindow { bool flat; Tall g; int hb, nbox; size_t bytes; };
+static bool tc_window(const ConvProb& p, int mode, TcWindow& w) {
+    w.flat = p.ksz == 1 && (p.stride == 1 || mode == CONV_DGRAD); w.hb = 0; w.nbox = 1; w.bytes = SLAB_BYTES;
+    if (w.flat) return true;
+    const bool s2 = p.stride == 2; const int pad = p.ksz == 3 ? 1 : 0;
+    if (!tall_of(s2 ? p.P : p.H, s2 ? p.Q : p.W, pad, s2 && mode == CONV_FWD ? 2 : 1, w.g)) return false;
+    int span = TILE_M;
+    if (pad && !s2) { w.hb = w.g.Wp + 1; span += 2 * w.hb; }
+    else if (pad && mode == CONV_FWD) { w.hb = w.g.Wp + 1; span += w.hb; }
+    else if (pad) span += w.g.Wp + 1;                            // one output phase of a stride-2 dgrad
+    w.nbox = boxes_for(span, w.g.box_pos); w.bytes = ((size_t)w.nbox * w.g.box_bytes + 1023) / 1024 * 1024;
+    return true;
+}
+
+constexpr size_t TC_SMEM_BUDGET = 204 * 1024;
+static size_t tc_budget(bool dgrad) { return dgrad ? TC_SMEM_BUDGET - 8 * 1024 : TC_SMEM_BUDGET; }      // dgrad keeps 8 KB of BN constants beside the rings
+static int tc_weight_tile(int n, int mode) { return mode == CONV_FWD ? n * 128 : ((n + 63) / 64) * 8192; }
+// The least a launch runs with: the two windows of a pair of tiles, one weight tile of n columns and a slab buffer per epilogue group, another
+// one per group when a BN of the output (evaluation) leaves through it.
+static bool tc_fits(size_t window, int n, int mode, bool bn) {
+    return 2 * window + ((size_t)tc_weight_tile(n, mode) + 1023) / 1024 * 1024 + 2 * (bn ? 2 : 1) * (size_t)SLAB_BYTES <= tc_budget(mode == CONV_DGRAD);
+}
+static int tc_narrowest(int ncol) { return std::min(64, (ncol + 15) / 16 * 16); }
+static int tc_columns(const ConvProb& p, int mode) { return mode == CONV_FWD ? p.K : p.C; }
+
 // Number of TcProb descriptors a forward / dgrad problem needs (0: not supported): one, or one per output phase of a stride-2 3x3 dgrad.
+// Maps so wide that two windows do not fit (3x3: about 120 positions and up) are left to the other kernel families.
 int conv_tc_count(const ConvProb& p, int mode) {
     if (mode == CONV_WGRAD || !encode_fn() || !tc_shape_ok(p)) return 0;
     if (((uintptr_t)p.act | (uintptr_t)p.wgt | (uintptr_t)p.out | (uintptr_t)p.add) & 15) return 0;
-    Tall t;
-    if (p.ksz == 3 && !tall_of(p.stride == 2 ? p.P : p.H, p.stride == 2 ? p.Q : p.W, 1, mode == CONV_FWD ? p.stride : 1, t)) return 0;
-    if (p.ksz == 1 && p.stride == 2 && mode == CONV_FWD && !tall_of(p.P, p.Q, 0, 2, t)) return 0;
+    TcWindow w;
+    if (!tc_window(p, mode, w) || !tc_fits(w.bytes, tc_narrowest(tc_columns(p, mode)), mode, p.bn_out != nullptr)) return 0;
     return (mode == CONV_DGRAD && p.ksz == 3 && p.stride == 2) ? 4 : 1;
+}
+// evaluation: is there room for the BN of the output in the epilogue?
+bool conv_tc_bn_fits(const ConvProb& p) {
+    TcWindow w; return tc_window(p, CONV_FWD, w) && tc_fits(w.bytes, tc_narrowest(p.K), CONV_FWD, true);
 }
 bool conv_tc_supported(const ConvProb& p, int mode) { return conv_tc_count(p, mode) > 0; }
 // 128-position tiles of a forward problem (the rows of ConvProb::stat_tiles)
@@ -1127,14 +1157,14 @@ int conv_tc_read_status() {
 // MMAs when two accumulators per tile fit TMEM (up to 128 columns).  Narrower tiles read every window once more, so they have to promise
 // 12 %, and from two full waves of the widest tiles on there is nothing to fill.  (50 images of 14 x 14 x 256, 3x3: 88 tiles of 256
 // columns are 88 busy SMs of 148; 74 -> 63 us for the layer call.  Evaluation of 50 ImageNet-shaped images 2.19 -> 1.95 ms.)
-static void pick_n_tile(TcHot& t, int ntaps, int group, int phases) {
+static void pick_n_tile(TcHot& t, int ntaps, int group, int phases, int mode, bool bn) {
     const int sms = device_sms();
     double best = 0; int best_n = 0; long long wide_pairs = 0;
     const int first = (t.ncol + 255) / 256;
     for (int tn = first; tn <= std::max(first, (t.ncol + 63) / 64); ++tn) {
         int n = (t.ncol + tn - 1) / tn;
         n = tn > 1 ? (n + 63) / 64 * 64 : (n + 15) / 16 * 16;
-        if ((t.ncol + n - 1) / n != tn) continue;
+        if ((t.ncol + n - 1) / n != tn || !tc_fits(((size_t)t.nbox * t.a_box_bytes + 1023) / 1024 * 1024, n, mode, bn)) continue;
         const double mma = n > 128 ? n / 2.0 : n > 64 ? 68 : 52, steps = (double)ntaps * t.slabs * std::min(4, (t.red + 15) / 16);
         const double epi = 20.0 * n + 500, a_bytes = (double)t.slabs * t.ngroups * t.nbox * t.a_box_bytes, b_bytes = (double)t.slabs * ntaps * n * 128;
         auto unit = [&](int tiles) {
@@ -1153,9 +1183,11 @@ static void pick_n_tile(TcHot& t, int ntaps, int group, int phases) {
 // Fills conv_tc_count() host-side TcProbs for this problem.  Returns the number written (0: not supported or encoding failed).
 int conv_tc_fill(const ConvProb& p, int mode, void* host_tc) {
     const int count = conv_tc_count(p, mode);
-    if (!count) return 0;
+    TcWindow win;
+    if (!count || !tc_window(p, mode, win)) return 0;
+    const Tall& g = win.g;
     const int taps = p.ksz * p.ksz;
-    const int chan_a = mode == CONV_FWD ? p.C : p.K, ncol = mode == CONV_FWD ? p.K : p.C;
+    const int chan_a = mode == CONV_FWD ? p.C : p.K, ncol = tc_columns(p, mode);
     for (int ph = 0; ph < count; ++ph) {
         TcProb tp; memset(&tp, 0, sizeof(tp)); TcHot& t = tp.h;
         t.add = (const __nv_bfloat16*)p.add; t.out = (__nv_bfloat16*)p.out; t.status = conv_tc_status_word();
@@ -1166,7 +1198,7 @@ int conv_tc_fill(const ConvProb& p, int mode, void* host_tc) {
         t.es = 1; t.pad = 0; t.os = 1; t.oy = 0; t.ox = 0; t.ngroups = 1; t.gbeg[0] = 0;
         const void* act = p.act;
         long long out_pixels = 0;
-        if (p.ksz == 1 && (p.stride == 1 || mode == CONV_DGRAD)) {
+        if (win.flat) {
             // plain GEMM over the pixels of the operand: forward at stride 1, dgrad at either stride (stride 2: over the P x Q pixels of dy)
             const int Hg = mode == CONV_DGRAD ? p.P : p.H, Wg = mode == CONV_DGRAD ? p.Q : p.W;
             t.a_flat = 1; t.Hp = Hg; t.Wp = Wg; t.R = 0; t.box_pos = TILE_M; t.nbox = 1; t.hb = 0; t.a_box_bytes = SLAB_BYTES;
@@ -1177,24 +1209,21 @@ int conv_tc_fill(const ConvProb& p, int mode, void* host_tc) {
             else { t.dense = 1; t.OH = Hg; t.OW = Wg; out_pixels = t.total_pos; }
         } else if (p.ksz == 1) {
             // forward of a stride-2 1x1 layer: the positions are the output pixels, the window gathers every second input pixel
-            Tall g; if (!tall_of(p.P, p.Q, 0, 2, g)) return 0;
-            t.a_flat = 0; t.dense = 1; t.es = 2; t.Hp = g.Hp; t.Wp = g.Wp; t.R = g.R; t.box_pos = g.box_pos; t.a_box_bytes = g.box_bytes; t.hb = 0;
-            t.nbox = boxes_for(TILE_M, g.box_pos); t.total_pos = p.N * g.Hp * g.Wp; t.OH = p.P; t.OW = p.Q; out_pixels = t.total_pos;
+            t.a_flat = 0; t.dense = 1; t.es = 2; t.Hp = g.Hp; t.Wp = g.Wp; t.R = g.R; t.box_pos = g.box_pos; t.a_box_bytes = g.box_bytes; t.hb = win.hb; t.nbox = win.nbox;
+            t.total_pos = p.N * g.Hp * g.Wp; t.OH = p.P; t.OW = p.Q; out_pixels = t.total_pos;
             { const int ti_ = 0; t.wtap[ti_] = 0; t.shift[ti_] = 0; } t.gbeg[1] = 1;
             if (!encode_tall(&tp.map_a, act, chan_a, p.N, p.H, p.W, g.Wp, g.box_h, g.box_n, 2)) return 0;
         } else if (p.stride == 1) {
             // 3x3 at stride 1: one window, nine taps; dgrad walks the taps mirrored
-            Tall g; if (!tall_of(p.H, p.W, 1, 1, g)) return 0;
-            t.a_flat = 0; t.dense = 0; t.pad = 1; t.Hp = g.Hp; t.Wp = g.Wp; t.R = g.R; t.box_pos = g.box_pos; t.a_box_bytes = g.box_bytes; t.hb = g.Wp + 1;
-            t.nbox = boxes_for(TILE_M + 2 * t.hb, g.box_pos); t.total_pos = p.N * g.Hp * g.Wp; t.OH = p.H; t.OW = p.W; out_pixels = (long long)p.N * p.H * p.W;
+            t.a_flat = 0; t.dense = 0; t.pad = 1; t.Hp = g.Hp; t.Wp = g.Wp; t.R = g.R; t.box_pos = g.box_pos; t.a_box_bytes = g.box_bytes; t.hb = win.hb; t.nbox = win.nbox;
+            t.total_pos = p.N * g.Hp * g.Wp; t.OH = p.H; t.OW = p.W; out_pixels = (long long)p.N * p.H * p.W;
             for (int w = 0; w < 9; ++w) { const int ti_ = w; t.wtap[ti_] = mode == CONV_DGRAD ? 8 - w : w; t.shift[ti_] = (w / 3) * g.Wp + (w % 3); }
             t.gbeg[1] = 9;
             if (!encode_tall(&tp.map_a, act, chan_a, p.N, p.H, p.W, g.Wp, g.box_h, g.box_n, 1)) return 0;
         } else if (mode == CONV_FWD) {
             // 3x3 at stride 2, forward: positions over the P x Q outputs, one window per input parity phase (element-strided fetch)
-            Tall g; if (!tall_of(p.P, p.Q, 1, 2, g)) return 0;
-            t.a_flat = 0; t.dense = 0; t.pad = 1; t.es = 2; t.Hp = g.Hp; t.Wp = g.Wp; t.R = g.R; t.box_pos = g.box_pos; t.a_box_bytes = g.box_bytes; t.hb = g.Wp + 1;
-            t.nbox = boxes_for(TILE_M + t.hb, g.box_pos); t.total_pos = p.N * g.Hp * g.Wp; t.OH = p.P; t.OW = p.Q; out_pixels = (long long)p.N * p.P * p.Q;
+            t.a_flat = 0; t.dense = 0; t.pad = 1; t.es = 2; t.Hp = g.Hp; t.Wp = g.Wp; t.R = g.R; t.box_pos = g.box_pos; t.a_box_bytes = g.box_bytes; t.hb = win.hb; t.nbox = win.nbox;
+            t.total_pos = p.N * g.Hp * g.Wp; t.OH = p.P; t.OW = p.Q; out_pixels = (long long)p.N * p.P * p.Q;
             int n = 0; t.ngroups = 0;
             for (int u = 0; u < 2; ++u) for (int v = 0; v < 2; ++v) {
                 int rs[4][2]; const int k = phase_taps(u, v, rs);
@@ -1210,9 +1239,8 @@ int conv_tc_fill(const ConvProb& p, int mode, void* host_tc) {
             // 3x3 at stride 2, dgrad: one problem per output parity phase (u, v), positions over the P x Q grid of dy; input row 2i + u
             // takes dy row i + (u + 1 - r) / 2 through tap r
             const int u = ph >> 1, v = ph & 1;
-            Tall g; if (!tall_of(p.P, p.Q, 1, 1, g)) return 0;
-            t.a_flat = 0; t.dense = 0; t.pad = 1; t.Hp = g.Hp; t.Wp = g.Wp; t.R = g.R; t.box_pos = g.box_pos; t.a_box_bytes = g.box_bytes; t.hb = 0;
-            t.nbox = boxes_for(TILE_M + g.Wp + 1, g.box_pos); t.total_pos = p.N * g.Hp * g.Wp;
+            t.a_flat = 0; t.dense = 0; t.pad = 1; t.Hp = g.Hp; t.Wp = g.Wp; t.R = g.R; t.box_pos = g.box_pos; t.a_box_bytes = g.box_bytes; t.hb = win.hb; t.nbox = win.nbox;
+            t.total_pos = p.N * g.Hp * g.Wp;
             t.OH = p.H; t.OW = p.W; t.os = 2; t.oy = u; t.ox = v; out_pixels = (long long)p.N * p.H * p.W;
             int rs[4][2]; const int k = phase_taps(u, v, rs);
             for (int i = 0; i < k; ++i) { const int ti_ = i; t.wtap[ti_] = rs[i][0] * 3 + rs[i][1]; t.shift[ti_] = ((u + 1 - rs[i][0]) / 2) * g.Wp + (v + 1 - rs[i][1]) / 2; }
@@ -1222,14 +1250,11 @@ int conv_tc_fill(const ConvProb& p, int mode, void* host_tc) {
         // residual
         t.add_mode = !p.add ? 0 : p.add_sub == 2 ? 3 : 2;
         const int ntaps = t.gbeg[t.ngroups];
-        auto b_tile = [&](int nt) { return mode == CONV_FWD ? nt * 128 : ((nt + 63) / 64) * 8192; };
-        auto b_total = [&](int nt) { return (size_t)t.slabs * ntaps * ((b_tile(nt) + 1023) / 1024 * 1024); };
         t.tiles_m = (t.total_pos + TILE_M - 1) / TILE_M;
         if (t.stat_tiles) t.stat_tiles += (long long)ph * t.tiles_m * 2 * ncol;        // one run of tiles per output phase
-        pick_n_tile(t, ntaps, p.group > 0 ? p.group : 1, count);
+        pick_n_tile(t, ntaps, p.group > 0 ? p.group : 1, count, mode, p.bn_out != nullptr);
         t.out_slabs = (t.n_tile + 63) / 64;
-        t.b_bytes = b_tile(t.n_tile);
-        t.b_total = (int)b_total(t.n_tile);
+        t.b_bytes = tc_weight_tile(t.n_tile, mode);
         // weights [K][taps][C] viewed as (C, tap, K).  Forward: a tile is n_tile output channels (rows) x 64 input channels.
         // dgrad: a block is 64 reduction channels k (rows) x 64 output columns c.
         { const uint64_t dims[3] = {(uint64_t)p.C, (uint64_t)taps, (uint64_t)p.K};
@@ -1251,42 +1276,29 @@ size_t conv_tc_prob_bytes() { return sizeof(TcProb); }
 // units of work of a problem: pairs of row tiles x column tiles
 int conv_tc_tiles(const void* host_tc) { const TcHot* t = &((const TcProb*)host_tc)->h; return ((t->tiles_m + 1) / 2) * t->tiles_n; }
 // packs what a launch has to know about its largest problem into one number: window KB (12 bits), weight-tile KB (12), flags
-// (4; 1: residual through TMA, 2: BN of the output, 4: dgrad), KB of all weight tiles of a column tile (16), MMA N (20)
+// (4; 1: residual through TMA, 2: BN of the output, 4: dgrad), MMA N (36)
 size_t conv_tc_smem(const void* host_tc) {
     const TcHot* t = &((const TcProb*)host_tc)->h;
     const size_t a_stage = ((size_t)t->nbox * t->a_box_bytes + 1023) / 1024, b_stage = ((size_t)t->b_bytes + 1023) / 1024;
-    return (a_stage << 52) | (b_stage << 40) | ((size_t)((t->res_tma ? 1 : 0) | (t->bn_out ? 2 : 0) | (t->b_mn_major ? 4 : 0)) << 36) | ((size_t)std::min(t->b_total / 1024, 0xFFFF) << 20) | (size_t)t->n_tile;
+    return (a_stage << 52) | (b_stage << 40) | ((size_t)((t->res_tma ? 1 : 0) | (t->bn_out ? 2 : 0) | (t->b_mn_major ? 4 : 0)) << 36) | (size_t)t->n_tile;
 }
 // field-wise maximum of two packed values
 size_t conv_tc_merge(size_t a, size_t b) {
     return (std::max(a >> 52, b >> 52) << 52) | (std::max((a >> 40) & 0xFFF, (b >> 40) & 0xFFF) << 40) | ((((a >> 36) | (b >> 36)) & 0xF) << 36) |
-           (std::max((a >> 20) & 0xFFFF, (b >> 20) & 0xFFFF) << 20) | std::max(a & 0xFFFFF, b & 0xFFFFF);
+           std::max(a & 0xFFFFFFFFF, b & 0xFFFFFFFFF);
 }
 
-constexpr size_t TC_SMEM_BUDGET = 204 * 1024;
-
-// total_tiles: an upper bound of the tiles of all problems of the launch (max_tiles * nprob); packed: conv_tc_merge over its problems
-// pdl: programmatic launch.  For evaluation, a chain of convolutions; in training the linked launches made the steps slower (ImageNet-shaped
-// 22.6 -> 24.4 ms with the forward half linked): between the convolutions run streaming kernels that want the whole SM.
-void launch_conv_tc_probs(const void* d_tc, int nprob, int max_tiles, size_t packed, cudaStream_t s, bool pdl) {
-    static bool configured = false; static int sms = 0;
-    if (!configured) {
-        cudaFuncSetAttribute(conv_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(TC_SMEM_BUDGET + 1024));
-        cudaFuncSetAttribute(conv_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(TC_SMEM_BUDGET - 8 * 1024 + 1024));
-        int dev = 0; cudaGetDevice(&dev); cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        configured = true;
-    }
-    TcLaunch L{};
-    L.nprob = nprob;
+// Shared memory and tensor memory of a launch; returns the dynamic shared memory (tc_fits says which problems get here).
+static size_t tc_layout(size_t packed, TcLaunch& L) {
     L.a_stage = (int)(packed >> 52) * 1024; L.b_stage = (int)((packed >> 40) & 0xFFF) * 1024;
-    const int n_tile = (int)(packed & 0xFFFFF);
+    const int n_tile = (int)(packed & 0xFFFFFFFFF);
     // Shared memory.  Two epilogue groups of L.eb 16 KB slab buffers: a residual is fetched into them ahead of its use and wants three
     // (one being added to, one being stored, one in flight), else two; a BN of the output takes one more per group.  A layer runs at the
     // bytes it keeps in flight.  1x1 layers: four windows (two pairs of tiles), then weight tiles.  3x3 layers read a window nine times,
     // so it is the weight tiles that stream: one slab buffer per group, two windows, four weight tiles, then more windows (measured
     // at 128 channels on 16 x 16 maps, 1024 images: 148 us with two weight tiles and four windows, 125 us with four and three).
     const size_t a = (size_t)L.a_stage, b = (size_t)L.b_stage;
-    const size_t budget = (packed >> 36) & 4 ? TC_SMEM_BUDGET - 8 * 1024 : TC_SMEM_BUDGET;      // dgrad keeps 8 KB of BN constants beside the rings
+    const size_t budget = tc_budget((packed >> 36) & 4);
     const int flags = (int)((packed >> 36) & 0xF), extra = flags & 2 ? 1 : 0;
     L.groups = 2; L.res = flags & 1;
     auto staging = [&] { return (size_t)L.groups * (L.eb + extra) * SLAB_BYTES; };
@@ -1308,13 +1320,30 @@ void launch_conv_tc_probs(const void* d_tc, int nprob, int max_tiles, size_t pac
     L.nbuf = L.acc_stride <= 128 ? 2 : 1;
     L.tmem_cols = 32; while (L.tmem_cols < 2 * L.nbuf * L.acc_stride) L.tmem_cols *= 2;
     // at least 120 KB of shared memory so that two CTAs that allocate tensor memory never share an SM
-    const size_t smem = std::max((size_t)L.na * a + (size_t)L.nb * b + staging(), (size_t)120 * 1024) + 1024;
+    return std::max((size_t)L.na * a + (size_t)L.nb * b + staging(), (size_t)120 * 1024) + 1024;
+}
+
+// total_tiles: an upper bound of the tiles of all problems of the launch (max_tiles * nprob); packed: conv_tc_merge over its problems
+// pdl: programmatic launch.  For evaluation, a chain of convolutions; in training the linked launches made the steps slower (ImageNet-shaped
+// 22.6 -> 24.4 ms with the forward half linked): between the convolutions run streaming kernels that want the whole SM.
+void launch_conv_tc_probs(const void* d_tc, int nprob, int max_tiles, size_t packed, cudaStream_t s, bool pdl) {
+    static bool configured = false; static int sms = 0;
+    if (!configured) {
+        cudaFuncSetAttribute(conv_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(tc_budget(false) + 1024));
+        cudaFuncSetAttribute(conv_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(tc_budget(true) + 1024));
+        int dev = 0; cudaGetDevice(&dev); cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        configured = true;
+    }
+    TcLaunch L{};
+    L.nprob = nprob;
+    const size_t smem = tc_layout(packed, L);
+    const bool dgrad = (packed >> 36) & 4;
     const long long total = (long long)max_tiles * nprob;
     const int grid = (int)std::max(1ll, std::min(total, (long long)sms));
     cudaLaunchConfig_t cfg = {}; cfg.gridDim = dim3(grid); cfg.blockDim = dim3(TC_CONV_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = s;
     cudaLaunchAttribute at[1]; at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization; at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at; cfg.numAttrs = pdl ? 1 : 0;
-    cudaLaunchKernelEx(&cfg, flags & 4 ? conv_tc_kernel<true> : conv_tc_kernel<false>, (const TcProb*)d_tc, (const TcLaunch)L);
+    cudaLaunchKernelEx(&cfg, dgrad ? conv_tc_kernel<true> : conv_tc_kernel<false>, (const TcProb*)d_tc, (const TcLaunch)L);
 }
 
 // ---- wgrad host side

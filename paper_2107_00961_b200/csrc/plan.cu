@@ -21,6 +21,7 @@ int conv_tc_stat_tiles(const ConvProb& p);
 int bn_fused_capacity(int backward);                                                    // kernels_ref.cu
 void launch_bn_finalize_tiles(const BnProb* d, int nprob, int max_c, int backward, cudaStream_t s);
 int conv_tc_dgrad_tiles(const ConvProb& p);
+bool conv_tc_bn_fits(const ConvProb& p);
 size_t conv_tc_prob_bytes();
 int conv_tc_tiles(const void* host_tc);
 size_t conv_tc_smem(const void* host_tc);
@@ -63,7 +64,9 @@ static int pick_backend(const ConvProb& p, int mode, int group, int target_ctas,
     // 3x3 layers of 64 channels and more run faster on tcgen05, followed by the streaming BN kernels, than on the warp-level MMA kernels
     // with the BN inside, once the launch has enough positions: ResNet-110's 8 x 8 stage at 4 x 128 images 3.44 -> 3.24 ms per step, its
     // evaluation of 1000 images 3.68 -> 3.32 ms; one worker's 84 images alone (5376 positions) 1.28 -> 1.46 ms, so they stay.
-    if (pref == RESIST_CONV_AUTO && p.C >= 64 && p.K >= 64 && p.ksz == 3 && (long long)group * p.N * p.H * p.W >= 24576) want_mma = false;
+    // Only where tcgen05 takes the layer: its two windows do not fit maps of more than about 120 columns.
+    if (pref == RESIST_CONV_AUTO && p.C >= 64 && p.K >= 64 && p.ksz == 3 && (long long)group * p.N * p.H * p.W >= 24576 &&
+        (mode == CONV_WGRAD ? conv_wgrad_tc_supported(p, target_ctas, nullptr) : conv_tc_supported(p, mode))) want_mma = false;
     if (mode == CONV_WGRAD) {
         if (want_mma && conv_wgrad_mma_supported(p, target_ctas, partial_bytes)) return 200 + conv_wgrad_mma_pick_variant(p, target_ctas);
         if (want_tc && conv_wgrad_tc_supported(p, target_ctas, partial_bytes)) return 1;
@@ -286,7 +289,7 @@ struct Builder {
             op.key = EVAL_STATS_KEY; op.kind = OP_BN_EVAL_STATS; ops->push_back(op);
             const int prod = producer >= 0 ? producer : tc_producer;
             if (prod >= 0 && (*ops)[prod].conv.out == x && (*ops)[prod].conv.K == r.c &&
-                (tc_producer >= 0 || (p.vec && conv_mma_can_fuse_bn((*ops)[prod].conv, CONV_FWD, r.c)))) {
+                (tc_producer >= 0 ? conv_tc_bn_fits((*ops)[prod].conv) : p.vec && conv_mma_can_fuse_bn((*ops)[prod].conv, CONV_FWD, r.c))) {
                 ConvProb& c = (*ops)[prod].conv;
                 c.bn_stat = stat; c.bn_gamma = p.gamma; c.bn_beta = p.beta; c.bn_out = a; c.bn_only = x_used ? 0 : 1;
                 return stat;

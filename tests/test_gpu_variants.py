@@ -49,6 +49,8 @@ CONVS = [
     (2, 4, 17, 15, 136, 72, 3, 1), (2, 2, 8, 8, 256, 256, 3, 1), (2, 3, 11, 13, 72, 200, 3, 2),
     # forward and data gradient: one tile, a last wave of single tiles (298 tiles), column tiles narrower than the channels
     (2, 1, 2, 2, 64, 64, 1, 1), (2, 4, 97, 98, 64, 72, 1, 1), (2, 5, 14, 14, 256, 256, 3, 1),
+    # maps so wide that two windows take most of the shared memory (one weight tile, narrower column tiles) or no longer fit (CUDA cores)
+    (2, 1, 3, 112, 64, 256, 3, 1), (2, 1, 3, 119, 72, 136, 3, 1), (2, 1, 3, 125, 64, 64, 3, 1), (2, 1, 3, 200, 64, 64, 3, 1), (2, 1, 5, 240, 64, 128, 3, 2),
 ]
 
 
@@ -211,6 +213,32 @@ def test_steps_on_different_streams_run_in_the_order_of_the_calls(m, replayed):
         got.append(ctx.get_params(0))
     for u, v in zip(*got):
         np.testing.assert_array_equal(u, v)
+
+
+# 64 columns: the BN's slabs fit beside the windows up to 104 positions per row, the windows alone up to 124; 160: 2 x 16 x 160 x 5 images pass
+# the size from which such layers go to tcgen05, which does not take them
+@pytest.mark.parametrize("w,B,backend", [(95, 2, 2), (104, 2, 2), (105, 2, 2), (112, 2, 2), (124, 2, 2), (126, 2, 2), (160, 10, 0)])
+def test_networks_on_wide_maps(m, w, B, backend):
+    """A step and an evaluation against this library's CUDA-core kernels, which transcribe the definitions."""
+    arch = net(16 if B > 2 else 5, w, 10, 64, 64, 0, depth=(2,))
+    p, buf = synth.perturbed_params(arch, 3)
+    x, y = to_dev(rnd(8, B, arch.in_h, w, 3), torch.bfloat16), to_dev((synth.splitmix64_words(9, B) % np.uint64(10)).astype(np.int32), None)
+    got = []
+    for be in (backend, 1):
+        ctx = m.Context(arch.to_int32(), dtype=m.BF16, conv_backend=be)
+        ctx.set_params(p, buf)
+        ctx.partition(1, 1)
+        logits, loss, _ = ctx.eval(x, y)
+        step = torch.zeros(1, device="cuda")
+        ctx.local_step(0, x, y, LR, step)
+        torch.cuda.synchronize()
+        got.append((logits.cpu().numpy(), loss.item(), step.item(), ctx.get_grads(0).astype(np.float64)))
+    # five layers of one-ulp differences, as for evaluation below; the gradients by direction only, as bf16 steps' are (a mask decided the other way)
+    assert norm_max_abs(got[0][0], got[1][0]) < 2e-2
+    for i in (1, 2):
+        assert abs(got[0][i] - got[1][i]) < 2e-2 * max(1.0, abs(got[1][i]))
+    g, h = got[0][3], got[1][3]
+    assert g @ h / (np.linalg.norm(g) * np.linalg.norm(h)) > 0.97
 
 
 @pytest.mark.parametrize("calls", [0, 3])
