@@ -1,11 +1,10 @@
 // Layer-level entry points: one convolution (forward, dgrad or wgrad) or one BN+ReLU (forward, backward)
 // on caller-owned device tensors, run by the same kernels the local step uses.
 #include <algorithm>
-#include <cstring>
-#include <mutex>
 #include <string>
 #include <vector>
 #include "runtime.h"
+#include "scratch.h"
 
 namespace resist {
 bool conv_tc_supported(const ConvProb& p, int mode);
@@ -45,71 +44,7 @@ using namespace resist;
 static thread_local std::string g_layer_error;
 extern "C" const char* resist_layer_last_error(void) { return g_layer_error.c_str(); }
 
-
-// Scratch of the layer-level calls.  cudaMalloc and cudaFree cost 100 to 300 us each (cudaFree also waits for the whole device), many
-// times the kernels of a small layer, so a call borrows a block and hands it back once its work is done (every call
-// synchronises its stream before it returns, so a block handed back is idle).  A block: device scratch plus pinned host memory for
-// the descriptors, which go up in one asynchronous copy.  A borrowed block belongs to one call alone, so any number of threads and
-// streams may be inside the calls.  Idle blocks are kept up to SCRATCH_IDLE_BYTES and SCRATCH_IDLE_BLOCKS over all devices, the rest is
-// freed at once; resist_layer_release_scratch() gives back the idle ones.
-namespace {
-constexpr size_t SCRATCH_IDLE_BYTES = (size_t)256 << 20, SCRATCH_HOST_BYTES = 16384;
-constexpr int SCRATCH_IDLE_BLOCKS = 16;
-struct ScratchBlock { char* dev = nullptr; char* host = nullptr; size_t bytes = 0; int device = -1; };
-std::mutex g_scratch_mutex;
-std::vector<ScratchBlock> g_scratch_idle;                     // guarded by the mutex
-
-void scratch_free(const ScratchBlock& b) { cudaFree(b.dev); cudaFreeHost(b.host); }
-
-struct Scratch {
-    ScratchBlock b;
-    cudaStream_t st; size_t staged = 0; bool busy = false;
-    explicit Scratch(cudaStream_t s) : st(s) {}
-    Scratch(const Scratch&) = delete;
-    cudaError_t take(size_t bytes) {
-        int dev = 0; cudaError_t e = cudaGetDevice(&dev); if (e != cudaSuccess) return e;
-        {
-            std::lock_guard<std::mutex> lock(g_scratch_mutex);
-            int best = -1;
-            for (int i = 0; i < (int)g_scratch_idle.size(); ++i)
-                if (g_scratch_idle[i].device == dev && g_scratch_idle[i].bytes >= bytes && (best < 0 || g_scratch_idle[i].bytes < g_scratch_idle[best].bytes)) best = i;
-            if (best >= 0) { b = g_scratch_idle[best]; g_scratch_idle.erase(g_scratch_idle.begin() + best); return cudaSuccess; }
-        }
-        size_t room = (size_t)1 << 20; while (room < bytes && room < ((size_t)64 << 20)) room *= 2;     // few sizes, so that blocks serve other layers too
-        b.bytes = std::max(room, bytes); b.device = dev;
-        e = cudaMalloc(&b.dev, b.bytes);
-        if (e == cudaSuccess) e = cudaHostAlloc(&b.host, SCRATCH_HOST_BYTES, cudaHostAllocPortable);
-        if (e != cudaSuccess) { cudaFree(b.dev); b = ScratchBlock(); }
-        return e;
-    }
-    // descriptors are laid out in the pinned memory at the offsets they have in the block, then sent as one copy
-    void stage(size_t at, const void* what, size_t bytes) { memcpy(b.host + at, what, bytes); staged = std::max(staged, at + bytes); }
-    cudaError_t send() { busy = true; return cudaMemcpyAsync(b.dev, b.host, staged, cudaMemcpyHostToDevice, st); }
-    cudaError_t wait() { const cudaError_t e = cudaStreamSynchronize(st); busy = false; return e; }
-    ~Scratch() {
-        if (!b.dev) return;
-        if (busy) cudaStreamSynchronize(st);                   // an error path left work in flight
-        std::vector<ScratchBlock> out;
-        {
-            std::lock_guard<std::mutex> lock(g_scratch_mutex);
-            g_scratch_idle.push_back(b);
-            size_t total = 0; for (const ScratchBlock& x : g_scratch_idle) total += x.bytes;
-            while (total > SCRATCH_IDLE_BYTES || (int)g_scratch_idle.size() > SCRATCH_IDLE_BLOCKS) {      // the largest goes first
-                int big = 0; for (int i = 1; i < (int)g_scratch_idle.size(); ++i) if (g_scratch_idle[i].bytes > g_scratch_idle[big].bytes) big = i;
-                total -= g_scratch_idle[big].bytes; out.push_back(g_scratch_idle[big]); g_scratch_idle.erase(g_scratch_idle.begin() + big);
-            }
-        }
-        for (const ScratchBlock& x : out) scratch_free(x);
-    }
-};
-}
-
-extern "C" int resist_layer_release_scratch(void) {
-    std::vector<ScratchBlock> out;
-    { std::lock_guard<std::mutex> lock(g_scratch_mutex); out.swap(g_scratch_idle); }
-    for (const ScratchBlock& x : out) scratch_free(x);
-    return RESIST_OK;
-}
+extern "C" int resist_layer_release_scratch(void) { scratch_release(); return RESIST_OK; }
 
 static int sm_count_of_device() {
     int sm = 148, dev = 0; cudaGetDevice(&dev); cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev); return sm;
