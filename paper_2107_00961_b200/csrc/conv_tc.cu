@@ -25,6 +25,7 @@
 // TMEM and returns.
 #include <cuda.h>
 #include <cstdio>
+#include <climits>
 #include <cstring>
 #include <algorithm>
 #include "internal.h"
@@ -823,7 +824,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) conv_wgrad_tc_kernel(const TcWg
                     for (int w = 0; w < 4096 && !mbar_try(bar_full + 8 * (c % stages), (uint32_t)(c / stages) & 1u); ++w) __nanosleep(64);
         }
     } else if (warp == 1) {
-        // The issuer: every tap of the group into its own accumulator, so each is summed over the positions in order.
+        // The issuer: every tap of the group into its own accumulator, so each is summed over the positions in order.  The last tap of an odd group
+        // has two, for the first and the second 64 positions of every chunk, which the epilogue adds: the tensor core's sums lose a little
+        // with every step of a chain (relative to 64 bits, 128 images of 32 x 32, 1x1 256 -> 64 channels: 5.8e-7 with one chain, 3.3e-7 with two).
         if (elect_one()) {
             // fp32 accumulate, bf16 x bf16, A and B MN-major, N = mma_n, M = 128
             const int mma_n = p.mma_n;
@@ -846,9 +849,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) conv_wgrad_tc_kernel(const TcWg
                 for (int q = 0; q < 4; ++q) {
                     if (q >= ntap) break;
                     const uint32_t d_t = tmem_d + (uint32_t)(q * mma_n), at = a_lo + sh[q];
+                    const bool halves = q == ntap - 1 && (ntap & 1);
+                    const uint32_t d_t2 = halves ? d_t + (uint32_t)mma_n : d_t, acc2 = halves ? acc : 1u;
 #pragma unroll
                     for (int k16 = 0; k16 < 8; ++k16)          // 16 positions = 16 rows of 128 bytes per step
-                        umma_bf16(d_t, f2_pack(dy_lo + 128u * (uint32_t)k16, desc_hi), f2_pack(at + 128u * (uint32_t)k16, desc_hi), idesc, k16 ? 1u : acc);
+                        umma_bf16(k16 < 4 ? d_t : d_t2, f2_pack(dy_lo + 128u * (uint32_t)k16, desc_hi), f2_pack(at + 128u * (uint32_t)k16, desc_hi), idesc, k16 == 0 ? acc : k16 == 4 ? acc2 : 1u);
                 }
                 acc = 1;
                 umma_commit(bar_empty + 8 * s);
@@ -905,6 +910,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1) conv_wgrad_tc_kernel(const TcWg
                     if (nc > 0) {
                         tmem_ld32(tmem_d + ((uint32_t)(quad * 32) << 16) + (uint32_t)(tt * n_tile + c0), v);
                         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                        if ((ntap & 1) && tt == ntap - 1) {      // first half + second half
+                            uint32_t v2[32];
+                            tmem_ld32(tmem_d + ((uint32_t)(quad * 32) << 16) + (uint32_t)(ntap * n_tile + c0), v2);
+                            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                            for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + __uint_as_float(v2[j]));
+                        }
                     } else { for (int j = 0; j < 32; ++j) v[j] = 0u; }
                     if (k < cout) {
 #pragma unroll
@@ -1349,7 +1361,7 @@ void launch_conv_tc_probs(const void* d_tc, int nprob, int max_tiles, size_t pac
 // ---- wgrad host side
 struct WgGeom { TcWgradProb t; size_t smem, partial_bytes; long long cost; int box_h, box_n; };
 
-static bool wg_geometry_box(const ConvProb& p, int target_ctas, WgGeom& w, int max_box, bool nine);
+static bool wg_geometry_box(const ConvProb& p, int target_ctas, WgGeom& w, int max_box, bool nine, int max_chain = INT_MAX);
 // Both operands of a 3x3 weight gradient are windows of boxes, so a stage is large and the boxes' rounding decides how many stages
 // fit: the largest boxes that still leave two stages are taken (fewer TMA issues), else the size with the most stages.
 // A stride-1 3x3 layer has two forms: 128 x 128 tiles with one filter row's three taps per CTA, or 64 x 64 tiles with all nine taps, which load
@@ -1358,20 +1370,25 @@ static bool wg_geometry_box(const ConvProb& p, int target_ctas, WgGeom& w, int m
 static bool wg_geometry(const ConvProb& p, int target_ctas, WgGeom& w) {
     if (p.ksz == 1) return wg_geometry_box(p, target_ctas, w, 96, false);
     const int caps[5] = {96, 64, 48, 32, 24};
-    bool found = false;
+    bool found = false; size_t partial = 0;
     for (int nine = 0; nine < (p.stride == 1 ? 2 : 1); ++nine) {
         WgGeom best; int best_stages = 0;
+        // its sums must not run longer than the other form's, one of whose three taps has chains of half the length: sqrt((1 + 1 + 1 / 4) / 3)
+        const int max_chain = found && nine ? (int)(0.866 * w.t.chunks_per_split) : INT_MAX;
         for (int i = 0; i < 5 && best_stages < 2; ++i) {
             WgGeom g;
-            if (!wg_geometry_box(p, target_ctas, g, caps[i], nine != 0)) continue;
+            if (!wg_geometry_box(p, target_ctas, g, caps[i], nine != 0, max_chain)) continue;
             if (g.t.stages > best_stages) { best = g; best_stages = g.t.stages; }
         }
-        if (!best_stages || (found && best.cost >= w.cost)) continue;
+        if (!best_stages) continue;
+        partial = std::max(partial, best.partial_bytes);         // a launch of more problems may take the other form
+        if (best.cost < 0 || (found && best.cost >= w.cost)) continue;
         w = best; found = true;
     }
+    w.partial_bytes = partial;
     return found;
 }
-static bool wg_geometry_box(const ConvProb& p, int target_ctas, WgGeom& w, int max_box, bool nine) {
+static bool wg_geometry_box(const ConvProb& p, int target_ctas, WgGeom& w, int max_box, bool nine, int max_chain) {
     if (!tc_shape_ok(p)) return false;
     if (((uintptr_t)p.act | (uintptr_t)p.wgt) & 15) return false;
     TcWgradProb& t = w.t; memset(&t, 0, sizeof(t));
@@ -1434,7 +1451,7 @@ static bool wg_geometry_box(const ConvProb& p, int target_ctas, WgGeom& w, int m
     t.a_slabs = (t.n_tile + 63) / 64;
     if (t.nine) { t.tap_groups = 1; t.gbeg[1] = 9; }
     else if (taps == 9 && p.stride == 1) { for (int g = 0; g < 3; ++g) { t.gbeg[g + 1] = 3 * (g + 1); t.gxs[g] = 0; t.gys[g] = 0; } t.tap_groups = 3; }
-    int max_acc = 0; for (int g = 0; g < t.tap_groups; ++g) max_acc = std::max(max_acc, t.gbeg[g + 1] - t.gbeg[g]);
+    int max_acc = 0; for (int g = 0; g < t.tap_groups; ++g) { const int n = t.gbeg[g + 1] - t.gbeg[g]; max_acc = std::max(max_acc, n + (n & 1)); }   // an odd group's last tap has two
     t.mma_n = t.nine ? 192 : t.n_tile;
     if (t.nine) max_acc = 2;
     t.tmem_cols = 32; while (t.tmem_cols < max_acc * t.mma_n) t.tmem_cols *= 2;
@@ -1455,6 +1472,7 @@ static bool wg_geometry_box(const ConvProb& p, int target_ctas, WgGeom& w, int m
     long long best_cost = -1; int best_cps = t.chunks;
     for (int sp = 1; sp <= want_max; ++sp) {
         const int cps = (t.chunks + sp - 1) / sp, eff = (t.chunks + cps - 1) / cps;
+        if (cps > max_chain) continue;
         const long long waves = ((long long)fixed * eff + share - 1) / share, cost = waves * ((t.nine ? 3 : 4) * (long long)cps + 24);
         if (best_cost < 0 || cost < best_cost) { best_cost = cost; best_cps = cps; }
     }

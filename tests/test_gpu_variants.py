@@ -69,6 +69,24 @@ def test_convolutions_at_the_edges_of_the_variants(m, case):
     assert max_rel_err(dw.cpu().numpy(), oracle.conv_wgrad(dy, a, k, s)) < F32_TOL
 
 
+# A running sum of the tensor core loses up to 2^-24 of itself with every step of 16 positions, and with non-negative operands always in one
+# direction: n steps end about n / 2 of 2^-25 low (the sum grows evenly).  128 x 32 x 32 positions of 1024 chunks over 37 CTAs are 28 chunks, 224 steps
+# in one chain (3.3e-6 low at the least) or 112 in each of two; likewise the last tap of a filter row, the single taps of stride 2.
+@pytest.mark.parametrize("geom,bound,taps", [((128, 32, 32, 256, 512, 1, 1), 6e-6, [0]), ((128, 8, 8, 256, 512, 3, 1), 1.8e-6, [2, 5, 8]), ((40, 56, 56, 512, 512, 1, 2), 2.3e-6, [0])])
+def test_weight_gradients_keep_two_running_sums_where_there_is_room(m, geom, bound, taps):
+    """Mean loss against 64 bits.  With one chain: 1.0e-5, 2.4e-6 to 3.0e-6, 3.8e-6; with two: 3.8e-6, 0.99e-6 to 1.2e-6, 1.5e-6.  The bounds lie between."""
+    N, H, W, C, K, k, s = geom
+    P = (H - 1) // s + 1
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    a = torch.rand(N, H, W, C, device="cuda", generator=gen).to(torch.bfloat16)
+    dy = torch.rand(N, P, P, K, device="cuda", generator=gen).to(torch.bfloat16)
+    dw = m.resist_conv2d(2, a, dy, geom, backend=2)[0].reshape(K, k * k, C).double()
+    d64, ap = dy.double().reshape(-1, K), torch.nn.functional.pad(a.double(), (0, 0, k // 2, k // 2, k // 2, k // 2))
+    for t in taps:
+        ref = d64.T @ ap[:, t // k:t // k + (P - 1) * s + 1:s, t % k:t % k + (P - 1) * s + 1:s].reshape(-1, C)
+        assert abs(((ref - dw[:, t]) / ref).mean().item()) < bound, t
+
+
 # a single tile of sums, two partial tiles, more tiles than one pass of loads holds, stride-1 3x3 over several column tiles
 @pytest.mark.parametrize("shape", [(1, 2, 3, 64, 64, 1), (1, 13, 11, 256, 64, 1), (2, 160, 207, 64, 64, 1), (3, 9, 7, 512, 128, 3)])
 def test_backward_sums_from_the_data_gradients_tiles(m, shape):
