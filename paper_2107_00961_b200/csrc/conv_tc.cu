@@ -613,7 +613,8 @@ __global__ void __launch_bounds__(TC_CONV_THREADS, 1) conv_tc_kernel(const TcPro
                 }
                 if (bwd_x) {
                     // the sums the BN backward needs, of the stored (rounded) da: dz = da where relu's input was positive, and dz * xhat.  A lane
-                    // has 8 columns of 8 rows; the four lanes of a column group are added in a fixed order, the warps as below.
+                    // has 8 columns of 8 rows in fp32; the four lanes of a column group are added in double, each lane ending with four of the
+                    // sixteen sums (half as many shuffles as a butterfly of all of them), the warps as below.
                     const int ch = lane & 7;
                     uint64_t nm[4], is[4], ga2[4], be2[4], su[4] = {0, 0, 0, 0}, sq[4] = {0, 0, 0, 0};
                     const uint32_t w0 = smem_u32(&bwd_s2[BWD ? grp : 0][0][0]) + (uint32_t)(s0 + ch * 8) * 4u;
@@ -637,15 +638,20 @@ __global__ void __launch_bounds__(TC_CONV_THREADS, 1) conv_tc_kernel(const TcPro
                         }
                     }
                     if (s0 + 64 < n_tile) load_x(s0 + 64);
+                    const bool sqs = lane & 8, hi = lane & 16;   // which kind of sum, and which four columns, this lane ends with
+                    auto pair = [&](int k, double* d) {          // columns 2k and 2k + 1 over the lane and its neighbour by bit 3
+                        const uint64_t other = __shfl_xor_sync(0xffffffffu, sqs ? su[k] : sq[k], 8), own = sqs ? sq[k] : su[k];
+                        float a0, a1, b0, b1; f2_unpack(own, a0, a1); f2_unpack(other, b0, b1);
+                        d[0] = (double)a0 + (double)b0; d[1] = (double)a1 + (double)b1;
+                    };
+                    float w[4];
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
+                    for (int k = 0; k < 2; ++k) {
+                        double lo2[2], hi2[2]; pair(k, lo2); pair(k + 2, hi2);
 #pragma unroll
-                        for (int d = 8; d < 32; d <<= 1) { su[k] = f2_add(su[k], __shfl_xor_sync(0xffffffffu, su[k], d)); sq[k] = f2_add(sq[k], __shfl_xor_sync(0xffffffffu, sq[k], d)); }
-                        if (lane < 8) {
-                            *reinterpret_cast<uint64_t*>(&stat_s[quad][0][s0 + ch * 8 + 2 * k]) = su[k];
-                            *reinterpret_cast<uint64_t*>(&stat_s[quad][1][s0 + ch * 8 + 2 * k]) = sq[k];
-                        }
+                        for (int j = 0; j < 2; ++j) w[2 * k + j] = (float)((hi ? hi2[j] : lo2[j]) + __shfl_xor_sync(0xffffffffu, hi ? lo2[j] : hi2[j], 16));
                     }
+                    *reinterpret_cast<float4*>(&stat_s[quad][sqs ? 1 : 0][s0 + ch * 8 + (hi ? 4 : 0)]) = make_float4(w[0], w[1], w[2], w[3]);
                 } else if (stat_tiles) {
                     // column sums of the stored (rounded) values: every warp over its own 32 rows, lane = two neighbouring columns;
                     // the four warps' sums are added in a fixed order once the tile's last slab is through
@@ -663,7 +669,12 @@ __global__ void __launch_bounds__(TC_CONV_THREADS, 1) conv_tc_kernel(const TcPro
             if (stat_tiles) {
                 bar_sync_epi(bid);                               // (the next tile's barrier behind its accumulator keeps these sums until they are read)
                 for (int c = et; c < n_tile; c += 128) {
-                    if (col0 + c < ncol) {
+                    if (BWD && bwd_x) {
+                        if (col0 + c < ncol)
+#pragma unroll
+                            for (int k = 0; k < 2; ++k)
+                                stat_tiles[((long long)tm * 2 + k) * ncol + col0 + c] = (float)((((double)stat_s[0][k][c] + (double)stat_s[1][k][c]) + (double)stat_s[2][k][c]) + (double)stat_s[3][k][c]);
+                    } else if (col0 + c < ncol) {
                         const float su = ((stat_s[0][0][c] + stat_s[1][0][c]) + stat_s[2][0][c]) + stat_s[3][0][c];
                         const float sq = ((stat_s[0][1][c] + stat_s[1][1][c]) + stat_s[2][1][c]) + stat_s[3][1][c];
                         stat_tiles[((long long)tm * 2 + 0) * ncol + col0 + c] = su;
