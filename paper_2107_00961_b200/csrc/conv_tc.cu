@@ -540,9 +540,8 @@ __global__ void __launch_bounds__(TC_CONV_THREADS, 1) conv_tc_kernel(const TcPro
             };
             if (bwd_x) {
                 load_x(0);
-                // the rows of the group's next tile are asked into L2 now, a whole tile ahead of their use (the 64 -> 256
-                // channel dgrad of 8 x 128 images of 32 x 32: 342 us with the sums, 131 + 193 us with a reduction pass of its own; the epilogue is the
-                // limit, and the little L1 beside 225 KB of shared memory; 3x3 layers at 128 channels 118 instead of 105 + 43 us)
+                // the rows of the group's next tile are asked into L2 now, a whole tile ahead of their use: the epilogue is the limit of the 1x1 layers,
+                // and the little L1 beside 225 KB of shared memory (which layers: conv_tc_bwd_sums)
                 const Unit nx = u + u_step < u_stop ? decode(u + u_step) : Unit{-1, 0, 0, 0};
                 if (nx.pi == pi && grp < nx.nt) {
                     const int px2 = pixel_of((nx.tm0 + grp) * TILE_M + m);
@@ -1152,11 +1151,20 @@ int conv_tc_stat_tiles(const ConvProb& p) {
     return (int)((pos + TILE_M - 1) / TILE_M);
 }
 
-// likewise of a dgrad problem, over its descriptors
+// likewise of a stride-1 dgrad problem
 int conv_tc_dgrad_tiles(const ConvProb& p) {
     if (p.ksz == 1) return (int)(((long long)p.N * p.P * p.Q + TILE_M - 1) / TILE_M);
-    Tall g; tall_of(p.stride == 2 ? p.P : p.H, p.stride == 2 ? p.Q : p.W, 1, 1, g);
-    return (int)(((long long)p.N * g.Hp * g.Wp + TILE_M - 1) / TILE_M) * (p.stride == 2 ? 4 : 1);
+    Tall g; tall_of(p.H, p.W, 1, 1, g);
+    return (int)(((long long)p.N * g.Hp * g.Wp + TILE_M - 1) / TILE_M);
+}
+
+// Are the BN backward's sums taken in this data gradient's epilogue?  `group`: problems of the launch.  Yes where x, read in the epilogue, is no more
+// than about twice the 126 MB L2; a reduction of its own streams more than that faster (data gradient + sums, us fused | apart: 256 <- 64 channels
+// 206 MB 154 | 165, 268 MB 202 | 194, 537 MB 361 | 331; 256 <- 128 157 MB 163 | 163, 268 MB 255 | 239, 537 MB 480 | 423; 512 <- 256 134 MB 151 | 157,
+// 268 MB 267 | 259; 1024 <- 256 134 MB 128 | 154).  Not below 64 channels, where half of the lanes have nothing to read (32 <- 128, 34 MB 93 | 75,
+// 134 MB 279 | 218).  Not at stride 2: the scattered rows of x cost the four phases 171 us where the pass took 130.
+bool conv_tc_bwd_sums(const ConvProb& p, int group) {
+    return p.stride == 1 && p.C >= 64 && (double)group * p.N * p.H * p.W * p.C * 2 <= 250e6;
 }
 
 // One status word per process in pinned host memory that every device can write: a kernel stores into it only when a bounded wait
@@ -1274,7 +1282,6 @@ int conv_tc_fill(const ConvProb& p, int mode, void* host_tc) {
         t.add_mode = !p.add ? 0 : p.add_sub == 2 ? 3 : 2;
         const int ntaps = t.gbeg[t.ngroups];
         t.tiles_m = (t.total_pos + TILE_M - 1) / TILE_M;
-        if (t.stat_tiles) t.stat_tiles += (long long)ph * t.tiles_m * 2 * ncol;        // one run of tiles per output phase
         pick_n_tile(t, ntaps, p.group > 0 ? p.group : 1, count, mode, p.bn_out != nullptr);
         t.out_slabs = (t.n_tile + 63) / 64;
         t.b_bytes = tc_weight_tile(t.n_tile, mode);

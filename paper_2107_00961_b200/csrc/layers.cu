@@ -209,13 +209,15 @@ size_t conv_mma_bn_partial_bytes(int C, int sms);
 int conv_tc_stat_tiles(const ConvProb& p);
 void launch_bn_finalize_tiles(const BnProb* d, int nprob, int max_c, int backward, cudaStream_t s);
 int conv_tc_dgrad_tiles(const ConvProb& p);
+bool conv_tc_bwd_sums(const ConvProb& p, int group);
 }
 
 // A convolution together with the BN+ReLU that consumes its output, launched the way the local step launches the pair (bf16):
 //   mode 0: y = scale * conv(a, w) + add;  a_out = relu(bn(y)) with batch statistics (stat, running statistics updated)
 //   mode 1: da = conv^T(dy, w) + add;      dx = BN+ReLU backward of the BN with input x and output gradient da (+ bn_add), dgamma, dbeta
 // Warp-MMA family (narrow layers): the BN runs inside the convolution's launch.  tcgen05 family: the statistics, or the
-// two sums of the backward, come from the per-tile sums of the convolution's epilogue (a finalize launch, then the elementwise pass).  *used_backend: 1 tcgen05, 2 warp-level MMA.
+// two sums of the backward where conv_tc_bwd_sums says so, come from the per-tile sums of the convolution's epilogue (a finalize launch, then the
+// elementwise pass); else the BN backward is the cooperative launch, or a reduction and the elementwise pass, behind the dgrad.  *used_backend: 1 tcgen05, 2 warp-level MMA.
 extern "C" int resist_conv2d_bn_relu(int32_t mode, int32_t backend, const void* act, const void* wgt, const void* add, void* out,
                                      int32_t N, int32_t H, int32_t W, int32_t C, int32_t K, int32_t ksz, int32_t stride, float scale,
                                      const void* x, const float* gamma, const float* beta, float* stat, float* run_mean, float* run_var,
@@ -246,7 +248,8 @@ extern "C" int resist_conv2d_bn_relu(int32_t mode, int32_t backend, const void* 
     else if (want_tc && conv_tc_supported(p, mode) && !(mode == CONV_DGRAD && ksz == 1 && stride == 2)) be = 1;
     if (used_backend) *used_backend = be;
     if (!be) { g_layer_error = "no tensor-core family takes this convolution with its BN"; return RESIST_EUNSUPPORTED; }
-    const int tiles = be != 1 ? 0 : mode == CONV_FWD ? conv_tc_stat_tiles(p) : conv_tc_dgrad_tiles(p);
+    const bool sums = be == 1 && (mode == CONV_FWD || conv_tc_bwd_sums(p, 1));      // the BN's sums come from the convolution's epilogue
+    const int tiles = !sums ? 0 : mode == CONV_FWD ? conv_tc_stat_tiles(p) : conv_tc_dgrad_tiles(p);
     const size_t partial_bytes = be == 2 ? conv_mma_bn_partial_bytes(bn.C, sm) : std::max((size_t)bn.chunks * 2 * bn.C * 8, (size_t)tiles * 2 * bn.C * 4);
     const int n_tc = be == 1 ? conv_tc_count(p, mode) : 1;
     std::vector<char> hd(be == 1 ? (size_t)n_tc * conv_tc_prob_bytes() : conv_mma_prob_bytes());
@@ -259,8 +262,8 @@ extern "C" int resist_conv2d_bn_relu(int32_t mode, int32_t backend, const void* 
     bool ok = true;
     if (be == 2) ok = conv_mma_fill(q, mode, hd.data(), &bn);
     else {
-        p.stat_tiles = (float*)bn.partial; bn.chunks = tiles;
-        if (mode == CONV_DGRAD) { p.bn_x = x; p.bn_stat = stat; p.bn_gamma = gamma; p.bn_beta = beta; }
+        if (sums) { p.stat_tiles = (float*)bn.partial; bn.chunks = tiles; }
+        if (sums && mode == CONV_DGRAD) { p.bn_x = x; p.bn_stat = stat; p.bn_gamma = gamma; p.bn_beta = beta; }
         ok = conv_tc_fill(p, mode, hd.data()) == n_tc;
     }
     if (!ok) { g_layer_error = "descriptor set-up failed"; return RESIST_ECUDA; }
@@ -275,9 +278,14 @@ extern "C" int resist_conv2d_bn_relu(int32_t mode, int32_t backend, const void* 
             int t = 0; size_t packed = 0;
             for (int i = 0; i < n_tc; ++i) { const char* h = hd.data() + (size_t)i * conv_tc_prob_bytes(); t = std::max(t, conv_tc_tiles(h)); packed = conv_tc_merge(packed, conv_tc_smem(h)); }
             launch_conv_tc_probs(blob + 1024, n_tc, t, packed, st);
-            launch_bn_finalize_tiles((BnProb*)blob, 1, bn.C, mode == CONV_FWD ? 0 : 1, st);
+            if (sums) launch_bn_finalize_tiles((BnProb*)blob, 1, bn.C, mode == CONV_FWD ? 0 : 1, st);
             if (mode == CONV_FWD) launch_bn_apply((BnProb*)blob, 1, bn.m * bn.C, true, true, st);
-            else launch_bn_bwd_apply((BnProb*)blob, 1, bn.m * bn.C, true, true, st);
+            else if (sums) launch_bn_bwd_apply((BnProb*)blob, 1, bn.m * bn.C, true, true, st);
+            else if (!(bn.C <= 512 && launch_bn_fused((BnProb*)blob, 1, bn.chunks, 1, st))) {
+                cudaGetLastError();
+                launch_bn_bwd_reduce((BnProb*)blob, 1, bn.chunks, bn.C, true, true, st);
+                launch_bn_bwd_apply((BnProb*)blob, 1, bn.m * bn.C, true, true, st);
+            }
         }
         e = cudaGetLastError();
     }

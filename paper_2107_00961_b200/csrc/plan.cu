@@ -22,6 +22,7 @@ int bn_fused_capacity(int backward);                                            
 void launch_bn_finalize_tiles(const BnProb* d, int nprob, int max_c, int backward, cudaStream_t s);
 int conv_tc_dgrad_tiles(const ConvProb& p);
 bool conv_tc_bn_fits(const ConvProb& p);
+bool conv_tc_bwd_sums(const ConvProb& p, int group);
 size_t conv_tc_prob_bytes();
 int conv_tc_tiles(const void* host_tc);
 size_t conv_tc_smem(const void* host_tc);
@@ -328,11 +329,9 @@ struct Builder {
         p.partial = bn_partial;
         const int producer = last_dgrad; last_dgrad = -1;
         const int tc_producer = last_tc_dgrad; last_tc_dgrad = -1;
-        if (tc_producer >= 0 && (*ops)[tc_producer].conv.out == da && (*ops)[tc_producer].conv.C == r.c && (*ops)[tc_producer].conv.stride == 1) {
+        if (tc_producer >= 0 && (*ops)[tc_producer].conv.out == da && (*ops)[tc_producer].conv.C == r.c && conv_tc_bwd_sums((*ops)[tc_producer].conv, group)) {
             // the tcgen05 data gradient that produces da reads x beside it and leaves the per-tile sums; one small launch adds them up, then
-            // one elementwise pass.  (The reduction as a pass of its own read x and da once more: 2.8 of 26 ms of the wide net's launches, and
-            // the cooperative form of small layers was 27 us of barrier and re-added partial sums whatever its size.  Not at stride 2: the
-            // scattered rows of x cost the four phases 171 us where the pass took 130.)
+            // one elementwise pass.  (The cooperative form of small layers was 27 us of barrier and re-added partial sums whatever its size.)
             ConvProb& c = (*ops)[tc_producer].conv;
             const int tiles = conv_tc_dgrad_tiles(c);
             bn_partial_need = std::max(bn_partial_need, (size_t)tiles * 2 * r.c * 4);

@@ -109,6 +109,28 @@ def test_backward_sums_of_wide_layers_are_as_exact_as_a_reduction_of_their_own(m
     assert sorted(err)[2] < 7.7e-8, err       # the third of six: an undecided relu mask (see above) costs a seed more than all of this
 
 
+# beside the data gradient rather than in it: x of more than 250 MB, fewer than 64 channels, stride 2; the last one just inside
+@pytest.mark.parametrize("shape", [(477, 32, 32, 256, 64, 1, 1), (8, 16, 16, 32, 128, 1, 1), (12, 16, 15, 128, 128, 3, 2), (476, 32, 32, 256, 64, 1, 1)])
+def test_backward_passes_on_both_sides_of_the_rule_for_the_sums(m, shape):
+    N, H, W, C, K, k, s = shape
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    r = lambda *z: torch.randn(*z, device="cuda", generator=gen)  # noqa: E731
+    w, dy = (r(K, k, k, C) * (2 / (k * k * C)) ** 0.5).to(torch.bfloat16), r(N, (H - 1) // s + 1, (W - 1) // s + 1, K).to(torch.bfloat16)
+    x, g, b = (1.7 * r(N, H, W, C) + r(C)).to(torch.bfloat16), 1 + 0.2 * r(C), 0.3 * r(C)
+    xd = x.double().reshape(-1, C)
+    stat = torch.zeros(4 * C, device="cuda")
+    stat[:C], stat[C:2 * C] = xd.mean(0).float(), (1 / torch.sqrt(xd.var(0, unbiased=False) + 1e-5)).float()
+    da, dx, dg, db, used = m.resist_conv2d_bn_relu(1, dy, w, shape, g, b, stat=stat, x=x, backend=2)
+    assert used == 1
+    assert torch.equal(da, m.resist_conv2d(1, dy, w, shape, backend=2)[0])
+    xh = (xd - stat[:C].double()) * stat[C:2 * C].double()
+    dz = torch.where(xh * g.double() + b.double() > 0, da.double().reshape(-1, C), torch.zeros_like(xh))
+    db_ref, dg_ref = dz.sum(0), (dz * xh).sum(0)
+    assert norm_max_abs(dg.cpu().numpy(), dg_ref.cpu().numpy()) < 2e-3 and norm_max_abs(db.cpu().numpy(), db_ref.cpu().numpy()) < 2e-3      # undecided masks, as below
+    dx_ref = g.double() * stat[C:2 * C].double() * (dz - db_ref / len(xd) - xh * dg_ref / len(xd))
+    assert ((dx.double().reshape(-1, C) - dx_ref).norm() / dx_ref.norm()).item() < BF16_TOL / 2      # one rounding: at most half an ulp of each element
+
+
 # a single tile of sums, two partial tiles, more tiles than one pass of loads holds, stride-1 3x3 over several column tiles
 @pytest.mark.parametrize("shape", [(1, 2, 3, 64, 64, 1), (1, 13, 11, 256, 64, 1), (2, 160, 207, 64, 64, 1), (3, 9, 7, 512, 128, 3)])
 def test_backward_sums_from_the_data_gradients_tiles(m, shape):
