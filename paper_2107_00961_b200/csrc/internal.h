@@ -156,7 +156,7 @@ int launch_head_bwd(const HeadProb* d, int nprob, int maxB, int maxC, int max_cl
 bool conv_small_ok(const ConvProb& p, int mode);
 int conv_small_ctas(const ConvProb& p, int mode);
 void launch_conv_small(const ConvProb* d, int nprob, int max_ctas, int mode, int ksz, bool bf16, cudaStream_t s);
-bool bn_small_ok(const BnProb& p);
+bool bn_small_ok(const BnProb& p, bool backward);
 void launch_bn_small(const BnProb* d, int nprob, int max_c, int backward, bool bf16, cudaStream_t s);
 
 // statistics, finalisation and apply of BN+ReLU in one cooperative launch (bf16 vector path, training mode); false if the grid cannot be co-resident

@@ -310,7 +310,7 @@ struct Builder {
             return stat;
         }
         if (p.vec && !eval && r.c <= 512 && (long long)p.chunks * ctx->S <= bn_fused_capacity(0)) { op.kind = OP_BN_FWD_FUSED; ops->push_back(op); return stat; }   // one cooperative launch
-        if (bn_small_ok(p)) { op.kind = OP_BN_FWD_SMALL; ops->push_back(op); return stat; }
+        if (bn_small_ok(p, false)) { op.kind = OP_BN_FWD_SMALL; ops->push_back(op); return stat; }
         ops->push_back(op);
         op.key = key + 1; op.kind = OP_BN_APPLY; ops->push_back(op);
         return stat;
@@ -340,7 +340,7 @@ struct Builder {
             op.key = key + 1; op.kind = OP_BN_BWD_APPLY; ops->push_back(op);
             return;
         }
-        if (bn_small_ok(p)) { op.kind = OP_BN_BWD_SMALL; ops->push_back(op); return; }
+        if (bn_small_ok(p, true)) { op.kind = OP_BN_BWD_SMALL; ops->push_back(op); return; }
         if (fusable(producer, da, p)) { fuse_into(producer, p, 2); return; }
         // one cooperative launch where all sub-ResNets' chunks can be resident together (the kernel holds 128 registers: one CTA
         // per SM), else the reduction and the elementwise pass as launches of their own

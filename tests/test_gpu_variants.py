@@ -347,6 +347,30 @@ def test_an_evaluation_is_refused_while_the_callers_stream_is_recorded(m):
     assert torch.equal(ctx.eval(x)[0].cpu(), ref)
 
 
+# channel counts without the vector path: up to 1024 rows both directions are one launch each, up to 4096 the forward is
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("B", [4, 5, 16, 17])
+def test_steps_on_both_sides_of_the_rules_for_a_bn_in_one_launch(m, dtype, B):
+    rows, arch = B * 256, net(16, 16, 10, 24, 24, 0, depth=(2,))
+    out = run_protocol_both(arch, 1, B, 1, 23, dtype, int(dtype == "bf16"), True, m, conv_backend=1)
+    for r in out["steps"][0]["subs"]:
+        if dtype == "f32":
+            assert max_rel_err(r["logits_gpu"], r["logits_cpu"]) < 1e-4
+            v, name = per_tensor(arch, r["grads_gpu"], r["grads_cpu"], max_rel_err)
+            assert v < 1e-4, (name, v)
+        else:                                                     # as for whole bf16 steps: gradients by direction
+            assert norm_max_abs(r["logits_gpu"], r["logits_cpu"]) < 2e-2
+            g, h = r["grads_gpu"].astype(np.float64), r["grads_cpu"].astype(np.float64)
+            assert g @ h / (np.linalg.norm(g) * np.linalg.norm(h)) > 0.97
+    ctx = out["ctx"]
+    ctx.set_profiling(True)
+    ctx.partition(3, 1)
+    x, y = to_dev(rnd(1, B, 16, 16, 3), ctx.act_dtype), torch.zeros(B, device="cuda", dtype=torch.int32)
+    ctx.local_step_grouped([x], [y], LR)
+    families = ctx.get_profile()
+    assert ("bn_relu_fwd_fused" in families) == (rows <= 4096) and ("bn_relu_bwd_fused" in families) == (rows <= 1024)
+
+
 # BN in the epilogues of evaluation's convolutions, three calls so that the recorded form runs too: warp-level layers, tcgen05 layers with more than
 # one slab and column tile, the pooled stem; 1 image, a ragged batch and one that fills several waves of tiles
 @pytest.mark.parametrize("kind,width,pool", [(synth.BASIC, 16, 0), (synth.BOTTLENECK, 64, 0), (synth.BOTTLENECK, 64, 1)])
