@@ -1353,7 +1353,7 @@ static size_t tc_layout(size_t packed, TcLaunch& L) {
     return std::max((size_t)L.na * a + (size_t)L.nb * b + staging(), (size_t)120 * 1024) + 1024;
 }
 
-// total_tiles: an upper bound of the tiles of all problems of the launch (max_tiles * nprob); packed: conv_tc_merge over its problems
+// max_tiles: the most units (pairs of row tiles x column tiles) of a problem; packed: conv_tc_merge over its problems
 // pdl: programmatic launch.  For evaluation, a chain of convolutions; in training the linked launches made the steps slower (ImageNet-shaped
 // 22.6 -> 24.4 ms with the forward half linked): between the convolutions run streaming kernels that want the whole SM.
 void launch_conv_tc_probs(const void* d_tc, int nprob, int max_tiles, size_t packed, cudaStream_t s, bool pdl) {
@@ -1368,8 +1368,8 @@ void launch_conv_tc_probs(const void* d_tc, int nprob, int max_tiles, size_t pac
     L.nprob = nprob;
     const size_t smem = tc_layout(packed, L);
     const bool dgrad = (packed >> 36) & 4;
-    const long long total = (long long)max_tiles * nprob;
-    const int grid = (int)std::max(1ll, std::min(total, (long long)sms));
+    // a CTA per row tile while there are SMs for them: the kernel then splits the pairs (of few units there is no full wave, only the last one)
+    const int grid = (int)std::max(1ll, std::min(2ll * max_tiles * nprob, (long long)sms));
     cudaLaunchConfig_t cfg = {}; cfg.gridDim = dim3(grid); cfg.blockDim = dim3(TC_CONV_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = s;
     cudaLaunchAttribute at[1]; at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization; at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at; cfg.numAttrs = pdl ? 1 : 0;

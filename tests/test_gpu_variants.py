@@ -49,6 +49,8 @@ CONVS = [
     (2, 4, 17, 15, 136, 72, 3, 1), (2, 2, 8, 8, 256, 256, 3, 1), (2, 3, 11, 13, 72, 200, 3, 2),
     # forward and data gradient: one tile, a last wave of single tiles (298 tiles), column tiles narrower than the channels
     (2, 1, 2, 2, 64, 64, 1, 1), (2, 4, 97, 98, 64, 72, 1, 1), (2, 5, 14, 14, 256, 256, 3, 1),
+    # fewer pairs of row tiles than half of the SMs, which run as single tiles: an odd number of them, one pair, several column tiles
+    (2, 3, 19, 19, 64, 320, 1, 1), (2, 1, 11, 14, 72, 64, 3, 1), (2, 2, 13, 21, 128, 192, 3, 1), (2, 2, 26, 23, 64, 96, 3, 2),
     # maps so wide that two windows take most of the shared memory (one weight tile, narrower column tiles) or no longer fit (CUDA cores)
     (2, 1, 3, 112, 64, 256, 3, 1), (2, 1, 3, 119, 72, 136, 3, 1), (2, 1, 3, 125, 64, 64, 3, 1), (2, 1, 3, 200, 64, 64, 3, 1), (2, 1, 5, 240, 64, 128, 3, 2),
 ]
