@@ -162,7 +162,8 @@ typedef struct {
 } resist_step_info;
 int resist_get_step_info(resist_ctx* ctx, resist_step_info* out);
 
-/* ---- Layer-level entry points: one layer on caller-owned device tensors, run by the kernels of the local step.
+/* ---- Layer-level entry points: one layer on caller-owned device tensors, run by the kernels of the local step
+ * (the family by the layer alone: a 3x3 layer of 64 channels stays on warp-level MMA here however large it is).
  * They take their scratch from a bounded pool of cudaMalloc'ed blocks (resist_layer_release_scratch() frees the idle ones),
  * synchronise the stream before returning, and report failures through resist_layer_last_error().  dtype: RESIST_F32 or RESIST_BF16 for activations and weights.
  *

@@ -20,7 +20,7 @@
 // the two tiles of the pair); warp 1 = MMA issuer, an accumulator in TMEM per tile; warps 2..9 = two epilogue groups of four warps,
 // one per tile of the pair (TMEM -> registers -> scale, residual add, bf16 -> staging slabs of 64 columns -> TMA store or row copy-out,
 // with per-tile column sums for the BN that follows); warp 10 = the residual, by TMA into the staging slabs.
-// The weight-gradient kernel (224 threads) has one producer warp, two issuer warps and four epilogue warps.
+// The weight-gradient kernel (224 threads) has a producer warp per operand (0: dy, 2: a), one issuer warp (1) and four epilogue warps.
 // Every wait is bounded: on expiry the kernel records the place in the status word, drains its copies and MMAs, frees its
 // TMEM and returns.
 #include <cuda.h>
@@ -764,7 +764,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) conv_wgrad_tc_kernel(const TcWg
     const int tn = id % n_tiles; const int tm = id / n_tiles;
     const int c_begin = split * chunks_per_split;
     const int c_end = min(c_begin + chunks_per_split, chunks);
-    const int tap0 = p.gbeg[tg], ntap = nine ? 2 : p.gbeg[tg + 1] - tap0;      // nine: one accumulator per issuing warp
+    const int tap0 = p.gbeg[tg], ntap = nine ? 2 : p.gbeg[tg + 1] - tap0;      // nine: two accumulators of 192 columns
     const int gx = p.gxs[tg], gy = p.gys[tg];
     const int hb = p.hb - tg * p.hb_step;                        // the group's window of a starts hb positions before the chunk
     const int nc = c_end - c_begin;
@@ -1186,8 +1186,8 @@ int conv_tc_read_status() {
 // single tiles (see the kernel).  Clocks per tile: the tensor core needs 128 / 68 / 52 per MMA of 256 / 128 / 64 columns; the rings are fed
 // from L2 at about 28 bytes per clock and SM (all SMs at once); an epilogue takes about 20 per column, and only runs under the next tile's
 // MMAs when two accumulators per tile fit TMEM (up to 128 columns).  Narrower tiles read every window once more, so they have to promise
-// 12 %, and from two full waves of the widest tiles on there is nothing to fill.  (50 images of 14 x 14 x 256, 3x3: 88 tiles of 256
-// columns are 88 busy SMs of 148; 74 -> 63 us for the layer call.  Evaluation of 50 ImageNet-shaped images 2.19 -> 1.95 ms.)
+// 12 %, and from two full waves of the widest tiles on there is nothing to fill.  (Evaluation of 50 ImageNet-shaped images 2.19 -> 1.95 ms;
+// with pairs really split where they are few, as this assumes, 1.87 -> 1.78, 4 images 0.98 -> 0.78.)
 static void pick_n_tile(TcHot& t, int ntaps, int group, int phases, int mode, bool bn) {
     const int sms = device_sms();
     double best = 0; int best_n = 0; long long wide_pairs = 0;
@@ -1377,7 +1377,7 @@ void launch_conv_tc_probs(const void* d_tc, int nprob, int max_tiles, size_t pac
 }
 
 // ---- wgrad host side
-struct WgGeom { TcWgradProb t; size_t smem, partial_bytes; long long cost; int box_h, box_n; };
+struct WgGeom { TcWgradProb t; size_t partial_bytes; long long cost; int box_h, box_n; };
 
 static bool wg_geometry_box(const ConvProb& p, int target_ctas, WgGeom& w, int max_box, bool nine, int max_chain = INT_MAX);
 // Both operands of a 3x3 weight gradient are windows of boxes, so a stage is large and the boxes' rounding decides how many stages
@@ -1480,7 +1480,6 @@ static bool wg_geometry_box(const ConvProb& p, int target_ctas, WgGeom& w, int m
     t.stage_bytes = t.dy_slabs * t.dy_slab_bytes + t.a_slabs * t.a_slab_bytes;
     t.stages = TC_MAX_STAGES; while (t.stages > 1 && (size_t)t.stages * t.stage_bytes > TC_SMEM_BUDGET) --t.stages;
     if ((size_t)t.stages * t.stage_bytes > TC_SMEM_BUDGET) return false;
-    w.smem = std::max((size_t)t.stages * t.stage_bytes, (size_t)120 * 1024) + 1024;
     // Split of the positions.  target_ctas is twice this problem's share of the SMs.  Every CTA pays a fixed cost (set-up, the
     // accumulators' way out) worth about six chunks, and a launch takes whole waves, so the split is the one that minimises
     // waves x (chunks per CTA + 6): mostly one full wave.  (A chunk of the nine-tap form takes 3/4 of the others' time.)  The partial buffer is sized for the most splits any share could pick.

@@ -145,8 +145,10 @@ __global__ void __launch_bounds__(1024) wgrad_small_kernel(const ConvProb* __res
     }
 }
 
-// The line: up to 64 M multiply-adds (about where one GEMM tile per SM exists and the tiles' reuse starts to pay), filters of at most nine
-// taps, and for the weight gradient at most 2048 positions (its CTAs walk all of them).
+// The line: up to 64 M multiply-adds, filters of at most nine taps, and for the weight gradient at most 2048 positions (its CTAs walk all of them).
+// us for the 3x3 layers of a four-block fp32 net, GEMM tiles | here, forward: 64 M 902 | 857 at 8 channels on 32 x 32 maps, 449 | 344 at 16,
+// 486 | 208 at 32, 1002 | 223 at 64 on 4 x 4; 255 M 3229 | 3217, 1464 | 1157, 798 | 618, 999 | 540, so the line lies on the safe side.  Weight gradient
+// (tiles with their split sums): 1728 positions 250 | 241 at 32 channels, 295 | 241 at 64; 3456 positions 320 | 421, 401 | 423.
 bool conv_small_ok(const ConvProb& p, int mode) {
     if ((p.ksz != 1 && p.ksz != 3) || (double)p.M * p.Ncol * p.Kred > 64e6) return false;
     if ((long long)p.N * p.H * p.W * p.C >= (1ll << 31) || (long long)p.N * p.P * p.Q * p.K >= (1ll << 31)) return false;

@@ -1,6 +1,6 @@
 // BN + ReLU forward for callers that must not allocate device memory.
 //
-// resist_bn_relu_forward() obtains its reduction scratch with cudaMalloc on every call.  Some callers cannot do
+// resist_bn_relu_forward() takes its reduction scratch from a pool that grows with cudaMalloc, and synchronises.  Some callers cannot do
 // that: code that runs inside a memory pool it may not grow, a real-time loop in which an allocation (and the
 // device-wide synchronisation cudaFree implies) is a latency spike, or a host framework that has handed all
 // device memory to its own allocator.  This file gives them the same operation with the scratch in a fixed

@@ -13,7 +13,6 @@ void* ctx_alloc(resist_ctx* ctx, size_t bytes);
 void ctx_free(resist_ctx* ctx, void* p);
 void held_segments(const resist_ctx* ctx, int sub, uint32_t bit, bool buffers, std::vector<Segment>& out, long long& chunks);
 int ensure_param_arrays(resist_ctx* ctx, int S);
-int ensure_seg_table(resist_ctx* ctx, int n);
 bool conv_tc_supported(const ConvProb& p, int mode);                                   // conv_tc.cu
 int conv_tc_fill(const ConvProb& p, int mode, void* host_tc);
 int conv_tc_count(const ConvProb& p, int mode);
@@ -64,7 +63,9 @@ static int pick_backend(const ConvProb& p, int mode, int group, int target_ctas,
     bool want_mma = pref == RESIST_CONV_AUTO || pref == RESIST_CONV_WARP_MMA || pref == RESIST_CONV_WARP_MMA_UNFUSED; const bool want_tc = pref == RESIST_CONV_AUTO || pref == RESIST_CONV_TCGEN05;
     // 3x3 layers of 64 channels and more run faster on tcgen05, followed by the streaming BN kernels, than on the warp-level MMA kernels
     // with the BN inside, once the launch has enough positions: ResNet-110's 8 x 8 stage at 4 x 128 images 3.44 -> 3.24 ms per step, its
-    // evaluation of 1000 images 3.68 -> 3.32 ms; one worker's 84 images alone (5376 positions) 1.28 -> 1.46 ms, so they stay.
+    // evaluation of 1000 images 3.68 -> 3.32 ms; one worker's 84 images alone (5376 positions) 1.28 -> 1.46 ms, so they stay.  Around the line, us per
+    // step tcgen05 | warp MMA: ResNet-110's worker at 14336 positions 2020 | 1977, 16384 2064 | 2121, 24576 2457 | 2788; six blocks of 64 channels on
+    // 16 x 16 maps 12288 715 | 645, 16384 706 | 830; 32 x 32 16384 771 | 732, 24576 789 | 844; 56 x 56 12544 748 | 719, 18816 785 | 932.
     // Only where tcgen05 takes the layer: its two windows do not fit maps of more than about 120 columns.
     if (pref == RESIST_CONV_AUTO && p.C >= 64 && p.K >= 64 && p.ksz == 3 && (long long)group * p.N * p.H * p.W >= 24576 &&
         (mode == CONV_WGRAD ? conv_wgrad_tc_supported(p, target_ctas, nullptr) : conv_tc_supported(p, mode))) want_mma = false;
@@ -116,7 +117,7 @@ struct Builder {
     std::vector<Op>* ops;
     // scratch shared by the operations of this sub-ResNet (they run one after another)
     double* bn_partial = nullptr; float* wgrad_partial = nullptr; size_t bn_partial_need = 0, wgrad_partial_need = 0;
-    char* up_buf = nullptr; size_t up_need = 0; const void* up_src = nullptr;      // zero-stuffed dy of the current stride-2 layer
+    char* up_buf = nullptr; size_t up_need = 0;      // zero-stuffed dy of the current stride-2 layer
     char* col_buf = nullptr; char* col_w = nullptr;                                 // im2col of the input images and the stem's weights packed alike
     static constexpr long long EVAL_STATS_KEY = -1;
     static constexpr int NGBUF = 12;           // rotating gradient buffers: the more, the further the main stream runs ahead of the weight gradients
@@ -468,7 +469,6 @@ static size_t unroll_subnet(resist_ctx* ctx, Builder& bd, const std::vector<char
         const long long key = BWD_BLOCK0 + 40LL * ((long long)n_aslots - 1 - aslot[slot]);
         const long long m_in = (long long)B * s.H * s.W, m_out = (long long)B * s.Ho * s.Wo;
         const char* dout = bd.gbuf[g_cur];
-        bd.up_src = nullptr;                                     // no zero-stuffed dy carries over from another block
         int g_sc = -1; bool sc_compact = false;
         if (K.has_projection) {
             bd.conv(key + 0, CONV_WGRAD, s.a1, r.proj, dout, nullptr, nullptr, B, s.H, s.W, 1.f);
@@ -959,7 +959,9 @@ static int enqueue_launches(resist_ctx* ctx, Plan& plan, bool update, bool overl
 
 // Records the plan's launches (everything but the patching of the call's pointers) as a graph.  A step is up to 400 launches, two
 // events around every weight gradient among them: enqueueing them costs the host 0.3 to 1 ms, and each dependent pair of launches
-// a few microseconds of idle GPU.  Failing to record is no error: the plan keeps being enqueued launch by launch.
+// a few microseconds of idle GPU.  Failing to record is no error: the plan keeps being enqueued launch by launch.  At the third run: recording and
+// instantiating cost 0.27 / 0.62 / 1.0 ms (smallest net / ResNet-110 / wide net, 8 x 32 images), a replay saves 0.12 / 0.31 / 0.43 ms, so by the
+// sixth run it has paid; rounds of one or two steps, which also exist, never pay.
 static void record_plan(resist_ctx* ctx, Plan& plan, bool update) {
     plan.graph_failed = true;
     cudaGraph_t g = nullptr;

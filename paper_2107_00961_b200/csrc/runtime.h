@@ -90,10 +90,6 @@ struct Plan {
     resist_step_info info{};
 };
 
-struct SubMem {           // device tensors of one sub-ResNet for one batch size (offsets into the workspace)
-    size_t bytes = 0;
-};
-
 }  // namespace resist
 
 struct resist_ctx {
