@@ -195,7 +195,7 @@ int resist_bn_relu_backward(int32_t dtype, const void* x, const void* da, const 
  *   mode 1: da = conv^T(dy, w) + add  [out];  dx = backward of the BN+ReLU with input x (a-shaped) and output gradient da,
  *           plus bn_add when non-NULL  [bn_out]; dgamma, dbeta; stat must hold that BN's mean and 1/sqrt(var+eps).
  * Layers of up to 64 channels run the BN inside the warp-MMA convolution's launch; wider ones take the statistics, or
- * the two sums of the backward (stride 1, up to 250 MB of x), from the per-tile sums of the tcgen05 convolution's epilogue.
+ * the two sums of the backward (stride 1, 64 channels and more, as long as x is about what L2 holds), from the per-tile sums of the tcgen05 convolution's epilogue.
  * *used_backend: 1 tcgen05, 2 warp-level MMA.  RESIST_EUNSUPPORTED when no tensor-core family takes the pair. */
 int resist_conv2d_bn_relu(int32_t mode, int32_t backend, const void* act, const void* wgt, const void* add, void* out,
                           int32_t N, int32_t H, int32_t W, int32_t C, int32_t K, int32_t ksz, int32_t stride, float scale,

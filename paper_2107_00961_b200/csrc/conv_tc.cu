@@ -727,7 +727,7 @@ void launch_zero_stuff(const UpProb* d, int nprob, long long max_vecs, cudaStrea
 // What bounds it: the tensor pipe, 74 % active at 64 channels and 1024 x 32 x 32 positions (a quarter of that is row 1 computed twice), then the
 // boxes' way into shared memory.  Before, one thread produced both operands with two divisions per box and a chunk of 1536 clocks of MMAs took
 // ~5500.  8 x 128 images, us: 64 channels 32 x 32 294 -> 94,
-// 128 16 x 16 143 -> 102, 256 8 x 8 205 -> 101, 512 4 x 4 171 -> 134.
+// 128 16 x 16 143 -> 103, 256 8 x 8 205 -> 146 (two splits; 101 with one, whose chains are too long), 512 4 x 4 171 -> 134.
 struct alignas(64) TcWgradProb {
     CUtensorMap map_dy;       // (channel k, pixel) or (channel k, x, y, image)
     CUtensorMap map_a;        // likewise for a, possibly element-strided
@@ -1158,13 +1158,18 @@ int conv_tc_dgrad_tiles(const ConvProb& p) {
     return (int)(((long long)p.N * g.Hp * g.Wp + TILE_M - 1) / TILE_M);
 }
 
-// Are the BN backward's sums taken in this data gradient's epilogue?  `group`: problems of the launch.  Yes where x, read in the epilogue, is no more
-// than about twice the 126 MB L2; a reduction of its own streams more than that faster (data gradient + sums, us fused | apart: 256 <- 64 channels
-// 206 MB 154 | 165, 268 MB 202 | 194, 537 MB 361 | 331; 256 <- 128 157 MB 163 | 163, 268 MB 255 | 239, 537 MB 480 | 423; 512 <- 256 134 MB 151 | 157,
-// 268 MB 267 | 259; 1024 <- 256 134 MB 128 | 154).  Not below 64 channels, where half of the lanes have nothing to read (32 <- 128, 34 MB 93 | 75,
-// 134 MB 279 | 218).  Not at stride 2: the scattered rows of x cost the four phases 171 us where the pass took 130.
+// Are the BN backward's sums taken in this data gradient's epilogue?  `group`: problems of the launch.  The epilogue then reads x, and is what the
+// launch waits for; a reduction of its own reads x and da once more, which from beyond L2 (126 MB) it does faster than an epilogue.  How far the
+// epilogue keeps up depends on the MMAs beside it and on the columns.  Data gradient + sums, us fused | apart (x of the launch in MB):
+//   1x1, 64 <- 256 channels 134 MB 175 | 200, 201 MB 243 | 273; 128 <- 512 101 MB 134 | 165; 1024 <- 256 134 MB 138 | 153, 201 MB 191 | 198: up to 250 MB;
+//   1x1 of fewer reduction than output channels, 256 <- 64 103 MB 101 | 104, 206 MB 165 | 167, 537 MB 384 | 331; 256 <- 128 103 MB 124 | 120, 206 MB 210 | 200,
+//   537 MB 514 | 427; 512 <- 256 103 MB 134 | 130, 201 MB 230 | 208; 3x3, 64 channels 103 MB 165 | 167, 134 MB 226 | 216, 201 MB 327 | 296; 128 channels
+//   101 MB 173 | 189: up to L2.
+// Not below 64 channels, where half of the lanes have nothing to read (32 <- 128, 34 MB 93 | 75, 134 MB 279 | 218).  Not at stride 2: the scattered rows
+// of x cost the four phases 171 us where the pass took 130.
 bool conv_tc_bwd_sums(const ConvProb& p, int group) {
-    return p.stride == 1 && p.C >= 64 && (double)group * p.N * p.H * p.W * p.C * 2 <= 250e6;
+    const double limit = p.ksz == 1 && (p.K >= p.C || p.C >= 1024) ? 250e6 : 126e6;
+    return p.stride == 1 && p.C >= 64 && (double)group * p.N * p.H * p.W * p.C * 2 <= limit;
 }
 
 // One status word per process in pinned host memory that every device can write: a kernel stores into it only when a bounded wait
@@ -1384,7 +1389,7 @@ static bool wg_geometry_box(const ConvProb& p, int target_ctas, WgGeom& w, int m
 // fit: the largest boxes that still leave two stages are taken (fewer TMA issues), else the size with the most stages.
 // A stride-1 3x3 layer has two forms: 128 x 128 tiles with one filter row's three taps per CTA, or 64 x 64 tiles with all nine taps, which load
 // both operands once and, at 64 channels, leave no half of the MMA's lanes idle.  The cheaper one by the split's cost is taken.  us at
-// 8 x 128 images, three taps | nine: 64 channels 32 x 32 294 | 94, 128 16 x 16 102 | 119, 256 8 x 8 146 | 101 (96 against 128 CTAs), 512 4 x 4 134 | 150.
+// 8 x 128 images, three taps | nine: 64 channels 32 x 32 294 | 94, 128 16 x 16 102 | 119, 256 8 x 8 146 | 101 with one split, 146 with two, 512 4 x 4 134 | 150.
 static bool wg_geometry(const ConvProb& p, int target_ctas, WgGeom& w) {
     if (p.ksz == 1) return wg_geometry_box(p, target_ctas, w, 96, false);
     const int caps[5] = {96, 64, 48, 32, 24};

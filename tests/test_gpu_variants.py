@@ -111,8 +111,8 @@ def test_backward_sums_of_wide_layers_are_as_exact_as_a_reduction_of_their_own(m
     assert sorted(err)[2] < 7.7e-8, err       # the third of six: an undecided relu mask (see above) costs a seed more than all of this
 
 
-# beside the data gradient rather than in it: x of more than 250 MB, fewer than 64 channels, stride 2; the last one just inside
-@pytest.mark.parametrize("shape", [(477, 32, 32, 256, 64, 1, 1), (8, 16, 16, 32, 128, 1, 1), (12, 16, 15, 128, 128, 3, 2), (476, 32, 32, 256, 64, 1, 1)])
+# beside the data gradient rather than in it: x of more than 126 MB, fewer than 64 channels, stride 2; the last one just inside
+@pytest.mark.parametrize("shape", [(241, 32, 32, 256, 64, 1, 1), (8, 16, 16, 32, 128, 1, 1), (12, 16, 15, 128, 128, 3, 2), (240, 32, 32, 256, 64, 1, 1)])
 def test_backward_passes_on_both_sides_of_the_rule_for_the_sums(m, shape):
     N, H, W, C, K, k, s = shape
     gen = torch.Generator(device="cuda").manual_seed(1)
