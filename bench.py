@@ -215,7 +215,7 @@ def run_ours(args):
         if state["step"] % LOCAL_STEPS == 0:
             ctx.aggregate()
             new_round()
-            state["launches"] += 3            # aggregate (one launch) + scatter (parameters, buffers)
+            state["launches"] += 2            # aggregate + scatter, one launch each
             state["boundaries"] += 1
 
     def barrier():

@@ -117,8 +117,8 @@ struct Segment {
     long long begin;      // offset in the flat vector
     long long len;
     long long chunk0;     // first chunk index of this segment in the launch
-    unsigned mask;        // aggregate: owners; scatter/sgd: unused
-    int sub;              // scatter/sgd: sub-ResNet index
+    unsigned mask;        // aggregate, scatter: owners; sgd: unused
+    int sub;              // sgd: sub-ResNet index; aggregate, scatter: 0 = parameters, 1 = BN running statistics
 };
 
 struct ParamArrays {      // device pointers of the flat arrays
@@ -168,10 +168,9 @@ void launch_zero_stuff(const UpProb* d, int nprob, long long max_vecs, cudaStrea
 // ---- launchers (kernels_bw.cu)
 void launch_sgd(const Segment* d, int nseg, long long nchunks, ParamArrays pa, const float* lr, float mu, float wd,
                 bool shadow, cudaStream_t s);
-void launch_scatter(const Segment* d, int nseg, long long nchunks, ParamArrays pa, bool zero_momentum, bool shadow,
+void launch_scatter(const Segment* d, int nseg, long long nchunks, ParamArrays pa, int S, bool zero_momentum, bool shadow,
                     cudaStream_t s);
 void launch_shadow(const float* src, __nv_bfloat16* dst, long long n, cudaStream_t s);   // dst = round(src); both 16-byte aligned
-void launch_scatter_buffers(const Segment* d, int nseg, long long nchunks, ParamArrays pa, cudaStream_t s);
 struct AggArrays { const float* sub_p; const float* sub_b; long long stride_p, stride_b; float* global_p; float* global_b; };   // _p parameters, _b BN running statistics
 void launch_aggregate(const Segment* d, int nseg, long long nchunks, const AggArrays& arr, int S, cudaStream_t s);
 

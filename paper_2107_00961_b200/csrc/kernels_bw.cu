@@ -56,27 +56,47 @@ __global__ void __launch_bounds__(256) sgd_kernel(const Segment* __restrict__ se
     }
 }
 
-// working copy <- global; momentum <- 0 (restart); bf16 copy <- round(global)
+// working copies <- global; momentum <- 0 (restart); bf16 copies <- round(global).  Bound by HBM, most of it the writes to the copies, so a CTA
+// takes a chunk of the GLOBAL vector, reads it once into registers (four 16-byte loads in flight per thread) and writes it to every owner.  Segments are
+// runs with the same owners; Segment::sub 0 = parameters, 1 = BN running statistics (one launch serves both).  With segments per working copy
+// a block held by k of them was read k times: ResNet-101 parameters at S = 8, 2.58 GB moved in 409 us; now 2.0 GB in 336, and a round's
+// boundary (aggregate and this) 605 -> 533.
 template <bool SHADOW, bool ZERO_V>
-__global__ void __launch_bounds__(256) scatter_kernel(const Segment* __restrict__ segs, int nseg, ParamArrays pa) {
+__global__ void __launch_bounds__(256) scatter_kernel(const Segment* __restrict__ segs, int nseg, ParamArrays pa, int S) {
     const Segment& sg = find_segment(segs, nseg, blockIdx.x);
     const Range r = chunk_range(sg, blockIdx.x);
-    const long long o = (long long)sg.sub * pa.n + r.base;
-    const float* __restrict__ src = pa.global + r.base;
-    float* __restrict__ w = pa.w + o; float* __restrict__ v = pa.v + o; __nv_bfloat16* __restrict__ wb = pa.wb + o;
+    const bool stats = sg.sub != 0;
+    const float* __restrict__ src = (stats ? pa.global_buf : pa.global) + r.base;
+    const long long stride = stats ? pa.nbuf : pa.n;
+    float* __restrict__ dst = stats ? pa.buf : pa.w;
+    const unsigned mask = sg.mask & (S >= 32 ? 0xffffffffu : ((1u << S) - 1u));
     int done = 0;
-    if (((o | r.base) & 3) == 0) {
+    if (((r.base | stride) & 3) == 0) {
         const int nq = r.len >> 2;
-        for (int q = threadIdx.x; q < nq; q += 256) {
-            float4 x = reinterpret_cast<const float4*>(src)[q];
-            reinterpret_cast<float4*>(w)[q] = x;
-            if (ZERO_V) reinterpret_cast<float4*>(v)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (SHADOW) reinterpret_cast<uint2*>(wb)[q] = make_uint2(pack_bf16x2(x.x, x.y), pack_bf16x2(x.z, x.w));
+        float4 x[SEG_CHUNK / 1024];
+#pragma unroll
+        for (int u = 0; u < SEG_CHUNK / 1024; ++u) { const int q = threadIdx.x + u * 256; x[u] = q < nq ? __ldg(reinterpret_cast<const float4*>(src) + q) : make_float4(0.f, 0.f, 0.f, 0.f); }
+        for (unsigned m = mask; m; m &= m - 1) {
+            const long long o = (long long)(__ffs(m) - 1) * stride + r.base;
+#pragma unroll
+            for (int u = 0; u < SEG_CHUNK / 1024; ++u) {
+                const int q = threadIdx.x + u * 256;
+                if (q >= nq) continue;
+                reinterpret_cast<float4*>(dst + o)[q] = x[u];
+                if (stats) continue;
+                if (ZERO_V) reinterpret_cast<float4*>(pa.v + o)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (SHADOW) reinterpret_cast<uint2*>(pa.wb + o)[q] = make_uint2(pack_bf16x2(x[u].x, x[u].y), pack_bf16x2(x[u].z, x[u].w));
+            }
         }
         done = nq << 2;
     }
     for (int i = done + threadIdx.x; i < r.len; i += 256) {
-        float x = src[i]; w[i] = x; if (ZERO_V) v[i] = 0.f; if (SHADOW) wb[i] = __float2bfloat16_rn(x);
+        const float x = src[i];
+        for (unsigned m = mask; m; m &= m - 1) {
+            const long long o = (long long)(__ffs(m) - 1) * stride + r.base + i;
+            dst[o] = x;
+            if (!stats) { if (ZERO_V) pa.v[o] = 0.f; if (SHADOW) pa.wb[o] = __float2bfloat16_rn(x); }
+        }
     }
 }
 
@@ -90,14 +110,6 @@ __global__ void __launch_bounds__(256) shadow_kernel(const float* __restrict__ s
         for (int u = 0; u < 4; ++u) if (q + u * step < nq) reinterpret_cast<uint2*>(dst)[q + u * step] = make_uint2(pack_bf16x2(x[u].x, x[u].y), pack_bf16x2(x[u].z, x[u].w));
     }
     for (long long i = 4 * nq + blockIdx.x * 256ll + threadIdx.x; i < n; i += step) dst[i] = __float2bfloat16_rn(src[i]);
-}
-
-__global__ void __launch_bounds__(256) scatter_buffers_kernel(const Segment* __restrict__ segs, int nseg, ParamArrays pa) {
-    const Segment& sg = find_segment(segs, nseg, blockIdx.x);
-    const Range r = chunk_range(sg, blockIdx.x);
-    const float* __restrict__ src = pa.global_buf + r.base;
-    float* __restrict__ dst = pa.buf + (long long)sg.sub * pa.nbuf + r.base;
-    for (int i = threadIdx.x; i < r.len; i += 256) dst[i] = src[i];
 }
 
 // global <- first + (sum over the other owners of (w_s - first)) / count, owners ascending; one owner: copy.
@@ -193,22 +205,18 @@ void launch_sgd(const Segment* d, int nseg, long long nchunks, ParamArrays pa, c
     if (shadow) sgd_kernel<true><<<(unsigned)nchunks, 256, 0, s>>>(d, nseg, pa, lr, mu, wd);
     else sgd_kernel<false><<<(unsigned)nchunks, 256, 0, s>>>(d, nseg, pa, lr, mu, wd);
 }
-void launch_scatter(const Segment* d, int nseg, long long nchunks, ParamArrays pa, bool zero_momentum, bool shadow,
+void launch_scatter(const Segment* d, int nseg, long long nchunks, ParamArrays pa, int S, bool zero_momentum, bool shadow,
                     cudaStream_t s) {
     if (nchunks <= 0) return;
     const unsigned g = (unsigned)nchunks;
-    if (shadow) { if (zero_momentum) scatter_kernel<true, true><<<g, 256, 0, s>>>(d, nseg, pa);
-                  else scatter_kernel<true, false><<<g, 256, 0, s>>>(d, nseg, pa); }
-    else { if (zero_momentum) scatter_kernel<false, true><<<g, 256, 0, s>>>(d, nseg, pa);
-           else scatter_kernel<false, false><<<g, 256, 0, s>>>(d, nseg, pa); }
+    if (shadow) { if (zero_momentum) scatter_kernel<true, true><<<g, 256, 0, s>>>(d, nseg, pa, S);
+                  else scatter_kernel<true, false><<<g, 256, 0, s>>>(d, nseg, pa, S); }
+    else { if (zero_momentum) scatter_kernel<false, true><<<g, 256, 0, s>>>(d, nseg, pa, S);
+           else scatter_kernel<false, false><<<g, 256, 0, s>>>(d, nseg, pa, S); }
 }
 void launch_shadow(const float* src, __nv_bfloat16* dst, long long n, cudaStream_t s) {
     const long long g = (n / 4 + 1023) / 1024;
     shadow_kernel<<<(unsigned)(g < 1 ? 1 : g > 148 * 8 ? 148 * 8 : g), 256, 0, s>>>(src, dst, n);
-}
-void launch_scatter_buffers(const Segment* d, int nseg, long long nchunks, ParamArrays pa, cudaStream_t s) {
-    if (nchunks <= 0) return;
-    scatter_buffers_kernel<<<(unsigned)nchunks, 256, 0, s>>>(d, nseg, pa);
 }
 void launch_aggregate(const Segment* d, int nseg, long long nchunks, const AggArrays& arr, int S, cudaStream_t s) {
     if (nchunks <= 0) return;

@@ -141,6 +141,22 @@ void held_segments(const resist_ctx* ctx, int sub, uint32_t bit, bool buffers, s
     flush(total);
 }
 
+// Runs of parameters (or BN running statistics) with the same owners, cut into chunks of `chunk` elements.
+static void owner_segments(const resist_ctx* ctx, bool buffers, int chunk, std::vector<Segment>& out, long long& chunks) {
+    const Layout& L = ctx->L; const int S = ctx->S;
+    const uint32_t all = S >= 32 ? 0xFFFFFFFFu : ((1u << S) - 1u);
+    const long long total = buffers ? L.n_buffers : L.n_params;
+    long long run = 0; uint32_t run_mask = all;
+    auto flush = [&](long long end) { if (end > run) { Segment s{run, end - run, chunks, run_mask, buffers ? 1 : 0}; chunks += (s.len + chunk - 1) / chunk; out.push_back(s); } run = end; };
+    for (size_t b = 0; b < L.blk.size(); ++b) {
+        if (ctx->mask[b] == run_mask) continue;               // extends the current run (block ranges are contiguous)
+        flush(buffers ? L.blk[b].buf_begin : L.blk[b].begin); run_mask = ctx->mask[b];
+    }
+    // the tail after the last block (final BN, head) is shared by all
+    if (!L.blk.empty() && run_mask != all) { flush(buffers ? L.blk.back().buf_end : L.blk.back().end); run_mask = all; }
+    flush(total);
+}
+
 }  // namespace resist
 
 extern "C" {
@@ -340,19 +356,19 @@ int resist_partition(resist_ctx* ctx, uint64_t round_seed, int32_t S, uint32_t* 
     ctx->S = S; ctx->mask = mask; ctx->generation++;
     if (member_mask) std::copy(mask.begin(), mask.end(), member_mask);
 
-    // scatter: global -> working copies of the blocks each sub-ResNet holds; momentum restarted
-    std::vector<Segment> segs, bsegs; long long chunks = 0, bchunks = 0;
-    for (int s = 0; s < S; ++s) { held_segments(ctx, s, 1u << s, false, segs, chunks); held_segments(ctx, s, 1u << s, true, bsegs, bchunks); }
-    rc = ensure_seg_table(ctx, (int)(segs.size() + bsegs.size()));
+    // scatter: global -> working copies of the blocks each sub-ResNet holds; momentum restarted.  One table, one launch: the statistics' chunks
+    // follow the parameters'
+    std::vector<Segment> segs; long long chunks = 0;
+    owner_segments(ctx, false, SEG_CHUNK, segs, chunks); owner_segments(ctx, true, SEG_CHUNK, segs, chunks);
+    rc = ensure_seg_table(ctx, (int)segs.size());
     if (rc) return rc;
     CK(cudaMemcpyAsync(ctx->d_seg, segs.data(), segs.size() * sizeof(Segment), cudaMemcpyHostToDevice, st));
-    CK(cudaMemcpyAsync(ctx->d_seg + segs.size(), bsegs.data(), bsegs.size() * sizeof(Segment), cudaMemcpyHostToDevice, st));
     const bool restart = ctx->opts.momentum_policy == RESIST_MOMENTUM_RESTART || ctx->state == 0;
-    double held_p = 0, heldb = 0; for (const Segment& g : segs) held_p += (double)g.len; for (const Segment& g : bsegs) heldb += (double)g.len;
     const bool bf = ctx->opts.dtype == RESIST_BF16;
-    ctx->prof.begin(PK_SCATTER, 2, held_p * (4.0 + 4.0 + (restart ? 4.0 : 0.0) + (bf ? 2.0 : 0.0)) + heldb * 8.0, 0, st);
-    launch_scatter(ctx->d_seg, (int)segs.size(), chunks, ctx->pa, restart, bf, st);
-    launch_scatter_buffers(ctx->d_seg + segs.size(), (int)bsegs.size(), bchunks, ctx->pa, st);
+    double bytes = 0;
+    for (const Segment& g : segs) bytes += (double)g.len * (4.0 + __builtin_popcount(g.mask) * (g.sub ? 4.0 : 4.0 + (restart ? 4.0 : 0.0) + (bf ? 2.0 : 0.0)));
+    ctx->prof.begin(PK_SCATTER, 1, bytes, 0, st);
+    launch_scatter(ctx->d_seg, (int)segs.size(), chunks, ctx->pa, S, restart, bf, st);
     ctx->prof.end(st); ctx->prof.collect(st);
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(st));     // the host-side segment vectors die here
@@ -364,26 +380,11 @@ int resist_aggregate(resist_ctx* ctx, resist_stream stream) {
     if (!ctx) return RESIST_EINVAL;
     if (ctx->state < 1) { ctx->err = "aggregate before partition"; return RESIST_ESTATE; }
     cudaStream_t st = (cudaStream_t)stream;
-    const Layout& L = ctx->L; const int S = ctx->S;
-    const uint32_t all = S >= 32 ? 0xFFFFFFFFu : ((1u << S) - 1u);
-    std::vector<Segment> segs, bsegs; long long chunks = 0, bchunks = 0;
-    auto build = [&](bool buffers, std::vector<Segment>& out, long long& ch) {
-        const long long total = buffers ? L.n_buffers : L.n_params;
-        long long run = 0; uint32_t run_mask = all;
-        auto flush = [&](long long end) { if (end > run) { Segment s{run, end - run, ch, run_mask, buffers ? 1 : 0}; ch += (s.len + AGG_CHUNK - 1) / AGG_CHUNK; out.push_back(s); } run = end; };
-        for (size_t b = 0; b < L.blk.size(); ++b) {
-            const long long bb = buffers ? L.blk[b].buf_begin : L.blk[b].begin, be = buffers ? L.blk[b].buf_end : L.blk[b].end;
-            if (ctx->mask[b] == run_mask) continue;           // extends the current run (block ranges are contiguous)
-            flush(bb); run_mask = ctx->mask[b]; (void)be;
-        }
-        // the tail after the last block (final BN, head) is shared by all
-        if (!L.blk.empty() && run_mask != all) { flush(buffers ? L.blk.back().buf_end : L.blk.back().end); run_mask = all; }
-        flush(total);
-    };
+    const int S = ctx->S;
+    std::vector<Segment> segs; long long chunks = 0;
     // BN running statistics: at every call, or at every bn_stat_period-th one (Sec. 5, ImageNet settings)
     const bool with_stats = ctx->opts.bn_stat_period <= 1 || (++ctx->aggregate_calls % ctx->opts.bn_stat_period) == 0;
-    build(false, segs, chunks); bchunks = chunks; if (with_stats) build(true, bsegs, bchunks);   // one table, one launch: the statistics' chunks follow the parameters'
-    segs.insert(segs.end(), bsegs.begin(), bsegs.end());
+    owner_segments(ctx, false, AGG_CHUNK, segs, chunks); if (with_stats) owner_segments(ctx, true, AGG_CHUNK, segs, chunks);   // one table, one launch, as the scatter
     int rc = ensure_seg_table(ctx, (int)segs.size());
     if (rc) return rc;
     CK(cudaMemcpyAsync(ctx->d_seg, segs.data(), segs.size() * sizeof(Segment), cudaMemcpyHostToDevice, st));
@@ -392,7 +393,7 @@ int resist_aggregate(resist_ctx* ctx, resist_stream stream) {
     if (ctx->ev_eval) CK(cudaStreamWaitEvent(st, ctx->ev_eval, 0));   // an evaluation in flight on another stream still reads what is overwritten here
     ctx->prof.begin(PK_AGGREGATE, 1, 4.0 * (rd + wr), 0, st);
     const AggArrays arr{ctx->pa.w, ctx->pa.buf, ctx->pa.n, ctx->pa.nbuf, ctx->pa.global, ctx->pa.global_buf};
-    launch_aggregate(ctx->d_seg, (int)segs.size(), bchunks, arr, S, st);
+    launch_aggregate(ctx->d_seg, (int)segs.size(), chunks, arr, S, st);
     ctx->prof.end(st); ctx->prof.collect(st);
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(st));
