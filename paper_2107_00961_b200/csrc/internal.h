@@ -112,6 +112,22 @@ struct HeadProb {         // global average pool + linear head + mean softmax cr
 // weights (32 KB at most, from L2).  Larger heads run as matrix products over the whole batch.
 inline bool head_small(int C, int classes) { return C <= 256 && classes <= 128 && C * classes <= 8192; }
 
+// Evaluation of a run of identity basic blocks by one launch (eval_chain.cu).
+struct ChainProb {
+    const __nv_bfloat16* x;                            // [N,H,W,C] input of the first block
+    __nv_bfloat16* x_out; __nv_bfloat16* a_out;        // output of the last block, and relu(bn(.)) of it; either may be nullptr
+    const uint4* wpk; const float* cst;                // filters in fragment order, constants of the layers + 1 BNs (eval_chain_pack_kernel)
+    int N, H, W, C, layers;                            // layers: convolutions, two per block
+    int pair, imgs, plane;                             // maps of up to 8 columns go in pairs; images per CTA; bytes of one image's 8-channel group
+};
+// One BN of a chain with the convolution whose output it normalises (none for the first, whose input is the chain's).
+struct ChainLayer {
+    const float* w;                                    // fp32 [C][9][C], or nullptr
+    const float *gamma, *beta, *mean, *var;            // gamma nullptr: no BN behind the last convolution
+    uint4* wdst; float* cdst;
+    float scale, eps; int C;                           // scale of the convolution
+};
+
 // A contiguous run of parameters treated alike by the bandwidth kernels.
 struct Segment {
     long long begin;      // offset in the flat vector
@@ -164,6 +180,14 @@ bool launch_bn_fused(const BnProb* d, int nprob, int max_chunks, int backward, c
 void launch_im2col(const ColProb* d, int nprob, const ColProb& shape, cudaStream_t s);      // shape: the largest problem's
 void launch_repack_rows(const ConvProb* d, int nprob, int max_elems, cudaStream_t s);     // kernels_ref.cu
 void launch_zero_stuff(const UpProb* d, int nprob, long long max_vecs, cudaStream_t s);   // conv_tc.cu
+
+// ---- launchers (eval_chain.cu)
+bool eval_chain_geometry(ChainProb& p);                    // from C, H, W: whether the chain kernel takes such blocks, and how
+size_t eval_chain_weight_bytes(int C, int layers);
+size_t eval_chain_const_bytes(int C, int layers);
+int eval_chain_set_floats(int C);                          // floats of one BN's constants
+void launch_eval_chain_pack(const ChainLayer* d, int n, int max_c, cudaStream_t s);
+bool launch_eval_chain(const ChainProb* d, const ChainProb& h, cudaStream_t s);
 
 // ---- launchers (kernels_bw.cu)
 void launch_sgd(const Segment* d, int nseg, long long nchunks, ParamArrays pa, const float* lr, float mu, float wd,

@@ -119,7 +119,7 @@ struct Builder {
     double* bn_partial = nullptr; float* wgrad_partial = nullptr; size_t bn_partial_need = 0, wgrad_partial_need = 0;
     char* up_buf = nullptr; size_t up_need = 0;      // zero-stuffed dy of the current stride-2 layer
     char* col_buf = nullptr; char* col_w = nullptr;                                 // im2col of the input images and the stem's weights packed alike
-    static constexpr long long EVAL_STATS_KEY = -1;
+    static constexpr long long EVAL_STATS_KEY = -1, EVAL_PACK_KEY = -2;
     static constexpr int NGBUF = 12;           // rotating gradient buffers: the more, the further the main stream runs ahead of the weight gradients
     char* gbuf[NGBUF] = {}; bool gused[NGBUF] = {}; size_t gbig = 0;
     float* logits = nullptr;
@@ -128,6 +128,7 @@ struct Builder {
     // output; backward: the BN backward whose da the data gradient produces).  Index of the candidate in *ops, or -1.
     int last_fwd_conv = -1, last_dgrad = -1;
     int last_tc_dgrad = -1;   // likewise the last data gradient, for the BN backward behind it
+    int last_chain = -1, last_chain_layer = -1;      // evaluation: the chain whose output is the current tensor, and its last layer's entry in *ops
     int last_tc_fwd = -1;     // the last forward convolution if it runs on tcgen05: its epilogue can leave the sums the BN of its output needs
     bool fusable(int idx, const void* tensor, const BnProb& p) const {
         if (idx < 0 || eval || ctx->opts.dtype != RESIST_BF16 || (ctx->opts.conv_backend != RESIST_CONV_AUTO && ctx->opts.conv_backend != RESIST_CONV_WARP_MMA)) return false;
@@ -285,6 +286,13 @@ struct Builder {
         p.partial = bn_partial;
         const int producer = last_fwd_conv; last_fwd_conv = -1;
         const int tc_producer = last_tc_fwd; last_tc_fwd = -1;
+        if (eval && last_chain >= 0 && (*ops)[last_chain].chain.x_out == x && (*ops)[last_chain].chain.C == r.c) {
+            // behind a chain: its last convolution applies this BN too
+            ChainProb& c = (*ops)[last_chain].chain; ChainLayer& l = (*ops)[last_chain_layer].layer; last_chain = -1;
+            c.a_out = (__nv_bfloat16*)a; if (!x_used) c.x_out = nullptr;
+            l.gamma = p.gamma; l.beta = p.beta; l.mean = p.run_mean; l.var = p.run_var;
+            return stat;
+        }
         if (eval) {
             // all layers' mean | 1/std come from one launch at the start; behind a tensor-core convolution the elementwise pass runs in
             // that convolution's epilogue
@@ -315,6 +323,37 @@ struct Builder {
         ops->push_back(op);
         op.key = key + 1; op.kind = OP_BN_APPLY; ops->push_back(op);
         return stat;
+    }
+    // Evaluation of the n identity basic blocks order[0 .. n) on x as one launch; false where the chain kernel does not take them.
+    static bool chainable(const resist_block& k) { return k.kind == RESIST_BASIC && !k.has_projection && k.stride == 1; }
+    bool chain(long long key, const int* order, int n, const void* x, int H, int Wd, float inv_S, void** out) {
+        const int C = ctx->blocks[order[0]].cin;
+        ChainProb c{}; c.N = B; c.H = H; c.W = Wd; c.C = C; c.layers = 2 * n;
+        if (!eval || ctx->opts.dtype != RESIST_BF16 || ctx->opts.conv_backend != RESIST_CONV_AUTO || !eval_chain_geometry(c)) return false;
+        char* const wpk = (char*)take(eval_chain_weight_bytes(C, c.layers)); float* const cst = (float*)take(eval_chain_const_bytes(C, c.layers));
+        *out = act((long long)B * H * Wd * C);
+        for (int l = 0; l <= c.layers; ++l) {                 // BN l behind convolution l - 1
+            Op op{}; op.key = EVAL_PACK_KEY; op.sub = sub; op.kind = OP_EVAL_CHAIN_PACK;
+            ChainLayer& y = op.layer; y.C = C; y.eps = ctx->opts.bn_eps; y.scale = 1.f;
+            y.cdst = cst + (size_t)l * eval_chain_set_floats(C);
+            if (l > 0) {
+                const int b = order[(l - 1) / 2];
+                y.w = W() + ctx->L.blk[b].conv[(l - 1) & 1].w; y.wdst = (uint4*)(wpk + eval_chain_weight_bytes(C, l - 1));
+                if (!(l & 1) && ctx->blocks[b].partitionable) y.scale = inv_S;
+                flops += 2LL * B * H * Wd * 9 * C * C; ++n_tc;
+            }
+            if (l < c.layers) {
+                const BNRef& r = ctx->L.blk[order[l / 2]].bn[l & 1];
+                y.gamma = W() + r.g; y.beta = W() + r.b; y.mean = Bf() + r.buf; y.var = Bf() + r.buf + r.c;
+            }
+            ops->push_back(op);
+        }
+        last_chain_layer = (int)ops->size() - 1;
+        Op op{}; op.key = key; op.sub = sub; op.kind = OP_EVAL_CHAIN;
+        c.x = (const __nv_bfloat16*)x; c.x_out = (__nv_bfloat16*)*out; c.wpk = (const uint4*)wpk; c.cst = cst;
+        op.chain = c; ops->push_back(op);
+        last_chain = (int)ops->size() - 1; last_fwd_conv = last_tc_fwd = -1;
+        return true;
     }
     void bn_bwd(long long key, const void* x, const void* da, void* dx, const void* add, const BNRef& r, float* stat, long long m) {
         Op op{}; op.key = key; op.sub = sub; op.kind = OP_BN_BWD_REDUCE;
@@ -420,6 +459,11 @@ static size_t unroll_subnet(resist_ctx* ctx, Builder& bd, const std::vector<char
         const int b = order[slot]; const resist_block& K = ctx->blocks[b]; const BlockRef& r = L.blk[b]; BlockMem& s = bm[b];
         bd.group = share[slot];
         const long long key = KEY_BLOCK0 + 20LL * (long long)aslot[slot];
+        if (bd.eval && Builder::chainable(K)) {
+            int n = 1; while (slot + n < order.size() && Builder::chainable(ctx->blocks[order[slot + n]])) ++n;
+            void* out = nullptr;
+            if (bd.chain(key, &order[slot], n, cur, cH, cW, inv_S, &out)) { cur = out; slot += n - 1; continue; }
+        }
         s.H = cH; s.W = cW; s.Ho = out_dim(cH, 3, K.stride); s.Wo = out_dim(cW, 3, K.stride);
         const long long m_in = (long long)B * s.H * s.W, m_out = (long long)B * s.Ho * s.Wo;
         const float scale = (bd.eval && K.partitionable) ? inv_S : 1.f;
@@ -559,6 +603,7 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
         return a.backend < b.backend; });
     const double es = ctx->opts.dtype == RESIST_BF16 ? 2.0 : 4.0;
     std::vector<ConvProb> conv; std::vector<BnProb> bn; std::vector<PoolProb> pool; std::vector<HeadProb> head; std::vector<UpProb> up; std::vector<ColProb> col;
+    std::vector<ChainProb> chain; std::vector<ChainLayer> layer;
     const size_t tcb = conv_tc_prob_bytes(); std::vector<char> tc; int n_tc = 0;
     const size_t wtcb = conv_wgrad_tc_prob_bytes(); std::vector<char> wtc; int n_wtc = 0;
     const size_t mmb = conv_mma_prob_bytes(); std::vector<char> mm; int n_mm = 0;
@@ -575,12 +620,24 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
             const ConvProb& c = ops[i].conv;
             snprintf(L.label, sizeof(L.label), "%dx%d C%d K%d HW%d s%d%s x%d", c.ksz, c.ksz, c.C, c.K, c.H, c.stride, c.dy_sub == 2 ? "*" : "", L.count);
         } else if (ops[i].kind != OP_HEAD_FWD && ops[i].kind != OP_HEAD_BWD && ops[i].kind != OP_POOL_FWD && ops[i].kind != OP_POOL_BWD &&
-                   ops[i].kind != OP_UPSAMPLE && ops[i].kind != OP_IM2COL && ops[i].kind != OP_SPLITK && ops[i].kind != OP_REPACK)
+                   ops[i].kind != OP_UPSAMPLE && ops[i].kind != OP_IM2COL && ops[i].kind != OP_SPLITK && ops[i].kind != OP_REPACK &&
+                   ops[i].kind != OP_EVAL_CHAIN_PACK && ops[i].kind != OP_EVAL_CHAIN)
             snprintf(L.label, sizeof(L.label), "bn m%lld C%d x%d", ops[i].bn.m, ops[i].bn.C, L.count);
         for (size_t k = i; k < j; ++k) {
             ops[k].conv.group = (int)(j - i);
             const Op& o = ops[k]; const int slot = single ? 0 : o.sub;
             switch (o.kind) {
+                case OP_EVAL_CHAIN_PACK:
+                    if (k == i) L.first = (int)layer.size();
+                    layer.push_back(o.layer); L.max_c = std::max(L.max_c, o.layer.C);
+                    if (o.layer.w) L.bytes += (4.0 + 2.0) * 9 * o.layer.C * o.layer.C;
+                    break;
+                case OP_EVAL_CHAIN: {
+                    L.first = (int)chain.size(); chain.push_back(o.chain); L.chain = o.chain;
+                    const ChainProb& p = o.chain; const double e = (double)p.N * p.H * p.W * p.C, w_e = 9.0 * p.C * p.C;
+                    L.flops += 2.0 * p.layers * e * 9 * p.C; L.bytes += es * (e * (1 + (p.x_out ? 1 : 0) + (p.a_out ? 1 : 0)) + p.layers * w_e);
+                    snprintf(L.label, sizeof(L.label), "%d blocks C%d HW%d", p.layers / 2, p.C, p.H);
+                    break; }
                 case OP_REPACK: {
                     if (k == i) L.first = (int)conv.size();
                     conv.push_back(o.conv);
@@ -755,6 +812,8 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
     const size_t o_mm = off;   off += align_up(mm.size(), 256);
     const size_t o_col = off;  off += align_up(col.size() * sizeof(ColProb), 256);
     const size_t o_wmm = off;  off += align_up(wmm.size(), 256);
+    const size_t o_chain = off; off += align_up(chain.size() * sizeof(ChainProb), 256);
+    const size_t o_layer = off; off += align_up(layer.size() * sizeof(ChainLayer), 256);
     if (plan.graph) cudaGraphExecDestroy(plan.graph);
     plan.graph = nullptr; plan.runs = 0; plan.graph_failed = false;
     ctx_free(ctx, plan.d_blob);
@@ -789,6 +848,9 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
     if (!up.empty()) memcpy(host.data() + o_up, up.data(), up.size() * sizeof(UpProb));
     if (!col.empty()) memcpy(host.data() + o_col, col.data(), col.size() * sizeof(ColProb));
     plan.d_up = (UpProb*)(base + o_up);
+    if (!chain.empty()) memcpy(host.data() + o_chain, chain.data(), chain.size() * sizeof(ChainProb));
+    if (!layer.empty()) memcpy(host.data() + o_layer, layer.data(), layer.size() * sizeof(ChainLayer));
+    plan.d_chain = (ChainProb*)(base + o_chain); plan.d_layer = (ChainLayer*)(base + o_layer);
     if (!mm.empty()) memcpy(host.data() + o_mm, mm.data(), mm.size());
     if (!wmm.empty()) memcpy(host.data() + o_wmm, wmm.data(), wmm.size());
     plan.d_mm = base + o_mm; plan.mm_stride = mmb; plan.d_wmm = base + o_wmm; plan.wmm_stride = wmmb;
@@ -902,6 +964,7 @@ static int enqueue_launches(resist_ctx* ctx, Plan& plan, bool update, bool overl
             case OP_BN_FWD_FUSED: case OP_BN_FWD_SMALL: pk = PK_BN_FWD_FUSED; break;
             case OP_BN_TILE_STATS: case OP_BN_BWD_TILE_SUMS: pk = PK_BN_TILE_STATS; break;
             case OP_BN_BWD_FUSED: case OP_BN_BWD_SMALL: pk = PK_BN_BWD_FUSED; break;
+            case OP_EVAL_CHAIN_PACK: case OP_EVAL_CHAIN: pk = PK_EVAL_CHAIN; break;
         }
         pf.begin(pk, nk, L.bytes, L.flops, st, L.label);
         switch (L.kind) {
@@ -931,6 +994,10 @@ static int enqueue_launches(resist_ctx* ctx, Plan& plan, bool update, bool overl
             case OP_HEAD_FWD: n_launch += launch_head_fwd(plan.d_head + L.first, L.count, L.max_b, L.max_c, L.max_classes, bf, st); break;
             case OP_HEAD_BWD: n_launch += launch_head_bwd(plan.d_head + L.first, L.count, L.max_b, L.max_c, L.max_classes, L.max_elems, bf, st); break;
             case OP_UPSAMPLE: launch_zero_stuff(plan.d_up + L.first, L.count, L.max_elems, st); ++n_launch; break;
+            case OP_EVAL_CHAIN_PACK: launch_eval_chain_pack(plan.d_layer + L.first, L.count, L.max_c, st); ++n_launch; break;
+            case OP_EVAL_CHAIN:
+                if (!launch_eval_chain(plan.d_chain + L.first, L.chain, st)) { ctx->err = "evaluation chain launch failed"; return RESIST_ECUDA; }
+                ++n_launch; break;
             case OP_IM2COL: launch_im2col(plan.d_col + L.first, L.count, L.col, st); ++n_launch; break;
             case OP_BN_TILE_STATS: launch_bn_finalize_tiles(plan.d_bn + L.first, L.count, L.max_c, 0, st); ++n_launch; break;
             case OP_BN_BWD_TILE_SUMS: launch_bn_finalize_tiles(plan.d_bn + L.first, L.count, L.max_c, 1, st); ++n_launch; break;

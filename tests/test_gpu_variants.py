@@ -393,3 +393,49 @@ def test_evaluation_with_bn_in_the_epilogues(m, kind, width, pool, B):
         # seven layers of one-ulp differences (2^-8 each of what they touch), averaged by the sums that follow: 2e-2 as for whole steps
         assert norm_max_abs(logits.cpu().numpy(), ref["logits"]) < 2e-2
         assert abs(loss.item() - ref["loss"]) < 2e-2 * max(1.0, abs(ref["loss"]))
+
+
+def chain_net(h, w, width, depth=(3, 2, 2)):
+    ws = tuple(width * 2 ** i for i in range(len(depth)))
+    return synth.Arch(h, w, 3, 10, 3, 1, width, 0, 0, synth._stack(synth.BASIC, width, depth, ws, ws, "stage_first_shared"))
+
+
+# runs of identity blocks evaluated image by image: maps of whole and ragged 16-column blocks and 4-row strips, up to 8 columns (pairs of images, the last
+# one alone) and 9, one to eight images per CTA, shared memory for one CTA per SM, and maps that do not fit (layer by layer)
+@pytest.mark.parametrize("h,w,width,B", [(32, 32, 16, 3), (28, 28, 16, 5), (36, 33, 16, 2), (24, 36, 16, 1), (18, 18, 16, 9), (5, 6, 16, 17), (4, 4, 16, 4), (9, 64, 16, 3),
+                                         (64, 64, 16, 2), (16, 16, 32, 7), (17, 9, 32, 2), (7, 7, 64, 5), (9, 10, 64, 3), (16, 16, 64, 2)])
+def test_evaluation_of_runs_of_identity_blocks(m, h, w, width, B):
+    arch = chain_net(h, w, width)
+    a = arch.to_int32()
+    p, buf = synth.perturbed_params(arch, 3)
+    ctx = m.Context(a, dtype=m.BF16)
+    ctx.set_params(p, buf)
+    ctx.partition(1, 2)
+    for call in range(3):                                         # launched twice, then replayed
+        x = rnd(8 + call, B, h, w, 3)
+        y = (synth.splitmix64_words(9 + call, B) % np.uint64(10)).astype(np.int32)
+        logits, loss, _ = ctx.eval(to_dev(x, torch.bfloat16), to_dev(y, None))
+        ref = oracle.evaluate(a, p, buf, 2, x, y, quant=1)
+        # fifteen layers of one-ulp differences: 2e-2 as for whole steps
+        assert norm_max_abs(logits.cpu().numpy(), ref["logits"]) < 2e-2
+        assert abs(loss.item() - ref["loss"]) < 2e-2 * max(1.0, abs(ref["loss"]))
+    ctx.set_profiling(True)
+    ctx.eval(to_dev(x, torch.bfloat16), to_dev(y, None))
+    families = {k.split("@")[0] for k in ctx.get_profile()}
+    assert ("eval_chain" in families) == ((h, w, width) not in [(64, 64, 16), (16, 16, 64)])
+
+
+def test_evaluation_of_a_run_whose_output_is_read_as_it_is(m):
+    """Behind the run stands a block whose skip path reads the run's output itself, beside its normalised form."""
+    blocks = [synth.Block(synth.BASIC, 0, 16, 16, 16, 1, 0, 0), synth.Block(synth.BASIC, 0, 16, 16, 16, 1, 0, 1),
+              synth.Block(synth.BOTTLENECK, 0, 16, 16, 16, 1, 0, 0), synth.Block(synth.BASIC, 0, 16, 16, 16, 1, 0, 0)]
+    arch = synth.Arch(11, 12, 3, 10, 3, 1, 16, 0, 0, blocks)
+    p, buf = synth.perturbed_params(arch, 3)
+    ctx = m.Context(arch.to_int32(), dtype=m.BF16)
+    ctx.set_params(p, buf)
+    ctx.partition(1, 1)
+    x, y = rnd(8, 3, 11, 12, 3), np.array([1, 2, 3], np.int32)
+    logits, loss, _ = ctx.eval(to_dev(x, torch.bfloat16), to_dev(y, None))
+    ref = oracle.evaluate(arch.to_int32(), p, buf, 1, x, y, quant=1)
+    assert norm_max_abs(logits.cpu().numpy(), ref["logits"]) < 2e-2
+    assert abs(loss.item() - ref["loss"]) < 2e-2 * max(1.0, abs(ref["loss"]))
