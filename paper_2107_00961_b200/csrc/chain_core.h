@@ -1,0 +1,98 @@
+// What the kernels that carry images through runs of identity basic blocks share: the layout of an image in shared memory and the 3x3 convolution on it.
+//
+// Layout: [8-channel group][position][8 channels], 16 bytes per position, so that the eight rows of an ldmatrix matrix are 128 consecutive bytes without
+// padding or swizzle.  Positions are a zero-bordered map of W + 1 columns (the column W of a row is the column -1 of the next) and of a row above the image and
+// at least one below; position (y, x) is (y + 1) * (W + 1) + x + 1.
+//
+// A task of a warp is 64 positions x 16 output channels, all its accumulators in registers: four rows of two groups of eight columns.  The second group lies
+// `half` bytes from the first: the next eight columns, the same columns four rows further down, or the same positions of the next image, whichever
+// wastes least of the map at hand.  A fragment of input row i shifted by filter column s serves the three output rows i - 1 .. i + 1 it is a tap of: 18 ldmatrix
+// per 72 MMAs of a 16-channel step, where one per tap and row would be 36 and take as long as the MMAs.  Filters come from L2 in the fragments'
+// own order, 16 bytes per lane; the registers of a filter row are refilled as soon as the last map row that uses them is through.
+//
+// Rates: mma.sync m16n8k16 takes 8 clocks of an SM sub-partition (one warp with six accumulators reaches it), 576 TFLOP/s over the chip.
+#pragma once
+#include "internal.h"
+
+namespace resist {
+namespace chain {
+
+__device__ __forceinline__ uint32_t sm_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void ldsm4(uint32_t addr, uint32_t* r) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void mma16(float* c, const uint32_t* a, uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ uint4 ldg_pinned(const uint4* p) {     // stays where it is written: the compiler would sink the load to its first use
+    uint4 v; asm volatile("ld.global.nc.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p)); return v;
+}
+__device__ __forceinline__ float bf_lo(uint32_t w) { return __uint_as_float(w << 16); }
+__device__ __forceinline__ float bf_hi(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
+__device__ __forceinline__ uint32_t bf_pack(float a, float b) { __nv_bfloat162 h = __floats2bfloat162_rn(a, b); return *reinterpret_cast<uint32_t*>(&h); }
+// two fp32 operations per instruction
+__device__ __forceinline__ uint64_t v2(float lo, float hi) { uint64_t r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi)); return r; }
+__device__ __forceinline__ void un2(uint64_t v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) { uint64_t r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) { uint64_t r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) { uint64_t r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+__device__ __forceinline__ uint64_t of_bf2(uint32_t w) { return v2(bf_lo(w), bf_hi(w)); }
+__device__ __forceinline__ uint32_t to_bf2(uint64_t v) { float a, b; un2(v, a, b); return bf_pack(a, b); }
+__device__ __forceinline__ uint32_t relu_bf2(uint32_t w) { uint32_t r; asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(w), "r"(0u)); return r; }   // NaN becomes 0, as in z > 0 ? z : 0
+// relu(bn(x)) of two rounded values: (x - mean) / std * gamma + beta
+__device__ __forceinline__ uint32_t bn_relu2(uint32_t x, uint64_t neg_mean, uint64_t istd, uint64_t gamma, uint64_t beta) {
+    return relu_bf2(to_bf2(fma2(mul2(add2(of_bf2(x), neg_mean), istd), gamma, beta)));
+}
+
+constexpr int R = 4;                                             // rows of a task's half
+
+// fragments of one filter row of (output group, input step): [filter column]
+template <int NG>
+__device__ __forceinline__ void load_frag(uint4 (&b)[3][3], const uint4* __restrict__ wpk, int lane, int layer, int ng, int k, int r) {
+    const uint4* w = wpk + ((long long)layer * NG * NG + ng * NG + k) * (9 * 32) + r * (3 * 32) + lane;
+#pragma unroll
+    for (int s = 0; s < 3; ++s) b[r][s] = ldg_pinned(w + s * 32);
+}
+
+// acc = 3x3 convolution of a task.  base: shared address of the lane's row of the ldmatrix at input row -1, column -1, channel step 0.  refill(k, r): filter row r is
+// through with channel step k.
+template <int NG, class F>
+__device__ __forceinline__ void conv_task(float (&acc)[R][2][4], uint4 (&b)[3][3], uint32_t base, uint32_t row_bytes, uint32_t plane, F&& refill) {
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) { acc[r][j][0] = acc[r][j][1] = acc[r][j][2] = acc[r][j][3] = 0.f; }
+    constexpr int STEPS = NG * (R + 2) * 3;
+    uint32_t a[2][4];
+    auto addr = [&](int st) { return base + (uint32_t)(2 * (st / (3 * (R + 2)))) * plane + (uint32_t)(st / 3 % (R + 2)) * row_bytes + (uint32_t)(st % 3) * 16u; };
+    ldsm4(addr(0), a[0]);
+#pragma unroll
+    for (int st = 0; st < STEPS; ++st) {
+        const int k = st / (3 * (R + 2)), i = st / 3 % (R + 2), s = st % 3;
+        if (st + 1 < STEPS) ldsm4(addr(st + 1), a[(st + 1) & 1]);
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            const int o = i - r;
+            if (o < 0 || o >= R) continue;
+            mma16(acc[o][0], a[st & 1], b[r][s].x, b[r][s].y);
+            mma16(acc[o][1], a[st & 1], b[r][s].z, b[r][s].w);
+        }
+        if (s == 2 && i >= R - 1) refill(k, i - (R - 1));
+    }
+}
+
+}  // namespace chain
+
+// ---- host: how a map is cut into tasks
+// mode 0: 16 columns; 1: 8 columns, two groups of rows; 2: 8 columns of two images
+inline ChainMap chain_map(int H, int W, int mode) {
+    ChainMap m; m.cols = mode == 0 ? 16 : 8; m.rows = mode == 1 ? 8 : 4; m.slot = mode == 2 ? 2 : 1;
+    m.strips = (H + m.rows - 1) / m.rows; m.xblocks = (W + m.cols - 1) / m.cols;
+    m.map_rows = m.strips * m.rows + 2;
+    const int npos = m.map_rows * (W + 1) + m.xblocks * m.cols - W + 1;     // the last read: last row, columns of the last block, one more for the last filter column
+    m.plane = (npos * 16 + 127) / 128 * 128 + 64;                // 64 beyond a multiple of 128: the two groups of sixteen channels fall on different banks
+    return m;
+}
+
+}  // namespace resist

@@ -112,13 +112,19 @@ struct HeadProb {         // global average pool + linear head + mean softmax cr
 // weights (32 KB at most, from L2).  Larger heads run as matrix products over the whole batch.
 inline bool head_small(int C, int classes) { return C <= 256 && classes <= 128 && C * classes <= 8192; }
 
+// How the map of an image is cut into the tasks of the chain kernels (chain_core.h).
+struct ChainMap {
+    int cols, rows;               // columns and rows of a task's block of positions: 16 x 4, 8 x 8, or 8 x 4 of two images
+    int strips, xblocks, slot;    // blocks down and across; images of a block (1 or 2)
+    int map_rows, plane;          // rows of the zero-bordered map; bytes of one image's 8-channel group
+};
 // Evaluation of a run of identity basic blocks by one launch (eval_chain.cu).
 struct ChainProb {
     const __nv_bfloat16* x;                            // [N,H,W,C] input of the first block
     __nv_bfloat16* x_out; __nv_bfloat16* a_out;        // output of the last block, and relu(bn(.)) of it; either may be nullptr
     const uint4* wpk; const float* cst;                // filters in fragment order, constants of the layers + 1 BNs (eval_chain_pack_kernel)
     int N, H, W, C, layers;                            // layers: convolutions, two per block
-    int pair, imgs, plane;                             // maps of up to 8 columns go in pairs; images per CTA; bytes of one image's 8-channel group
+    ChainMap map; int imgs, warps;                     // images and warps per CTA
 };
 // One BN of a chain with the convolution whose output it normalises (none for the first, whose input is the chain's).
 struct ChainLayer {

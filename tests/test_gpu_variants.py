@@ -401,7 +401,7 @@ def chain_net(h, w, width, depth=(3, 2, 2)):
 
 
 # runs of identity blocks evaluated image by image: maps of whole and ragged 16-column blocks and 4-row strips, up to 8 columns (pairs of images, the last
-# one alone) and 9, one to eight images per CTA, shared memory for one CTA per SM, and maps that do not fit (layer by layer)
+# one alone) and 9, two rows of blocks in a task, one to eight images per CTA, shared memory for one CTA per SM, maps that do not fit (layer by layer)
 @pytest.mark.parametrize("h,w,width,B", [(32, 32, 16, 3), (28, 28, 16, 5), (36, 33, 16, 2), (24, 36, 16, 1), (18, 18, 16, 9), (5, 6, 16, 17), (4, 4, 16, 4), (9, 64, 16, 3),
                                          (64, 64, 16, 2), (16, 16, 32, 7), (17, 9, 32, 2), (7, 7, 64, 5), (9, 10, 64, 3), (16, 16, 64, 2)])
 def test_evaluation_of_runs_of_identity_blocks(m, h, w, width, B):
@@ -422,7 +422,7 @@ def test_evaluation_of_runs_of_identity_blocks(m, h, w, width, B):
     ctx.set_profiling(True)
     ctx.eval(to_dev(x, torch.bfloat16), to_dev(y, None))
     families = {k.split("@")[0] for k in ctx.get_profile()}
-    assert ("eval_chain" in families) == ((h, w, width) not in [(64, 64, 16), (16, 16, 64)])
+    assert ("eval_chain" in families) == ((h, w, width) != (16, 16, 64))
 
 
 def test_evaluation_of_a_run_whose_output_is_read_as_it_is(m):
