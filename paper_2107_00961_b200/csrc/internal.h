@@ -134,6 +134,26 @@ struct ChainLayer {
     float scale, eps; int C;                           // scale of the convolution
 };
 
+// Training through a run of identity basic blocks (train_chain.cu): one convolution and the BN + ReLU behind it, forward, or the data gradient of a
+// convolution and the backward of the BN + ReLU before it.
+struct TrainLayer {
+    const uint4* wpk;                                  // filter in fragment order of this direction
+    const __nv_bfloat16* res;                          // added to the convolution's output (forward) or to dx (backward), or nullptr
+    const __nv_bfloat16* x;                            // backward: input of the BN
+    __nv_bfloat16* y; __nv_bfloat16* a;                // forward: convolution's output and relu(bn(.)) of it; backward: a is dx
+    const float* gamma; const float* beta; float* stat; float* run_mean; float* run_var; float* dgamma; float* dbeta;
+};
+struct TrainChain {
+    const __nv_bfloat16* in;                           // input of the first convolution (forward), gradient of the run's output (backward)
+    const TrainLayer* layers; int nlayers;
+    uint4* packets;                                    // [2][CTAs][2][C]: the CTAs' sums, numbered
+    unsigned* arrive; int* status;                     // where the step's packet numbers start
+    int N, H, W, C; ChainMap map;
+    int imgs, cta0, ctas;                              // images per CTA; the problem's CTAs in the launch
+    float eps, momentum;
+};
+struct TrainPack { const __nv_bfloat16* w; uint4* fwd; uint4* bwd; int C; };      // w [C][9][C]
+
 // A contiguous run of parameters treated alike by the bandwidth kernels.
 struct Segment {
     long long begin;      // offset in the flat vector
@@ -194,6 +214,15 @@ size_t eval_chain_const_bytes(int C, int layers);
 int eval_chain_set_floats(int C);                          // floats of one BN's constants
 void launch_eval_chain_pack(const ChainLayer* d, int n, int max_c, cudaStream_t s);
 bool launch_eval_chain(const ChainProb* d, const ChainProb& h, cudaStream_t s);
+
+// ---- launchers (train_chain.cu)
+bool train_chain_geometry(int C, int H, int W, ChainMap& map);
+int train_chain_max_imgs(int C, const ChainMap& map);
+int train_chain_max_layers();
+bool train_chain_assign(TrainChain* p, int n, int sms);
+size_t train_chain_launch_smem(const TrainChain* p, int n);
+void launch_train_chain_pack(const TrainPack* d, int n, int max_c, unsigned* counters, int ncounters, cudaStream_t s);
+bool launch_train_chain(const TrainChain* d, int nprob, int C, bool backward, int ctas, size_t smem, cudaStream_t s);
 
 // ---- launchers (kernels_bw.cu)
 void launch_sgd(const Segment* d, int nseg, long long nchunks, ParamArrays pa, const float* lr, float mu, float wd,

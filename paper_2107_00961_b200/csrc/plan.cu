@@ -55,6 +55,7 @@ size_t conv_wgrad_mma_smem(const void* h);
 long long conv_wgrad_mma_out_elems(const void* h);
 void launch_conv_wgrad_mma_probs(const void* d, int nprob, int max_ctas, size_t max_smem, long long max_out, int variant, cudaStream_t s, bool pdl = false);
 int conv_wgrad_mma_pick_variant(const ConvProb& p, int target_ctas);
+int* conv_tc_status_word();
 
 // Which kernel family takes a bf16 convolution: 0 = CUDA cores, 1 = tcgen05, >= 200 = warp-level MMA (wgrad: 200 +
 // output channels; forward and dgrad: 1000 + the kernel variant, so that the value also separates launches by what
@@ -113,13 +114,13 @@ __global__ void patch_kernel(const PatchSite* sites, int n, PatchArgs a) {
 // ------------------------------------------------------------------------------------------------
 struct Builder {
     resist_ctx* ctx; int B; int sub; int copy; bool eval; int group;      // group: sub-ResNets that share the launches now being built
-    char* base; size_t off = 0; size_t es;
+    char* base; size_t off = 0; size_t es; bool group_all = group > 1;                // group_all: the plan is of all sub-ResNets (`group` itself changes from slot to slot)
     std::vector<Op>* ops;
     // scratch shared by the operations of this sub-ResNet (they run one after another)
     double* bn_partial = nullptr; float* wgrad_partial = nullptr; size_t bn_partial_need = 0, wgrad_partial_need = 0;
     char* up_buf = nullptr; size_t up_need = 0;      // zero-stuffed dy of the current stride-2 layer
     char* col_buf = nullptr; char* col_w = nullptr;                                 // im2col of the input images and the stem's weights packed alike
-    static constexpr long long EVAL_STATS_KEY = -1, EVAL_PACK_KEY = -2;
+    static constexpr long long EVAL_STATS_KEY = -1, PACK_KEY = -2;
     static constexpr int NGBUF = 12;           // rotating gradient buffers: the more, the further the main stream runs ahead of the weight gradients
     char* gbuf[NGBUF] = {}; bool gused[NGBUF] = {}; size_t gbig = 0;
     float* logits = nullptr;
@@ -129,6 +130,7 @@ struct Builder {
     int last_fwd_conv = -1, last_dgrad = -1;
     int last_tc_dgrad = -1;   // likewise the last data gradient, for the BN backward behind it
     int last_chain = -1, last_chain_layer = -1;      // evaluation: the chain whose output is the current tensor, and its last layer's entry in *ops
+    int last_tchain = -1;     // training: the chain whose output is the current tensor
     int last_tc_fwd = -1;     // the last forward convolution if it runs on tcgen05: its epilogue can leave the sums the BN of its output needs
     bool fusable(int idx, const void* tensor, const BnProb& p) const {
         if (idx < 0 || eval || ctx->opts.dtype != RESIST_BF16 || (ctx->opts.conv_backend != RESIST_CONV_AUTO && ctx->opts.conv_backend != RESIST_CONV_WARP_MMA)) return false;
@@ -307,6 +309,11 @@ struct Builder {
             op.key = key + 1; op.kind = OP_BN_APPLY; ops->push_back(op);
             return stat;
         }
+        if (last_tchain >= 0 && (*ops)[last_tchain].tlayers.back().y == x && (*ops)[last_tchain].tchain.C == r.c) {
+            TrainLayer& l = (*ops)[last_tchain].tlayers.back(); last_tchain = -1;                           // behind a chain: its last layer's
+            l.a = (__nv_bfloat16*)a; l.gamma = p.gamma; l.beta = p.beta; l.stat = stat; l.run_mean = p.run_mean; l.run_var = p.run_var;
+            return stat;
+        }
         if (fusable(producer, x, p)) { fuse_into(producer, p, 1); return stat; }                            // inside the producing convolution's launch
         if (!eval && p.vec && tc_producer >= 0 && (*ops)[tc_producer].conv.out == x && (*ops)[tc_producer].conv.K == r.c) {
             // the tcgen05 convolution that produces x leaves per-tile column sums: a small launch turns them into statistics, then one elementwise pass
@@ -333,7 +340,7 @@ struct Builder {
         char* const wpk = (char*)take(eval_chain_weight_bytes(C, c.layers)); float* const cst = (float*)take(eval_chain_const_bytes(C, c.layers));
         *out = act((long long)B * H * Wd * C);
         for (int l = 0; l <= c.layers; ++l) {                 // BN l behind convolution l - 1
-            Op op{}; op.key = EVAL_PACK_KEY; op.sub = sub; op.kind = OP_EVAL_CHAIN_PACK;
+            Op op{}; op.key = PACK_KEY; op.sub = sub; op.kind = OP_EVAL_CHAIN_PACK;
             ChainLayer& y = op.layer; y.C = C; y.eps = ctx->opts.bn_eps; y.scale = 1.f;
             y.cdst = cst + (size_t)l * eval_chain_set_floats(C);
             if (l > 0) {
@@ -354,6 +361,32 @@ struct Builder {
         op.chain = c; ops->push_back(op);
         last_chain = (int)ops->size() - 1; last_fwd_conv = last_tc_fwd = -1;
         return true;
+    }
+    // Training through the n identity basic blocks order[0 .. n) as one launch per direction: whether the chain kernel takes them, for `share` sub-ResNets
+    // in the launch (all their CTAs have to be resident together, one per SM).
+    bool tchain_ok(const resist_block& k, int H, int Wd, int share, ChainMap& map) const {
+        if (eval || ctx->opts.dtype != RESIST_BF16 || ctx->opts.conv_backend != RESIST_CONV_AUTO || !chainable(k) || !train_chain_geometry(k.cin, H, Wd, map)) return false;
+        const int cap = train_chain_max_imgs(k.cin, map);
+        if (cap < 1 || (long long)std::max(1, share) * ((B + cap - 1) / cap) > ctx->sm_count) return false;
+        ConvProb p = wgrad_prob(k.cin, H, Wd); size_t pb = 0;
+        return pick_backend(p, CONV_WGRAD, group, 8, &pb) != 0;
+    }
+    ConvProb wgrad_prob(int C, int H, int Wd) const {
+        ConvProb p{}; p.N = B; p.H = p.P = H; p.W = p.Q = Wd; p.C = p.K = C; p.ksz = 3; p.stride = 1; p.pad = 1; p.scale = 1.f;
+        p.M = C; p.Ncol = 9 * C; p.Kred = B * H * Wd;
+        p.tiles_m = (p.M + 63) / 64; p.tiles_n = (p.Ncol + 63) / 64; p.splits = 1; p.ktiles_per_split = (p.Kred + 15) / 16;
+        return p;
+    }
+    // a chain's weight gradients share one launch: each its own partial sums, the GPU's CTAs split among `many`
+    void chain_wgrad(long long key, const void* a, const void* dy, const ConvRef& cr, int H, int Wd, int many) {
+        Op op{}; op.key = key; op.sub = sub; op.kind = OP_CONV_WGRAD;
+        op.conv = wgrad_prob(cr.cin, H, Wd); op.conv.act = a; op.conv.wgt = dy; op.conv.out = G() + cr.w;
+        op.wg_target = wgrad_target_ctas(ctx, many);
+        size_t pb = 0;
+        op.backend = pick_backend(op.conv, CONV_WGRAD, group, op.wg_target, &pb);
+        op.conv.partial = (float*)take(pb);
+        flops += 2LL * B * H * Wd * 9 * cr.cin * cr.cout; ++n_tc;
+        ops->push_back(op);
     }
     void bn_bwd(long long key, const void* x, const void* da, void* dx, const void* add, const BNRef& r, float* stat, long long m) {
         Op op{}; op.key = key; op.sub = sub; op.kind = OP_BN_BWD_REDUCE;
@@ -398,7 +431,7 @@ struct Builder {
     }
 };
 
-struct BlockMem { int H, W, Ho, Wo; void *x, *a1, *y1, *a2, *y2, *a3; float* stat[3]; };
+struct BlockMem { int H, W, Ho, Wo; void *x, *a1, *y1, *a2, *y2, *a3; float* stat[3]; int chain_n, chain_first; const uint4* dpk[2]; };   // chain_n: blocks of the training chain that starts / ends here
 
 // Returns the workspace bytes this sub-ResNet needs.  `present` has one entry per block.
 static size_t unroll_subnet(resist_ctx* ctx, Builder& bd, const std::vector<char>& present, float inv_S) {
@@ -464,6 +497,41 @@ static size_t unroll_subnet(resist_ctx* ctx, Builder& bd, const std::vector<char
             void* out = nullptr;
             if (bd.chain(key, &order[slot], n, cur, cH, cW, inv_S, &out)) { cur = out; slot += n - 1; continue; }
         }
+        ChainMap cmap{};
+        if (bd.tchain_ok(K, cH, cW, share[slot], cmap)) {
+            int n = 1; while (slot + n < order.size() && 2 * n < train_chain_max_layers() && Builder::chainable(ctx->blocks[order[slot + n]])) ++n;
+            const long long rows = (long long)B * cH * cW; const int C = K.cin;
+            void* x = cur; void* a1 = bd.act(rows * C);
+            float* st1 = bd.bn_fwd(key + 0, x, a1, r.bn[0], rows, true);
+            Op op{}; op.key = key + 3; op.sub = bd.sub; op.kind = OP_TRAIN_CHAIN_FWD;
+            TrainChain& t = op.tchain;
+            t.in = (const __nv_bfloat16*)a1; t.nlayers = 2 * n; t.N = B; t.H = cH; t.W = cW; t.C = C; t.map = cmap;
+            t.eps = ctx->opts.bn_eps; t.momentum = ctx->opts.bn_momentum;
+            for (int i = 0; i < n; ++i) {
+                const int bi = order[slot + i]; const BlockRef& q = L.blk[bi]; BlockMem& e = bm[bi];
+                e.H = e.Ho = cH; e.W = e.Wo = cW; e.x = x; e.a1 = a1; e.stat[0] = st1; e.chain_n = i == n - 1 ? n : 0; e.chain_first = (int)slot;
+                e.y1 = bd.act(rows * C); e.a2 = bd.act(rows * C); void* out = bd.act(rows * C);
+                e.stat[1] = (float*)bd.take((size_t)4 * C * 4);
+                for (int j = 0; j < 2; ++j) {
+                    Op pk{}; pk.key = Builder::PACK_KEY; pk.sub = bd.sub; pk.kind = OP_TRAIN_CHAIN_PACK;
+                    uint4* f = (uint4*)bd.take((size_t)9 * C * C * 2); uint4* d = (uint4*)bd.take((size_t)9 * C * C * 2);
+                    pk.tpack = TrainPack{(const __nv_bfloat16*)bd.CW(q.conv[j].w), f, d, C}; bd.ops->push_back(pk); e.dpk[j] = d;
+                    TrainLayer l{}; l.wpk = f; l.res = j ? (const __nv_bfloat16*)x : nullptr; l.y = (__nv_bfloat16*)(j ? out : e.y1);
+                    bd.flops += 2LL * rows * 9 * C * C; ++bd.n_tc;
+                    if (j == 0 || i < n - 1) {                // the BN behind it; the last layer's comes with whatever follows the chain
+                        const int nb2 = j ? order[slot + i + 1] : bi; const BNRef& br = L.blk[nb2].bn[j ? 0 : 1];
+                        float* stat = e.stat[1]; void* a = e.a2;
+                        if (j) { a1 = a = bd.act(rows * C); st1 = stat = (float*)bd.take((size_t)4 * C * 4); }
+                        l.a = (__nv_bfloat16*)a; l.gamma = bd.W() + br.g; l.beta = bd.W() + br.b; l.stat = stat; l.run_mean = bd.Bf() + br.buf; l.run_var = bd.Bf() + br.buf + br.c;
+                    }
+                    op.tlayers.push_back(l);
+                }
+                x = out;
+            }
+            bd.ops->push_back(op);
+            bd.last_tchain = (int)bd.ops->size() - 1; bd.last_fwd_conv = bd.last_tc_fwd = -1;
+            cur = x; slot += n - 1; continue;
+        }
         s.H = cH; s.W = cW; s.Ho = out_dim(cH, 3, K.stride); s.Wo = out_dim(cW, 3, K.stride);
         const long long m_in = (long long)B * s.H * s.W, m_out = (long long)B * s.Ho * s.Wo;
         const float scale = (bd.eval && K.partitionable) ? inv_S : 1.f;
@@ -513,6 +581,43 @@ static size_t unroll_subnet(resist_ctx* ctx, Builder& bd, const std::vector<char
         const long long key = BWD_BLOCK0 + 40LL * ((long long)n_aslots - 1 - aslot[slot]);
         const long long m_in = (long long)B * s.H * s.W, m_out = (long long)B * s.Ho * s.Wo;
         const char* dout = bd.gbuf[g_cur];
+        if (s.chain_n) {
+            const int n = s.chain_n, first = s.chain_first, C = K.cin; const long long rows = m_in;
+            bd.group = share[first];
+            // the launch's key is the first block's: the same for all sub-ResNets, however many blocks they hold
+            const long long ckey = BWD_BLOCK0 + 40LL * ((long long)n_aslots - 1 - aslot[first]);
+            int many = 0;                                     // weight gradients in the launch: the stage's identity blocks of every sub-ResNet of the plan
+            for (int s2 = 0; s2 < ctx->S; ++s2)
+                if (bd.group_all || s2 == bd.sub)
+                    for (int b2 = 0; b2 < nb; ++b2) if ((ctx->mask[b2] >> s2 & 1u) && ctx->blocks[b2].stage == K.stage && Builder::chainable(ctx->blocks[b2])) many += 2;
+            Op op{}; op.key = ckey; op.sub = bd.sub; op.kind = OP_TRAIN_CHAIN_BWD;
+            TrainChain& t = op.tchain; ChainMap cmap{}; train_chain_geometry(C, s.H, s.W, cmap);
+            t.in = (const __nv_bfloat16*)dout; t.nlayers = 2 * n; t.N = B; t.H = s.H; t.W = s.W; t.C = C; t.map = cmap;
+            std::vector<const void*> dys;                     // gradient of every convolution's output, last first
+            const int g_dx = bd.gtake();
+            const void* d2 = dout;
+            for (int i = n - 1; i >= 0; --i) {
+                const int bi = order[first + i]; const BlockRef& q = L.blk[bi]; BlockMem& e = bm[bi];
+                void* dy1 = bd.act(rows * C); void* dxb = i ? bd.act(rows * C) : (void*)bd.gbuf[g_dx];
+                dys.push_back(d2); dys.push_back(dy1);
+                for (int j = 1; j >= 0; --j) {
+                    TrainLayer l{}; const BNRef& br = q.bn[j];
+                    l.wpk = e.dpk[j]; l.x = (const __nv_bfloat16*)(j ? e.y1 : e.x); l.a = (__nv_bfloat16*)(j ? dy1 : dxb); l.res = j ? nullptr : (const __nv_bfloat16*)d2;
+                    l.gamma = bd.W() + br.g; l.beta = bd.W() + br.b; l.stat = e.stat[j]; l.dgamma = bd.G() + br.g; l.dbeta = bd.G() + br.b;
+                    bd.flops += 2LL * rows * 9 * C * C; ++bd.n_tc;
+                    op.tlayers.push_back(l);
+                }
+                d2 = dxb;
+            }
+            bd.ops->push_back(op);
+            for (int i = n - 1, k = 0; i >= 0; --i, k += 2) {
+                const BlockRef& q = L.blk[order[first + i]]; BlockMem& e = bm[order[first + i]];
+                bd.chain_wgrad(ckey + 1, e.a2, dys[k], q.conv[1], s.H, s.W, many);
+                bd.chain_wgrad(ckey + 1, e.a1, dys[k + 1], q.conv[0], s.H, s.W, many);
+            }
+            bd.grel(g_cur); g_cur = g_dx; bd.last_dgrad = bd.last_tc_dgrad = -1;
+            slot = first; continue;
+        }
         int g_sc = -1; bool sc_compact = false;
         if (K.has_projection) {
             bd.conv(key + 0, CONV_WGRAD, s.a1, r.proj, dout, nullptr, nullptr, B, s.H, s.W, 1.f);
@@ -604,6 +709,7 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
     const double es = ctx->opts.dtype == RESIST_BF16 ? 2.0 : 4.0;
     std::vector<ConvProb> conv; std::vector<BnProb> bn; std::vector<PoolProb> pool; std::vector<HeadProb> head; std::vector<UpProb> up; std::vector<ColProb> col;
     std::vector<ChainProb> chain; std::vector<ChainLayer> layer;
+    std::vector<TrainChain> tchain; std::vector<TrainLayer> tlayer; std::vector<TrainPack> tpack; std::vector<size_t> tfirst;   // tfirst: a chain's first entry of tlayer
     const size_t tcb = conv_tc_prob_bytes(); std::vector<char> tc; int n_tc = 0;
     const size_t wtcb = conv_wgrad_tc_prob_bytes(); std::vector<char> wtc; int n_wtc = 0;
     const size_t mmb = conv_mma_prob_bytes(); std::vector<char> mm; int n_mm = 0;
@@ -621,12 +727,30 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
             snprintf(L.label, sizeof(L.label), "%dx%d C%d K%d HW%d s%d%s x%d", c.ksz, c.ksz, c.C, c.K, c.H, c.stride, c.dy_sub == 2 ? "*" : "", L.count);
         } else if (ops[i].kind != OP_HEAD_FWD && ops[i].kind != OP_HEAD_BWD && ops[i].kind != OP_POOL_FWD && ops[i].kind != OP_POOL_BWD &&
                    ops[i].kind != OP_UPSAMPLE && ops[i].kind != OP_IM2COL && ops[i].kind != OP_SPLITK && ops[i].kind != OP_REPACK &&
-                   ops[i].kind != OP_EVAL_CHAIN_PACK && ops[i].kind != OP_EVAL_CHAIN)
+                   ops[i].kind != OP_EVAL_CHAIN_PACK && ops[i].kind != OP_EVAL_CHAIN && ops[i].kind != OP_TRAIN_CHAIN_PACK && ops[i].kind != OP_TRAIN_CHAIN_FWD && ops[i].kind != OP_TRAIN_CHAIN_BWD)
             snprintf(L.label, sizeof(L.label), "bn m%lld C%d x%d", ops[i].bn.m, ops[i].bn.C, L.count);
         for (size_t k = i; k < j; ++k) {
             ops[k].conv.group = (int)(j - i);
             const Op& o = ops[k]; const int slot = single ? 0 : o.sub;
             switch (o.kind) {
+                case OP_TRAIN_CHAIN_PACK:
+                    if (k == i) L.first = (int)tpack.size();
+                    tpack.push_back(o.tpack); L.max_c = std::max(L.max_c, o.tpack.C); L.bytes += 6.0 * 9 * o.tpack.C * o.tpack.C;
+                    break;
+                case OP_TRAIN_CHAIN_FWD: case OP_TRAIN_CHAIN_BWD: {
+                    if (k == i) L.first = (int)tchain.size();
+                    tchain.push_back(o.tchain); tfirst.push_back(tlayer.size()); tlayer.insert(tlayer.end(), o.tlayers.begin(), o.tlayers.end());
+                    const TrainChain& p = o.tchain; const double e = (double)p.N * p.H * p.W * p.C;
+                    L.flops += 2.0 * p.nlayers * e * 9 * p.C; L.max_c = p.C;
+                    // forward: every layer writes y and a, every other one reads the residual; backward: every layer reads x and writes dx, every other one reads the skip gradient
+                    L.bytes += es * (e * (1 + 2.5 * p.nlayers) + p.nlayers * 9.0 * p.C * p.C);
+                    snprintf(L.label, sizeof(L.label), "%d layers C%d HW%d x%d", p.nlayers, p.C, p.H, L.count);
+                    if (k == j - 1) {
+                        TrainChain* t = tchain.data() + L.first;
+                        if (!train_chain_assign(t, L.count, ctx->sm_count)) { ctx->err = "internal: a chain's CTAs do not fit"; return RESIST_EINVAL; }
+                        L.gx = t[L.count - 1].cta0 + t[L.count - 1].ctas; L.smem = train_chain_launch_smem(t, L.count);
+                    }
+                    break; }
                 case OP_EVAL_CHAIN_PACK:
                     if (k == i) L.first = (int)layer.size();
                     layer.push_back(o.layer); L.max_c = std::max(L.max_c, o.layer.C);
@@ -652,7 +776,7 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
                         if (o.kind == OP_CONV_WGRAD) {
                             if (k == i) L.first = n_wmm;
                             wmm.resize((size_t)(n_wmm + 1) * wmmb); char* h = wmm.data() + (size_t)n_wmm * wmmb;
-                            if (!conv_wgrad_mma_fill(o.conv, wgrad_target_ctas(ctx, (int)(j - i)), h)) { ctx->err = "wgrad descriptor failed"; return RESIST_EINVAL; }
+                            if (!conv_wgrad_mma_fill(o.conv, o.wg_target ? o.wg_target : wgrad_target_ctas(ctx, (int)(j - i)), h)) { ctx->err = "wgrad descriptor failed"; return RESIST_EINVAL; }
                             L.gx = std::max(L.gx, conv_wgrad_mma_ctas(h));
                             L.max_elems = std::max<long long>(L.max_elems, (long long)conv_wgrad_mma_smem(h));
                             L.max_b = (int)std::max<long long>(L.max_b, conv_wgrad_mma_out_elems(h));
@@ -675,7 +799,7 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
                         if (k == i) L.first = n_wtc;
                         wtc.resize((size_t)(n_wtc + 1) * wtcb);
                         char* h = wtc.data() + (size_t)n_wtc * wtcb;
-                        if (!conv_wgrad_tc_fill(o.conv, wgrad_target_ctas(ctx, (int)(j - i)), h)) { ctx->err = "tensor map encoding failed"; return RESIST_ECUDA; }
+                        if (!conv_wgrad_tc_fill(o.conv, o.wg_target ? o.wg_target : wgrad_target_ctas(ctx, (int)(j - i)), h)) { ctx->err = "tensor map encoding failed"; return RESIST_ECUDA; }
                         L.gx = std::max(L.gx, conv_wgrad_tc_ctas(h));
                         L.max_elems = std::max<long long>(L.max_elems, (long long)conv_wgrad_tc_smem(h));
                         L.max_b = (int)std::max<long long>(L.max_b, conv_wgrad_tc_out_elems(h));
@@ -777,7 +901,8 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
                     case OP_CONV_FWD: case OP_CONV_DGRAD: wr.push_back(o.conv.out);
                         if (o.fuse == 1) wr.push_back(o.bn.a); else if (o.fuse == 2) wr.push_back(o.bn.dx);
                         break;
-                    case OP_CONV_WGRAD: case OP_SPLITK: case OP_REPACK: break;
+                    case OP_CONV_WGRAD: case OP_SPLITK: case OP_REPACK: case OP_TRAIN_CHAIN_PACK: break;
+                    case OP_TRAIN_CHAIN_FWD: case OP_TRAIN_CHAIN_BWD: for (const TrainLayer& l : o.tlayers) { wr.push_back(l.y); wr.push_back(l.a); } break;
                     case OP_BN_STATS: case OP_BN_BWD_REDUCE: case OP_BN_TILE_STATS: case OP_BN_EVAL_STATS: case OP_BN_BWD_TILE_SUMS: break;
                     case OP_BN_APPLY: case OP_BN_FWD_FUSED: case OP_BN_FWD_SMALL: wr.push_back(o.bn.a); break;
                     case OP_BN_BWD_APPLY: case OP_BN_BWD_FUSED: case OP_BN_BWD_SMALL: wr.push_back(o.bn.dx); break;
@@ -813,11 +938,17 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
     const size_t o_col = off;  off += align_up(col.size() * sizeof(ColProb), 256);
     const size_t o_wmm = off;  off += align_up(wmm.size(), 256);
     const size_t o_chain = off; off += align_up(chain.size() * sizeof(ChainProb), 256);
+    const size_t o_tchain = off; off += align_up(tchain.size() * sizeof(TrainChain), 256);
+    const size_t o_tlayer = off; off += align_up(tlayer.size() * sizeof(TrainLayer), 256);
+    const size_t o_tpack = off; off += align_up(tpack.size() * sizeof(TrainPack), 256);
+    const size_t o_arrive = off; off += align_up(tchain.size() * 32 * sizeof(unsigned), 256);   // a number per chain, 128 bytes apart
     const size_t o_layer = off; off += align_up(layer.size() * sizeof(ChainLayer), 256);
+    std::vector<size_t> o_packets; size_t packets = 0;        // the chains' packets: behind the tables, zeroed, not copied
+    for (const TrainChain& t : tchain) { o_packets.push_back(off + 256 + packets); packets += align_up((size_t)2 * t.ctas * 2 * t.C * sizeof(uint4), 256); }
     if (plan.graph) cudaGraphExecDestroy(plan.graph);
     plan.graph = nullptr; plan.runs = 0; plan.graph_failed = false;
     ctx_free(ctx, plan.d_blob);
-    plan.d_blob = ctx_alloc(ctx, off + 256); plan.blob_bytes = off; plan.d_lr = (float*)((char*)plan.d_blob + off);
+    plan.d_blob = ctx_alloc(ctx, off + 256 + packets); plan.blob_bytes = off; plan.d_lr = (float*)((char*)plan.d_blob + off);
     if (!plan.d_blob) { ctx->err = "allocator returned NULL for the launch plan"; return RESIST_ENOMEM; }
     char* base = (char*)plan.d_blob;
     plan.d_conv = (ConvProb*)(base + o_conv); plan.d_bn = (BnProb*)(base + o_bn); plan.d_pool = (PoolProb*)(base + o_pool);
@@ -850,11 +981,17 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
     plan.d_up = (UpProb*)(base + o_up);
     if (!chain.empty()) memcpy(host.data() + o_chain, chain.data(), chain.size() * sizeof(ChainProb));
     if (!layer.empty()) memcpy(host.data() + o_layer, layer.data(), layer.size() * sizeof(ChainLayer));
+    plan.d_tchain = (TrainChain*)(base + o_tchain); plan.d_tpack = (TrainPack*)(base + o_tpack); plan.d_arrive = (unsigned*)(base + o_arrive); plan.n_arrive = (int)tchain.size() * 32;
+    for (size_t t = 0; t < tchain.size(); ++t) { tchain[t].layers = (const TrainLayer*)(base + o_tlayer) + tfirst[t]; tchain[t].arrive = plan.d_arrive + t * 32; tchain[t].packets = (uint4*)(base + o_packets[t]); tchain[t].status = conv_tc_status_word(); }
+    if (!tchain.empty()) memcpy(host.data() + o_tchain, tchain.data(), tchain.size() * sizeof(TrainChain));
+    if (!tlayer.empty()) memcpy(host.data() + o_tlayer, tlayer.data(), tlayer.size() * sizeof(TrainLayer));
+    if (!tpack.empty()) memcpy(host.data() + o_tpack, tpack.data(), tpack.size() * sizeof(TrainPack));
     plan.d_chain = (ChainProb*)(base + o_chain); plan.d_layer = (ChainLayer*)(base + o_layer);
     if (!mm.empty()) memcpy(host.data() + o_mm, mm.data(), mm.size());
     if (!wmm.empty()) memcpy(host.data() + o_wmm, wmm.data(), wmm.size());
     plan.d_mm = base + o_mm; plan.mm_stride = mmb; plan.d_wmm = base + o_wmm; plan.wmm_stride = wmmb;
     cudaError_t e = cudaMemcpyAsync(plan.d_blob, host.data(), off, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess && packets) e = cudaMemsetAsync(base + off + 256, 0, packets, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) { ctx->err = std::string("plan upload: ") + cudaGetErrorString(e); return RESIST_ECUDA; }
     plan.nsites = (int)dsites.size(); plan.n_sgd_seg = (int)segs.size(); plan.sgd_chunks = chunks;
@@ -965,6 +1102,8 @@ static int enqueue_launches(resist_ctx* ctx, Plan& plan, bool update, bool overl
             case OP_BN_TILE_STATS: case OP_BN_BWD_TILE_SUMS: pk = PK_BN_TILE_STATS; break;
             case OP_BN_BWD_FUSED: case OP_BN_BWD_SMALL: pk = PK_BN_BWD_FUSED; break;
             case OP_EVAL_CHAIN_PACK: case OP_EVAL_CHAIN: pk = PK_EVAL_CHAIN; break;
+            case OP_TRAIN_CHAIN_PACK: case OP_TRAIN_CHAIN_FWD: pk = PK_TRAIN_CHAIN_FWD; break;
+            case OP_TRAIN_CHAIN_BWD: pk = PK_TRAIN_CHAIN_BWD; break;
         }
         pf.begin(pk, nk, L.bytes, L.flops, st, L.label);
         switch (L.kind) {
@@ -994,6 +1133,10 @@ static int enqueue_launches(resist_ctx* ctx, Plan& plan, bool update, bool overl
             case OP_HEAD_FWD: n_launch += launch_head_fwd(plan.d_head + L.first, L.count, L.max_b, L.max_c, L.max_classes, bf, st); break;
             case OP_HEAD_BWD: n_launch += launch_head_bwd(plan.d_head + L.first, L.count, L.max_b, L.max_c, L.max_classes, L.max_elems, bf, st); break;
             case OP_UPSAMPLE: launch_zero_stuff(plan.d_up + L.first, L.count, L.max_elems, st); ++n_launch; break;
+            case OP_TRAIN_CHAIN_PACK: launch_train_chain_pack(plan.d_tpack + L.first, L.count, L.max_c, plan.d_arrive, plan.n_arrive, st); ++n_launch; break;
+            case OP_TRAIN_CHAIN_FWD: case OP_TRAIN_CHAIN_BWD:
+                if (!launch_train_chain(plan.d_tchain + L.first, L.count, L.max_c, L.kind == OP_TRAIN_CHAIN_BWD, L.gx, L.smem, st)) { ctx->err = "training chain launch failed"; cudaGetLastError(); return RESIST_ECUDA; }
+                ++n_launch; break;
             case OP_EVAL_CHAIN_PACK: launch_eval_chain_pack(plan.d_layer + L.first, L.count, L.max_c, st); ++n_launch; break;
             case OP_EVAL_CHAIN:
                 if (!launch_eval_chain(plan.d_chain + L.first, L.chain, st)) { ctx->err = "evaluation chain launch failed"; return RESIST_ECUDA; }

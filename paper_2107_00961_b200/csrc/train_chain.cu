@@ -1,0 +1,384 @@
+// Training through a run of identity basic blocks of a narrow stage: one launch forward, one backward (Algorithm 1, inner loop; Sec. 2.1).
+//
+// At these sizes a layer is a few microseconds of work, and a launch per layer spends most of its time on what does not depend on the work: tables, the
+// filter, the first window, a grid barrier, the re-added sums, a pass over a tensor that has just been written.  Here the images of a sub-ResNet are dealt out to
+// CTAs, one CTA per SM, and stay in shared memory through all layers of the run; what remains per layer is the convolution on them, the sums the BN
+// needs, a barrier among the CTAs of THIS sub-ResNet (they alone share its statistics; different sub-ResNets run through their blocks at
+// their own pace), and an elementwise pass in shared memory that also writes what the other direction or the weight gradients read.
+//
+// A layer is a convolution and the BN + ReLU behind it.  Forward: y = conv(a) (+ x), then a' = relu(bn(y)); y and a' are stored.  Backward: da = conv^T(dy), then dx =
+// backward of the BN whose output gradient da is (+ the skip path's gradient); dx is stored, and is the next layer's dy.  Rounding points are those of the
+// kernels per layer: y, a', da and dx are bf16, sums are of the rounded values, in fp32 over one task (8 values), in double from there on.
+//
+// The exchange: a CTA's sums go to every other CTA of its sub-ResNet as 16-byte packets of a double's halves, each beside the number of the layer, and are
+// polled for where they are added; the packets are data and barrier in one, and no fence has to wait for the tensors being written meanwhile.  (A
+// counter with release and acquire, then the sums: 10.5 us per layer where a worker has an image per CTA, 9.0 now.)  Two buffers by parity: a
+// CTA that writes layer l + 2 has read everyone's l + 1, who had all read l.
+//
+// In place: the warps compute a round of tasks (at most one each), keep the rounded results in 16 registers, and store them over the round's input once
+// every warp has arrived at the round's mbarrier, which it does as soon as its MMAs have read the input.  The residual (forward) or the BN's input (backward) of a task comes by cp.async into the warp's own 2 KB while it
+// computes.  Layout of an image and the convolution on it: chain_core.h.
+//
+// Measured, us per step: ResNet-110, 4 x 128 images of 32 x 32 (a launch per layer and direction before) 3290 -> 2440; one worker's 84 images 1160 -> 818; 256
+// images and all 54 blocks in one network 6720 -> 3684.
+#include <algorithm>
+#include <vector>
+#include "chain_core.h"
+
+namespace resist {
+using namespace chain;
+
+constexpr int TRAIN_THREADS = 512, TRAIN_WARPS = 16, STAGE_BYTES = 2048, TRAIN_MAX_ROUNDS = 32, TRAIN_MAX_LAYERS = 64;
+
+// Filters of the bf16 copy in fragment order, for the forward convolution and for the data gradient (channels exchanged, taps reversed); the chains' packets of
+// this step are numbered from 256 further on.
+__global__ void __launch_bounds__(256) train_chain_pack_kernel(const TrainPack* __restrict__ packs, unsigned* __restrict__ counters, int ncounters) {
+    if (blockIdx.x == 0 && blockIdx.y == 0) for (int i = threadIdx.x; i < ncounters; i += 256) counters[i] += 256u;
+    const TrainPack l = packs[blockIdx.y];
+    const int C = l.C, steps = C / 16;
+    const unsigned short* __restrict__ w = reinterpret_cast<const unsigned short*>(l.w);
+    for (int i = blockIdx.x * 256 + threadIdx.x; i < steps * steps * 9 * 32; i += gridDim.x * 256) {
+        const int lane = i & 31, t = (i >> 5) % 9, kn = (i >> 5) / 9, k = kn % steps, n = kn / steps, g8 = lane >> 2, t4 = lane & 3;
+        uint32_t f[4], d[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {                             // j: (column block, upper half of the 16 reduction channels)
+            const int out = n * 16 + (g8 >> 1) * 4 + 2 * (j >> 1) + (g8 & 1), in = k * 16 + t4 * 2 + 8 * (j & 1);
+            f[j] = (uint32_t)w[(out * 9 + t) * C + in] | ((uint32_t)w[(out * 9 + t) * C + in + 1] << 16);
+            d[j] = (uint32_t)w[(in * 9 + 8 - t) * C + out] | ((uint32_t)w[((in + 1) * 9 + 8 - t) * C + out] << 16);
+        }
+        l.fwd[i] = make_uint4(f[0], f[1], f[2], f[3]); l.bwd[i] = make_uint4(d[0], d[1], d[2], d[3]);
+    }
+}
+
+__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) { asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory"); }
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) { asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory"); }
+__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok != 0;
+}
+__device__ __forceinline__ uint4 ld_poll(const uint4* p) { uint4 v; asm volatile("ld.volatile.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory"); return v; }
+__device__ __forceinline__ void st_packet(uint4* p, double a, uint32_t n) {
+    asm volatile("st.volatile.global.v4.u32 [%0], {%1,%2,%3,%4};" ::"l"(p), "r"((uint32_t)__double2loint(a)), "r"(n), "r"((uint32_t)__double2hiint(a)), "r"(n) : "memory");
+}
+__device__ __forceinline__ void cp16(uint32_t dst, const void* src) { asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory"); }
+
+template <int C, bool BWD>
+__global__ void __launch_bounds__(TRAIN_THREADS, 1) train_chain_kernel(const TrainChain* __restrict__ probs, int nprob) {
+    constexpr int NG = C / 16, G = C / 8;
+    extern __shared__ __align__(128) uint8_t sm[];
+    __shared__ double s_red[TRAIN_WARPS][2][16];                  // a warp's sums of its sixteen channels over the layer
+    __shared__ double s_sum[TRAIN_THREADS];
+    __shared__ __align__(16) float s_bn2[2][6][C];                // by parity of the layer: -mean, 1/std, gamma, beta; backward: sum dz / m, sum dz * xhat / m
+    __shared__ int s_abort;
+    __shared__ __align__(8) uint64_t s_bar[TRAIN_MAX_ROUNDS];     // per round: the warps whose MMAs have read its input
+    int pi = 0; while (pi + 1 < nprob && (int)blockIdx.x >= probs[pi + 1].cta0) ++pi;
+    const TrainChain& pr = probs[pi];
+    const int N = pr.N, H = pr.H, W = pr.W, HW = H * W, Wp = W + 1, ctas = pr.ctas, cta = (int)blockIdx.x - pr.cta0, layers = pr.nlayers;
+    const int cols = pr.map.cols, trows = pr.map.rows, slot_imgs = pr.map.slot, strips = pr.map.strips, xblocks = pr.map.xblocks;
+    const int imgs = pr.imgs, img0 = cta * imgs, n_img = min(imgs, N - img0);
+    const uint32_t plane = (uint32_t)pr.map.plane, img_bytes = G * plane, row_bytes = (uint32_t)Wp * 16u;
+    uint4* const packets = pr.packets; const uint32_t number0 = __ldg(pr.arrive);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g8 = lane >> 2, t4 = lane & 3;
+    uint8_t* const s_stage = sm + imgs * img_bytes + warp * STAGE_BYTES;
+    TrainLayer* const lays = reinterpret_cast<TrainLayer*>(sm + imgs * img_bytes + TRAIN_WARPS * STAGE_BYTES);
+    for (int i = tid; i < layers * (int)(sizeof(TrainLayer) / 8); i += TRAIN_THREADS) reinterpret_cast<uint64_t*>(lays)[i] = __ldg(reinterpret_cast<const uint64_t*>(pr.layers) + i);
+    if (tid < TRAIN_MAX_ROUNDS) mbar_init(sm_u32(&s_bar[tid]), TRAIN_WARPS);
+    const double m = (double)N * HW; const float inv_m = 1.f / (float)((long long)N * HW);
+
+    // ---- zero the maps, then the input of the first convolution
+    for (uint32_t i = tid * 16; i < imgs * img_bytes; i += TRAIN_THREADS * 16) *reinterpret_cast<uint4*>(sm + i) = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = tid; i < TRAIN_WARPS * 32; i += TRAIN_THREADS) (&s_red[0][0][0])[i] = 0.0;
+    if (tid == 0) s_abort = 0;
+    __syncthreads();
+    // rows of the CTA's images, a warp per row; chunk i of a row: pixel i / G, group i % G = lane % G
+    const int all_rows = n_img * H, row_chunks = W * G;
+    for (int r = warp; r < all_rows; r += TRAIN_WARPS) {
+        const int im = r / H, y = r - im * H;
+        const uint4* src = reinterpret_cast<const uint4*>(pr.in + ((long long)(img0 + im) * HW + y * W) * C);
+        uint8_t* d = sm + im * img_bytes + (lane % G) * plane + ((y + 1) * Wp + 1) * 16;
+        for (int i = lane; i < row_chunks; i += 32) *reinterpret_cast<uint4*>(d + (i / G) * 16) = __ldg(src + i);
+    }
+
+    // ---- this warp's place in a round of tasks: slot and block of positions are the same in every round but for the slot's number
+    const int tps = NG * strips * xblocks, spr = TRAIN_WARPS / tps, wslot = warp / tps, wt = warp - wslot * tps;
+    const bool on = wslot < spr;
+    const int ng = wt % NG, x0 = wt / NG % xblocks * cols, y0 = wt / NG / xblocks * trows;
+    const int dx = cols == 16 ? 8 : 0, dy = trows == 8 ? 4 : 0, di = slot_imgs - 1;
+    const uint32_t half = di ? img_bytes : (uint32_t)(dx * 16) + (uint32_t)dy * row_bytes;
+    const uint32_t a_lane = sm_u32(sm) + (uint32_t)(lane >> 4) * plane + (uint32_t)((lane >> 3) & 1) * half + (uint32_t)(lane & 7) * 16u + (uint32_t)(y0 * Wp + x0) * 16u;
+    const int slots = (imgs + di) / slot_imgs, rounds = (slots + spr - 1) / spr;
+    const int c0 = ng * 16 + t4 * 4;                              // the thread's four channels
+    // rows of either half that are of the map at this thread's column
+    int vrows[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) vrows[h] = x0 + g8 + dx * h < W ? min(R, H - y0 - dy * h) : 0;
+
+    uint4 b[3][3];
+    auto frag = [&](int l, int k, int r) { load_frag<NG>(b, lays[min(l, layers - 1)].wpk, lane, 0, ng, k, r); };
+    if (on) { frag(0, 0, 0); frag(0, 0, 1); frag(0, 0, 2); }
+    for (int l = 0; l < layers; ++l) {
+        const TrainLayer& L = lays[l];
+        float (*const s_bn)[C] = s_bn2[l & 1];                    // a warp may still be reading the last layer's
+        const __nv_bfloat16* const extra = BWD ? L.x : L.res;     // read per task: the BN's input, or the residual
+        // constants of the BN: backward needs them in the epilogue, forward behind the exchange (asked for now, as are the running statistics)
+        float k0 = 0.f, k1 = 0.f, k2 = 0.f, k3 = 0.f;
+        if (tid < C) {
+            k2 = __ldg(L.gamma + tid); k3 = __ldg(L.beta + tid);
+            if (BWD) { s_bn[0][tid] = -__ldcg(L.stat + tid); s_bn[1][tid] = __ldcg(L.stat + C + tid); s_bn[2][tid] = k2; s_bn[3][tid] = k3; }
+            else if (cta == 0) { k0 = __ldcg(L.run_mean + tid); k1 = __ldcg(L.run_var + tid); }
+        }
+        __syncthreads();                                          // the layer's input (and constants) are in shared memory
+        for (int rd = 0; rd < rounds; ++rd) {
+            const int im = (rd * spr + wslot) * slot_imgs;        // first image of the task
+            const bool work = on && im < n_img;
+            const bool have1 = im + di < n_img;                   // the second image of a pair exists
+            uint32_t y[2 * R][2];
+            if (work) {
+                if (extra) {
+                    // 128 chunks [half][row][column][16-byte part]; the ones outside the map are left as they are and not used
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int c = lane + 32 * j, part = c & 1, px = (c >> 1) & 7, o = (c >> 4) & 3, h = c >> 6;
+                        const int yy = y0 + o + dy * h, xx = x0 + px + dx * h;
+                        if (yy < H && xx < W && (h == 0 || have1))
+                            cp16(sm_u32(s_stage) + c * 16, extra + ((long long)(img0 + im + di * h) * HW + yy * W + xx) * C + ng * 16 + part * 8);
+                    }
+                    asm volatile("cp.async.commit_group;" ::: "memory");
+                }
+                float acc[R][2][4];
+                const bool next_round = ((rd + 1) * spr + wslot) * slot_imgs < n_img;       // of this warp
+                conv_task<NG>(acc, b, a_lane + im * img_bytes, row_bytes, plane, [&](int k, int r) {
+                    const bool end = k == NG - 1;
+                    if (NG > 1 || !next_round) frag(end && !next_round ? l + 1 : l, end ? 0 : k + 1, r);
+                });
+                __syncwarp();
+                if (lane == 0) mbar_arrive(sm_u32(&s_bar[rd]));
+                if (extra) { asm volatile("cp.async.wait_group 0;" ::: "memory"); __syncwarp(); }
+                // ---- epilogue: thread (g8, t4) holds column g8 of both halves of each row, channels c0 .. c0 + 3
+                uint64_t s0 = 0, s1 = 0, q0 = 0, q1 = 0;
+                const int pix0 = y0 * W + x0 + g8;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int rows = h == 1 && !have1 ? 0 : vrows[h];
+                    __nv_bfloat16* const yo = BWD ? nullptr : L.y + ((long long)(img0 + im + di * h) * HW + pix0 + dx * h + dy * h * W) * C + c0;
+#pragma unroll
+                    for (int o = 0; o < R; ++o) {
+                        uint64_t v0 = v2(acc[o][0][2 * h], acc[o][0][2 * h + 1]), v1 = v2(acc[o][1][2 * h], acc[o][1][2 * h + 1]);
+                        uint2 e = make_uint2(0u, 0u);
+                        if (extra) e = *reinterpret_cast<const uint2*>(s_stage + ((h * R + o) * 8 + g8) * 32 + t4 * 8);
+                        if (!BWD && extra) { v0 = add2(v0, of_bf2(e.x)); v1 = add2(v1, of_bf2(e.y)); }
+                        const uint2 w = make_uint2(to_bf2(v0), to_bf2(v1));
+                        y[h * R + o][0] = w.x; y[h * R + o][1] = w.y;
+                        if (o >= rows) continue;
+                        if (!BWD) {
+                            *reinterpret_cast<uint2*>(yo + o * W * C) = w;
+                            const uint64_t r0 = of_bf2(w.x), r1 = of_bf2(w.y);
+                            s0 = add2(s0, r0); s1 = add2(s1, r1); q0 = fma2(r0, r0, q0); q1 = fma2(r1, r1, q1);
+                        } else {
+                            const ulonglong2 nm = *reinterpret_cast<const ulonglong2*>(&s_bn[0][c0]), is = *reinterpret_cast<const ulonglong2*>(&s_bn[1][c0]);
+                            const ulonglong2 ga = *reinterpret_cast<const ulonglong2*>(&s_bn[2][c0]), be = *reinterpret_cast<const ulonglong2*>(&s_bn[3][c0]);
+                            const uint64_t h0 = mul2(add2(of_bf2(e.x), nm.x), is.x), h1 = mul2(add2(of_bf2(e.y), nm.y), is.y);
+                            float z0, z1, z2, z3; un2(fma2(h0, ga.x, be.x), z0, z1); un2(fma2(h1, ga.y, be.y), z2, z3);
+                            const uint64_t d0 = of_bf2(w.x & ((z0 > 0.f ? 0x0000FFFFu : 0u) | (z1 > 0.f ? 0xFFFF0000u : 0u)));
+                            const uint64_t d1 = of_bf2(w.y & ((z2 > 0.f ? 0x0000FFFFu : 0u) | (z3 > 0.f ? 0xFFFF0000u : 0u)));
+                            s0 = add2(s0, d0); s1 = add2(s1, d1); q0 = fma2(d0, h0, q0); q1 = fma2(d1, h1, q1);
+                        }
+                    }
+                }
+                // the eight lanes of the same channels, fixed butterfly; the first keeps the warp's running sums
+                float f[8]; un2(s0, f[0], f[1]); un2(s1, f[2], f[3]); un2(q0, f[4], f[5]); un2(q1, f[6], f[7]);
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+#pragma unroll
+                    for (int off = 4; off < 32; off <<= 1) f[i] += __shfl_xor_sync(0xffffffffu, f[i], off);
+                if (g8 == 0)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) { s_red[warp][0][t4 * 4 + i] += (double)f[i]; s_red[warp][1][t4 * 4 + i] += (double)f[4 + i]; }
+            }
+            else if (lane == 0) mbar_arrive(sm_u32(&s_bar[rd]));
+            if (work) {
+                // every warp has arrived at its own pace; bounded like every wait
+                for (uint32_t i = 0; !mbar_try(sm_u32(&s_bar[rd]), (uint32_t)l & 1u); ++i) if (i > (1u << 22)) { s_abort = 1; break; }
+                uint8_t* const d = sm + im * img_bytes + (ng * 2 + (t4 >> 1)) * plane + ((y0 + 1) * Wp + x0 + 1 + g8) * 16 + (t4 & 1) * 8;
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int o = 0; o < R; ++o)
+                        if (o < vrows[h]) *reinterpret_cast<uint2*>(d + (h ? half : 0u) + o * row_bytes) = make_uint2(y[h * R + o][0], y[h * R + o][1]);
+            }
+        }
+        __syncthreads();
+        // ---- this CTA's sums, warps in order, as packets; then everyone's, in the same order everywhere
+        uint4* const box = packets + (long long)(l & 1) * ctas * 2 * C;
+        const uint32_t number = number0 + (uint32_t)l + 1u;
+        if (tid < 2 * C) {
+            const int k = tid / C, c = tid % C;
+            double a = 0.0;
+            for (int w = c / 16; w < spr * tps; w += NG) a += s_red[w][k][c & 15];      // the warps of the channel's group (tps is a multiple of the groups)
+            st_packet(box + (long long)cta * 2 * C + tid, a, number);
+        }
+        {
+            constexpr int Q = TRAIN_THREADS / (2 * C);
+            const int q = tid / (2 * C), c2 = tid % (2 * C);
+            double a = 0.0; bool ok = true;
+            for (int k = q; k < ctas && ok; k += 4 * Q) {
+                uint4 v[4];
+                for (uint32_t i = 0;; ++i) {
+                    bool all = true;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) v[u] = ld_poll(box + (long long)min(k + u * Q, ctas - 1) * 2 * C + c2);      // past the end: the last one again, not added
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) all &= v[u].y == number && v[u].w == number;
+                    if (all) break;
+                    if (i > (1u << 20)) { ok = false; break; }
+                    if (i > 256) __nanosleep(100);
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) if (k + u * Q < ctas) a += __hiloint2double((int)v[u].z, (int)v[u].x);
+            }
+            s_sum[tid] = a;
+            if (!ok) { s_abort = 1; *(volatile int*)pr.status = 21; __threadfence_system(); }
+            __syncthreads();
+            if (s_abort) return;                                  // the same for all: written before the barrier only
+            for (int i = tid; i < TRAIN_WARPS * 32; i += TRAIN_THREADS) (&s_red[0][0][0])[i] = 0.0;
+            if (tid < C) {
+                const int c = tid;
+                double t0 = 0.0, t1 = 0.0;
+#pragma unroll
+                for (int u = 0; u < Q; ++u) { t0 += s_sum[u * 2 * C + c]; t1 += s_sum[u * 2 * C + C + c]; }
+                if (!BWD) {
+                    const double mean = t0 / m; double var = t1 / m - mean * mean; if (var < 0.0) var = 0.0;
+                    const float fm = (float)mean, fi = (float)(1.0 / sqrt(var + (double)pr.eps));
+                    s_bn[0][c] = -fm; s_bn[1][c] = fi; s_bn[2][c] = k2; s_bn[3][c] = k3;
+                    if (cta == 0) {
+                        L.stat[c] = fm; L.stat[C + c] = fi;
+                        const double unb = m > 1.0 ? var * m / (m - 1.0) : var, mo = (double)pr.momentum;
+                        L.run_mean[c] = (float)((1.0 - mo) * (double)k0 + mo * mean);
+                        L.run_var[c] = (float)((1.0 - mo) * (double)k1 + mo * unb);
+                    }
+                } else {
+                    const float b0 = (float)t0, b1 = (float)t1;
+                    s_bn[4][c] = b0 * inv_m; s_bn[5][c] = b1 * inv_m;
+                    if (cta == 0) { L.stat[2 * C + c] = b0; L.stat[3 * C + c] = b1; L.dbeta[c] = b0; L.dgamma[c] = b1; }
+                }
+            }
+            __syncthreads();
+        }
+        // ---- elementwise pass in place: 8 channels per access, two pixels at a time; the constants are read where they are used
+        {
+            const int g = lane % G;
+            const uint64_t* const cst = reinterpret_cast<const uint64_t*>(&s_bn[0][g * 8]);
+            for (int r = warp; r < all_rows; r += TRAIN_WARPS) {
+                const int im = r / H, yy = r - im * H;
+                const long long at = ((long long)(img0 + im) * HW + yy * W) * C;
+                uint8_t* const d = sm + im * img_bytes + g * plane + ((yy + 1) * Wp + 1) * 16;
+                uint4* const out = reinterpret_cast<uint4*>(L.a + at);
+                const uint4* const xv = BWD ? reinterpret_cast<const uint4*>(L.x + at) : nullptr;
+                const uint4* const av = BWD && L.res ? reinterpret_cast<const uint4*>(L.res + at) : nullptr;
+                for (int i0 = lane; i0 < row_chunks; i0 += 64) {
+                    uint32_t v[2][4], x[2][4], e[2][4], o[2][4]; uint8_t* sp[2];
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        const int i = i0 + 32 * u < row_chunks ? i0 + 32 * u : i0;
+                        if (BWD) {
+                            const uint4 t = __ldcg(xv + i); x[u][0] = t.x; x[u][1] = t.y; x[u][2] = t.z; x[u][3] = t.w;
+                            if (av) { const uint4 w = __ldcg(av + i); e[u][0] = w.x; e[u][1] = w.y; e[u][2] = w.z; e[u][3] = w.w; }
+                        }
+                        sp[u] = d + (i / G) * 16;
+                        const uint4 t = *reinterpret_cast<const uint4*>(sp[u]); v[u][0] = t.x; v[u][1] = t.y; v[u][2] = t.z; v[u][3] = t.w;
+                    }
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const uint64_t nm = cst[k], is = cst[C / 2 + k], ga = cst[C + k], be = cst[3 * C / 2 + k];
+                        if (!BWD) { o[0][k] = bn_relu2(v[0][k], nm, is, ga, be); o[1][k] = bn_relu2(v[1][k], nm, is, ga, be); }
+                        else {
+                            const uint64_t nsb = cst[2 * C + k] ^ 0x8000000080000000ull, nsg = cst[5 * C / 2 + k] ^ 0x8000000080000000ull, gi = mul2(ga, is);
+#pragma unroll
+                            for (int u = 0; u < 2; ++u) {
+                                const uint64_t xh = mul2(add2(of_bf2(x[u][k]), nm), is);
+                                float z0, z1; un2(fma2(xh, ga, be), z0, z1);
+                                const uint64_t dz = of_bf2(v[u][k] & ((z0 > 0.f ? 0x0000FFFFu : 0u) | (z1 > 0.f ? 0xFFFF0000u : 0u)));
+                                uint64_t t = mul2(gi, fma2(xh, nsg, add2(dz, nsb)));
+                                if (av) t = add2(t, of_bf2(e[u][k]));
+                                o[u][k] = to_bf2(t);
+                            }
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        if (i0 + 32 * u >= row_chunks) break;
+                        const uint4 w = make_uint4(o[u][0], o[u][1], o[u][2], o[u][3]);
+                        *reinterpret_cast<uint4*>(sp[u]) = w; out[i0 + 32 * u] = w;
+                    }
+                }
+            }
+        }
+    }
+}
+
+// ------------------------------------------------------------------------------------------------ host side
+// The form of a task with the fewest blocks of positions per image among those of which a round of sixteen warps takes a whole slot.
+bool train_chain_geometry(int C, int H, int W, ChainMap& best) {
+    if ((C != 16 && C != 32 && C != 64) || H < 2 || W < 2 || H > 64 || W > 64) return false;
+    double least = 0;
+    for (int mode = 0; mode < 3; ++mode) {
+        const ChainMap m = chain_map(H, W, mode);
+        const int tps = C / 16 * m.strips * m.xblocks;
+        if (tps > TRAIN_WARPS) continue;
+        const double cost = 1.0 / (TRAIN_WARPS / tps * m.slot);
+        if (least == 0 || cost < least) { least = cost; best = m; }
+    }
+    return least > 0;
+}
+constexpr size_t TRAIN_SMEM = 214 * 1024, TRAIN_FIXED = TRAIN_WARPS * STAGE_BYTES + TRAIN_MAX_LAYERS * sizeof(TrainLayer);      // 11 KB more are static
+static size_t train_smem(int C, const ChainMap& m, int imgs) { return (size_t)imgs * (C / 8) * m.plane + TRAIN_FIXED; }
+int train_chain_max_layers() { return TRAIN_MAX_LAYERS; }
+// images a CTA can hold
+int train_chain_max_imgs(int C, const ChainMap& m) {
+    const int tps = C / 16 * m.strips * m.xblocks, spr = TRAIN_WARPS / tps;
+    const int n = std::min((int)((TRAIN_SMEM - TRAIN_FIXED) / ((size_t)(C / 8) * m.plane)), TRAIN_MAX_ROUNDS * spr * m.slot);
+    return n / m.slot * m.slot;
+}
+// Deals the SMs to the problems of a launch: images per CTA so that all CTAs fit, with the least time of the slowest problem, a layer taken as a fixed part (barrier, sums)
+// of about four images' worth and its rounds.
+bool train_chain_assign(TrainChain* p, int n, int sms) {
+    auto rounds = [](const TrainChain& t, int imgs) { const int tps = t.C / 16 * t.map.strips * t.map.xblocks, spr = TRAIN_WARPS / tps; return ((imgs + t.map.slot - 1) / t.map.slot + spr - 1) / spr; };
+    const int cap = train_chain_max_imgs(p[0].C, p[0].map);
+    if (cap < 1) return false;
+    std::vector<int> k(n, p[0].map.slot);
+    auto ctas = [&](int i) { return (p[i].N + k[i] - 1) / k[i]; };
+    for (;;) {
+        int total = 0; for (int i = 0; i < n; ++i) total += ctas(i);
+        if (total <= sms) break;
+        int who = -1; double least = 0;                           // the problem whose time stays lowest with another slot per CTA
+        for (int i = 0; i < n; ++i) {
+            if (k[i] + p[i].map.slot > cap) continue;
+            const double t = p[i].nlayers * (4.0 + rounds(p[i], k[i] + p[i].map.slot) * 1.0);
+            if (who < 0 || t < least) { who = i; least = t; }
+        }
+        if (who < 0) return false;
+        k[who] += p[who].map.slot;
+    }
+    int at = 0;
+    for (int i = 0; i < n; ++i) { p[i].imgs = k[i]; p[i].ctas = ctas(i); p[i].cta0 = at; at += p[i].ctas; }
+    return true;
+}
+size_t train_chain_launch_smem(const TrainChain* p, int n) { size_t s = 0; for (int i = 0; i < n; ++i) s = std::max(s, train_smem(p[i].C, p[i].map, p[i].imgs)); return s; }
+void launch_train_chain_pack(const TrainPack* d, int n, int max_c, unsigned* counters, int ncounters, cudaStream_t s) {
+    const int steps = max_c / 16;
+    train_chain_pack_kernel<<<dim3((steps * steps * 9 * 32 + 255) / 256, n), 256, 0, s>>>(d, counters, ncounters);
+}
+template <int C, bool BWD> static bool launch_chain(const TrainChain* d, int nprob, int ctas, size_t smem, cudaStream_t s) {
+    if (cudaFuncSetAttribute(train_chain_kernel<C, BWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TRAIN_SMEM) != cudaSuccess) { cudaGetLastError(); return false; }
+    cudaLaunchConfig_t cfg = {}; cfg.gridDim = dim3(ctas); cfg.blockDim = dim3(TRAIN_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = s;
+    cudaLaunchAttribute at[1]; at[0].id = cudaLaunchAttributeCooperative; at[0].val.cooperative = 1; cfg.attrs = at; cfg.numAttrs = 1;      // its CTAs wait for one another
+    return cudaLaunchKernelEx(&cfg, train_chain_kernel<C, BWD>, d, nprob) == cudaSuccess;
+}
+bool launch_train_chain(const TrainChain* d, int nprob, int C, bool backward, int ctas, size_t smem, cudaStream_t s) {
+    if (C == 16) return backward ? launch_chain<16, true>(d, nprob, ctas, smem, s) : launch_chain<16, false>(d, nprob, ctas, smem, s);
+    if (C == 32) return backward ? launch_chain<32, true>(d, nprob, ctas, smem, s) : launch_chain<32, false>(d, nprob, ctas, smem, s);
+    return backward ? launch_chain<64, true>(d, nprob, ctas, smem, s) : launch_chain<64, false>(d, nprob, ctas, smem, s);
+}
+
+}  // namespace resist
