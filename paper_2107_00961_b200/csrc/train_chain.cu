@@ -12,15 +12,15 @@
 //
 // The exchange: a CTA's sums go to every other CTA of its sub-ResNet as 16-byte packets of a double's halves, each beside the number of the layer, and are
 // polled for where they are added; the packets are data and barrier in one, and no fence has to wait for the tensors being written meanwhile.  (A
-// counter with release and acquire, then the sums: 10.5 us per layer where a worker has an image per CTA, 9.0 now.)  Two buffers by parity: a
+// counter with release and acquire, then the sums: 10.5 us per layer where a worker has an image per CTA, 8.2 now.)  Two buffers by parity: a
 // CTA that writes layer l + 2 has read everyone's l + 1, who had all read l.
 //
 // In place: the warps compute a round of tasks (at most one each), keep the rounded results in 16 registers, and store them over the round's input once
 // every warp has arrived at the round's mbarrier, which it does as soon as its MMAs have read the input.  The residual (forward) or the BN's input (backward) of a task comes by cp.async into the warp's own 2 KB while it
 // computes.  Layout of an image and the convolution on it: chain_core.h.
 //
-// Measured, us per step: ResNet-110, 4 x 128 images of 32 x 32 (a launch per layer and direction before) 3290 -> 2440; one worker's 84 images 1160 -> 818; 256
-// images and all 54 blocks in one network 6720 -> 3684.
+// Measured, us per step: ResNet-110, 4 x 128 images of 32 x 32 (a launch per layer and direction before) 3290 -> 2353; one worker's 84 images 1160 -> 807; 256
+// images and all 54 blocks in one network 6720 -> 3760.
 #include <algorithm>
 #include <vector>
 #include "chain_core.h"
@@ -28,7 +28,7 @@
 namespace resist {
 using namespace chain;
 
-constexpr int TRAIN_THREADS = 512, TRAIN_WARPS = 16, STAGE_BYTES = 2048, TRAIN_MAX_ROUNDS = 32, TRAIN_MAX_LAYERS = 64;
+constexpr int TRAIN_THREADS = 512, TRAIN_WARPS = 16, STAGE_BYTES = 2048, TRAIN_MAX_ROUNDS = 32, TRAIN_MAX_LAYERS = 48;
 
 // Filters of the bf16 copy in fragment order, for the forward convolution and for the data gradient (channels exchanged, taps reversed); the chains' packets of
 // this step are numbered from 256 further on.
@@ -69,7 +69,8 @@ __global__ void __launch_bounds__(TRAIN_THREADS, 1) train_chain_kernel(const Tra
     extern __shared__ __align__(128) uint8_t sm[];
     __shared__ double s_red[TRAIN_WARPS][2][16];                  // a warp's sums of its sixteen channels over the layer
     __shared__ double s_sum[TRAIN_THREADS];
-    __shared__ __align__(16) float s_bn2[2][6][C];                // by parity of the layer: -mean, 1/std, gamma, beta; backward: sum dz / m, sum dz * xhat / m
+    // by parity of the layer.  Forward: -mean, gamma / std, beta.  Backward: -mean, 1/std, gamma, beta, sum dz / m, sum dz * xhat / m
+    __shared__ __align__(16) float s_bn2[2][6][C];
     __shared__ int s_abort;
     __shared__ __align__(8) uint64_t s_bar[TRAIN_MAX_ROUNDS];     // per round: the warps whose MMAs have read its input
     int pi = 0; while (pi + 1 < nprob && (int)blockIdx.x >= probs[pi + 1].cta0) ++pi;
@@ -81,10 +82,12 @@ __global__ void __launch_bounds__(TRAIN_THREADS, 1) train_chain_kernel(const Tra
     uint4* const packets = pr.packets; const uint32_t number0 = __ldg(pr.arrive);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g8 = lane >> 2, t4 = lane & 3;
     uint8_t* const s_stage = sm + imgs * img_bytes + warp * STAGE_BYTES;
-    TrainLayer* const lays = reinterpret_cast<TrainLayer*>(sm + imgs * img_bytes + TRAIN_WARPS * STAGE_BYTES);
+    uint8_t* const s_w = sm + imgs * img_bytes + TRAIN_WARPS * STAGE_BYTES;       // the layer's filter in fragment order
+    TrainLayer* const lays = reinterpret_cast<TrainLayer*>(s_w + 18 * C * C);
     for (int i = tid; i < layers * (int)(sizeof(TrainLayer) / 8); i += TRAIN_THREADS) reinterpret_cast<uint64_t*>(lays)[i] = __ldg(reinterpret_cast<const uint64_t*>(pr.layers) + i);
     if (tid < TRAIN_MAX_ROUNDS) mbar_init(sm_u32(&s_bar[tid]), TRAIN_WARPS);
-    const double m = (double)N * HW; const float inv_m = 1.f / (float)((long long)N * HW);
+    const double inv_md = 1.0 / ((double)N * HW), unbiased = (double)N * HW / ((double)N * HW > 1.0 ? (double)N * HW - 1.0 : 1.0);
+    const float inv_m = 1.f / (float)((long long)N * HW);
 
     // ---- zero the maps, then the input of the first convolution
     for (uint32_t i = tid * 16; i < imgs * img_bytes; i += TRAIN_THREADS * 16) *reinterpret_cast<uint4*>(sm + i) = make_uint4(0u, 0u, 0u, 0u);
@@ -99,6 +102,22 @@ __global__ void __launch_bounds__(TRAIN_THREADS, 1) train_chain_kernel(const Tra
         uint8_t* d = sm + im * img_bytes + (lane % G) * plane + ((y + 1) * Wp + 1) * 16;
         for (int i = lane; i < row_chunks; i += 32) *reinterpret_cast<uint4*>(d + (i / G) * 16) = __ldg(src + i);
     }
+    auto fetch_filter = [&](int l) {
+        const uint8_t* w = reinterpret_cast<const uint8_t*>(lays[l].wpk);
+        for (int i = tid; i < 18 * C * C / 16; i += TRAIN_THREADS) cp16(sm_u32(s_w) + i * 16, w + i * 16);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    // the BN constants a layer's epilogue (backward) or elementwise pass (forward) needs, by the threads that finish the sums: thread 8c for channel c
+    const bool fin = (tid & 7) == 0 && tid < 8 * C;
+    const int fc = tid >> 3;
+    auto backward_constants = [&](int l) {
+        if (fin) {
+            float (*const d)[C] = s_bn2[l & 1];
+            d[0][fc] = -__ldcg(lays[l].stat + fc); d[1][fc] = __ldcg(lays[l].stat + C + fc); d[2][fc] = __ldg(lays[l].gamma + fc); d[3][fc] = __ldg(lays[l].beta + fc);
+        }
+    };
+    fetch_filter(0);
+    if (BWD) backward_constants(0);
 
     // ---- this warp's place in a round of tasks: slot and block of positions are the same in every round but for the slot's number
     const int tps = NG * strips * xblocks, spr = TRAIN_WARPS / tps, wslot = warp / tps, wt = warp - wslot * tps;
@@ -110,102 +129,115 @@ __global__ void __launch_bounds__(TRAIN_THREADS, 1) train_chain_kernel(const Tra
     const int slots = (imgs + di) / slot_imgs, rounds = (slots + spr - 1) / spr;
     const int c0 = ng * 16 + t4 * 4;                              // the thread's four channels
     // rows of either half that are of the map at this thread's column
-    int vrows[2];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) vrows[h] = x0 + g8 + dx * h < W ? min(R, H - y0 - dy * h) : 0;
+    const int vr0 = x0 + g8 < W ? min(R, H - y0) : 0, vr1 = x0 + g8 + dx < W ? min(R, H - y0 - dy) : 0;
+    const bool whole = x0 + cols <= W && y0 + trows <= H;
 
+    const uint32_t w_lane = sm_u32(s_w) + (uint32_t)(ng * NG * 9 * 512 + lane * 16);
     uint4 b[3][3];
-    auto frag = [&](int l, int k, int r) { load_frag<NG>(b, lays[min(l, layers - 1)].wpk, lane, 0, ng, k, r); };
-    if (on) { frag(0, 0, 0); frag(0, 0, 1); frag(0, 0, 2); }
+    auto frag = [&](int k, int r) {
+#pragma unroll
+        for (int s = 0; s < 3; ++s) {
+            uint4& v = b[r][s];
+            asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(w_lane + (uint32_t)((k * 9 + r * 3 + s) * 512)));
+        }
+    };
     for (int l = 0; l < layers; ++l) {
         const TrainLayer& L = lays[l];
         float (*const s_bn)[C] = s_bn2[l & 1];                    // a warp may still be reading the last layer's
         const __nv_bfloat16* const extra = BWD ? L.x : L.res;     // read per task: the BN's input, or the residual
-        // constants of the BN: backward needs them in the epilogue, forward behind the exchange (asked for now, as are the running statistics)
-        float k0 = 0.f, k1 = 0.f, k2 = 0.f, k3 = 0.f;
-        if (tid < C) {
-            k2 = __ldg(L.gamma + tid); k3 = __ldg(L.beta + tid);
-            if (BWD) { s_bn[0][tid] = -__ldcg(L.stat + tid); s_bn[1][tid] = __ldcg(L.stat + C + tid); s_bn[2][tid] = k2; s_bn[3][tid] = k3; }
-            else if (cta == 0) { k0 = __ldcg(L.run_mean + tid); k1 = __ldcg(L.run_var + tid); }
-        }
-        __syncthreads();                                          // the layer's input (and constants) are in shared memory
+        float k0 = 0.f, k1 = 0.f, k2 = 0.f, k3 = 0.f;             // forward: gamma, beta, running statistics, asked for now
+        if (!BWD && fin) { k2 = __ldg(L.gamma + fc); k3 = __ldg(L.beta + fc); if (cta == 0) { k0 = __ldcg(L.run_mean + fc); k1 = __ldcg(L.run_var + fc); } }
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();                                          // the layer's input, filter and constants are in shared memory
+        if (NG == 1 && on) { frag(0, 0); frag(0, 1); frag(0, 2); }
         for (int rd = 0; rd < rounds; ++rd) {
             const int im = (rd * spr + wslot) * slot_imgs;        // first image of the task
             const bool work = on && im < n_img;
-            const bool have1 = im + di < n_img;                   // the second image of a pair exists
             uint32_t y[2 * R][2];
             if (work) {
+                const bool have1 = im + di < n_img;               // the second image of a pair exists
+                const long long base = ((long long)(img0 + im) * HW + y0 * W + x0) * C + ng * 16;
+                const int half_e = (di * HW + dx + dy * W) * C;   // elements from the first half to the second
                 if (extra) {
-                    // 128 chunks [half][row][column][16-byte part]; the ones outside the map are left as they are and not used
+                    // 128 chunks [half][row][column][16-byte part], zero outside the map
+                    const int part = lane & 1, px = (lane >> 1) & 7, o0 = lane >> 4;
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        const int c = lane + 32 * j, part = c & 1, px = (c >> 1) & 7, o = (c >> 4) & 3, h = c >> 6;
-                        const int yy = y0 + o + dy * h, xx = x0 + px + dx * h;
-                        if (yy < H && xx < W && (h == 0 || have1))
-                            cp16(sm_u32(s_stage) + c * 16, extra + ((long long)(img0 + im + di * h) * HW + yy * W + xx) * C + ng * 16 + part * 8);
+                        const int o = o0 + 2 * (j & 1), h = j >> 1;
+                        const bool in = whole ? h == 0 || have1 : y0 + o + dy * h < H && x0 + px + dx * h < W && (h == 0 || have1);
+                        const __nv_bfloat16* src = extra + base + (in ? half_e * h + (o * W + px) * C + part * 8 : 0);
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(sm_u32(s_stage) + (lane + 32 * j) * 16), "l"(src), "r"(in ? 16u : 0u) : "memory");
                     }
                     asm volatile("cp.async.commit_group;" ::: "memory");
                 }
+                if (NG > 1) { frag(0, 0); frag(0, 1); frag(0, 2); }
                 float acc[R][2][4];
-                const bool next_round = ((rd + 1) * spr + wslot) * slot_imgs < n_img;       // of this warp
-                conv_task<NG>(acc, b, a_lane + im * img_bytes, row_bytes, plane, [&](int k, int r) {
-                    const bool end = k == NG - 1;
-                    if (NG > 1 || !next_round) frag(end && !next_round ? l + 1 : l, end ? 0 : k + 1, r);
-                });
+                conv_task<NG>(acc, b, a_lane + im * img_bytes, row_bytes, plane, [&](int k, int r) { if (k < NG - 1) frag(k + 1, r); });
                 __syncwarp();
                 if (lane == 0) mbar_arrive(sm_u32(&s_bar[rd]));
                 if (extra) { asm volatile("cp.async.wait_group 0;" ::: "memory"); __syncwarp(); }
-                // ---- epilogue: thread (g8, t4) holds column g8 of both halves of each row, channels c0 .. c0 + 3
+                // ---- epilogue: thread (g8, t4) holds column g8 of both halves of each row, channels c0 .. c0 + 3.  What lies outside the map is zero from
+                // here on (and so is what is added to it), so it adds nothing to the sums
+                if (!(whole && have1)) {
+#pragma unroll
+                    for (int o = 0; o < R; ++o) {
+                        if (o >= vr0) acc[o][0][0] = acc[o][0][1] = acc[o][1][0] = acc[o][1][1] = 0.f;
+                        if (o >= (have1 ? vr1 : 0)) acc[o][0][2] = acc[o][0][3] = acc[o][1][2] = acc[o][1][3] = 0.f;
+                    }
+                }
                 uint64_t s0 = 0, s1 = 0, q0 = 0, q1 = 0;
-                const int pix0 = y0 * W + x0 + g8;
+                ulonglong2 nm, is, ga, be;
+                if (BWD) {
+                    nm = *reinterpret_cast<const ulonglong2*>(&s_bn[0][c0]); is = *reinterpret_cast<const ulonglong2*>(&s_bn[1][c0]);
+                    ga = *reinterpret_cast<const ulonglong2*>(&s_bn[2][c0]); be = *reinterpret_cast<const ulonglong2*>(&s_bn[3][c0]);
+                }
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    const int rows = h == 1 && !have1 ? 0 : vrows[h];
-                    __nv_bfloat16* const yo = BWD ? nullptr : L.y + ((long long)(img0 + im + di * h) * HW + pix0 + dx * h + dy * h * W) * C + c0;
+                    const int rows = h ? (have1 ? vr1 : 0) : vr0;
+                    __nv_bfloat16* yo = BWD ? nullptr : L.y + base + g8 * C + t4 * 4 + half_e * h;
+                    const uint8_t* es = s_stage + (h * R * 8 + g8) * 32 + t4 * 8;
 #pragma unroll
                     for (int o = 0; o < R; ++o) {
                         uint64_t v0 = v2(acc[o][0][2 * h], acc[o][0][2 * h + 1]), v1 = v2(acc[o][1][2 * h], acc[o][1][2 * h + 1]);
-                        uint2 e = make_uint2(0u, 0u);
-                        if (extra) e = *reinterpret_cast<const uint2*>(s_stage + ((h * R + o) * 8 + g8) * 32 + t4 * 8);
+                        uint2 e;
+                        if (BWD || extra) e = *reinterpret_cast<const uint2*>(es + o * 256);
                         if (!BWD && extra) { v0 = add2(v0, of_bf2(e.x)); v1 = add2(v1, of_bf2(e.y)); }
                         const uint2 w = make_uint2(to_bf2(v0), to_bf2(v1));
                         y[h * R + o][0] = w.x; y[h * R + o][1] = w.y;
-                        if (o >= rows) continue;
                         if (!BWD) {
-                            *reinterpret_cast<uint2*>(yo + o * W * C) = w;
+                            if (o < rows) *reinterpret_cast<uint2*>(yo) = w;
+                            yo += W * C;
                             const uint64_t r0 = of_bf2(w.x), r1 = of_bf2(w.y);
                             s0 = add2(s0, r0); s1 = add2(s1, r1); q0 = fma2(r0, r0, q0); q1 = fma2(r1, r1, q1);
                         } else {
-                            const ulonglong2 nm = *reinterpret_cast<const ulonglong2*>(&s_bn[0][c0]), is = *reinterpret_cast<const ulonglong2*>(&s_bn[1][c0]);
-                            const ulonglong2 ga = *reinterpret_cast<const ulonglong2*>(&s_bn[2][c0]), be = *reinterpret_cast<const ulonglong2*>(&s_bn[3][c0]);
                             const uint64_t h0 = mul2(add2(of_bf2(e.x), nm.x), is.x), h1 = mul2(add2(of_bf2(e.y), nm.y), is.y);
                             float z0, z1, z2, z3; un2(fma2(h0, ga.x, be.x), z0, z1); un2(fma2(h1, ga.y, be.y), z2, z3);
-                            const uint64_t d0 = of_bf2(w.x & ((z0 > 0.f ? 0x0000FFFFu : 0u) | (z1 > 0.f ? 0xFFFF0000u : 0u)));
-                            const uint64_t d1 = of_bf2(w.y & ((z2 > 0.f ? 0x0000FFFFu : 0u) | (z3 > 0.f ? 0xFFFF0000u : 0u)));
+                            const uint64_t d0 = v2(z0 > 0.f ? bf_lo(w.x) : 0.f, z1 > 0.f ? bf_hi(w.x) : 0.f), d1 = v2(z2 > 0.f ? bf_lo(w.y) : 0.f, z3 > 0.f ? bf_hi(w.y) : 0.f);
                             s0 = add2(s0, d0); s1 = add2(s1, d1); q0 = fma2(d0, h0, q0); q1 = fma2(d1, h1, q1);
                         }
                     }
                 }
-                // the eight lanes of the same channels, fixed butterfly; the first keeps the warp's running sums
-                float f[8]; un2(s0, f[0], f[1]); un2(s1, f[2], f[3]); un2(q0, f[4], f[5]); un2(q1, f[6], f[7]);
-#pragma unroll
-                for (int i = 0; i < 8; ++i)
-#pragma unroll
-                    for (int off = 4; off < 32; off <<= 1) f[i] += __shfl_xor_sync(0xffffffffu, f[i], off);
-                if (g8 == 0)
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) { s_red[warp][0][t4 * 4 + i] += (double)f[i]; s_red[warp][1][t4 * 4 + i] += (double)f[4 + i]; }
-            }
-            else if (lane == 0) mbar_arrive(sm_u32(&s_bar[rd]));
+                // the eight lanes of the same channels: each step halves what a lane keeps; lane g8 ends with one of the eight sums
+                {
+                    const bool q = lane & 16, hi = lane & 8, odd = lane & 4;
+                    const uint64_t a0 = __shfl_xor_sync(0xffffffffu, q ? s0 : q0, 16), a1 = __shfl_xor_sync(0xffffffffu, q ? s1 : q1, 16);
+                    const uint64_t r0 = add2(q ? q0 : s0, a0), r1 = add2(q ? q1 : s1, a1);
+                    const uint64_t r = add2(hi ? r1 : r0, __shfl_xor_sync(0xffffffffu, hi ? r0 : r1, 8));
+                    float f0, f1; un2(r, f0, f1);
+                    const float f = (odd ? f1 : f0) + __shfl_xor_sync(0xffffffffu, odd ? f0 : f1, 4);
+                    s_red[warp][q ? 1 : 0][t4 * 4 + (hi ? 2 : 0) + (odd ? 1 : 0)] += (double)f;
+                }
+            } else if (lane == 0) mbar_arrive(sm_u32(&s_bar[rd]));
             if (work) {
                 // every warp has arrived at its own pace; bounded like every wait
                 for (uint32_t i = 0; !mbar_try(sm_u32(&s_bar[rd]), (uint32_t)l & 1u); ++i) if (i > (1u << 22)) { s_abort = 1; break; }
-                uint8_t* const d = sm + im * img_bytes + (ng * 2 + (t4 >> 1)) * plane + ((y0 + 1) * Wp + x0 + 1 + g8) * 16 + (t4 & 1) * 8;
+                uint8_t* d = sm + im * img_bytes + (ng * 2 + (t4 >> 1)) * plane + ((y0 + 1) * Wp + x0 + 1 + g8) * 16 + (t4 & 1) * 8;
 #pragma unroll
-                for (int h = 0; h < 2; ++h)
-#pragma unroll
-                    for (int o = 0; o < R; ++o)
-                        if (o < vrows[h]) *reinterpret_cast<uint2*>(d + (h ? half : 0u) + o * row_bytes) = make_uint2(y[h * R + o][0], y[h * R + o][1]);
+                for (int o = 0; o < R; ++o) {
+                    if (o < vr0) *reinterpret_cast<uint2*>(d) = make_uint2(y[o][0], y[o][1]);
+                    if (o < vr1) *reinterpret_cast<uint2*>(d + half) = make_uint2(y[R + o][0], y[R + o][1]);
+                    d += row_bytes;
+                }
             }
         }
         __syncthreads();
@@ -218,6 +250,7 @@ __global__ void __launch_bounds__(TRAIN_THREADS, 1) train_chain_kernel(const Tra
             for (int w = c / 16; w < spr * tps; w += NG) a += s_red[w][k][c & 15];      // the warps of the channel's group (tps is a multiple of the groups)
             st_packet(box + (long long)cta * 2 * C + tid, a, number);
         }
+        if (l + 1 < layers) { fetch_filter(l + 1); if (BWD) backward_constants(l + 1); }
         {
             constexpr int Q = TRAIN_THREADS / (2 * C);
             const int q = tid / (2 * C), c2 = tid % (2 * C);
@@ -240,35 +273,47 @@ __global__ void __launch_bounds__(TRAIN_THREADS, 1) train_chain_kernel(const Tra
             s_sum[tid] = a;
             if (!ok) { s_abort = 1; *(volatile int*)pr.status = 21; __threadfence_system(); }
             __syncthreads();
-            if (s_abort) return;                                  // the same for all: written before the barrier only
+            if (s_abort) { asm volatile("cp.async.wait_group 0;" ::: "memory"); return; }      // the same for all: written before the barrier only
             for (int i = tid; i < TRAIN_WARPS * 32; i += TRAIN_THREADS) (&s_red[0][0][0])[i] = 0.0;
-            if (tid < C) {
-                const int c = tid;
-                double t0 = 0.0, t1 = 0.0;
+            if (tid < 8 * C) {                                    // eight lanes per channel: four parts of either sum
+                const int kind = (tid >> 2) & 1, part = tid & 3;
+                double t = 0.0;
 #pragma unroll
-                for (int u = 0; u < Q; ++u) { t0 += s_sum[u * 2 * C + c]; t1 += s_sum[u * 2 * C + C + c]; }
-                if (!BWD) {
-                    const double mean = t0 / m; double var = t1 / m - mean * mean; if (var < 0.0) var = 0.0;
-                    const float fm = (float)mean, fi = (float)(1.0 / sqrt(var + (double)pr.eps));
-                    s_bn[0][c] = -fm; s_bn[1][c] = fi; s_bn[2][c] = k2; s_bn[3][c] = k3;
+                for (int u = 0; u < Q / 4; ++u) t += s_sum[(part + 4 * u) * 2 * C + kind * C + fc];
+                t += __shfl_xor_sync(0xffffffffu, t, 1); t += __shfl_xor_sync(0xffffffffu, t, 2);
+                const double t1 = __shfl_xor_sync(0xffffffffu, t, 4);
+                if (fin && !BWD) {
+                    const double mean = t * inv_md; double var = t1 * inv_md - mean * mean; if (var < 0.0) var = 0.0;
+                    const float fm = (float)mean, fi = (float)rsqrt(var + (double)pr.eps);
+                    s_bn[0][fc] = -fm; s_bn[1][fc] = fi * k2; s_bn[2][fc] = k3;
                     if (cta == 0) {
-                        L.stat[c] = fm; L.stat[C + c] = fi;
-                        const double unb = m > 1.0 ? var * m / (m - 1.0) : var, mo = (double)pr.momentum;
-                        L.run_mean[c] = (float)((1.0 - mo) * (double)k0 + mo * mean);
-                        L.run_var[c] = (float)((1.0 - mo) * (double)k1 + mo * unb);
+                        L.stat[fc] = fm; L.stat[C + fc] = fi;
+                        const double mo = (double)pr.momentum;
+                        L.run_mean[fc] = (float)((1.0 - mo) * (double)k0 + mo * mean);
+                        L.run_var[fc] = (float)((1.0 - mo) * (double)k1 + mo * var * unbiased);
                     }
-                } else {
-                    const float b0 = (float)t0, b1 = (float)t1;
-                    s_bn[4][c] = b0 * inv_m; s_bn[5][c] = b1 * inv_m;
-                    if (cta == 0) { L.stat[2 * C + c] = b0; L.stat[3 * C + c] = b1; L.dbeta[c] = b0; L.dgamma[c] = b1; }
+                } else if (fin) {
+                    const float b0 = (float)t, b1 = (float)t1;
+                    s_bn[4][fc] = b0 * inv_m; s_bn[5][fc] = b1 * inv_m;
+                    if (cta == 0) { L.stat[2 * C + fc] = b0; L.stat[3 * C + fc] = b1; L.dbeta[fc] = b0; L.dgamma[fc] = b1; }
                 }
             }
             __syncthreads();
         }
-        // ---- elementwise pass in place: 8 channels per access, two pixels at a time; the constants are read where they are used
+        // ---- elementwise pass in place: 8 channels per access, two pixels at a time; a lane keeps its group's constants in registers
         {
             const int g = lane % G;
             const uint64_t* const cst = reinterpret_cast<const uint64_t*>(&s_bn[0][g * 8]);
+            uint64_t nm[4], sc[4], be[4], is[BWD ? 4 : 1], ga[BWD ? 4 : 1], nsb[BWD ? 4 : 1], nsg[BWD ? 4 : 1];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                nm[k] = cst[k];
+                if (!BWD) { sc[k] = cst[C / 2 + k]; be[k] = cst[C + k]; }
+                else {
+                    is[k] = cst[C / 2 + k]; ga[k] = cst[C + k]; be[k] = cst[3 * C / 2 + k]; sc[k] = mul2(ga[k], is[k]);
+                    nsb[k] = cst[2 * C + k] ^ 0x8000000080000000ull; nsg[k] = cst[5 * C / 2 + k] ^ 0x8000000080000000ull;
+                }
+            }
             for (int r = warp; r < all_rows; r += TRAIN_WARPS) {
                 const int im = r / H, yy = r - im * H;
                 const long long at = ((long long)(img0 + im) * HW + yy * W) * C;
@@ -277,7 +322,7 @@ __global__ void __launch_bounds__(TRAIN_THREADS, 1) train_chain_kernel(const Tra
                 const uint4* const xv = BWD ? reinterpret_cast<const uint4*>(L.x + at) : nullptr;
                 const uint4* const av = BWD && L.res ? reinterpret_cast<const uint4*>(L.res + at) : nullptr;
                 for (int i0 = lane; i0 < row_chunks; i0 += 64) {
-                    uint32_t v[2][4], x[2][4], e[2][4], o[2][4]; uint8_t* sp[2];
+                    uint32_t v[2][4], x[2][4], e[2][4]; uint8_t* sp[2];
 #pragma unroll
                     for (int u = 0; u < 2; ++u) {
                         const int i = i0 + 32 * u < row_chunks ? i0 + 32 * u : i0;
@@ -289,26 +334,22 @@ __global__ void __launch_bounds__(TRAIN_THREADS, 1) train_chain_kernel(const Tra
                         const uint4 t = *reinterpret_cast<const uint4*>(sp[u]); v[u][0] = t.x; v[u][1] = t.y; v[u][2] = t.z; v[u][3] = t.w;
                     }
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const uint64_t nm = cst[k], is = cst[C / 2 + k], ga = cst[C + k], be = cst[3 * C / 2 + k];
-                        if (!BWD) { o[0][k] = bn_relu2(v[0][k], nm, is, ga, be); o[1][k] = bn_relu2(v[1][k], nm, is, ga, be); }
-                        else {
-                            const uint64_t nsb = cst[2 * C + k] ^ 0x8000000080000000ull, nsg = cst[5 * C / 2 + k] ^ 0x8000000080000000ull, gi = mul2(ga, is);
+                    for (int u = 0; u < 2; ++u) {
+                        uint32_t o[4];
 #pragma unroll
-                            for (int u = 0; u < 2; ++u) {
-                                const uint64_t xh = mul2(add2(of_bf2(x[u][k]), nm), is);
-                                float z0, z1; un2(fma2(xh, ga, be), z0, z1);
-                                const uint64_t dz = of_bf2(v[u][k] & ((z0 > 0.f ? 0x0000FFFFu : 0u) | (z1 > 0.f ? 0xFFFF0000u : 0u)));
-                                uint64_t t = mul2(gi, fma2(xh, nsg, add2(dz, nsb)));
+                        for (int k = 0; k < 4; ++k) {
+                            if (!BWD) o[k] = relu_bf2(to_bf2(fma2(add2(of_bf2(v[u][k]), nm[k]), sc[k], be[k])));
+                            else {
+                                const uint64_t xh = mul2(add2(of_bf2(x[u][k]), nm[k]), is[k]);
+                                float z0, z1; un2(fma2(xh, ga[k], be[k]), z0, z1);
+                                const uint64_t dz = v2(z0 > 0.f ? bf_lo(v[u][k]) : 0.f, z1 > 0.f ? bf_hi(v[u][k]) : 0.f);
+                                uint64_t t = mul2(sc[k], fma2(xh, nsg[k], add2(dz, nsb[k])));
                                 if (av) t = add2(t, of_bf2(e[u][k]));
-                                o[u][k] = to_bf2(t);
+                                o[k] = to_bf2(t);
                             }
                         }
-                    }
-#pragma unroll
-                    for (int u = 0; u < 2; ++u) {
                         if (i0 + 32 * u >= row_chunks) break;
-                        const uint4 w = make_uint4(o[u][0], o[u][1], o[u][2], o[u][3]);
+                        const uint4 w = make_uint4(o[0], o[1], o[2], o[3]);
                         *reinterpret_cast<uint4*>(sp[u]) = w; out[i0 + 32 * u] = w;
                     }
                 }
@@ -331,13 +372,15 @@ bool train_chain_geometry(int C, int H, int W, ChainMap& best) {
     }
     return least > 0;
 }
-constexpr size_t TRAIN_SMEM = 214 * 1024, TRAIN_FIXED = TRAIN_WARPS * STAGE_BYTES + TRAIN_MAX_LAYERS * sizeof(TrainLayer);      // 11 KB more are static
-static size_t train_smem(int C, const ChainMap& m, int imgs) { return (size_t)imgs * (C / 8) * m.plane + TRAIN_FIXED; }
+// dynamic shared memory: maps, the warps' staging, the filter, the layers' descriptors; the kernel's static arrays take 9 to 12 KB of the 227
+static size_t train_fixed(int C) { return TRAIN_WARPS * STAGE_BYTES + 18 * C * C + TRAIN_MAX_LAYERS * sizeof(TrainLayer); }
+static size_t train_room(int C) { return 227 * 1024 - 8704 - 48 * C; }
+static size_t train_smem(int C, const ChainMap& m, int imgs) { return (size_t)imgs * (C / 8) * m.plane + train_fixed(C); }
 int train_chain_max_layers() { return TRAIN_MAX_LAYERS; }
 // images a CTA can hold
 int train_chain_max_imgs(int C, const ChainMap& m) {
     const int tps = C / 16 * m.strips * m.xblocks, spr = TRAIN_WARPS / tps;
-    const int n = std::min((int)((TRAIN_SMEM - TRAIN_FIXED) / ((size_t)(C / 8) * m.plane)), TRAIN_MAX_ROUNDS * spr * m.slot);
+    const int n = std::min((int)((train_room(C) - train_fixed(C)) / ((size_t)(C / 8) * m.plane)), TRAIN_MAX_ROUNDS * spr * m.slot);
     return n / m.slot * m.slot;
 }
 // Deals the SMs to the problems of a launch: images per CTA so that all CTAs fit, with the least time of the slowest problem, a layer taken as a fixed part (barrier, sums)
@@ -370,7 +413,7 @@ void launch_train_chain_pack(const TrainPack* d, int n, int max_c, unsigned* cou
     train_chain_pack_kernel<<<dim3((steps * steps * 9 * 32 + 255) / 256, n), 256, 0, s>>>(d, counters, ncounters);
 }
 template <int C, bool BWD> static bool launch_chain(const TrainChain* d, int nprob, int ctas, size_t smem, cudaStream_t s) {
-    if (cudaFuncSetAttribute(train_chain_kernel<C, BWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TRAIN_SMEM) != cudaSuccess) { cudaGetLastError(); return false; }
+    if (cudaFuncSetAttribute(train_chain_kernel<C, BWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)train_room(C)) != cudaSuccess) { cudaGetLastError(); return false; }
     cudaLaunchConfig_t cfg = {}; cfg.gridDim = dim3(ctas); cfg.blockDim = dim3(TRAIN_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = s;
     cudaLaunchAttribute at[1]; at[0].id = cudaLaunchAttributeCooperative; at[0].val.cooperative = 1; cfg.attrs = at; cfg.numAttrs = 1;      // its CTAs wait for one another
     return cudaLaunchKernelEx(&cfg, train_chain_kernel<C, BWD>, d, nprob) == cudaSuccess;
