@@ -154,6 +154,16 @@ struct TrainChain {
 };
 struct TrainPack { const __nv_bfloat16* w; uint4* fwd; uint4* bwd; int C; };      // w [C][9][C]
 
+// Weight gradients of a run's layers (wgrad_chain.cu).
+struct WgChainProb { const __nv_bfloat16* a; const __nv_bfloat16* dy; float* out; };
+struct WgChainLaunch {
+    int C, H, W, N;                                    // all problems of a launch alike
+    int cols, rs, strips, xblocks;                     // columns of a block (16, or 8 with two groups of rows), steps of a chain, blocks down and across
+    int dy_cols, a_plane, d_plane;                     // columns of the gradient's map; bytes of an image's 8-channel group of either tensor
+    int imgs, units, nq, max_parts;                    // images per unit, units per problem, problems (halves of them at 64 channels), CTAs that touch one at most
+    float* partial;
+};
+
 // A contiguous run of parameters treated alike by the bandwidth kernels.
 struct Segment {
     long long begin;      // offset in the flat vector
@@ -223,6 +233,11 @@ bool train_chain_assign(TrainChain* p, int n, int sms);
 size_t train_chain_launch_smem(const TrainChain* p, int n);
 void launch_train_chain_pack(const TrainPack* d, int n, int max_c, unsigned* counters, int ncounters, cudaStream_t s);
 bool launch_train_chain(const TrainChain* d, int nprob, int C, bool backward, int ctas, size_t smem, cudaStream_t s);
+
+// ---- launchers (wgrad_chain.cu)
+bool wgrad_chain_geometry(int C, int H, int W, int N, WgChainLaunch& g);
+int wgrad_chain_plan(WgChainLaunch& g, int nprob, int sms, size_t* partial_bytes);
+bool launch_wgrad_chain(const WgChainProb* d, const WgChainLaunch& g, int ctas, cudaStream_t s);
 
 // ---- launchers (kernels_bw.cu)
 void launch_sgd(const Segment* d, int nseg, long long nchunks, ParamArrays pa, const float* lr, float mu, float wd,

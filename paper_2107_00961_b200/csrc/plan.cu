@@ -114,7 +114,7 @@ __global__ void patch_kernel(const PatchSite* sites, int n, PatchArgs a) {
 // ------------------------------------------------------------------------------------------------
 struct Builder {
     resist_ctx* ctx; int B; int sub; int copy; bool eval; int group;      // group: sub-ResNets that share the launches now being built
-    char* base; size_t off = 0; size_t es; bool group_all = group > 1;                // group_all: the plan is of all sub-ResNets (`group` itself changes from slot to slot)
+    char* base; size_t off = 0; size_t es; 
     std::vector<Op>* ops;
     // scratch shared by the operations of this sub-ResNet (they run one after another)
     double* bn_partial = nullptr; float* wgrad_partial = nullptr; size_t bn_partial_need = 0, wgrad_partial_need = 0;
@@ -368,25 +368,8 @@ struct Builder {
         if (eval || ctx->opts.dtype != RESIST_BF16 || ctx->opts.conv_backend != RESIST_CONV_AUTO || !chainable(k) || !train_chain_geometry(k.cin, H, Wd, map)) return false;
         const int cap = train_chain_max_imgs(k.cin, map);
         if (cap < 1 || (long long)std::max(1, share) * ((B + cap - 1) / cap) > ctx->sm_count) return false;
-        ConvProb p = wgrad_prob(k.cin, H, Wd); size_t pb = 0;
-        return pick_backend(p, CONV_WGRAD, group, 8, &pb) != 0;
-    }
-    ConvProb wgrad_prob(int C, int H, int Wd) const {
-        ConvProb p{}; p.N = B; p.H = p.P = H; p.W = p.Q = Wd; p.C = p.K = C; p.ksz = 3; p.stride = 1; p.pad = 1; p.scale = 1.f;
-        p.M = C; p.Ncol = 9 * C; p.Kred = B * H * Wd;
-        p.tiles_m = (p.M + 63) / 64; p.tiles_n = (p.Ncol + 63) / 64; p.splits = 1; p.ktiles_per_split = (p.Kred + 15) / 16;
-        return p;
-    }
-    // a chain's weight gradients share one launch: each its own partial sums, the GPU's CTAs split among `many`
-    void chain_wgrad(long long key, const void* a, const void* dy, const ConvRef& cr, int H, int Wd, int many) {
-        Op op{}; op.key = key; op.sub = sub; op.kind = OP_CONV_WGRAD;
-        op.conv = wgrad_prob(cr.cin, H, Wd); op.conv.act = a; op.conv.wgt = dy; op.conv.out = G() + cr.w;
-        op.wg_target = wgrad_target_ctas(ctx, many);
-        size_t pb = 0;
-        op.backend = pick_backend(op.conv, CONV_WGRAD, group, op.wg_target, &pb);
-        op.conv.partial = (float*)take(pb);
-        flops += 2LL * B * H * Wd * 9 * cr.cin * cr.cout; ++n_tc;
-        ops->push_back(op);
+        WgChainLaunch g;
+        return wgrad_chain_geometry(k.cin, H, Wd, B, g);
     }
     void bn_bwd(long long key, const void* x, const void* da, void* dx, const void* add, const BNRef& r, float* stat, long long m) {
         Op op{}; op.key = key; op.sub = sub; op.kind = OP_BN_BWD_REDUCE;
@@ -583,13 +566,8 @@ static size_t unroll_subnet(resist_ctx* ctx, Builder& bd, const std::vector<char
         const char* dout = bd.gbuf[g_cur];
         if (s.chain_n) {
             const int n = s.chain_n, first = s.chain_first, C = K.cin; const long long rows = m_in;
-            bd.group = share[first];
             // the launch's key is the first block's: the same for all sub-ResNets, however many blocks they hold
             const long long ckey = BWD_BLOCK0 + 40LL * ((long long)n_aslots - 1 - aslot[first]);
-            int many = 0;                                     // weight gradients in the launch: the stage's identity blocks of every sub-ResNet of the plan
-            for (int s2 = 0; s2 < ctx->S; ++s2)
-                if (bd.group_all || s2 == bd.sub)
-                    for (int b2 = 0; b2 < nb; ++b2) if ((ctx->mask[b2] >> s2 & 1u) && ctx->blocks[b2].stage == K.stage && Builder::chainable(ctx->blocks[b2])) many += 2;
             Op op{}; op.key = ckey; op.sub = bd.sub; op.kind = OP_TRAIN_CHAIN_BWD;
             TrainChain& t = op.tchain; ChainMap cmap{}; train_chain_geometry(C, s.H, s.W, cmap);
             t.in = (const __nv_bfloat16*)dout; t.nlayers = 2 * n; t.N = B; t.H = s.H; t.W = s.W; t.C = C; t.map = cmap;
@@ -610,11 +588,15 @@ static size_t unroll_subnet(resist_ctx* ctx, Builder& bd, const std::vector<char
                 d2 = dxb;
             }
             bd.ops->push_back(op);
-            for (int i = n - 1, k = 0; i >= 0; --i, k += 2) {
-                const BlockRef& q = L.blk[order[first + i]]; BlockMem& e = bm[order[first + i]];
-                bd.chain_wgrad(ckey + 1, e.a2, dys[k], q.conv[1], s.H, s.W, many);
-                bd.chain_wgrad(ckey + 1, e.a1, dys[k + 1], q.conv[0], s.H, s.W, many);
-            }
+            for (int i = n - 1, k = 0; i >= 0; --i)
+                for (int j = 1; j >= 0; --j, ++k) {
+                    const BlockMem& e = bm[order[first + i]];
+                    Op wg{}; wg.key = ckey + 1; wg.sub = bd.sub; wg.kind = OP_CHAIN_WGRAD;
+                    wg.wgc = WgChainProb{(const __nv_bfloat16*)(j ? e.a2 : e.a1), (const __nv_bfloat16*)dys[k], bd.G() + L.blk[order[first + i]].conv[j].w};
+                    wg.conv.act = wg.wgc.a; wg.conv.wgt = wg.wgc.dy; wg.conv.N = B; wg.conv.H = s.H; wg.conv.W = s.W; wg.conv.C = C;
+                    bd.flops += 2LL * rows * 9 * C * C; ++bd.n_tc;
+                    bd.ops->push_back(wg);
+                }
             bd.grel(g_cur); g_cur = g_dx; bd.last_dgrad = bd.last_tc_dgrad = -1;
             slot = first; continue;
         }
@@ -710,6 +692,7 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
     std::vector<ConvProb> conv; std::vector<BnProb> bn; std::vector<PoolProb> pool; std::vector<HeadProb> head; std::vector<UpProb> up; std::vector<ColProb> col;
     std::vector<ChainProb> chain; std::vector<ChainLayer> layer;
     std::vector<TrainChain> tchain; std::vector<TrainLayer> tlayer; std::vector<TrainPack> tpack; std::vector<size_t> tfirst;   // tfirst: a chain's first entry of tlayer
+    std::vector<WgChainProb> wgc; size_t wgc_partial = 0;
     const size_t tcb = conv_tc_prob_bytes(); std::vector<char> tc; int n_tc = 0;
     const size_t wtcb = conv_wgrad_tc_prob_bytes(); std::vector<char> wtc; int n_wtc = 0;
     const size_t mmb = conv_mma_prob_bytes(); std::vector<char> mm; int n_mm = 0;
@@ -727,12 +710,23 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
             snprintf(L.label, sizeof(L.label), "%dx%d C%d K%d HW%d s%d%s x%d", c.ksz, c.ksz, c.C, c.K, c.H, c.stride, c.dy_sub == 2 ? "*" : "", L.count);
         } else if (ops[i].kind != OP_HEAD_FWD && ops[i].kind != OP_HEAD_BWD && ops[i].kind != OP_POOL_FWD && ops[i].kind != OP_POOL_BWD &&
                    ops[i].kind != OP_UPSAMPLE && ops[i].kind != OP_IM2COL && ops[i].kind != OP_SPLITK && ops[i].kind != OP_REPACK &&
-                   ops[i].kind != OP_EVAL_CHAIN_PACK && ops[i].kind != OP_EVAL_CHAIN && ops[i].kind != OP_TRAIN_CHAIN_PACK && ops[i].kind != OP_TRAIN_CHAIN_FWD && ops[i].kind != OP_TRAIN_CHAIN_BWD)
+                   ops[i].kind != OP_EVAL_CHAIN_PACK && ops[i].kind != OP_EVAL_CHAIN && ops[i].kind != OP_TRAIN_CHAIN_PACK && ops[i].kind != OP_TRAIN_CHAIN_FWD && ops[i].kind != OP_TRAIN_CHAIN_BWD && ops[i].kind != OP_CHAIN_WGRAD)
             snprintf(L.label, sizeof(L.label), "bn m%lld C%d x%d", ops[i].bn.m, ops[i].bn.C, L.count);
         for (size_t k = i; k < j; ++k) {
             ops[k].conv.group = (int)(j - i);
             const Op& o = ops[k]; const int slot = single ? 0 : o.sub;
             switch (o.kind) {
+                case OP_CHAIN_WGRAD: {
+                    if (k == i) {
+                        L.first = (int)wgc.size(); size_t pb = 0;
+                        if (!wgrad_chain_geometry(o.conv.C, o.conv.H, o.conv.W, o.conv.N, L.wgc)) { ctx->err = "internal: a chain's weight gradients do not fit"; return RESIST_EINVAL; }
+                        L.gx = wgrad_chain_plan(L.wgc, L.count, ctx->sm_count, &pb); wgc_partial = std::max(wgc_partial, pb);      // one launch at a time uses it
+                        snprintf(L.label, sizeof(L.label), "3x3 C%d HW%d x%d", o.conv.C, o.conv.H, L.count);
+                    }
+                    wgc.push_back(o.wgc);
+                    const double e = (double)o.conv.N * o.conv.H * o.conv.W * o.conv.C, w_e = 9.0 * o.conv.C * o.conv.C;
+                    L.flops += 2.0 * e * 9 * o.conv.C; L.bytes += es * 2 * e + 4.0 * w_e;
+                    break; }
                 case OP_TRAIN_CHAIN_PACK:
                     if (k == i) L.first = (int)tpack.size();
                     tpack.push_back(o.tpack); L.max_c = std::max(L.max_c, o.tpack.C); L.bytes += 6.0 * 9 * o.tpack.C * o.tpack.C;
@@ -776,7 +770,7 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
                         if (o.kind == OP_CONV_WGRAD) {
                             if (k == i) L.first = n_wmm;
                             wmm.resize((size_t)(n_wmm + 1) * wmmb); char* h = wmm.data() + (size_t)n_wmm * wmmb;
-                            if (!conv_wgrad_mma_fill(o.conv, o.wg_target ? o.wg_target : wgrad_target_ctas(ctx, (int)(j - i)), h)) { ctx->err = "wgrad descriptor failed"; return RESIST_EINVAL; }
+                            if (!conv_wgrad_mma_fill(o.conv, wgrad_target_ctas(ctx, (int)(j - i)), h)) { ctx->err = "wgrad descriptor failed"; return RESIST_EINVAL; }
                             L.gx = std::max(L.gx, conv_wgrad_mma_ctas(h));
                             L.max_elems = std::max<long long>(L.max_elems, (long long)conv_wgrad_mma_smem(h));
                             L.max_b = (int)std::max<long long>(L.max_b, conv_wgrad_mma_out_elems(h));
@@ -799,7 +793,7 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
                         if (k == i) L.first = n_wtc;
                         wtc.resize((size_t)(n_wtc + 1) * wtcb);
                         char* h = wtc.data() + (size_t)n_wtc * wtcb;
-                        if (!conv_wgrad_tc_fill(o.conv, o.wg_target ? o.wg_target : wgrad_target_ctas(ctx, (int)(j - i)), h)) { ctx->err = "tensor map encoding failed"; return RESIST_ECUDA; }
+                        if (!conv_wgrad_tc_fill(o.conv, wgrad_target_ctas(ctx, (int)(j - i)), h)) { ctx->err = "tensor map encoding failed"; return RESIST_ECUDA; }
                         L.gx = std::max(L.gx, conv_wgrad_tc_ctas(h));
                         L.max_elems = std::max<long long>(L.max_elems, (long long)conv_wgrad_tc_smem(h));
                         L.max_b = (int)std::max<long long>(L.max_b, conv_wgrad_tc_out_elems(h));
@@ -901,7 +895,7 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
                     case OP_CONV_FWD: case OP_CONV_DGRAD: wr.push_back(o.conv.out);
                         if (o.fuse == 1) wr.push_back(o.bn.a); else if (o.fuse == 2) wr.push_back(o.bn.dx);
                         break;
-                    case OP_CONV_WGRAD: case OP_SPLITK: case OP_REPACK: case OP_TRAIN_CHAIN_PACK: break;
+                    case OP_CONV_WGRAD: case OP_CHAIN_WGRAD: case OP_SPLITK: case OP_REPACK: case OP_TRAIN_CHAIN_PACK: break;
                     case OP_TRAIN_CHAIN_FWD: case OP_TRAIN_CHAIN_BWD: for (const TrainLayer& l : o.tlayers) { wr.push_back(l.y); wr.push_back(l.a); } break;
                     case OP_BN_STATS: case OP_BN_BWD_REDUCE: case OP_BN_TILE_STATS: case OP_BN_EVAL_STATS: case OP_BN_BWD_TILE_SUMS: break;
                     case OP_BN_APPLY: case OP_BN_FWD_FUSED: case OP_BN_FWD_SMALL: wr.push_back(o.bn.a); break;
@@ -910,7 +904,7 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
                 }
             }
             L.join_before = false;
-            if (L.kind == OP_CONV_WGRAD) { for (size_t k = i; k < j; ++k) { inflight.push_back(ops[k].conv.act); inflight.push_back(ops[k].conv.wgt); } }
+            if (L.kind == OP_CONV_WGRAD || L.kind == OP_CHAIN_WGRAD) { for (size_t k = i; k < j; ++k) { inflight.push_back(ops[k].conv.act); inflight.push_back(ops[k].conv.wgt); } }
             else if (L.kind != OP_SPLITK && L.kind != OP_REPACK && !inflight.empty()) {
                 bool hit = always;
                 for (const void* w : wr) for (const void* r : inflight) if (w == r) hit = true;
@@ -940,6 +934,7 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
     const size_t o_chain = off; off += align_up(chain.size() * sizeof(ChainProb), 256);
     const size_t o_tchain = off; off += align_up(tchain.size() * sizeof(TrainChain), 256);
     const size_t o_tlayer = off; off += align_up(tlayer.size() * sizeof(TrainLayer), 256);
+    const size_t o_wgc = off; off += align_up(wgc.size() * sizeof(WgChainProb), 256);
     const size_t o_tpack = off; off += align_up(tpack.size() * sizeof(TrainPack), 256);
     const size_t o_arrive = off; off += align_up(tchain.size() * 32 * sizeof(unsigned), 256);   // a number per chain, 128 bytes apart
     const size_t o_layer = off; off += align_up(layer.size() * sizeof(ChainLayer), 256);
@@ -948,7 +943,7 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
     if (plan.graph) cudaGraphExecDestroy(plan.graph);
     plan.graph = nullptr; plan.runs = 0; plan.graph_failed = false;
     ctx_free(ctx, plan.d_blob);
-    plan.d_blob = ctx_alloc(ctx, off + 256 + packets); plan.blob_bytes = off; plan.d_lr = (float*)((char*)plan.d_blob + off);
+    plan.d_blob = ctx_alloc(ctx, off + 256 + packets + wgc_partial); plan.blob_bytes = off; plan.d_lr = (float*)((char*)plan.d_blob + off);
     if (!plan.d_blob) { ctx->err = "allocator returned NULL for the launch plan"; return RESIST_ENOMEM; }
     char* base = (char*)plan.d_blob;
     plan.d_conv = (ConvProb*)(base + o_conv); plan.d_bn = (BnProb*)(base + o_bn); plan.d_pool = (PoolProb*)(base + o_pool);
@@ -983,6 +978,9 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
     if (!layer.empty()) memcpy(host.data() + o_layer, layer.data(), layer.size() * sizeof(ChainLayer));
     plan.d_tchain = (TrainChain*)(base + o_tchain); plan.d_tpack = (TrainPack*)(base + o_tpack); plan.d_arrive = (unsigned*)(base + o_arrive); plan.n_arrive = (int)tchain.size() * 32;
     for (size_t t = 0; t < tchain.size(); ++t) { tchain[t].layers = (const TrainLayer*)(base + o_tlayer) + tfirst[t]; tchain[t].arrive = plan.d_arrive + t * 32; tchain[t].packets = (uint4*)(base + o_packets[t]); tchain[t].status = conv_tc_status_word(); }
+    plan.d_wgc = (WgChainProb*)(base + o_wgc);
+    if (!wgc.empty()) memcpy(host.data() + o_wgc, wgc.data(), wgc.size() * sizeof(WgChainProb));
+    for (Launch& l : plan.launches) if (l.kind == OP_CHAIN_WGRAD) l.wgc.partial = (float*)(base + off + 256 + packets);
     if (!tchain.empty()) memcpy(host.data() + o_tchain, tchain.data(), tchain.size() * sizeof(TrainChain));
     if (!tlayer.empty()) memcpy(host.data() + o_tlayer, tlayer.data(), tlayer.size() * sizeof(TrainLayer));
     if (!tpack.empty()) memcpy(host.data() + o_tpack, tpack.data(), tpack.size() * sizeof(TrainPack));
@@ -1073,7 +1071,7 @@ static int enqueue_launches(resist_ctx* ctx, Plan& plan, bool update, bool overl
     for (const Launch& L : plan.launches) {
         // early start of a warp-MMA convolution: not behind the im2col pass that writes the stem's packed weights, not while profiling
         const bool pdl_ok = !pf.on && prev_kind != OP_IM2COL; prev_kind = L.kind;
-        const bool on_side = overlap && (L.kind == OP_CONV_WGRAD || ((L.kind == OP_SPLITK || L.kind == OP_REPACK) && side_pending));
+        const bool on_side = overlap && (L.kind == OP_CONV_WGRAD || L.kind == OP_CHAIN_WGRAD || ((L.kind == OP_SPLITK || L.kind == OP_REPACK) && side_pending));
         if (on_side) {
             cudaEventRecord(ctx->ev_fork, main_st); cudaStreamWaitEvent(ctx->side_stream, ctx->ev_fork, 0);
             st = ctx->side_stream;
@@ -1104,6 +1102,7 @@ static int enqueue_launches(resist_ctx* ctx, Plan& plan, bool update, bool overl
             case OP_EVAL_CHAIN_PACK: case OP_EVAL_CHAIN: pk = PK_EVAL_CHAIN; break;
             case OP_TRAIN_CHAIN_PACK: case OP_TRAIN_CHAIN_FWD: pk = PK_TRAIN_CHAIN_FWD; break;
             case OP_TRAIN_CHAIN_BWD: pk = PK_TRAIN_CHAIN_BWD; break;
+            case OP_CHAIN_WGRAD: pk = PK_CHAIN_WGRAD; nk = 2; break;
         }
         pf.begin(pk, nk, L.bytes, L.flops, st, L.label);
         switch (L.kind) {
@@ -1133,6 +1132,9 @@ static int enqueue_launches(resist_ctx* ctx, Plan& plan, bool update, bool overl
             case OP_HEAD_FWD: n_launch += launch_head_fwd(plan.d_head + L.first, L.count, L.max_b, L.max_c, L.max_classes, bf, st); break;
             case OP_HEAD_BWD: n_launch += launch_head_bwd(plan.d_head + L.first, L.count, L.max_b, L.max_c, L.max_classes, L.max_elems, bf, st); break;
             case OP_UPSAMPLE: launch_zero_stuff(plan.d_up + L.first, L.count, L.max_elems, st); ++n_launch; break;
+            case OP_CHAIN_WGRAD:
+                if (!launch_wgrad_chain(plan.d_wgc + L.first, L.wgc, L.gx, st)) { ctx->err = "weight gradient launch failed"; return RESIST_ECUDA; }
+                n_launch += 2; break;
             case OP_TRAIN_CHAIN_PACK: launch_train_chain_pack(plan.d_tpack + L.first, L.count, L.max_c, plan.d_arrive, plan.n_arrive, st); ++n_launch; break;
             case OP_TRAIN_CHAIN_FWD: case OP_TRAIN_CHAIN_BWD:
                 if (!launch_train_chain(plan.d_tchain + L.first, L.count, L.max_c, L.kind == OP_TRAIN_CHAIN_BWD, L.gx, L.smem, st)) { ctx->err = "training chain launch failed"; cudaGetLastError(); return RESIST_ECUDA; }

@@ -20,7 +20,7 @@ Layout make_layout(const resist_arch& a, const std::vector<resist_block>& blocks
 enum OpKind {
     OP_CONV_FWD, OP_CONV_DGRAD, OP_CONV_WGRAD, OP_SPLITK, OP_BN_STATS, OP_BN_APPLY, OP_BN_BWD_REDUCE, OP_BN_BWD_APPLY,
     OP_POOL_FWD, OP_POOL_BWD, OP_HEAD_FWD, OP_HEAD_BWD, OP_UPSAMPLE, OP_IM2COL, OP_BN_FWD_FUSED, OP_BN_BWD_FUSED, OP_BN_TILE_STATS, OP_REPACK, OP_BN_EVAL_STATS, OP_BN_FWD_SMALL, OP_BN_BWD_SMALL, OP_BN_BWD_TILE_SUMS,
-    OP_EVAL_CHAIN_PACK, OP_EVAL_CHAIN, OP_TRAIN_CHAIN_PACK, OP_TRAIN_CHAIN_FWD, OP_TRAIN_CHAIN_BWD
+    OP_EVAL_CHAIN_PACK, OP_EVAL_CHAIN, OP_TRAIN_CHAIN_PACK, OP_TRAIN_CHAIN_FWD, OP_TRAIN_CHAIN_BWD, OP_CHAIN_WGRAD
 };
 
 // One operation of one sub-ResNet, keyed so that equal keys of different sub-ResNets share a launch.
@@ -28,7 +28,7 @@ struct Op {
     long long key; OpKind kind; int sub;
     ConvProb conv; BnProb bn; PoolProb pool; HeadProb head; UpProb up; ColProb col; ChainProb chain; ChainLayer layer;
     TrainChain tchain; std::vector<TrainLayer> tlayers; TrainPack tpack;
-    int wg_target;        // weight gradients launched many at a time: CTAs of this one (0: by the launch)
+    WgChainProb wgc;
     int backend;          // convolutions: 0 = CUDA cores, 1 = tensor cores
     int patch_images;     // conv.act must be replaced by the caller's image pointer
     int fuse;             // warp-MMA convolutions: 1 = `bn` is the BN+ReLU forward of the output, 2 = the BN+ReLU backward whose da is the output; it runs in the same launch
@@ -46,14 +46,14 @@ struct Launch {
     int small_ctas, ksz;                                      // CUDA-core convolutions: CTAs per problem of the small-layer kernels (0: not all problems are small)
     ColProb col;                                              // im2col: the geometry its problems share
     ChainProb chain;
-    size_t smem;
+    size_t smem; WgChainLaunch wgc;
     char label[40];                                           // shape of the launch's first problem, for the per-launch trace
 };
 
 enum ProfKind {
     PK_CONV_FWD_CC, PK_CONV_DGRAD_CC, PK_CONV_WGRAD_CC, PK_CONV_FWD_TC, PK_CONV_DGRAD_TC, PK_CONV_WGRAD_TC, PK_SPLITK,
     PK_BN_STATS, PK_BN_APPLY, PK_BN_BWD_REDUCE, PK_BN_BWD_APPLY, PK_POOL_FWD, PK_POOL_BWD, PK_HEAD_FWD, PK_HEAD_BWD,
-    PK_SGD, PK_PATCH, PK_SCATTER, PK_AGGREGATE, PK_UPSAMPLE, PK_CONV_FWD_MMA, PK_CONV_DGRAD_MMA, PK_CONV_WGRAD_MMA, PK_IM2COL, PK_BN_FWD_FUSED, PK_BN_BWD_FUSED, PK_CONV_FWD_MMA_BN, PK_CONV_DGRAD_MMA_BN, PK_BN_TILE_STATS, PK_EVAL_CHAIN, PK_TRAIN_CHAIN_FWD, PK_TRAIN_CHAIN_BWD, PK_COUNT
+    PK_SGD, PK_PATCH, PK_SCATTER, PK_AGGREGATE, PK_UPSAMPLE, PK_CONV_FWD_MMA, PK_CONV_DGRAD_MMA, PK_CONV_WGRAD_MMA, PK_IM2COL, PK_BN_FWD_FUSED, PK_BN_BWD_FUSED, PK_CONV_FWD_MMA_BN, PK_CONV_DGRAD_MMA_BN, PK_BN_TILE_STATS, PK_EVAL_CHAIN, PK_TRAIN_CHAIN_FWD, PK_TRAIN_CHAIN_BWD, PK_CHAIN_WGRAD, PK_COUNT
 };
 constexpr double PROFILE_RIDGE = 250.0;          // FLOP per byte at which a B200's bf16 tensor peak meets its HBM bandwidth (about 1.63e15 / 6.5e12)
 struct Profiler {
@@ -85,7 +85,7 @@ struct Plan {
     void* d_blob = nullptr; size_t blob_bytes = 0;            // descriptor arrays in one device allocation
     ConvProb* d_conv = nullptr; BnProb* d_bn = nullptr; PoolProb* d_pool = nullptr; HeadProb* d_head = nullptr; UpProb* d_up = nullptr; ColProb* d_col = nullptr;
     ChainProb* d_chain = nullptr; ChainLayer* d_layer = nullptr;
-    TrainChain* d_tchain = nullptr; TrainPack* d_tpack = nullptr; unsigned* d_arrive = nullptr; int n_arrive = 0;
+    TrainChain* d_tchain = nullptr; TrainPack* d_tpack = nullptr; WgChainProb* d_wgc = nullptr; unsigned* d_arrive = nullptr; int n_arrive = 0;
     PatchSite* d_sites = nullptr; int nsites = 0;
     void* d_tc = nullptr; size_t tc_stride = 0;              // tensor-core convolution descriptors
     void* d_wtc = nullptr; size_t wtc_stride = 0;            // tensor-core wgrad descriptors
