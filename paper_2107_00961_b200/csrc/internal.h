@@ -160,7 +160,7 @@ struct WgChainLaunch {
     int C, H, W, N;                                    // all problems of a launch alike
     int cols, rs, strips, xblocks;                     // columns of a block (16, or 8 with two groups of rows), steps of a chain, blocks down and across
     int dy_cols, a_plane, d_plane;                     // columns of the gradient's map; bytes of an image's 8-channel group of either tensor
-    int imgs, units, nq, max_parts;                    // images per unit, units per problem, problems (halves of them at 64 channels), CTAs that touch one at most
+    int stages, imgs, units, nq, max_parts;            // units in shared memory, images per unit, units per problem, problems, CTAs that touch one at most
     float* partial;
 };
 
@@ -235,7 +235,7 @@ void launch_train_chain_pack(const TrainPack* d, int n, int max_c, unsigned* cou
 bool launch_train_chain(const TrainChain* d, int nprob, int C, bool backward, int ctas, size_t smem, cudaStream_t s);
 
 // ---- launchers (wgrad_chain.cu)
-bool wgrad_chain_geometry(int C, int H, int W, int N, WgChainLaunch& g);
+bool wgrad_chain_geometry(int C, int H, int W, int N, int nprob, int sms, WgChainLaunch& g);
 int wgrad_chain_plan(WgChainLaunch& g, int nprob, int sms, size_t* partial_bytes);
 bool launch_wgrad_chain(const WgChainProb* d, const WgChainLaunch& g, int ctas, cudaStream_t s);
 

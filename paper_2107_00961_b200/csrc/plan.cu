@@ -369,7 +369,7 @@ struct Builder {
         const int cap = train_chain_max_imgs(k.cin, map);
         if (cap < 1 || (long long)std::max(1, share) * ((B + cap - 1) / cap) > ctx->sm_count) return false;
         WgChainLaunch g;
-        return wgrad_chain_geometry(k.cin, H, Wd, B, g);
+        return wgrad_chain_geometry(k.cin, H, Wd, B, 1, ctx->sm_count, g);
     }
     void bn_bwd(long long key, const void* x, const void* da, void* dx, const void* add, const BNRef& r, float* stat, long long m) {
         Op op{}; op.key = key; op.sub = sub; op.kind = OP_BN_BWD_REDUCE;
@@ -719,7 +719,7 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool s
                 case OP_CHAIN_WGRAD: {
                     if (k == i) {
                         L.first = (int)wgc.size(); size_t pb = 0;
-                        if (!wgrad_chain_geometry(o.conv.C, o.conv.H, o.conv.W, o.conv.N, L.wgc)) { ctx->err = "internal: a chain's weight gradients do not fit"; return RESIST_EINVAL; }
+                        if (!wgrad_chain_geometry(o.conv.C, o.conv.H, o.conv.W, o.conv.N, L.count, ctx->sm_count, L.wgc)) { ctx->err = "internal: a chain's weight gradients do not fit"; return RESIST_EINVAL; }
                         L.gx = wgrad_chain_plan(L.wgc, L.count, ctx->sm_count, &pb); wgc_partial = std::max(wgc_partial, pb);      // one launch at a time uses it
                         snprintf(L.label, sizeof(L.label), "3x3 C%d HW%d x%d", o.conv.C, o.conv.H, L.count);
                     }
