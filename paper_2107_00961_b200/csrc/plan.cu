@@ -663,14 +663,14 @@ static size_t unroll_subnet(resist_ctx* ctx, Builder& bd, const std::vector<char
 struct Needs { size_t bn_partial = 0, wgrad_partial = 0, gbig = 0, up = 0, total = 0; };
 
 static Needs measure_subnet(resist_ctx* ctx, int sub, int copy, const std::vector<char>& present, int B, bool eval, float inv_S, int group) {
-    std::vector<Op> scratch;
+    std::vector<Op> scratch; scratch.reserve(64 + 24 * present.size());
     Builder b1{ctx, B, sub, copy, eval, group, nullptr}; b1.es = ctx->opts.dtype == RESIST_BF16 ? 2 : 4; b1.ops = &scratch;
-    unroll_subnet(ctx, b1, present, inv_S);
+    const size_t used = unroll_subnet(ctx, b1, present, inv_S);
     Needs n; n.bn_partial = b1.bn_partial_need; n.wgrad_partial = b1.wgrad_partial_need; n.gbig = b1.gbig; n.up = b1.up_need;
-    scratch.clear();
-    Builder b2{ctx, B, sub, copy, eval, group, nullptr}; b2.es = b1.es; b2.ops = &scratch;
-    b2.bn_partial_need = n.bn_partial; b2.wgrad_partial_need = n.wgrad_partial; b2.gbig = n.gbig; b2.up_need = n.up;
-    n.total = align_up(unroll_subnet(ctx, b2, present, inv_S), 256);
+    // with the scratch laid out first everything behind it moves by its sizes: each piece starts 256-byte aligned
+    size_t shift = align_up(n.bn_partial, 256) + align_up(n.wgrad_partial, 256) + align_up(n.up, 256);
+    if (!eval) shift += Builder::NGBUF * align_up(n.gbig, 256);
+    n.total = align_up(used + shift, 256);
     return n;
 }
 
@@ -680,14 +680,18 @@ static std::vector<char> present_of(const resist_ctx* ctx, int sub) {
     return p;
 }
 
-static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& ops, bool single, cudaStream_t st) {
+static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& all_ops, bool single, cudaStream_t st) {
     // equal keys of different sub-ResNets become neighbours; a zero-stuffing or im2col op shares the key of the first
-    // convolution that reads its output and sorts in front of it
-    std::stable_sort(ops.begin(), ops.end(), [](const Op& a, const Op& b) {
-        if (a.key != b.key) return a.key < b.key;
-        const bool pa = a.kind == OP_UPSAMPLE || a.kind == OP_IM2COL, pb = b.kind == OP_UPSAMPLE || b.kind == OP_IM2COL;
+    // convolution that reads its output and sorts in front of it.  (Pointers are sorted: an Op is a kilobyte, and moving 1500 of them about took longer than all else that
+    // building a plan does.)
+    struct { std::vector<Op*> at; Op& operator[](size_t i) const { return *at[i]; } size_t size() const { return at.size(); } } ops;
+    ops.at.reserve(all_ops.size());
+    for (Op& o : all_ops) ops.at.push_back(&o);
+    std::stable_sort(ops.at.begin(), ops.at.end(), [](const Op* a, const Op* b) {
+        if (a->key != b->key) return a->key < b->key;
+        const bool pa = a->kind == OP_UPSAMPLE || a->kind == OP_IM2COL, pb = b->kind == OP_UPSAMPLE || b->kind == OP_IM2COL;
         if (pa != pb) return pa;
-        return a.backend < b.backend; });
+        return a->backend < b->backend; });
     const double es = ctx->opts.dtype == RESIST_BF16 ? 2.0 : 4.0;
     std::vector<ConvProb> conv; std::vector<BnProb> bn; std::vector<PoolProb> pool; std::vector<HeadProb> head; std::vector<UpProb> up; std::vector<ColProb> col;
     std::vector<ChainProb> chain; std::vector<ChainLayer> layer;
@@ -1021,6 +1025,7 @@ static int build_plan(resist_ctx* ctx, Plan& plan, int sub, int B, cudaStream_t 
     int rc = ensure_workspace(ctx, B, group, needs);
     if (rc) return rc;
     std::vector<Op> ops; plan.info = resist_step_info{};
+    ops.reserve((size_t)(sub >= 0 ? 1 : ctx->S) * (64 + 24 * ctx->arch.num_blocks));
     const int s0 = sub >= 0 ? sub : 0, s1 = sub >= 0 ? sub + 1 : ctx->S;
     for (int s = s0; s < s1; ++s) {
         Builder bd{ctx, B, s, s, false, group, (char*)ctx->d_ws + (size_t)s * ctx->ws_slice};
