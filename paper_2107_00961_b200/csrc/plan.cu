@@ -362,14 +362,14 @@ struct Builder {
         last_chain = (int)ops->size() - 1; last_fwd_conv = last_tc_fwd = -1;
         return true;
     }
-    // Training through the n identity basic blocks order[0 .. n) as one launch per direction: whether the chain kernel takes them, for `share` sub-ResNets
-    // in the launch (all their CTAs have to be resident together, one per SM).
-    bool tchain_ok(const resist_block& k, int H, int Wd, int share, ChainMap& map) const {
-        if (eval || ctx->opts.dtype != RESIST_BF16 || ctx->opts.conv_backend != RESIST_CONV_AUTO || !chainable(k) || !train_chain_geometry(k.cin, H, Wd, map)) return false;
-        const int cap = train_chain_max_imgs(k.cin, map);
+    // Training through a run of 3x3 layers of C channels as one launch per direction: whether the chain kernel takes them, for `share` sub-ResNets in the launch (all
+    // their CTAs have to be resident together, one per SM).
+    bool tchain_ok(int C, int H, int Wd, int share, ChainMap& map) const {
+        if (eval || ctx->opts.dtype != RESIST_BF16 || ctx->opts.conv_backend != RESIST_CONV_AUTO || !train_chain_geometry(C, H, Wd, map)) return false;
+        const int cap = train_chain_max_imgs(C, map);
         if (cap < 1 || (long long)std::max(1, share) * ((B + cap - 1) / cap) > ctx->sm_count) return false;
         WgChainLaunch g;
-        return wgrad_chain_geometry(k.cin, H, Wd, B, 1, ctx->sm_count, g);
+        return wgrad_chain_geometry(C, H, Wd, B, 1, ctx->sm_count, g);
     }
     void bn_bwd(long long key, const void* x, const void* da, void* dx, const void* add, const BNRef& r, float* stat, long long m) {
         Op op{}; op.key = key; op.sub = sub; op.kind = OP_BN_BWD_REDUCE;
@@ -414,7 +414,10 @@ struct Builder {
     }
 };
 
-struct BlockMem { int H, W, Ho, Wo; void *x, *a1, *y1, *a2, *y2, *a3; float* stat[3]; int chain_n, chain_first; const uint4* dpk[2]; };   // chain_n: blocks of the training chain that starts / ends here
+struct BlockMem { int H, W, Ho, Wo; void *x, *a1, *y1, *a2, *y2, *a3; float* stat[3];
+    // training chains: the data gradients' filters of either convolution; on a chain's last block: its identity blocks order[chain_first .. + chain_n) and the block
+    // whose second convolution leads it (-1: none); on that block, once the chain has run backward: gradients of its output and of its first convolution's output
+    const uint4* dpk[2]; int chain_last, chain_n, chain_first, chain_head; int chain_done; const void *chain_dout, *chain_dy1; };
 
 // Returns the workspace bytes this sub-ResNet needs.  `present` has one entry per block.
 static size_t unroll_subnet(resist_ctx* ctx, Builder& bd, const std::vector<char>& present, float inv_S) {
@@ -480,40 +483,55 @@ static size_t unroll_subnet(resist_ctx* ctx, Builder& bd, const std::vector<char
             void* out = nullptr;
             if (bd.chain(key, &order[slot], n, cur, cH, cW, inv_S, &out)) { cur = out; slot += n - 1; continue; }
         }
-        ChainMap cmap{};
-        if (bd.tchain_ok(K, cH, cW, share[slot], cmap)) {
-            int n = 1; while (slot + n < order.size() && 2 * n < train_chain_max_layers() && Builder::chainable(ctx->blocks[order[slot + n]])) ++n;
-            const long long rows = (long long)B * cH * cW; const int C = K.cin;
-            void* x = cur; void* a1 = bd.act(rows * C);
-            float* st1 = bd.bn_fwd(key + 0, x, a1, r.bn[0], rows, true);
-            Op op{}; op.key = key + 3; op.sub = bd.sub; op.kind = OP_TRAIN_CHAIN_FWD;
+        // Training: a run of 3x3 layers of one width and resolution as one chain: the identity blocks from slot `first` on, led (head >= 0) by the second convolution of the
+        // block before them.  in: input of its first convolution; x, a1, st1 (no head): the first block's input, its BN's output and statistics; res: (head) the skip path
+        auto chain_forward = [&](long long ckey, size_t first, int head, void* in, void* x, void* res, float* st1, int C, int H, int Wd, const ChainMap& cmap) -> void* {
+            const long long rows = (long long)B * H * Wd;
+            int n = 0; while (first + n < order.size() && 2 * (n + 1) < train_chain_max_layers() && Builder::chainable(ctx->blocks[order[first + n]])) ++n;
+            Op op{}; op.key = ckey; op.sub = bd.sub; op.kind = OP_TRAIN_CHAIN_FWD;
             TrainChain& t = op.tchain;
-            t.in = (const __nv_bfloat16*)a1; t.nlayers = 2 * n; t.N = B; t.H = cH; t.W = cW; t.C = C; t.map = cmap;
+            t.in = (const __nv_bfloat16*)in; t.nlayers = 2 * n + (head >= 0); t.N = B; t.H = H; t.W = Wd; t.C = C; t.map = cmap;
             t.eps = ctx->opts.bn_eps; t.momentum = ctx->opts.bn_momentum;
+            auto layer = [&](int bi, int j, const void* add, void* y, void* a, const BNRef* br, float* stat) {      // br: the BN behind it (nullptr: it comes with whatever follows the chain)
+                Op pk{}; pk.key = Builder::PACK_KEY; pk.sub = bd.sub; pk.kind = OP_TRAIN_CHAIN_PACK;
+                uint4* f = (uint4*)bd.take((size_t)9 * C * C * 2); uint4* d = (uint4*)bd.take((size_t)9 * C * C * 2);
+                pk.tpack = TrainPack{(const __nv_bfloat16*)bd.CW(L.blk[bi].conv[j].w), f, d, C}; bd.ops->push_back(pk); bm[bi].dpk[j] = d;
+                TrainLayer l{}; l.wpk = f; l.res = (const __nv_bfloat16*)add; l.y = (__nv_bfloat16*)y;
+                if (br) { l.a = (__nv_bfloat16*)a; l.gamma = bd.W() + br->g; l.beta = bd.W() + br->b; l.stat = stat; l.run_mean = bd.Bf() + br->buf; l.run_var = bd.Bf() + br->buf + br->c; }
+                bd.flops += 2LL * rows * 9 * C * C; ++bd.n_tc;
+                op.tlayers.push_back(l);
+            };
+            void* a1 = in;
+            if (head >= 0) {
+                x = bd.act(rows * C); a1 = nullptr;
+                if (n) { a1 = bd.act(rows * C); st1 = (float*)bd.take((size_t)4 * C * 4); }
+                layer(head, 1, res, x, a1, n ? &L.blk[order[first]].bn[0] : nullptr, st1);
+            }
             for (int i = 0; i < n; ++i) {
-                const int bi = order[slot + i]; const BlockRef& q = L.blk[bi]; BlockMem& e = bm[bi];
-                e.H = e.Ho = cH; e.W = e.Wo = cW; e.x = x; e.a1 = a1; e.stat[0] = st1; e.chain_n = i == n - 1 ? n : 0; e.chain_first = (int)slot;
+                const int bi = order[first + i]; BlockMem& e = bm[bi];
+                e.H = e.Ho = H; e.W = e.Wo = Wd; e.x = x; e.a1 = a1; e.stat[0] = st1;
                 e.y1 = bd.act(rows * C); e.a2 = bd.act(rows * C); void* out = bd.act(rows * C);
                 e.stat[1] = (float*)bd.take((size_t)4 * C * 4);
-                for (int j = 0; j < 2; ++j) {
-                    Op pk{}; pk.key = Builder::PACK_KEY; pk.sub = bd.sub; pk.kind = OP_TRAIN_CHAIN_PACK;
-                    uint4* f = (uint4*)bd.take((size_t)9 * C * C * 2); uint4* d = (uint4*)bd.take((size_t)9 * C * C * 2);
-                    pk.tpack = TrainPack{(const __nv_bfloat16*)bd.CW(q.conv[j].w), f, d, C}; bd.ops->push_back(pk); e.dpk[j] = d;
-                    TrainLayer l{}; l.wpk = f; l.res = j ? (const __nv_bfloat16*)x : nullptr; l.y = (__nv_bfloat16*)(j ? out : e.y1);
-                    bd.flops += 2LL * rows * 9 * C * C; ++bd.n_tc;
-                    if (j == 0 || i < n - 1) {                // the BN behind it; the last layer's comes with whatever follows the chain
-                        const int nb2 = j ? order[slot + i + 1] : bi; const BNRef& br = L.blk[nb2].bn[j ? 0 : 1];
-                        float* stat = e.stat[1]; void* a = e.a2;
-                        if (j) { a1 = a = bd.act(rows * C); st1 = stat = (float*)bd.take((size_t)4 * C * 4); }
-                        l.a = (__nv_bfloat16*)a; l.gamma = bd.W() + br.g; l.beta = bd.W() + br.b; l.stat = stat; l.run_mean = bd.Bf() + br.buf; l.run_var = bd.Bf() + br.buf + br.c;
-                    }
-                    op.tlayers.push_back(l);
-                }
+                layer(bi, 0, nullptr, e.y1, e.a2, &L.blk[bi].bn[1], e.stat[1]);
+                const bool more = i + 1 < n;
+                if (more) { a1 = bd.act(rows * C); st1 = (float*)bd.take((size_t)4 * C * 4); }
+                layer(bi, 1, x, out, a1, more ? &L.blk[order[first + i + 1]].bn[0] : nullptr, st1);
                 x = out;
             }
+            BlockMem& e = bm[n ? order[first + n - 1] : head];
+            e.chain_last = 1; e.chain_n = n; e.chain_first = (int)first; e.chain_head = head;
             bd.ops->push_back(op);
             bd.last_tchain = (int)bd.ops->size() - 1; bd.last_fwd_conv = bd.last_tc_fwd = -1;
-            cur = x; slot += n - 1; continue;
+            slot = first + n - 1;
+            return x;
+        };
+        ChainMap cmap{};
+        if (Builder::chainable(K) && bd.tchain_ok(K.cin, cH, cW, share[slot], cmap)) {
+            const long long rows = (long long)B * cH * cW;
+            void* a1 = bd.act(rows * K.cin);
+            float* st1 = bd.bn_fwd(key + 0, cur, a1, r.bn[0], rows, true);
+            cur = chain_forward(key + 3, slot, -1, a1, cur, nullptr, st1, K.cin, cH, cW, cmap); cC = K.cin;
+            continue;
         }
         s.H = cH; s.W = cW; s.Ho = out_dim(cH, 3, K.stride); s.Wo = out_dim(cW, 3, K.stride);
         const long long m_in = (long long)B * s.H * s.W, m_out = (long long)B * s.Ho * s.Wo;
@@ -522,6 +540,14 @@ static size_t unroll_subnet(resist_ctx* ctx, Builder& bd, const std::vector<char
         s.stat[0] = bd.bn_fwd(key + 0, s.x, s.a1, r.bn[0], m_in, !K.has_projection);
         const void* sc = s.x;
         if (K.has_projection) { void* scb = bd.act(m_out * K.cout); bd.conv(key + 2, CONV_FWD, s.a1, r.proj, nullptr, nullptr, scb, B, s.H, s.W, 1.f); sc = scb; }
+        if (K.kind == RESIST_BASIC && bd.tchain_ok(K.cout, s.Ho, s.Wo, share[slot], cmap)) {      // its second convolution leads the run behind it
+            s.y1 = bd.act(m_out * K.cout); s.a2 = bd.act(m_out * K.cout);
+            bd.conv(key + 3, CONV_FWD, s.a1, r.conv[0], nullptr, nullptr, s.y1, B, s.H, s.W, 1.f);
+            s.stat[1] = bd.bn_fwd(key + 4, s.y1, s.a2, r.bn[1], m_out, false);
+            const int Ho = s.Ho, Wo = s.Wo;
+            cur = chain_forward(key + 6, slot + 1, b, s.a2, nullptr, const_cast<void*>(sc), nullptr, K.cout, Ho, Wo, cmap); cH = Ho; cW = Wo; cC = K.cout;
+            continue;
+        }
         void* out = bd.act(m_out * K.cout);
         if (K.kind == RESIST_BASIC) {
             s.y1 = bd.act(m_out * K.cout); s.a2 = bd.act(m_out * K.cout);
@@ -563,43 +589,47 @@ static size_t unroll_subnet(resist_ctx* ctx, Builder& bd, const std::vector<char
         bd.group = share[slot];
         const long long key = BWD_BLOCK0 + 40LL * ((long long)n_aslots - 1 - aslot[slot]);
         const long long m_in = (long long)B * s.H * s.W, m_out = (long long)B * s.Ho * s.Wo;
-        const char* dout = bd.gbuf[g_cur];
-        if (s.chain_n) {
-            const int n = s.chain_n, first = s.chain_first, C = K.cin; const long long rows = m_in;
-            // the launch's key is the first block's: the same for all sub-ResNets, however many blocks they hold
-            const long long ckey = BWD_BLOCK0 + 40LL * ((long long)n_aslots - 1 - aslot[first]);
+        if (s.chain_last) {
+            const int n = s.chain_n, first = s.chain_first, head = s.chain_head, C = K.cout; const long long rows = m_out;
+            // keyed by the block it starts with, which is the same for all sub-ResNets however many blocks they hold; a head's own operations follow
+            const long long ckey = head >= 0 ? BWD_BLOCK0 + 40LL * ((long long)n_aslots - 1 - aslot[first - 1]) - 3 : BWD_BLOCK0 + 40LL * ((long long)n_aslots - 1 - aslot[first]);
             Op op{}; op.key = ckey; op.sub = bd.sub; op.kind = OP_TRAIN_CHAIN_BWD;
-            TrainChain& t = op.tchain; ChainMap cmap{}; train_chain_geometry(C, s.H, s.W, cmap);
-            t.in = (const __nv_bfloat16*)dout; t.nlayers = 2 * n; t.N = B; t.H = s.H; t.W = s.W; t.C = C; t.map = cmap;
-            std::vector<const void*> dys;                     // gradient of every convolution's output, last first
-            const int g_dx = bd.gtake();
-            const void* d2 = dout;
+            TrainChain& t = op.tchain; ChainMap cmap{}; train_chain_geometry(C, s.Ho, s.Wo, cmap);
+            const void* d2 = bd.gbuf[g_cur];                  // gradient of the tensor at hand
+            t.in = (const __nv_bfloat16*)d2; t.nlayers = 2 * n + (head >= 0); t.N = B; t.H = s.Ho; t.W = s.Wo; t.C = C; t.map = cmap;
+            std::vector<Op> wgs;
+            auto layer = [&](int bi, int j, const void* dy, void* dx, const void* add) {      // data gradient of a convolution, backward of the BN before it, weight gradient
+                const BlockRef& q = L.blk[bi]; const BlockMem& e = bm[bi]; const BNRef& br = q.bn[j];
+                TrainLayer l{};
+                l.wpk = e.dpk[j]; l.x = (const __nv_bfloat16*)(j ? e.y1 : e.x); l.a = (__nv_bfloat16*)dx; l.res = (const __nv_bfloat16*)add;
+                l.gamma = bd.W() + br.g; l.beta = bd.W() + br.b; l.stat = e.stat[j]; l.dgamma = bd.G() + br.g; l.dbeta = bd.G() + br.b;
+                op.tlayers.push_back(l);
+                Op wg{}; wg.key = ckey + 1; wg.sub = bd.sub; wg.kind = OP_CHAIN_WGRAD;
+                wg.wgc = WgChainProb{(const __nv_bfloat16*)(j ? e.a2 : e.a1), (const __nv_bfloat16*)dy, bd.G() + q.conv[j].w};
+                wg.conv.act = wg.wgc.a; wg.conv.wgt = wg.wgc.dy; wg.conv.N = B; wg.conv.H = s.Ho; wg.conv.W = s.Wo; wg.conv.C = C;
+                wgs.push_back(wg);
+                bd.flops += 4LL * rows * 9 * C * C; bd.n_tc += 2;
+            };
+            const int g_dx = head >= 0 ? -1 : bd.gtake();
             for (int i = n - 1; i >= 0; --i) {
-                const int bi = order[first + i]; const BlockRef& q = L.blk[bi]; BlockMem& e = bm[bi];
-                void* dy1 = bd.act(rows * C); void* dxb = i ? bd.act(rows * C) : (void*)bd.gbuf[g_dx];
-                dys.push_back(d2); dys.push_back(dy1);
-                for (int j = 1; j >= 0; --j) {
-                    TrainLayer l{}; const BNRef& br = q.bn[j];
-                    l.wpk = e.dpk[j]; l.x = (const __nv_bfloat16*)(j ? e.y1 : e.x); l.a = (__nv_bfloat16*)(j ? dy1 : dxb); l.res = j ? nullptr : (const __nv_bfloat16*)d2;
-                    l.gamma = bd.W() + br.g; l.beta = bd.W() + br.b; l.stat = e.stat[j]; l.dgamma = bd.G() + br.g; l.dbeta = bd.G() + br.b;
-                    bd.flops += 2LL * rows * 9 * C * C; ++bd.n_tc;
-                    op.tlayers.push_back(l);
-                }
+                const int bi = order[first + i];
+                void* dy1 = bd.act(rows * C); void* dxb = i || head >= 0 ? bd.act(rows * C) : (void*)bd.gbuf[g_dx];
+                layer(bi, 1, d2, dy1, nullptr); layer(bi, 0, dy1, dxb, d2);
                 d2 = dxb;
             }
+            if (head >= 0) {
+                BlockMem& e = bm[head];
+                void* dy1 = bd.act(rows * C);
+                layer(head, 1, d2, dy1, nullptr);
+                e.chain_done = 1; e.chain_dout = d2; e.chain_dy1 = dy1;
+            }
             bd.ops->push_back(op);
-            for (int i = n - 1, k = 0; i >= 0; --i)
-                for (int j = 1; j >= 0; --j, ++k) {
-                    const BlockMem& e = bm[order[first + i]];
-                    Op wg{}; wg.key = ckey + 1; wg.sub = bd.sub; wg.kind = OP_CHAIN_WGRAD;
-                    wg.wgc = WgChainProb{(const __nv_bfloat16*)(j ? e.a2 : e.a1), (const __nv_bfloat16*)dys[k], bd.G() + L.blk[order[first + i]].conv[j].w};
-                    wg.conv.act = wg.wgc.a; wg.conv.wgt = wg.wgc.dy; wg.conv.N = B; wg.conv.H = s.H; wg.conv.W = s.W; wg.conv.C = C;
-                    bd.flops += 2LL * rows * 9 * C * C; ++bd.n_tc;
-                    bd.ops->push_back(wg);
-                }
-            bd.grel(g_cur); g_cur = g_dx; bd.last_dgrad = bd.last_tc_dgrad = -1;
-            slot = first; continue;
+            for (const Op& wg : wgs) bd.ops->push_back(wg);
+            bd.last_dgrad = bd.last_tc_dgrad = -1;
+            if (head < 0) { bd.grel(g_cur); g_cur = g_dx; slot = first; continue; }
+            if (n) { bd.grel(g_cur); g_cur = -1; slot = first; continue; }      // the head's own part comes next
         }
+        const char* dout = s.chain_done ? (const char*)s.chain_dout : bd.gbuf[g_cur];
         int g_sc = -1; bool sc_compact = false;
         if (K.has_projection) {
             bd.conv(key + 0, CONV_WGRAD, s.a1, r.proj, dout, nullptr, nullptr, B, s.H, s.W, 1.f);
@@ -608,15 +638,18 @@ static size_t unroll_subnet(resist_ctx* ctx, Builder& bd, const std::vector<char
         }
         int g_da1 = -1;
         if (K.kind == RESIST_BASIC) {
-            const int g_da2 = bd.gtake();
-            bd.conv(key + 3, CONV_WGRAD, s.a2, r.conv[1], dout, nullptr, nullptr, B, s.Ho, s.Wo, 1.f);
-            bd.conv(key + 5, CONV_DGRAD, nullptr, r.conv[1], dout, nullptr, bd.gbuf[g_da2], B, s.Ho, s.Wo, 1.f);
-            const int g_dy1 = bd.gtake();
-            bd.bn_bwd(key + 6, s.y1, bd.gbuf[g_da2], bd.gbuf[g_dy1], nullptr, r.bn[1], s.stat[1], m_out);
-            bd.grel(g_da2);
-            bd.conv(key + 8, CONV_WGRAD, s.a1, r.conv[0], bd.gbuf[g_dy1], nullptr, nullptr, B, s.H, s.W, 1.f);
+            int g_dy1 = -1; const void* dy1 = s.chain_dy1;
+            if (!s.chain_done) {
+                const int g_da2 = bd.gtake();
+                bd.conv(key + 3, CONV_WGRAD, s.a2, r.conv[1], dout, nullptr, nullptr, B, s.Ho, s.Wo, 1.f);
+                bd.conv(key + 5, CONV_DGRAD, nullptr, r.conv[1], dout, nullptr, bd.gbuf[g_da2], B, s.Ho, s.Wo, 1.f);
+                g_dy1 = bd.gtake(); dy1 = bd.gbuf[g_dy1];
+                bd.bn_bwd(key + 6, s.y1, bd.gbuf[g_da2], bd.gbuf[g_dy1], nullptr, r.bn[1], s.stat[1], m_out);
+                bd.grel(g_da2);
+            }
+            bd.conv(key + 8, CONV_WGRAD, s.a1, r.conv[0], dy1, nullptr, nullptr, B, s.H, s.W, 1.f);
             g_da1 = bd.gtake();
-            bd.conv(key + 10, CONV_DGRAD, nullptr, r.conv[0], bd.gbuf[g_dy1], g_sc >= 0 ? bd.gbuf[g_sc] : nullptr, bd.gbuf[g_da1], B, s.H, s.W, 1.f, false, sc_compact);
+            bd.conv(key + 10, CONV_DGRAD, nullptr, r.conv[0], dy1, g_sc >= 0 ? bd.gbuf[g_sc] : nullptr, bd.gbuf[g_da1], B, s.H, s.W, 1.f, false, sc_compact);
             bd.grel(g_dy1);
         } else {
             const int g_da3 = bd.gtake();

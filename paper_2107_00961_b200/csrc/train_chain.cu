@@ -19,8 +19,8 @@
 // every warp has arrived at the round's mbarrier, which it does as soon as its MMAs have read the input.  The residual (forward) or the BN's input (backward) of a task comes by cp.async into the warp's own 2 KB while it
 // computes.  Layout of an image and the convolution on it: chain_core.h.
 //
-// Measured, us per step: ResNet-110, 4 x 128 images of 32 x 32 (a launch per layer and direction before) 3290 -> 2353; one worker's 84 images 1160 -> 807; 256
-// images and all 54 blocks in one network 6720 -> 3760.
+// Measured, us per step: ResNet-110, 4 x 128 images of 32 x 32 (a launch per layer and direction before) 3290 -> 1983; one worker's 84 images 1160 -> 800; 256
+// images and all 54 blocks in one network 6700 -> 3528.
 #include <algorithm>
 #include <vector>
 #include "chain_core.h"
