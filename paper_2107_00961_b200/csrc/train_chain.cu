@@ -16,11 +16,12 @@
 // CTA that writes layer l + 2 has read everyone's l + 1, who had all read l.
 //
 // In place: the warps compute a round of tasks (at most one each), keep the rounded results in 16 registers, and store them over the round's input once
-// every warp has arrived at the round's mbarrier, which it does as soon as its MMAs have read the input.  The residual (forward) or the BN's input (backward) of a task comes by cp.async into the warp's own 2 KB while it
+// every warp has arrived at the round's mbarrier, which it does as soon as its MMAs have read the input.  Backward, what the elementwise pass needs of the BN's
+// input waits in tensor memory: sixteen columns of the warp's 128 per round, hence eight rounds at most.  The residual (forward) or the BN's input (backward) of a task comes by cp.async into the warp's own 2 KB while it
 // computes.  Layout of an image and the convolution on it: chain_core.h.
 //
-// Measured, us per step: ResNet-110, 4 x 128 images of 32 x 32 (a launch per layer and direction before) 3290 -> 1983; one worker's 84 images 1160 -> 800; 256
-// images and all 54 blocks in one network 6700 -> 3528.
+// Measured, us per step: ResNet-110, 4 x 128 images of 32 x 32 (a launch per layer and direction before) 3290 -> 1838; one worker's 84 images 1160 -> 778; 256
+// images and all 54 blocks in one network 6700 -> 3301.
 #include <algorithm>
 #include <vector>
 #include "chain_core.h"
@@ -28,7 +29,7 @@
 namespace resist {
 using namespace chain;
 
-constexpr int TRAIN_THREADS = 512, TRAIN_WARPS = 16, STAGE_BYTES = 2048, TRAIN_MAX_ROUNDS = 32, TRAIN_MAX_LAYERS = 48;
+constexpr int TRAIN_THREADS = 512, TRAIN_WARPS = 16, STAGE_BYTES = 2048, TRAIN_MAX_ROUNDS = 8, TRAIN_MAX_LAYERS = 48;
 
 // Filters of the bf16 copy in fragment order, for the forward convolution and for the data gradient (channels exchanged, taps reversed); the chains' packets of
 // this step are numbered from 256 further on.
@@ -63,6 +64,18 @@ __device__ __forceinline__ void st_packet(uint4* p, double a, uint32_t n) {
 }
 __device__ __forceinline__ void cp16(uint32_t dst, const void* src) { asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory"); }
 
+// sixteen registers of a warp's lanes to and from sixteen columns of tensor memory
+__device__ __forceinline__ void tm_st16(uint32_t at, const uint32_t* v) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+                 ::"r"(at), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]),
+                   "r"(v[13]), "r"(v[14]), "r"(v[15]) : "memory");
+}
+__device__ __forceinline__ void tm_ld16(uint32_t at, uint32_t* v) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]),
+                   "=r"(v[13]), "=r"(v[14]), "=r"(v[15]) : "r"(at));
+}
+
 template <int C, bool BWD>
 __global__ void __launch_bounds__(TRAIN_THREADS, 1) train_chain_kernel(const TrainChain* __restrict__ probs, int nprob) {
     constexpr int NG = C / 16, G = C / 8;
@@ -72,6 +85,7 @@ __global__ void __launch_bounds__(TRAIN_THREADS, 1) train_chain_kernel(const Tra
     // by parity of the layer.  Forward: -mean, gamma / std, beta.  Backward: -mean, 1/std, gamma, beta, sum dz / m, sum dz * xhat / m
     __shared__ __align__(16) float s_bn2[2][6][C];
     __shared__ int s_abort;
+    __shared__ uint32_t s_tmem;
     __shared__ __align__(8) uint64_t s_bar[TRAIN_MAX_ROUNDS];     // per round: the warps whose MMAs have read its input
     int pi = 0; while (pi + 1 < nprob && (int)blockIdx.x >= probs[pi + 1].cta0) ++pi;
     const TrainChain& pr = probs[pi];
@@ -80,11 +94,15 @@ __global__ void __launch_bounds__(TRAIN_THREADS, 1) train_chain_kernel(const Tra
     const int imgs = pr.imgs, img0 = cta * imgs, n_img = min(imgs, N - img0);
     const uint32_t plane = (uint32_t)pr.map.plane, img_bytes = G * plane, row_bytes = (uint32_t)Wp * 16u;
     uint4* const packets = pr.packets; const uint32_t number0 = __ldg(pr.arrive);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g8 = lane >> 2, t4 = lane & 3;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31, g8 = lane >> 2, t4 = lane & 3;
     uint8_t* const s_stage = sm + imgs * img_bytes + warp * STAGE_BYTES;
     uint8_t* const s_w = sm + imgs * img_bytes + TRAIN_WARPS * STAGE_BYTES;       // the layer's filter in fragment order
     TrainLayer* const lays = reinterpret_cast<TrainLayer*>(s_w + 18 * C * C);
     for (int i = tid; i < layers * (int)(sizeof(TrainLayer) / 8); i += TRAIN_THREADS) reinterpret_cast<uint64_t*>(lays)[i] = __ldg(reinterpret_cast<const uint64_t*>(pr.layers) + i);
+    if (BWD && warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(sm_u32(&s_tmem)) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
     if (tid < TRAIN_MAX_ROUNDS) mbar_init(sm_u32(&s_bar[tid]), TRAIN_WARPS);
     const double inv_md = 1.0 / ((double)N * HW), unbiased = (double)N * HW / ((double)N * HW > 1.0 ? (double)N * HW - 1.0 : 1.0);
     const float inv_m = 1.f / (float)((long long)N * HW);
@@ -93,7 +111,10 @@ __global__ void __launch_bounds__(TRAIN_THREADS, 1) train_chain_kernel(const Tra
     for (uint32_t i = tid * 16; i < imgs * img_bytes; i += TRAIN_THREADS * 16) *reinterpret_cast<uint4*>(sm + i) = make_uint4(0u, 0u, 0u, 0u);
     for (int i = tid; i < TRAIN_WARPS * 32; i += TRAIN_THREADS) (&s_red[0][0][0])[i] = 0.0;
     if (tid == 0) s_abort = 0;
+    if (BWD) asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    if (BWD) asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tm = BWD ? s_tmem + ((uint32_t)(warp & 3) << 21) + (uint32_t)(warp >> 2) * 128u : 0u;      // the warp's lanes and its 128 columns
     // rows of the CTA's images, a warp per row; chunk i of a row: pixel i / G, group i % G = lane % G
     const int all_rows = n_img * H, row_chunks = W * G;
     for (int r = warp; r < all_rows; r += TRAIN_WARPS) {
@@ -186,6 +207,7 @@ __global__ void __launch_bounds__(TRAIN_THREADS, 1) train_chain_kernel(const Tra
                     }
                 }
                 uint64_t s0 = 0, s1 = 0, q0 = 0, q1 = 0;
+                uint32_t ex[BWD ? 4 * R : 1];                     // the BN's input once more for the elementwise pass: to tensor memory
                 ulonglong2 nm, is, ga, be;
                 if (BWD) {
                     nm = *reinterpret_cast<const ulonglong2*>(&s_bn[0][c0]); is = *reinterpret_cast<const ulonglong2*>(&s_bn[1][c0]);
@@ -210,6 +232,7 @@ __global__ void __launch_bounds__(TRAIN_THREADS, 1) train_chain_kernel(const Tra
                             const uint64_t r0 = of_bf2(w.x), r1 = of_bf2(w.y);
                             s0 = add2(s0, r0); s1 = add2(s1, r1); q0 = fma2(r0, r0, q0); q1 = fma2(r1, r1, q1);
                         } else {
+                            ex[(h * R + o) * 2] = e.x; ex[(h * R + o) * 2 + 1] = e.y;
                             const uint64_t h0 = mul2(add2(of_bf2(e.x), nm.x), is.x), h1 = mul2(add2(of_bf2(e.y), nm.y), is.y);
                             float z0, z1, z2, z3; un2(fma2(h0, ga.x, be.x), z0, z1); un2(fma2(h1, ga.y, be.y), z2, z3);
                             const uint64_t d0 = v2(z0 > 0.f ? bf_lo(w.x) : 0.f, z1 > 0.f ? bf_hi(w.x) : 0.f), d1 = v2(z2 > 0.f ? bf_lo(w.y) : 0.f, z3 > 0.f ? bf_hi(w.y) : 0.f);
@@ -217,6 +240,7 @@ __global__ void __launch_bounds__(TRAIN_THREADS, 1) train_chain_kernel(const Tra
                         }
                     }
                 }
+                if (BWD) tm_st16(tm + (uint32_t)rd * 16u, ex);
                 // the eight lanes of the same channels: each step halves what a lane keeps; lane g8 ends with one of the eight sums
                 {
                     const bool q = lane & 16, hi = lane & 8, odd = lane & 4;
@@ -273,7 +297,7 @@ __global__ void __launch_bounds__(TRAIN_THREADS, 1) train_chain_kernel(const Tra
             s_sum[tid] = a;
             if (!ok) { s_abort = 1; *(volatile int*)pr.status = 21; __threadfence_system(); }
             __syncthreads();
-            if (s_abort) { asm volatile("cp.async.wait_group 0;" ::: "memory"); return; }      // the same for all: written before the barrier only
+            if (s_abort) { asm volatile("cp.async.wait_group 0;" ::: "memory"); break; }       // the same for all: written before the barrier only
             for (int i = tid; i < TRAIN_WARPS * 32; i += TRAIN_THREADS) (&s_red[0][0][0])[i] = 0.0;
             if (tid < 8 * C) {                                    // eight lanes per channel: four parts of either sum
                 const int kind = (tid >> 2) & 1, part = tid & 3;
@@ -300,60 +324,92 @@ __global__ void __launch_bounds__(TRAIN_THREADS, 1) train_chain_kernel(const Tra
             }
             __syncthreads();
         }
-        // ---- elementwise pass in place: 8 channels per access, two pixels at a time; a lane keeps its group's constants in registers
-        {
-            const int g = lane % G;
-            const uint64_t* const cst = reinterpret_cast<const uint64_t*>(&s_bn[0][g * 8]);
-            uint64_t nm[4], sc[4], be[4], is[BWD ? 4 : 1], ga[BWD ? 4 : 1], nsb[BWD ? 4 : 1], nsg[BWD ? 4 : 1];
+        if constexpr (BWD) {
+            // ---- elementwise pass in place, by the tasks' own positions: da from the maps, the BN's input from tensor memory, only the skip path's gradient from L2.  (A
+            // pass by rows that read the BN's input from L2 again took 16800 clocks of a layer's 39000 at five images of 32 x 32 x 16 per CTA.)
+            ulonglong2 nm = *reinterpret_cast<const ulonglong2*>(&s_bn[0][c0]), is = *reinterpret_cast<const ulonglong2*>(&s_bn[1][c0]);
+            ulonglong2 ga = *reinterpret_cast<const ulonglong2*>(&s_bn[2][c0]), be = *reinterpret_cast<const ulonglong2*>(&s_bn[3][c0]);
+            ulonglong2 sb = *reinterpret_cast<const ulonglong2*>(&s_bn[4][c0]), sg = *reinterpret_cast<const ulonglong2*>(&s_bn[5][c0]);
+            sb.x ^= 0x8000000080000000ull; sb.y ^= 0x8000000080000000ull; sg.x ^= 0x8000000080000000ull; sg.y ^= 0x8000000080000000ull;      // negated
+            const uint64_t gi0 = mul2(ga.x, is.x), gi1 = mul2(ga.y, is.y);
+            const __nv_bfloat16* const skip = L.res;
+            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+            for (int rd = 0; rd < rounds; ++rd) {
+                const int im = (rd * spr + wslot) * slot_imgs;
+                if (!on || im >= n_img) continue;
+                const bool have1 = im + di < n_img;
+                const long long base = ((long long)(img0 + im) * HW + y0 * W + x0 + g8) * C + c0;
+                const int half_e = (di * HW + dx + dy * W) * C;
+                const int r0 = vr0, r1 = have1 ? vr1 : 0;
+                uint32_t ex[4 * R]; uint2 sk[2 * R];
+                tm_ld16(tm + (uint32_t)rd * 16u, ex);
+                if (skip) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                nm[k] = cst[k];
-                if (!BWD) { sc[k] = cst[C / 2 + k]; be[k] = cst[C + k]; }
-                else {
-                    is[k] = cst[C / 2 + k]; ga[k] = cst[C + k]; be[k] = cst[3 * C / 2 + k]; sc[k] = mul2(ga[k], is[k]);
-                    nsb[k] = cst[2 * C + k] ^ 0x8000000080000000ull; nsg[k] = cst[5 * C / 2 + k] ^ 0x8000000080000000ull;
+                    for (int o = 0; o < R; ++o) {
+                        sk[o] = sk[R + o] = make_uint2(0u, 0u);
+                        if (o < r0) sk[o] = __ldcg(reinterpret_cast<const uint2*>(skip + base + o * W * C));
+                        if (o < r1) sk[R + o] = __ldcg(reinterpret_cast<const uint2*>(skip + base + half_e + o * W * C));
+                    }
+                }
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                uint8_t* const d = sm + im * img_bytes + (ng * 2 + (t4 >> 1)) * plane + ((y0 + 1) * Wp + x0 + 1 + g8) * 16 + (t4 & 1) * 8;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    uint8_t* dh = d + (h ? half : 0u); __nv_bfloat16* oh = L.a + base + (h ? half_e : 0);
+                    const int rows = h ? r1 : r0;
+#pragma unroll
+                    for (int o = 0; o < R; ++o, dh += row_bytes, oh += W * C) {
+                        if (o >= rows) break;
+                        const uint2 v = *reinterpret_cast<const uint2*>(dh);
+                        const uint32_t ea = ex[(h * R + o) * 2], eb = ex[(h * R + o) * 2 + 1];
+                        const uint64_t h0 = mul2(add2(of_bf2(ea), nm.x), is.x), h1 = mul2(add2(of_bf2(eb), nm.y), is.y);
+                        float z0, z1, z2, z3; un2(fma2(h0, ga.x, be.x), z0, z1); un2(fma2(h1, ga.y, be.y), z2, z3);
+                        const uint64_t d0 = v2(z0 > 0.f ? bf_lo(v.x) : 0.f, z1 > 0.f ? bf_hi(v.x) : 0.f), d1 = v2(z2 > 0.f ? bf_lo(v.y) : 0.f, z3 > 0.f ? bf_hi(v.y) : 0.f);
+                        uint64_t t0 = mul2(gi0, fma2(h0, sg.x, add2(d0, sb.x))), t1 = mul2(gi1, fma2(h1, sg.y, add2(d1, sb.y)));
+                        if (skip) { t0 = add2(t0, of_bf2(sk[h * R + o].x)); t1 = add2(t1, of_bf2(sk[h * R + o].y)); }
+                        const uint2 w = make_uint2(to_bf2(t0), to_bf2(t1));
+                        *reinterpret_cast<uint2*>(dh) = w; *reinterpret_cast<uint2*>(oh) = w;
+                    }
                 }
             }
+        } else {
+            // ---- elementwise pass in place: 8 channels per access, two pixels at a time; a lane keeps its group's constants in registers
+            const int g = lane % G;
+            const uint64_t* const cst = reinterpret_cast<const uint64_t*>(&s_bn[0][g * 8]);
+            uint64_t nm[4], sc[4], be[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) { nm[k] = cst[k]; sc[k] = cst[C / 2 + k]; be[k] = cst[C + k]; }
             for (int r = warp; r < all_rows; r += TRAIN_WARPS) {
                 const int im = r / H, yy = r - im * H;
-                const long long at = ((long long)(img0 + im) * HW + yy * W) * C;
                 uint8_t* const d = sm + im * img_bytes + g * plane + ((yy + 1) * Wp + 1) * 16;
-                uint4* const out = reinterpret_cast<uint4*>(L.a + at);
-                const uint4* const xv = BWD ? reinterpret_cast<const uint4*>(L.x + at) : nullptr;
-                const uint4* const av = BWD && L.res ? reinterpret_cast<const uint4*>(L.res + at) : nullptr;
+                uint4* const out = reinterpret_cast<uint4*>(L.a + ((long long)(img0 + im) * HW + yy * W) * C);
                 for (int i0 = lane; i0 < row_chunks; i0 += 64) {
-                    uint32_t v[2][4], x[2][4], e[2][4]; uint8_t* sp[2];
+                    uint4 v[2]; uint8_t* sp[2];
 #pragma unroll
                     for (int u = 0; u < 2; ++u) {
                         const int i = i0 + 32 * u < row_chunks ? i0 + 32 * u : i0;
-                        if (BWD) {
-                            const uint4 t = __ldcg(xv + i); x[u][0] = t.x; x[u][1] = t.y; x[u][2] = t.z; x[u][3] = t.w;
-                            if (av) { const uint4 w = __ldcg(av + i); e[u][0] = w.x; e[u][1] = w.y; e[u][2] = w.z; e[u][3] = w.w; }
-                        }
-                        sp[u] = d + (i / G) * 16;
-                        const uint4 t = *reinterpret_cast<const uint4*>(sp[u]); v[u][0] = t.x; v[u][1] = t.y; v[u][2] = t.z; v[u][3] = t.w;
+                        sp[u] = d + (i / G) * 16; v[u] = *reinterpret_cast<const uint4*>(sp[u]);
                     }
 #pragma unroll
                     for (int u = 0; u < 2; ++u) {
-                        uint32_t o[4];
+                        const uint32_t vw[4] = {v[u].x, v[u].y, v[u].z, v[u].w}; uint32_t o[4];
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            if (!BWD) o[k] = relu_bf2(to_bf2(fma2(add2(of_bf2(v[u][k]), nm[k]), sc[k], be[k])));
-                            else {
-                                const uint64_t xh = mul2(add2(of_bf2(x[u][k]), nm[k]), is[k]);
-                                float z0, z1; un2(fma2(xh, ga[k], be[k]), z0, z1);
-                                const uint64_t dz = v2(z0 > 0.f ? bf_lo(v[u][k]) : 0.f, z1 > 0.f ? bf_hi(v[u][k]) : 0.f);
-                                uint64_t t = mul2(sc[k], fma2(xh, nsg[k], add2(dz, nsb[k])));
-                                if (av) t = add2(t, of_bf2(e[u][k]));
-                                o[k] = to_bf2(t);
-                            }
-                        }
+                        for (int k = 0; k < 4; ++k) o[k] = relu_bf2(to_bf2(fma2(add2(of_bf2(vw[k]), nm[k]), sc[k], be[k])));
                         if (i0 + 32 * u >= row_chunks) break;
                         const uint4 w = make_uint4(o[0], o[1], o[2], o[3]);
                         *reinterpret_cast<uint4*>(sp[u]) = w; out[i0 + 32 * u] = w;
                     }
                 }
             }
+        }
+    }
+    if (BWD) {
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncthreads();
+        if (warp == 0) {
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(s_tmem) : "memory");
         }
     }
 }
