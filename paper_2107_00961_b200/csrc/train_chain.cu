@@ -12,7 +12,7 @@
 //
 // The exchange: a CTA's sums go to every other CTA of its sub-ResNet as 16-byte packets of a double's halves, each beside the number of the layer, and are
 // polled for where they are added; the packets are data and barrier in one, and no fence has to wait for the tensors being written meanwhile.  (A
-// counter with release and acquire, then the sums: 10.5 us per layer where a worker has an image per CTA, 8.2 now.)  Two buffers by parity: a
+// counter with release and acquire, then the sums: 10.5 us per layer where a worker has an image per CTA, 8 now; with unused loads all asking for the last packet 3 % more.)  Two buffers by parity: a
 // CTA that writes layer l + 2 has read everyone's l + 1, who had all read l.
 //
 // In place: the warps compute a round of tasks (at most one each), keep the rounded results in 16 registers, and store them over the round's input once
@@ -20,7 +20,7 @@
 // input waits in tensor memory: sixteen columns of the warp's 128 per round, hence eight rounds at most.  The residual (forward) or the BN's input (backward) of a task comes by cp.async into the warp's own 2 KB while it
 // computes.  Layout of an image and the convolution on it: chain_core.h.
 //
-// Measured, us per step: ResNet-110, 4 x 128 images of 32 x 32 (a launch per layer and direction before) 3290 -> 1838; one worker's 84 images 1160 -> 778; 256
+// Measured, us per step: ResNet-110, 4 x 128 images of 32 x 32 (a launch per layer and direction before) 3290 -> 1826; one worker's 84 images 1160 -> 760; 256
 // images and all 54 blocks in one network 6700 -> 3301.
 #include <algorithm>
 #include <vector>
@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(TRAIN_THREADS, 1) train_chain_kernel(const Tra
                 for (uint32_t i = 0;; ++i) {
                     bool all = true;
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) v[u] = ld_poll(box + (long long)min(k + u * Q, ctas - 1) * 2 * C + c2);      // past the end: the last one again, not added
+                    for (int u = 0; u < 4; ++u) v[u] = ld_poll(box + (long long)(k + u * Q < ctas ? k + u * Q : k) * 2 * C + c2);      // past the end: the thread's first again, not added
 #pragma unroll
                     for (int u = 0; u < 4; ++u) all &= v[u].y == number && v[u].w == number;
                     if (all) break;
@@ -439,8 +439,8 @@ int train_chain_max_imgs(int C, const ChainMap& m) {
     const int n = std::min((int)((train_room(C) - train_fixed(C)) / ((size_t)(C / 8) * m.plane)), TRAIN_MAX_ROUNDS * spr * m.slot);
     return n / m.slot * m.slot;
 }
-// Deals the SMs to the problems of a launch: images per CTA so that all CTAs fit, with the least time of the slowest problem, a layer taken as a fixed part (barrier, sums)
-// of about four images' worth and its rounds.
+// Deals the SMs to the problems of a launch: images per CTA so that all CTAs fit, with the least time of the slowest problem.  A layer is taken as its rounds and a fixed part
+// (exchange, sums): about 5500 clocks, where a round of tasks takes about 4800 at 16 channels and grows with them.
 bool train_chain_assign(TrainChain* p, int n, int sms) {
     auto rounds = [](const TrainChain& t, int imgs) { const int tps = t.C / 16 * t.map.strips * t.map.xblocks, spr = TRAIN_WARPS / tps; return ((imgs + t.map.slot - 1) / t.map.slot + spr - 1) / spr; };
     const int cap = train_chain_max_imgs(p[0].C, p[0].map);
@@ -453,7 +453,7 @@ bool train_chain_assign(TrainChain* p, int n, int sms) {
         int who = -1; double least = 0;                           // the problem whose time stays lowest with another slot per CTA
         for (int i = 0; i < n; ++i) {
             if (k[i] + p[i].map.slot > cap) continue;
-            const double t = p[i].nlayers * (4.0 + rounds(p[i], k[i] + p[i].map.slot) * 1.0);
+            const double t = p[i].nlayers * (18.0 / p[i].C + rounds(p[i], k[i] + p[i].map.slot));
             if (who < 0 || t < least) { who = i; least = t; }
         }
         if (who < 0) return false;
