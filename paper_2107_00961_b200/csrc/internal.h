@@ -70,7 +70,7 @@ inline void bn_chunking(BnProb& p, bool bf16, int target_chunks = 0) {
     if (p.vec && target_chunks > 0 && (m + rpc - 1) / rpc < target_chunks) {      // more, smaller chunks (whole sweeps of the CTA's rows)
         const int R = 256 / G;
         rpc = ((m + target_chunks - 1) / target_chunks + R - 1) / R * R;
-        if (rpc < 32 * R) rpc = 32 * R;            // every CTA of the cooperative kernels re-adds all chunks' sums: few chunks for small problems
+        if (rpc < 32 * R) rpc = 32 * R;            // few chunks for small problems: their sums are added up once more
     }
     p.rows_per_chunk = (int)rpc; p.chunks = (int)((m + rpc - 1) / rpc);
 }
@@ -211,8 +211,6 @@ void launch_conv_small(const ConvProb* d, int nprob, int max_ctas, int mode, int
 bool bn_small_ok(const BnProb& p, bool backward);
 void launch_bn_small(const BnProb* d, int nprob, int max_c, int backward, bool bf16, cudaStream_t s);
 
-// statistics, finalisation and apply of BN+ReLU in one cooperative launch (bf16 vector path, training mode); false if the grid cannot be co-resident
-bool launch_bn_fused(const BnProb* d, int nprob, int max_chunks, int backward, cudaStream_t s);   // kernels_ref.cu
 void launch_im2col(const ColProb* d, int nprob, const ColProb& shape, cudaStream_t s);      // shape: the largest problem's
 void launch_repack_rows(const ConvProb* d, int nprob, int max_elems, cudaStream_t s);     // kernels_ref.cu
 void launch_zero_stuff(const UpProb* d, int nprob, long long max_vecs, cudaStream_t s);   // conv_tc.cu

@@ -3,10 +3,8 @@
 // tensor-core kernels do not take (3-channel stems, odd shapes) and the small head/loss kernels.
 // All reductions have a fixed order: results are reproducible run to run.
 #include <algorithm>
-#include <cooperative_groups.h>
 #include "internal.h"
 
-namespace cg = cooperative_groups;
 namespace resist {
 
 template <class T> __device__ __forceinline__ float ldf(const void* p, long long i);
@@ -479,81 +477,6 @@ template <class T, bool VEC>
 __global__ void __launch_bounds__(256, 2) bn_bwd_apply_kernel(const BnProb* __restrict__ probs) {
     const BnProb& p = probs[blockIdx.y];
     if constexpr (VEC) bn_stream_vec<1>(p, p.stat); else if (bn_by_four<T>(p)) bn_stream_lanes<T, 1, 4>(p); else bn_stream_lanes<T, 1, 1>(p);
-}
-
-// ------------------------------------------------------------------------------------------------ fused BN+ReLU (cooperative)
-// One launch per BN layer and direction: partial sums per chunk, a grid-wide barrier, then EVERY CTA adds the
-// partials of its problem in the same fixed order (so all CTAs hold identical statistics without a second barrier;
-// CTA 0 of the problem also stores them) and takes its share of the elementwise pass, whose re-read of x comes
-// from L2.  bf16 vector path, training mode only.
-template <int MODE>
-__global__ void __launch_bounds__(256, 2) bn_fused_kernel(const BnProb* __restrict__ probs) {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // a convolution launched behind this kernel may start its prologue
-    const BnProb& p = probs[blockIdx.y];
-    __shared__ __align__(16) float s_stat[4 * 512];               // callers keep C <= 512
-    if ((int)blockIdx.x < p.chunks) bn_reduce_vec<MODE>(p);
-    __threadfence();
-    cg::this_grid().sync();
-    // every CTA adds the partial sums of all chunks in the same fixed order: thread (c, q) adds chunks q, q+Q, ...
-    // (independent loads), then thread c adds the Q sums in order
-    const int C = p.C;
-    __shared__ double s_red[2][256];
-    for (int cb = 0; cb < C; cb += 256) {
-        const int nl = C - cb < 256 ? C - cb : 256, Q = 256 / nl;
-        const int c = cb + (int)threadIdx.x % nl, q = (int)threadIdx.x / nl;
-        double a0 = 0.0, a1 = 0.0;
-        if (q < Q) {
-#pragma unroll 4
-            for (int k = q; k < p.chunks; k += Q) { a0 += __ldcg(p.partial + ((long long)k * 2 + 0) * C + c); a1 += __ldcg(p.partial + ((long long)k * 2 + 1) * C + c); }
-        }
-        __syncthreads();
-        s_red[0][threadIdx.x] = a0; s_red[1][threadIdx.x] = a1;
-        __syncthreads();
-        if (q != 0) continue;
-        a0 = 0.0; a1 = 0.0;
-        for (int k = 0; k < Q; ++k) { a0 += s_red[0][k * nl + (c - cb)]; a1 += s_red[1][k * nl + (c - cb)]; }
-        if (MODE == 0) {
-            const double m = (double)p.m, dm = a0 / m;             // sums are of x - x[0,c]
-            double var = a1 / m - dm * dm; if (var < 0.0) var = 0.0;
-            const double mean = dm + (double)__bfloat162float(((const __nv_bfloat16*)p.x)[c]);
-            const float fm = (float)mean, fi = (float)(1.0 / sqrt(var + (double)p.eps));
-            s_stat[c] = fm; s_stat[C + c] = fi;
-            if (blockIdx.x == 0) {
-                p.stat[c] = fm; p.stat[C + c] = fi;
-                if (p.run_mean) {
-                    const double unb = p.m > 1 ? var * m / (m - 1.0) : var, mo = (double)p.momentum;
-                    p.run_mean[c] = (float)((1.0 - mo) * (double)p.run_mean[c] + mo * mean);
-                    p.run_var[c] = (float)((1.0 - mo) * (double)p.run_var[c] + mo * unb);
-                }
-            }
-        } else {
-            s_stat[c] = p.stat[c]; s_stat[C + c] = p.stat[C + c];
-            s_stat[2 * C + c] = (float)a0; s_stat[3 * C + c] = (float)a1;
-            if (blockIdx.x == 0) { p.stat[2 * C + c] = (float)a0; p.stat[3 * C + c] = (float)a1; p.dbeta[c] = (float)a0; p.dgamma[c] = (float)a1; }
-        }
-    }
-    __syncthreads();
-    bn_stream_vec<MODE>(p, s_stat);
-}
-
-// CTAs of the cooperative kernel that can be resident together on this device (its largest grid)
-int bn_fused_capacity(int backward) {
-    static int cap[2] = {0, 0};
-    if (!cap[backward]) {
-        int dev = 0, sms = 0, per = 0; cudaGetDevice(&dev); cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (backward) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, bn_fused_kernel<1>, 256, 0);
-        else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, bn_fused_kernel<0>, 256, 0);
-        cap[backward] = per * sms > 0 ? per * sms : -1;
-    }
-    return cap[backward];
-}
-bool launch_bn_fused(const BnProb* d, int nprob, int max_chunks, int backward, cudaStream_t s) {
-    if ((long long)max_chunks * nprob > bn_fused_capacity(backward)) return false;
-    void* args[] = {(void*)&d};
-    const dim3 grid(max_chunks, nprob), block(256);
-    const cudaError_t e = backward ? cudaLaunchCooperativeKernel((void*)bn_fused_kernel<1>, grid, block, args, 0, s)
-                                   : cudaLaunchCooperativeKernel((void*)bn_fused_kernel<0>, grid, block, args, 0, s);
-    return e == cudaSuccess;
 }
 
 static int ew_grid(long long n) { long long g = (n + 255) / 256; if (g > 148 * 16) g = 148 * 16; if (g < 1) g = 1; return (int)g; }

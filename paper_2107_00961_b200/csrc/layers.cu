@@ -217,7 +217,7 @@ bool conv_tc_bwd_sums(const ConvProb& p, int group);
 //   mode 1: da = conv^T(dy, w) + add;      dx = BN+ReLU backward of the BN with input x and output gradient da (+ bn_add), dgamma, dbeta
 // Warp-MMA family (narrow layers): the BN runs inside the convolution's launch.  tcgen05 family: the statistics, or the
 // two sums of the backward where conv_tc_bwd_sums says so, come from the per-tile sums of the convolution's epilogue (a finalize launch, then the
-// elementwise pass); else the BN backward is the cooperative launch, or a reduction and the elementwise pass, behind the dgrad.  *used_backend: 1 tcgen05, 2 warp-level MMA.
+// elementwise pass); else the BN backward is a reduction and the elementwise pass behind the dgrad.  *used_backend: 1 tcgen05, 2 warp-level MMA.
 extern "C" int resist_conv2d_bn_relu(int32_t mode, int32_t backend, const void* act, const void* wgt, const void* add, void* out,
                                      int32_t N, int32_t H, int32_t W, int32_t C, int32_t K, int32_t ksz, int32_t stride, float scale,
                                      const void* x, const float* gamma, const float* beta, float* stat, float* run_mean, float* run_var,
@@ -281,8 +281,7 @@ extern "C" int resist_conv2d_bn_relu(int32_t mode, int32_t backend, const void* 
             if (sums) launch_bn_finalize_tiles((BnProb*)blob, 1, bn.C, mode == CONV_FWD ? 0 : 1, st);
             if (mode == CONV_FWD) launch_bn_apply((BnProb*)blob, 1, bn.m * bn.C, true, true, st);
             else if (sums) launch_bn_bwd_apply((BnProb*)blob, 1, bn.m * bn.C, true, true, st);
-            else if (!(bn.C <= 512 && launch_bn_fused((BnProb*)blob, 1, bn.chunks, 1, st))) {
-                cudaGetLastError();
+            else {
                 launch_bn_bwd_reduce((BnProb*)blob, 1, bn.chunks, bn.C, true, true, st);
                 launch_bn_bwd_apply((BnProb*)blob, 1, bn.m * bn.C, true, true, st);
             }

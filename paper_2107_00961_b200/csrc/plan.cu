@@ -17,7 +17,6 @@ bool conv_tc_supported(const ConvProb& p, int mode);                            
 int conv_tc_fill(const ConvProb& p, int mode, void* host_tc);
 int conv_tc_count(const ConvProb& p, int mode);
 int conv_tc_stat_tiles(const ConvProb& p);
-int bn_fused_capacity(int backward);                                                    // kernels_ref.cu
 void launch_bn_finalize_tiles(const BnProb* d, int nprob, int max_c, int backward, cudaStream_t s);
 int conv_tc_dgrad_tiles(const ConvProb& p);
 bool conv_tc_bn_fits(const ConvProb& p);
@@ -273,8 +272,8 @@ struct Builder {
         }
     }
 
-    // chunks per BN problem that give the fused (cooperative) kernels about two CTAs per SM over all sub-ResNets
-    int fused_chunks() const { return std::max(8, 2 * ctx->sm_count / std::max(1, ctx->S)); }
+    // chunks per BN problem that give the reductions about two CTAs per SM over all sub-ResNets
+    int bn_chunks() const { return std::max(8, 2 * ctx->sm_count / std::max(1, ctx->S)); }
     // forward BN+ReLU: statistics (or running statistics in evaluation) then apply.  x_used: x is read by more than this BN
     float* bn_fwd(long long key, const void* x, void* a, const BNRef& r, long long m, bool x_used) {
         float* stat = (float*)take((size_t)4 * r.c * 4);
@@ -283,7 +282,7 @@ struct Builder {
         p.x = x; p.a = a; p.gamma = W() + r.g; p.beta = W() + r.b; p.dgamma = G() + r.g; p.dbeta = G() + r.b;
         p.run_mean = Bf() + r.buf; p.run_var = Bf() + r.buf + r.c; p.stat = stat; p.m = m; p.C = r.c;
         p.eps = ctx->opts.bn_eps; p.momentum = ctx->opts.bn_momentum; p.eval = eval ? 1 : 0;
-        bn_chunking(p, ctx->opts.dtype == RESIST_BF16, fused_chunks());
+        bn_chunking(p, ctx->opts.dtype == RESIST_BF16, bn_chunks());
         bn_partial_need = std::max(bn_partial_need, (size_t)p.chunks * 2 * r.c * 8);
         p.partial = bn_partial;
         const int producer = last_fwd_conv; last_fwd_conv = -1;
@@ -325,7 +324,6 @@ struct Builder {
             op.key = key + 1; op.kind = OP_BN_APPLY; ops->push_back(op);
             return stat;
         }
-        if (p.vec && !eval && r.c <= 512 && (long long)p.chunks * ctx->S <= bn_fused_capacity(0)) { op.kind = OP_BN_FWD_FUSED; ops->push_back(op); return stat; }   // one cooperative launch
         if (bn_small_ok(p, false)) { op.kind = OP_BN_FWD_SMALL; ops->push_back(op); return stat; }
         ops->push_back(op);
         op.key = key + 1; op.kind = OP_BN_APPLY; ops->push_back(op);
@@ -376,18 +374,15 @@ struct Builder {
         BnProb& p = op.bn;
         p.x = x; p.da = da; p.dx = dx; p.add = add; p.gamma = W() + r.g; p.beta = W() + r.b; p.dgamma = G() + r.g; p.dbeta = G() + r.b;
         p.stat = stat; p.m = m; p.C = r.c; p.eps = ctx->opts.bn_eps; p.momentum = ctx->opts.bn_momentum; p.eval = 0;
-        // (measured on 8 x 67 MB tensors, far beyond L2: reduction + elementwise pass as two streaming launches, each with twelve
-        // 16-byte loads in flight per thread and two CTAs per SM, take 194 + 323 us; the cooperative kernel with three CTAs per SM and one
-        // row in flight took 794 us; both move the same five passes over HBM, so the cooperative form only pays for tensors that
-        // stay in L2 between its two passes)
-        bn_chunking(p, ctx->opts.dtype == RESIST_BF16, fused_chunks());
+        // (A cooperative kernel with both phases around a grid barrier was slower at every size: 27 against 19 us at 5376 x 64, 794 against 586 at 8 x 131072 x 256.)
+        bn_chunking(p, ctx->opts.dtype == RESIST_BF16, bn_chunks());
         bn_partial_need = std::max(bn_partial_need, (size_t)p.chunks * 2 * r.c * 8);
         p.partial = bn_partial;
         const int producer = last_dgrad; last_dgrad = -1;
         const int tc_producer = last_tc_dgrad; last_tc_dgrad = -1;
         if (tc_producer >= 0 && (*ops)[tc_producer].conv.out == da && (*ops)[tc_producer].conv.C == r.c && conv_tc_bwd_sums((*ops)[tc_producer].conv, group)) {
             // the tcgen05 data gradient that produces da reads x beside it and leaves the per-tile sums; one small launch adds them up, then
-            // one elementwise pass.  (The cooperative form of small layers was 27 us of barrier and re-added partial sums whatever its size.)
+            // one elementwise pass. 
             ConvProb& c = (*ops)[tc_producer].conv;
             const int tiles = conv_tc_dgrad_tiles(c);
             bn_partial_need = std::max(bn_partial_need, (size_t)tiles * 2 * r.c * 4);
@@ -398,14 +393,11 @@ struct Builder {
         }
         if (bn_small_ok(p, true)) { op.kind = OP_BN_BWD_SMALL; ops->push_back(op); return; }
         if (fusable(producer, da, p)) { fuse_into(producer, p, 2); return; }
-        // one cooperative launch where all sub-ResNets' chunks can be resident together (the kernel holds 128 registers: one CTA
-        // per SM), else the reduction and the elementwise pass as launches of their own
-        if (p.vec && r.c <= 512 && (long long)p.chunks * ctx->S <= bn_fused_capacity(1)) { op.kind = OP_BN_BWD_FUSED; ops->push_back(op); return; }
         if (p.vec) {
             // the reduction as a launch of its own: about four waves of CTAs over all sub-ResNets (long enough chunks for the batched
             // loads to pipeline, enough of them for the SMs to even out the tail)
             const int R = 256 / (r.c / 8);
-            long long rpc = (m + 4 * fused_chunks() - 1) / (4 * fused_chunks());
+            long long rpc = (m + 4 * bn_chunks() - 1) / (4 * bn_chunks());
             rpc = (rpc + R - 1) / R * R; if (rpc < 32 * R) rpc = 32 * R;
             if (rpc > p.rows_per_chunk) { p.rows_per_chunk = (int)rpc; p.chunks = (int)((m + rpc - 1) / rpc); }
         }
@@ -873,7 +865,7 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& all_ops, bo
                         if (o.kind == OP_CONV_WGRAD) L.bytes += es * (in_e + out_e) + 4.0 * w_e;
                         else L.bytes += es * (in_e + out_e + w_e + (p.add ? (o.kind == OP_CONV_FWD ? out_e : in_e) : 0.0)); }
                     break; }
-                case OP_BN_STATS: case OP_BN_APPLY: case OP_BN_BWD_REDUCE: case OP_BN_BWD_APPLY: case OP_BN_FWD_FUSED: case OP_BN_BWD_FUSED: case OP_BN_TILE_STATS: case OP_BN_EVAL_STATS: case OP_BN_FWD_SMALL: case OP_BN_BWD_SMALL: case OP_BN_BWD_TILE_SUMS: {
+                case OP_BN_STATS: case OP_BN_APPLY: case OP_BN_BWD_REDUCE: case OP_BN_BWD_APPLY: case OP_BN_TILE_STATS: case OP_BN_EVAL_STATS: case OP_BN_FWD_SMALL: case OP_BN_BWD_SMALL: case OP_BN_BWD_TILE_SUMS: {
                     if (k == i) L.first = (int)bn.size();
                     bn.push_back(o.bn);
                     L.gx = std::max(L.gx, o.bn.chunks); L.max_c = std::max(L.max_c, o.bn.C); L.non_vec |= !o.bn.vec;
@@ -884,8 +876,7 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& all_ops, bo
                       else if (o.kind == OP_BN_STATS) L.bytes += es * e;
                       else if (o.kind == OP_BN_APPLY) L.bytes += 2 * es * e;
                       else if (o.kind == OP_BN_BWD_REDUCE) L.bytes += 2 * es * e;
-                      else if (o.kind == OP_BN_FWD_FUSED || o.kind == OP_BN_FWD_SMALL) L.bytes += 2 * es * e;          // x once from HBM (the second read is an L2 hit), a once
-                      else if (o.kind == OP_BN_BWD_FUSED) L.bytes += es * e * (o.bn.add ? 4 : 3);
+                      else if (o.kind == OP_BN_FWD_SMALL) L.bytes += 2 * es * e;          // x once from HBM (the second read is an L2 hit), a once
                       else L.bytes += es * e * (o.bn.add ? 4 : 3); }
                     break; }
                 case OP_IM2COL: {
@@ -935,8 +926,8 @@ static int upload_plan(resist_ctx* ctx, Plan& plan, std::vector<Op>& all_ops, bo
                     case OP_CONV_WGRAD: case OP_CHAIN_WGRAD: case OP_SPLITK: case OP_REPACK: case OP_TRAIN_CHAIN_PACK: break;
                     case OP_TRAIN_CHAIN_FWD: case OP_TRAIN_CHAIN_BWD: for (const TrainLayer& l : o.tlayers) { wr.push_back(l.y); wr.push_back(l.a); } break;
                     case OP_BN_STATS: case OP_BN_BWD_REDUCE: case OP_BN_TILE_STATS: case OP_BN_EVAL_STATS: case OP_BN_BWD_TILE_SUMS: break;
-                    case OP_BN_APPLY: case OP_BN_FWD_FUSED: case OP_BN_FWD_SMALL: wr.push_back(o.bn.a); break;
-                    case OP_BN_BWD_APPLY: case OP_BN_BWD_FUSED: case OP_BN_BWD_SMALL: wr.push_back(o.bn.dx); break;
+                    case OP_BN_APPLY: case OP_BN_FWD_SMALL: wr.push_back(o.bn.a); break;
+                    case OP_BN_BWD_APPLY: case OP_BN_BWD_SMALL: wr.push_back(o.bn.dx); break;
                     default: always = true; break;
                 }
             }
@@ -1134,9 +1125,9 @@ static int enqueue_launches(resist_ctx* ctx, Plan& plan, bool update, bool overl
             case OP_HEAD_BWD: pk = PK_HEAD_BWD; nk = head_small(L.max_c, L.max_classes) ? 1 : 3; break;
             case OP_UPSAMPLE: pk = PK_UPSAMPLE; break;
             case OP_IM2COL: pk = PK_IM2COL; break;
-            case OP_BN_FWD_FUSED: case OP_BN_FWD_SMALL: pk = PK_BN_FWD_FUSED; break;
+            case OP_BN_FWD_SMALL: pk = PK_BN_FWD_FUSED; break;
             case OP_BN_TILE_STATS: case OP_BN_BWD_TILE_SUMS: pk = PK_BN_TILE_STATS; break;
-            case OP_BN_BWD_FUSED: case OP_BN_BWD_SMALL: pk = PK_BN_BWD_FUSED; break;
+            case OP_BN_BWD_SMALL: pk = PK_BN_BWD_FUSED; break;
             case OP_EVAL_CHAIN_PACK: case OP_EVAL_CHAIN: pk = PK_EVAL_CHAIN; break;
             case OP_TRAIN_CHAIN_PACK: case OP_TRAIN_CHAIN_FWD: pk = PK_TRAIN_CHAIN_FWD; break;
             case OP_TRAIN_CHAIN_BWD: pk = PK_TRAIN_CHAIN_BWD; break;
@@ -1184,14 +1175,6 @@ static int enqueue_launches(resist_ctx* ctx, Plan& plan, bool update, bool overl
             case OP_IM2COL: launch_im2col(plan.d_col + L.first, L.count, L.col, st); ++n_launch; break;
             case OP_BN_TILE_STATS: launch_bn_finalize_tiles(plan.d_bn + L.first, L.count, L.max_c, 0, st); ++n_launch; break;
             case OP_BN_BWD_TILE_SUMS: launch_bn_finalize_tiles(plan.d_bn + L.first, L.count, L.max_c, 1, st); ++n_launch; break;
-            case OP_BN_FWD_FUSED:
-                if (launch_bn_fused(plan.d_bn + L.first, L.count, L.gx, 0, st)) ++n_launch;
-                else { launch_bn_stats(plan.d_bn + L.first, L.count, L.gx, L.max_c, bf, !L.non_vec, st); launch_bn_apply(plan.d_bn + L.first, L.count, L.max_elems, bf, !L.non_vec, st); n_launch += 3; }
-                break;
-            case OP_BN_BWD_FUSED:
-                if (launch_bn_fused(plan.d_bn + L.first, L.count, L.gx, 1, st)) ++n_launch;
-                else { launch_bn_bwd_reduce(plan.d_bn + L.first, L.count, L.gx, L.max_c, bf, !L.non_vec, st); launch_bn_bwd_apply(plan.d_bn + L.first, L.count, L.max_elems, bf, !L.non_vec, st); n_launch += 3; }
-                break;
         }
         pf.end(st);
         if (on_side) { cudaEventRecord(ctx->ev_side_done, ctx->side_stream); side_pending = true; }
