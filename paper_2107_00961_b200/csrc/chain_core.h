@@ -40,10 +40,8 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) { uint64_t r; a
 __device__ __forceinline__ uint64_t of_bf2(uint32_t w) { return v2(bf_lo(w), bf_hi(w)); }
 __device__ __forceinline__ uint32_t to_bf2(uint64_t v) { float a, b; un2(v, a, b); return bf_pack(a, b); }
 __device__ __forceinline__ uint32_t relu_bf2(uint32_t w) { uint32_t r; asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(w), "r"(0u)); return r; }   // NaN becomes 0, as in z > 0 ? z : 0
-// relu(bn(x)) of two rounded values: (x - mean) / std * gamma + beta
-__device__ __forceinline__ uint32_t bn_relu2(uint32_t x, uint64_t neg_mean, uint64_t istd, uint64_t gamma, uint64_t beta) {
-    return relu_bf2(to_bf2(fma2(mul2(add2(of_bf2(x), neg_mean), istd), gamma, beta)));
-}
+// relu(bn(x)) of two rounded values: (x - mean) * (gamma / std) + beta
+__device__ __forceinline__ uint32_t bn_relu2(uint32_t x, uint64_t neg_mean, uint64_t scale, uint64_t beta) { return relu_bf2(to_bf2(fma2(add2(of_bf2(x), neg_mean), scale, beta))); }
 
 constexpr int R = 4;                                             // rows of a task's half
 

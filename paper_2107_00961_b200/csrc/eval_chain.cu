@@ -7,15 +7,15 @@
 //
 // What bounds it: mma.sync and the issue slots of the epilogue beside it.  The layout of an image and the convolution on it: chain_core.h.
 //
-// Measured: evaluation of ResNet-110 on 1000 images 3290 -> 1851 us, its 52 identity blocks 1592 us of that (0.27 to 0.34 PFLOP/s); 115 launches -> 15.  One
-// image 656 -> 421 us, 512 images of 36 x 36 with 30 blocks 1387 -> 1237.
+// Measured: evaluation of ResNet-110 on 1000 images 3290 -> 1809 us, its 52 identity blocks 1555 us of that (0.28 to 0.35 PFLOP/s); 115 launches -> 15.  One
+// image 656 -> 421 us, 512 images of 36 x 36 with 30 blocks 1387 -> 1216.
 #include <algorithm>
 #include "chain_core.h"
 
 namespace resist {
 using namespace chain;
 
-static int chain_set(int C) { return 4 * C + 16; }                // floats of a BN's constants: mean | 1/std | gamma | beta, then the scale of the convolution before it
+static int chain_set(int C) { return 3 * C + 16; }                // floats of a BN's constants: -mean | gamma / std | beta, then the scale of the convolution before it
 
 // Filters to bf16 in fragment order [16 output channels][16 input channels][tap][lane]: the lane's four registers of two MMAs' B operands (the
 // columns permuted so that a thread's accumulators are four consecutive channels); constants of the BN.
@@ -36,16 +36,16 @@ __global__ void __launch_bounds__(256) eval_chain_pack_kernel(const ChainLayer* 
         }
     if (blockIdx.x == 0) {
         for (int c = threadIdx.x; c < C; c += 256) {
-            l.cdst[c] = l.gamma ? l.mean[c] : 0.f; l.cdst[C + c] = l.gamma ? (float)(1.0 / sqrt((double)l.var[c] + (double)l.eps)) : 1.f;
-            l.cdst[2 * C + c] = l.gamma ? l.gamma[c] : 1.f; l.cdst[3 * C + c] = l.gamma ? l.beta[c] : 0.f;
+            l.cdst[c] = l.gamma ? -l.mean[c] : 0.f; l.cdst[C + c] = l.gamma ? (float)(1.0 / sqrt((double)l.var[c] + (double)l.eps)) * l.gamma[c] : 1.f;
+            l.cdst[2 * C + c] = l.gamma ? l.beta[c] : 0.f;
         }
-        if (threadIdx.x == 0) l.cdst[4 * C] = l.scale;
+        if (threadIdx.x == 0) l.cdst[3 * C] = l.scale;
     }
 }
 
 template <int C>
 __global__ void __launch_bounds__(512) eval_chain_kernel(const ChainProb* __restrict__ probs) {
-    constexpr int NG = C / 16, SET = 4 * C + 16;
+    constexpr int NG = C / 16, SET = 3 * C + 16;
     extern __shared__ __align__(128) uint8_t sm[];
     const ChainProb p = *probs;
     const int H = p.H, W = p.W, HW = H * W, Wp = W + 1, imgs = p.imgs, img0 = blockIdx.x * imgs;
@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(512) eval_chain_kernel(const ChainProb* __rest
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     const int c = g * 8 + 2 * k;
-                    o[k] = bn_relu2(w[k], v2(-s_c[c], -s_c[c + 1]), v2(s_c[C + c], s_c[C + c + 1]), v2(s_c[2 * C + c], s_c[2 * C + c + 1]), v2(s_c[3 * C + c], s_c[3 * C + c + 1]));
+                    o[k] = bn_relu2(w[k], v2(s_c[c], s_c[c + 1]), v2(s_c[C + c], s_c[C + c + 1]), v2(s_c[2 * C + c], s_c[2 * C + c + 1]));
                 }
                 *reinterpret_cast<uint4*>(s_a + im * img_bytes + g * plane + ((y + 1) * Wp + x + 1) * 16) = make_uint4(o[0], o[1], o[2], o[3]);
             }
@@ -113,11 +113,8 @@ __global__ void __launch_bounds__(512) eval_chain_kernel(const ChainProb* __rest
             });
             // ---- epilogue: thread (g8, t4) holds column g8 of both halves of each row, channels t4 * 4 .. + 3 of the sixteen
             const int c0 = ng * 16 + t4 * 4;
-            const float4 mean = *reinterpret_cast<const float4*>(cs + c0), istd = *reinterpret_cast<const float4*>(cs + C + c0);
-            const float4 ga = *reinterpret_cast<const float4*>(cs + 2 * C + c0), be = *reinterpret_cast<const float4*>(cs + 3 * C + c0);
-            const uint64_t nm0 = v2(-mean.x, -mean.y), nm1 = v2(-mean.z, -mean.w), is0 = v2(istd.x, istd.y), is1 = v2(istd.z, istd.w);
-            const uint64_t ga0 = v2(ga.x, ga.y), ga1 = v2(ga.z, ga.w), be0 = v2(be.x, be.y), be1 = v2(be.z, be.w);
-            const float sc = cs[4 * C]; const uint64_t scale = v2(sc, sc);
+            const ulonglong2 nm = *reinterpret_cast<const ulonglong2*>(cs + c0), gi = *reinterpret_cast<const ulonglong2*>(cs + C + c0), be = *reinterpret_cast<const ulonglong2*>(cs + 2 * C + c0);
+            const float sc = cs[3 * C]; const uint64_t scale = v2(sc, sc);
             const int pix0 = y0 * W + x0 + g8;
             uint8_t* const xs = s_x + ((im * NG + ng) * HW + pix0) * 32 + t4 * 8;
             uint8_t* const dst = s_a + (second ? 0u : buf_bytes) + im * img_bytes + (ng * 2 + (t4 >> 1)) * plane + ((y0 + 1) * Wp + x0 + 1 + g8) * 16 + (t4 & 1) * 8;
@@ -132,7 +129,7 @@ __global__ void __launch_bounds__(512) eval_chain_kernel(const ChainProb* __rest
                     uint2* const xp = reinterpret_cast<uint2*>(xh + o * W * 32);
                     if (second) { const uint2 xv = *xp; v0 = fma2(v0, scale, of_bf2(xv.x)); v1 = fma2(v1, scale, of_bf2(xv.y)); }
                     const uint2 w = make_uint2(to_bf2(v0), to_bf2(v1));
-                    const uint2 a = make_uint2(bn_relu2(w.x, nm0, is0, ga0, be0), bn_relu2(w.y, nm1, is1, ga1, be1));
+                    const uint2 a = make_uint2(bn_relu2(w.x, nm.x, gi.x, be.x), bn_relu2(w.y, nm.y, gi.y, be.y));
                     if (!last) {
                         if (second) *xp = w;
                         *reinterpret_cast<uint2*>(dh + o * row_bytes) = a;
@@ -155,7 +152,7 @@ __global__ void __launch_bounds__(512) eval_chain_kernel(const ChainProb* __rest
 static size_t chain_smem(const ChainProb& p) { return (size_t)2 * p.imgs * (p.C / 8) * p.map.plane + (size_t)p.imgs * p.H * p.W * p.C * 2 + 2 * chain_set(p.C) * 4; }
 // How the blocks are cut: the form of a task, the images of a CTA and its warps with the least work per image, where an SM holds two CTAs of eight warps (up to 113 KB)
 // or one of sixteen; the cost of a launch is the larger of what the fullest SM computes and, for few images, one CTA's chain of layers on its own (a
-// CTA alone on its SM was measured at about 1.3 times its share of a full one).  C = 64 maps are taken only as far as two CTAs fit (larger ones run
+// CTA alone on its SM was measured at about 1.3 times its share of a full one).  C = 64 maps are taken below 16 x 16, as far as two CTAs fit (larger ones run
 // faster on tcgen05, layer by layer).
 bool eval_chain_geometry(ChainProb& p) {
     if (p.C != 16 && p.C != 32 && p.C != 64) return false;
@@ -166,7 +163,7 @@ bool eval_chain_geometry(ChainProb& p) {
         p.map = chain_map(p.H, p.W, mode);
         for (p.imgs = p.map.slot; p.imgs <= 8; p.imgs *= 2) {
             const size_t smem = chain_smem(p);
-            if (smem > (p.C == 64 ? 113u : 226u) * 1024) break;
+            if (smem > (p.C == 64 ? 112u : 226u) * 1024) break;
             p.warps = smem <= 113 * 1024 ? 8 : 16;
             const int per_sm = p.warps == 8 ? 2 : 1, ctas = (p.N + p.imgs - 1) / p.imgs;
             const int rounds = (p.C / 16 * p.map.strips * p.map.xblocks * (p.imgs / p.map.slot) + p.warps - 1) / p.warps;

@@ -394,7 +394,7 @@ __global__ void __launch_bounds__(TRAIN_THREADS, 1) train_chain_kernel(const Tra
                     for (int u = 0; u < 2; ++u) {
                         const uint32_t vw[4] = {v[u].x, v[u].y, v[u].z, v[u].w}; uint32_t o[4];
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) o[k] = relu_bf2(to_bf2(fma2(add2(of_bf2(vw[k]), nm[k]), sc[k], be[k])));
+                        for (int k = 0; k < 4; ++k) o[k] = bn_relu2(vw[k], nm[k], sc[k], be[k]);
                         if (i0 + 32 * u >= row_chunks) break;
                         const uint4 w = make_uint4(o[0], o[1], o[2], o[3]);
                         *reinterpret_cast<uint4*>(sp[u]) = w; out[i0 + 32 * u] = w;
