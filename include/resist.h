@@ -87,7 +87,8 @@ typedef struct {
     int32_t min_depth;       /* >0: top sub-ResNets up to this many partitioned blocks (Sec. 2.6) */
     int32_t momentum_policy; /* RESIST_MOMENTUM_RESTART: zero the momentum at every partition */
     int32_t conv_backend;    /* RESIST_CONV_AUTO: warp-level MMA for narrow layers (<= 64 channels), tcgen05 for wide ones,
-                                CUDA cores for the rest; _CUDA_CORES: never tensor cores; _TCGEN05 / _WARP_MMA: only that
+                                CUDA cores for the rest, and runs of 3x3 layers of 16, 32 or 64 channels (basic blocks) in one launch per
+                                direction with the images in shared memory, as long as all images of the call fit there; _CUDA_CORES: never tensor cores; _TCGEN05 / _WARP_MMA: only that
                                 tensor-core family where the shape allows, CUDA cores elsewhere.  With _AUTO and _WARP_MMA
                                 the BN+ReLU (forward or backward) that consumes a warp-MMA convolution's output runs inside
                                 that convolution's launch; _WARP_MMA_UNFUSED keeps BN in launches of its own */
