@@ -3,12 +3,12 @@
 // With running statistics every image is independent of the others, and a map of 32 x 32 x 16, 16 x 16 x 32 or 8 x 8 x 64 elements fits shared
 // memory three times over (the residual stream x and the inputs a1, a2 of the two convolutions of a block).  So a CTA takes one image (two to
 // eight small ones) and carries it through ALL blocks of the run: nothing between the run's input and the BN+ReLU of its output goes through L2, and a
-// barrier of the CTA stands where a launch per convolution stood.
+// barrier of the CTA stands where a launch per convolution stood.  A run may be led by the second convolution of the block before it (the one that changes resolution).
 //
 // What bounds it: mma.sync and the issue slots of the epilogue beside it.  The layout of an image and the convolution on it: chain_core.h.
 //
-// Measured: evaluation of ResNet-110 on 1000 images 3290 -> 1809 us, its 52 identity blocks 1555 us of that (0.28 to 0.35 PFLOP/s); 115 launches -> 15.  One
-// image 656 -> 421 us, 512 images of 36 x 36 with 30 blocks 1387 -> 1216.
+// Measured: evaluation of ResNet-110 on 1000 images 3290 -> 1778 us, 1561 us of that in the three runs (0.28 to 0.35 PFLOP/s); 115 launches -> 13.  One
+// image 656 -> 421 us, 512 images of 36 x 36 with 30 blocks 1387 -> 1197.
 #include <algorithm>
 #include "chain_core.h"
 
@@ -57,7 +57,8 @@ __global__ void __launch_bounds__(512) eval_chain_kernel(const ChainProb* __rest
 
     // ---- borders (and everything else) to zero, the first BN's constants, then x and a1 = relu(bn(x))
     for (uint32_t i = tid * 16; i < 2 * buf_bytes; i += nthr * 16) *reinterpret_cast<uint4*>(s_a + i) = make_uint4(0u, 0u, 0u, 0u);
-    for (int i = tid; i < 2 * SET; i += nthr) s_c[i] = __ldg(p.cst + i);
+    const int first = p.first;                                    // the constants of BNs `first` (the input's; not used when led) and first + 1, by parity
+    for (int i = tid; i < SET; i += nthr) { s_c[first * SET + i] = __ldg(p.cst + first * SET + i); s_c[(1 - first) * SET + i] = __ldg(p.cst + (first + 1) * SET + i); }
     __syncthreads();
     {
         const int n_img = min(imgs, p.N - img0), chunks = n_img * HW * (C / 8);
@@ -72,13 +73,15 @@ __global__ void __launch_bounds__(512) eval_chain_kernel(const ChainProb* __rest
                 if (i >= chunks) break;
                 const int g = i % (C / 8), q = i / (C / 8), im = q / HW, pix = q - im * HW, y = pix / W, x = pix - y * W;
                 *reinterpret_cast<uint4*>(s_x + ((size_t)(im * NG + (g >> 1)) * HW + pix) * 32 + (g & 1) * 16) = v[u];
+                uint8_t* const to = s_a + im * img_bytes + g * plane + ((y + 1) * Wp + x + 1) * 16;
+                if (first) { *reinterpret_cast<uint4*>(to + buf_bytes) = __ldg(reinterpret_cast<const uint4*>(p.a2 + (long long)img0 * HW * C) + i); continue; }
                 const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w}; uint32_t o[4];
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     const int c = g * 8 + 2 * k;
                     o[k] = bn_relu2(w[k], v2(s_c[c], s_c[c + 1]), v2(s_c[C + c], s_c[C + c + 1]), v2(s_c[2 * C + c], s_c[2 * C + c + 1]));
                 }
-                *reinterpret_cast<uint4*>(s_a + im * img_bytes + g * plane + ((y + 1) * Wp + x + 1) * 16) = make_uint4(o[0], o[1], o[2], o[3]);
+                *reinterpret_cast<uint4*>(to) = make_uint4(o[0], o[1], o[2], o[3]);
             }
         }
     }
@@ -92,10 +95,10 @@ __global__ void __launch_bounds__(512) eval_chain_kernel(const ChainProb* __rest
     uint4 b[3][3];
     if (warp < tasks) {
 #pragma unroll
-        for (int r = 0; r < 3; ++r) load_frag<NG>(b, p.wpk, lane, 0, warp % NG, 0, r);
+        for (int r = 0; r < 3; ++r) load_frag<NG>(b, p.wpk, lane, first, warp % NG, 0, r);
     }
     const int layers = p.layers;
-    for (int l = 0; l < layers; ++l) {
+    for (int l = first; l < layers; ++l) {
         __syncthreads();                                          // this layer's input and constants are in shared memory
         const bool second = l & 1, last = l + 1 == layers;
         const float* const cs = s_c + ((l + 1) & 1) * SET;

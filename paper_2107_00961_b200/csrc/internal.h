@@ -120,7 +120,8 @@ struct ChainMap {
 };
 // Evaluation of a run of identity basic blocks by one launch (eval_chain.cu).
 struct ChainProb {
-    const __nv_bfloat16* x;                            // [N,H,W,C] input of the first block
+    const __nv_bfloat16* x;                            // [N,H,W,C] input of the first block; led (first 1): the skip path of the block whose second convolution leads
+    const __nv_bfloat16* a2; int first;                // led: that convolution's input; the first convolution (0 or 1)
     __nv_bfloat16* x_out; __nv_bfloat16* a_out;        // output of the last block, and relu(bn(.)) of it; either may be nullptr
     const uint4* wpk; const float* cst;                // filters in fragment order, constants of the layers + 1 BNs (eval_chain_pack_kernel)
     int N, H, W, C, layers;                            // layers: convolutions, two per block

@@ -331,13 +331,15 @@ struct Builder {
     }
     // Evaluation of the n identity basic blocks order[0 .. n) on x as one launch; false where the chain kernel does not take them.
     static bool chainable(const resist_block& k) { return k.kind == RESIST_BASIC && !k.has_projection && k.stride == 1; }
-    bool chain(long long key, const int* order, int n, const void* x, int H, int Wd, float inv_S, void** out) {
-        const int C = ctx->blocks[order[0]].cin;
+    // a2: led by the second convolution of order[0], whose input this is (x: its skip path).
+    bool chain(long long key, const int* order, int n, const void* x, const void* a2, bool led, int H, int Wd, float inv_S, void** out) {
+        const int C = ctx->blocks[order[0]].cout;
         ChainProb c{}; c.N = B; c.H = H; c.W = Wd; c.C = C; c.layers = 2 * n;
         if (!eval || ctx->opts.dtype != RESIST_BF16 || ctx->opts.conv_backend != RESIST_CONV_AUTO || !eval_chain_geometry(c)) return false;
         char* const wpk = (char*)take(eval_chain_weight_bytes(C, c.layers)); float* const cst = (float*)take(eval_chain_const_bytes(C, c.layers));
         *out = act((long long)B * H * Wd * C);
-        for (int l = 0; l <= c.layers; ++l) {                 // BN l behind convolution l - 1
+        c.first = led ? 1 : 0; c.a2 = (const __nv_bfloat16*)a2;
+        for (int l = led ? 2 : 0; l <= c.layers; ++l) {       // BN l behind convolution l - 1
             Op op{}; op.key = PACK_KEY; op.sub = sub; op.kind = OP_EVAL_CHAIN_PACK;
             ChainLayer& y = op.layer; y.C = C; y.eps = ctx->opts.bn_eps; y.scale = 1.f;
             y.cdst = cst + (size_t)l * eval_chain_set_floats(C);
@@ -473,7 +475,7 @@ static size_t unroll_subnet(resist_ctx* ctx, Builder& bd, const std::vector<char
         if (bd.eval && Builder::chainable(K)) {
             int n = 1; while (slot + n < order.size() && Builder::chainable(ctx->blocks[order[slot + n]])) ++n;
             void* out = nullptr;
-            if (bd.chain(key, &order[slot], n, cur, cH, cW, inv_S, &out)) { cur = out; slot += n - 1; continue; }
+            if (bd.chain(key, &order[slot], n, cur, nullptr, false, cH, cW, inv_S, &out)) { cur = out; slot += n - 1; continue; }
         }
         // Training: a run of 3x3 layers of one width and resolution as one chain: the identity blocks from slot `first` on, led (head >= 0) by the second convolution of the
         // block before them.  in: input of its first convolution; x, a1, st1 (no head): the first block's input, its BN's output and statistics; res: (head) the skip path
@@ -539,6 +541,19 @@ static size_t unroll_subnet(resist_ctx* ctx, Builder& bd, const std::vector<char
             const int Ho = s.Ho, Wo = s.Wo;
             cur = chain_forward(key + 6, slot + 1, b, s.a2, nullptr, const_cast<void*>(sc), nullptr, K.cout, Ho, Wo, cmap); cH = Ho; cW = Wo; cC = K.cout;
             continue;
+        }
+        if (bd.eval && K.kind == RESIST_BASIC) {              // likewise
+            ChainProb fits{}; fits.N = B; fits.H = s.Ho; fits.W = s.Wo; fits.C = K.cout;
+            if (ctx->opts.dtype == RESIST_BF16 && ctx->opts.conv_backend == RESIST_CONV_AUTO && eval_chain_geometry(fits)) {
+                int n = 1; while (slot + n < order.size() && Builder::chainable(ctx->blocks[order[slot + n]])) ++n;
+                s.y1 = bd.act(m_out * K.cout); s.a2 = bd.act(m_out * K.cout); void* out = nullptr;
+                bd.conv(key + 3, CONV_FWD, s.a1, r.conv[0], nullptr, nullptr, s.y1, B, s.H, s.W, 1.f);
+                bd.bn_fwd(key + 4, s.y1, s.a2, r.bn[1], m_out, false);
+                const int Ho = s.Ho, Wo = s.Wo;
+                bd.chain(key + 6, &order[slot], n, sc, s.a2, true, Ho, Wo, inv_S, &out);
+                cur = out; cH = Ho; cW = Wo; cC = K.cout; slot += n - 1;
+                continue;
+            }
         }
         void* out = bd.act(m_out * K.cout);
         if (K.kind == RESIST_BASIC) {
