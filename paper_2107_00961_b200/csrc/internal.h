@@ -227,6 +227,7 @@ bool launch_eval_chain(const ChainProb* d, const ChainProb& h, cudaStream_t s);
 // ---- launchers (train_chain.cu)
 bool train_chain_geometry(int C, int H, int W, ChainMap& map);
 int train_chain_max_imgs(int C, const ChainMap& map);
+int train_chain_round_imgs(int C, const ChainMap& map);                                       // images a round of a CTA's warps takes
 int train_chain_max_layers();
 bool train_chain_assign(TrainChain* p, int n, int sms);
 size_t train_chain_launch_smem(const TrainChain* p, int n);

@@ -415,7 +415,7 @@ __global__ void __launch_bounds__(TRAIN_THREADS, 1) train_chain_kernel(const Tra
 }
 
 // ------------------------------------------------------------------------------------------------ host side
-// The form of a task with the fewest blocks of positions per image among those of which a round of sixteen warps takes a whole slot.
+// The form of a task with the fewest blocks of positions per image among those of which a round of sixteen warps (1024 positions x 16 channels) takes a whole slot.
 bool train_chain_geometry(int C, int H, int W, ChainMap& best) {
     if ((C != 16 && C != 32 && C != 64) || H < 2 || W < 2 || H > 64 || W > 64) return false;
     double least = 0;
@@ -433,10 +433,10 @@ static size_t train_fixed(int C) { return TRAIN_WARPS * STAGE_BYTES + 18 * C * C
 static size_t train_room(int C) { return 227 * 1024 - 8704 - 48 * C; }
 static size_t train_smem(int C, const ChainMap& m, int imgs) { return (size_t)imgs * (C / 8) * m.plane + train_fixed(C); }
 int train_chain_max_layers() { return TRAIN_MAX_LAYERS; }
+int train_chain_round_imgs(int C, const ChainMap& m) { return TRAIN_WARPS / (C / 16 * m.strips * m.xblocks) * m.slot; }
 // images a CTA can hold
 int train_chain_max_imgs(int C, const ChainMap& m) {
-    const int tps = C / 16 * m.strips * m.xblocks, spr = TRAIN_WARPS / tps;
-    const int n = std::min((int)((train_room(C) - train_fixed(C)) / ((size_t)(C / 8) * m.plane)), TRAIN_MAX_ROUNDS * spr * m.slot);
+    const int n = std::min((int)((train_room(C) - train_fixed(C)) / ((size_t)(C / 8) * m.plane)), TRAIN_MAX_ROUNDS * train_chain_round_imgs(C, m));
     return n / m.slot * m.slot;
 }
 // Deals the SMs to the problems of a launch: images per CTA so that all CTAs fit, with the least time of the slowest problem.  A layer is taken as its rounds and a fixed part
