@@ -71,6 +71,19 @@ def test_convolutions_at_the_edges_of_the_variants(m, case):
     assert max_rel_err(dw.cpu().numpy(), oracle.conv_wgrad(dy, a, k, s)) < F32_TOL
 
 
+# the sums of a weight gradient's splits: four values per thread, one where the result does not begin on 16 bytes.  Same bits.
+@pytest.mark.parametrize("geom", [(20, 32, 32, 64, 64, 1, 1), (20, 32, 32, 64, 64, 3, 1), (23, 32, 31, 72, 136, 1, 1), (20, 31, 33, 72, 136, 3, 2)])
+def test_weight_gradients_at_any_address(m, geom):
+    N, H, W, C, K, k, s = geom
+    a, dy = dev(rnd(1, N, H, W, C)), dev(rnd(4, N, (H - 1) // s + 1, (W - 1) // s + 1, K))
+    want = m.resist_conv2d(2, a, dy, geom, backend=2)[0].reshape(-1)
+    for off in (1, 2):
+        out = torch.zeros(want.numel() + off, device="cuda")
+        assert m.lib().resist_conv2d(2, m.BF16, 2, a.data_ptr(), dy.data_ptr(), 0, out.data_ptr() + 4 * off, *geom, 1.0, 0, torch.cuda.current_stream().cuda_stream) == 0
+        torch.cuda.synchronize()
+        assert torch.equal(out[off:], want)
+
+
 # A running sum of the tensor core loses up to 2^-24 of itself with every step of 16 positions, and with non-negative operands always in one
 # direction: n steps end about n / 2 of 2^-25 low (the sum grows evenly).  128 x 32 x 32 positions of 1024 chunks over 37 CTAs are 28 chunks, 224 steps
 # in one chain (3.3e-6 low at the least) or 112 in each of two; likewise the last tap of a filter row, the single taps of stride 2.
