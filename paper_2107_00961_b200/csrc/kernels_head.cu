@@ -1,6 +1,7 @@
 // The ends of the network: im2col of few-channel stems, the 3x3 stride-2 max-pool, and the head (global average pool, linear
 // layer, mean softmax cross-entropy and their gradients).  fp32 arithmetic on T = float or bf16 storage; every sum has a fixed order.
 #include <algorithm>
+#include <cooperative_groups.h>
 #include "internal.h"
 
 namespace resist {
@@ -248,14 +249,20 @@ __global__ void __launch_bounds__(256) avgpool_kernel(const HeadProb* __restrict
 // The head's three matrix products in fp32 on CUDA cores: tiles of 32 x 64 with a 32-deep slice in shared memory, 4 x 4 results per
 // thread, the next slice's loads in flight while one is used; the reduction runs in ascending order.  (One thread or warp per
 // result, as before, read both operands from L2 for every result: 220 + 650 us for 4 x 64 samples of 2048 channels and 1000 classes.)
+// A slice takes about 1.2 us, most of it the loads' latency, and the logits have few tiles and 64 slices at 2048 channels.  So from 16 slices on a cluster of HEAD_SPLIT
+// CTAs shares a tile of logits: each adds its part of the reduction, then each adds its rows of the eight partial tiles, in the order of the parts, out of the others' shared
+// memory.  Pooling, logits and loss of 8 x 128 samples and 100 classes 118 -> 68 us, of 50 samples and 1000 classes 109 -> 52, of 16 and 100 98 -> 36.
 //   PROD 0: logits[b][k] = pooled[b] . w[k] + bias    1: dw[k][c] = sum_b dlogits[b][k] pooled[b][c], and db    2: dpooled[b][c] = sum_k dlogits[b][k] w[k][c] / HW
-template <int PROD>
+template <int PROD, int SPLIT>
 __global__ void __launch_bounds__(128) head_gemm_kernel(const HeadProb* __restrict__ probs) {
-    const HeadProb& p = probs[blockIdx.z];
+    static_assert(PROD == 0 || SPLIT == 1, "only the logits' reduction is shared");
+    const HeadProb& p = probs[blockIdx.z / SPLIT];
+    const int part = blockIdx.z % SPLIT;
     const int C = p.C, classes = p.classes, B = p.B;
     const int M = PROD == 1 ? classes : B, N = PROD == 0 ? classes : C, K = PROD == 0 ? C : PROD == 1 ? B : classes;
     const int m0 = blockIdx.y * 32, n0 = blockIdx.x * 64;
-    if (m0 >= M || n0 >= N) return;
+    if (m0 >= M || n0 >= N) return;                               // a cluster leaves as a whole
+    const int per = ((K + 31) / 32 + SPLIT - 1) / SPLIT * 32, k_first = part * per, k_end = min(K, k_first + per);
     const float* __restrict__ A = PROD == 0 ? p.pooled : p.dlogits;
     const float* __restrict__ Bm = PROD == 1 ? p.pooled : p.w;
     const int lda = PROD == 0 ? C : classes, ldb = C;
@@ -272,15 +279,15 @@ __global__ void __launch_bounds__(128) head_gemm_kernel(const HeadProb* __restri
             rb[i] = k < K && n < N ? Bm[PROD == 0 ? (long long)n * ldb + k : (long long)k * ldb + n] : 0.f; }
     };
     float acc[4][4] = {}, bias = 0.f;
-    load(0);
-    for (int k0 = 0; k0 < K; k0 += 32) {
+    load(k_first);
+    for (int k0 = k_first; k0 < k_end; k0 += 32) {
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < 8; ++i) { const int e = tid + i * 128; if (PROD == 1) As[e >> 5][e & 31] = ra[i]; else As[e & 31][e >> 5] = ra[i]; }
 #pragma unroll
         for (int i = 0; i < 16; ++i) { const int e = tid + i * 128; if (PROD == 0) Bs[e & 31][e >> 5] = rb[i]; else Bs[e >> 6][e & 63] = rb[i]; }
         __syncthreads();
-        if (k0 + 32 < K) load(k0 + 32);
+        if (k0 + 32 < k_end) load(k0 + 32);
 #pragma unroll 8
         for (int k = 0; k < 32; ++k) {
             const float4 a = *reinterpret_cast<const float4*>(&As[k][tm * 4]), b = *reinterpret_cast<const float4*>(&Bs[k][tn * 4]);
@@ -294,18 +301,49 @@ __global__ void __launch_bounds__(128) head_gemm_kernel(const HeadProb* __restri
             for (int k = 0; k < 32; ++k) bias += As[k][tid];
     }
     if (PROD == 1 && blockIdx.x == 0 && tid < 32 && m0 + tid < M) p.db[m0 + tid] = bias;
+    auto put = [&](int m, int n, float v) {
+        if (m >= M || n >= N) return;
+        const long long o = (long long)m * N + n;
+        if (PROD == 0) { v += p.b[n]; p.logits[o] = v; if (p.logits_user) p.logits_user[o] = v; }
+        else if (PROD == 1) p.dw[o] = v;
+        else p.dpooled[o] = v / (float)p.HW;
+    };
+    if (SPLIT == 1) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int m = m0 + tm * 4 + i; if (m >= M) continue;
+        for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int n = n0 + tn * 4 + j; if (n >= N) continue;
-            const long long o = (long long)m * N + n;
-            if (PROD == 0) { const float v = acc[i][j] + p.b[n]; p.logits[o] = v; if (p.logits_user) p.logits_user[o] = v; }
-            else if (PROD == 1) p.dw[o] = acc[i][j];
-            else p.dpooled[o] = acc[i][j] / (float)p.HW;
-        }
+            for (int j = 0; j < 4; ++j) put(m0 + tm * 4 + i, n0 + tn * 4 + j, acc[i][j]);
+        return;
     }
+    cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+    __syncthreads();
+    float* mine = &Bs[0][0];                                      // [32][64]
+#pragma unroll
+    for (int i = 0; i < 4; ++i) *reinterpret_cast<float4*>(mine + (tm * 4 + i) * 64 + tn * 4) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+    cluster.sync();
+    constexpr int ROWS = 32 / SPLIT;
+    for (int e = tid; e < ROWS * 32; e += 128) {
+        const int m = part * ROWS + (e >> 5), n = (e & 31) * 2;
+        float2 v[SPLIT];
+#pragma unroll
+        for (int r = 0; r < SPLIT; ++r) v[r] = *reinterpret_cast<const float2*>(cluster.map_shared_rank(mine, r) + m * 64 + n);
+        float2 sum = v[0];
+#pragma unroll
+        for (int r = 1; r < SPLIT; ++r) { sum.x += v[r].x; sum.y += v[r].y; }
+        put(m0 + m, n0 + n, sum.x); put(m0 + m, n0 + n + 1, sum.y);
+    }
+    cluster.sync();                                               // no CTA leaves while another reads its tile
+}
+constexpr int HEAD_SPLIT = 8;
+// The rule looks at the channels alone, so that a sub-ResNet's results do not depend on how many others share the launch.  (The input gradient, a reduction over the classes
+// with a tile per 64 channels, has CTAs enough: 119 -> 124 us for the three backward kernels of 4 x 64 samples and 1000 classes with eight CTAs per tile there too.)
+static void launch_head_logits(const HeadProb* d, int nprob, int B, int classes, int C, cudaStream_t s) {
+    const dim3 grid((classes + 63) / 64, (B + 31) / 32, nprob);
+    if (C < 16 * 32) { head_gemm_kernel<0, 1><<<grid, 128, 0, s>>>(d); return; }
+    cudaLaunchConfig_t cfg = {}; cfg.gridDim = dim3(grid.x, grid.y, nprob * HEAD_SPLIT); cfg.blockDim = dim3(128); cfg.stream = s;
+    cudaLaunchAttribute at[1]; at[0].id = cudaLaunchAttributeClusterDimension; at[0].val.clusterDim.x = 1; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = HEAD_SPLIT;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, head_gemm_kernel<0, HEAD_SPLIT>, d);
 }
 // eight samples per CTA, one warp each; the last CTA of a problem adds the samples' losses in order
 __global__ void __launch_bounds__(256) loss_kernel(HeadProb* __restrict__ probs) {
@@ -379,15 +417,15 @@ int launch_head_fwd(const HeadProb* d, int nprob, int maxB, int maxC, int max_cl
     }
     if (bf16) avgpool_kernel<__nv_bfloat16><<<dim3(ew_grid((long long)maxB * ((maxC + 7) / 8)), nprob), 256, 0, s>>>(d);
     else avgpool_kernel<float><<<dim3(ew_grid((long long)maxB * maxC), nprob), 256, 0, s>>>(d);
-    head_gemm_kernel<0><<<dim3((max_classes + 63) / 64, (maxB + 31) / 32, nprob), 128, 0, s>>>(d);
+    launch_head_logits(d, nprob, maxB, max_classes, maxC, s);
     loss_kernel<<<dim3((maxB + 7) / 8, nprob), 256, 0, s>>>(dm);
     return 3;
 }
 int launch_head_bwd(const HeadProb* d, int nprob, int maxB, int maxC, int max_classes, long long max_elems,
                     bool bf16, cudaStream_t s) {
-    head_gemm_kernel<1><<<dim3((maxC + 63) / 64, (max_classes + 31) / 32, nprob), 128, 0, s>>>(d);
+    head_gemm_kernel<1, 1><<<dim3((maxC + 63) / 64, (max_classes + 31) / 32, nprob), 128, 0, s>>>(d);
     if (head_small(maxC, max_classes)) return 1;                  // the forward kernel has made the input gradient
-    head_gemm_kernel<2><<<dim3((maxC + 63) / 64, (maxB + 31) / 32, nprob), 128, 0, s>>>(d);
+    head_gemm_kernel<2, 1><<<dim3((maxC + 63) / 64, (maxB + 31) / 32, nprob), 128, 0, s>>>(d);
     if (bf16) avgpool_bwd_kernel<__nv_bfloat16><<<dim3(ew_grid((max_elems + 7) / 8), nprob), 256, 0, s>>>(d);
     else avgpool_bwd_kernel<float><<<dim3(ew_grid(max_elems), nprob), 256, 0, s>>>(d);
     return 3;

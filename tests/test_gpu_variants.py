@@ -230,6 +230,15 @@ def test_heads_and_pooling_in_a_step(m, arch):
         assert v < tol, (name, v)
 
 
+# logits whose reduction eight CTAs share, from 512 channels on: the first size, the last below it, a ragged last slice with nothing left for the eighth part (1032 = 6 x 160 + 72),
+# fewer parts than slices divide into (960), several tiles
+@pytest.mark.parametrize("width,classes", [(64, 10), (63, 129), (129, 33), (120, 130)])
+def test_logits_with_a_shared_reduction(m, width, classes):
+    out = run_protocol_both(net(4, 4, classes, 8, width, 0, kind=synth.BOTTLENECK), 2, 35, 1, 23, "f32", 0, True, m)
+    for r in out["steps"][0]["subs"]:
+        assert max_rel_err(r["logits_gpu"], r["logits_cpu"]) < 1e-4
+
+
 @pytest.mark.parametrize("dtype,grouped", [("f32", True), ("bf16", True), ("bf16", False)])
 def test_recorded_steps_equal_launched_steps(m, dtype, grouped):
     """Two rounds of four steps, new tensors and a new learning rate each: a plan is launched twice and replayed from its recording from then
